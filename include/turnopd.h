@@ -242,8 +242,9 @@ turnopd_status turnopd_loss_fwd_bwd_static(const void *z_student, const void *z_
 /*
  * turnopd_fused_lmhead_fwd_bwd -- the OPD loss with the two LM heads fused in:
  * student logits z_s = h_s W_s^T and teacher logits z_t = h_t W_t^T of the
- * supervised tokens are formed tile by tile on the tensor cores and consumed
- * by the loss without ever being stored (Eq. opd-rkl, full vocabulary).
+ * supervised tokens are formed tile by tile on the tensor cores and folded into
+ * the loss there; at most one chunk of rows is ever stored, in the workspace
+ * (Eq. opd-rkl, full vocabulary).
  * Outputs l_i, L = sum_i w_i l_i and dL/dh_s = G W_s with G = dL/dz_s (the
  * chain rule through z_s = h_s W_s^T; G is formed in fp32 and rounded to bf16
  * for the second tensor-core product).
@@ -261,7 +262,10 @@ turnopd_status turnopd_loss_fwd_bwd_static(const void *z_student, const void *z_
  * Workspace: turnopd_fused_workspace_bytes(num_tokens, vocab, d_s, d_t) bytes,
  *   queried with the device that will run the call current (gathered hidden
  *   rows, per-row partial statistics, G in bf16 and per-SM partial dH tiles:
- *   about 2 num_tokens vocab bytes + 256 KiB per SM).
+ *   about 2 num_tokens vocab bytes + 256 KiB per SM; then the logits of one
+ *   chunk of at most 2048 supervised rows in fp32, about 8 vocab bytes a row).
+ *   A workspace without room for the last part is accepted too: the backward
+ *   pass then computes the logits a second time, which is slower.
  * Device errors: TURNOPD_ERR_NONFINITE, TURNOPD_ERR_TIMEOUT (bounded waits).
  */
 turnopd_status turnopd_fused_lmhead_fwd_bwd(const void *h_s, const void *W_s, int64_t d_s,

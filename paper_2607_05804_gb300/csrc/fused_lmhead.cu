@@ -1,6 +1,6 @@
 // Fused LM heads + OPD loss (sm_103a): the student and teacher logits of the
-// supervised tokens are produced tile by tile on the tensor cores and consumed
-// in the epilogue, never stored.
+// supervised tokens are produced tile by tile on the tensor cores and folded
+// into the loss statistics in the epilogue; no whole logit matrix is stored.
 //
 //   forward   Z_t = H_t W_t^T (K = d_t), then Z_s = H_s W_s^T (K = d_s), per
 //             256-row x 256-vocab tile, accumulated in tensor memory (512 fp32
@@ -8,9 +8,15 @@
 //             folds each tile into per-row online statistics (max, sum exp,
 //             sum exp (z_s - z_t)) for both models over a group of tiles;
 //   merge     per row: LSE_s, LSE_t, KL = E_p[z_s - z_t] - (LSE_s - LSE_t);
-//   backward  the same tiles are recomputed; the epilogue forms
-//             G = w p_s ((z_s - z_t) - E_p[z_s - z_t]) = dL/dz_s and stores it in
-//             bf16 (the gradient w.r.t. the logits, not the logits);
+//   backward  G = w p_s ((z_s - z_t) - E_p[z_s - z_t]) = dL/dz_s in bf16.  The
+//             rows are taken in chunks of at most kChunkTiles row tiles: the
+//             forward epilogue of a chunk also leaves z_s and z_s - z_t (fp32,
+//             the very values it folded) in a chunk-sized scratch, and k_fused_g
+//             turns them into G.  A workspace without that scratch recomputes
+//             the tiles instead (k_fused_lm<kRecompute>).  Recomputing costs as much
+//             tensor work as the whole forward pass, the scratch 18 bytes of HBM per
+//             logit: 9,826 rows x 151,936, d 4096 / 5120, dH: 43.2 -> 27.1 ms; 308
+//             rows with dW: 3.65 -> 2.65 ms;
 //   dH_s      = G W_s by a second tensor-core GEMM over the vocabulary, W_s read
 //             in place as an MN-major operand.
 //
@@ -67,7 +73,8 @@ constexpr int kColQuarters = kEpiWarps / 4;      // column slices of a tile
 constexpr int kEpiCols = BN / kColQuarters;      // 64 columns per epilogue thread
 constexpr int kThreads = 32 * (2 + kEpiWarps);
 constexpr uint32_t kLimit = 1u << 24;
-constexpr int kTilesPerGroup = 10;  // vocabulary tiles one work unit folds into one partial
+constexpr int kTilesPerGroup = 10;  // vocabulary tiles one work unit folds into one partial, at most
+constexpr int kMinTilesPerGroup = 4;
 constexpr uint32_t kColT = 0, kColS = 256;  // tensor-memory columns of Z_t and Z_s
 constexpr uint16_t kPairMask = 0x3;
 
@@ -77,9 +84,12 @@ struct FusedArgs {
     int d_s, d_t;
     const int4 *rows;      // compacted supervised rows {token, row, y, w bits}
     const int32_t *nvalid;
-    int n_groups;          // vocabulary groups (units per M tile)
-    float *part;           // [n_groups][kColQuarters][cap rows][8] partial statistics
-    int64_t cap;           // row capacity of the gathered buffers (multiple of BMP)
+    int pairs;             // 2-CTA pairs of the launch (pick_group)
+    int chunk, chunk_tiles;  // this launch's row tiles: chunk_range(m_tiles, chunk_tiles, chunk)
+    int min_group;         // least vocabulary tiles per group that `part` has room for
+    float *part;           // [groups][kColQuarters][part_rows][8] partial statistics
+    int64_t part_rows;     // rows of `part`: those of the chunk
+    float4 *z;             // chunk scratch (kForwardStore), see z_index
     const float *rowc;     // [cap][4]: lse_s * log2e - log2 |w|, E_p[z_s - z_t], sign w, -
     __nv_bfloat16 *G;      // [cap][vpad] backward output
     int32_t *status;
@@ -245,10 +255,49 @@ __device__ __forceinline__ void unit_coords(int u, int m_tiles, int n_groups, in
     *mt = b * mb + rest % h;
 }
 
+// Vocabulary tiles per group: the largest of kTilesPerGroup .. min_group that gives the
+// fewest tile steps to the pair with the most work.  A unit is indivisible, so a fixed
+// group of 10 left the last wave of units nearly empty on few row tiles (2 row tiles of
+// V = 151,936 on 76 pairs: 120 units, 20 tile steps for the busiest pair where 15.6
+// would be even; groups of 8 take 16).
+__device__ __forceinline__ int pick_group(int m_tiles, int n_tiles, int pairs, int min_group)
+{
+    int best = kTilesPerGroup, cost = INT32_MAX;
+    for (int gs = kTilesPerGroup; gs >= min_group; --gs) {
+        const int units = m_tiles * ((n_tiles + gs - 1) / gs);
+        const int c = (units + pairs - 1) / pairs * gs;
+        if (c < cost) {
+            cost = c;
+            best = gs;
+        }
+    }
+    return best;
+}
+
+// Row tiles [*lo, *hi) of chunk c: the row tiles in the fewest chunks of at most
+// chunk_tiles, as even as they come (empty past the last).
+__device__ __forceinline__ void chunk_range(int m_tiles, int chunk_tiles, int c, int *lo, int *hi)
+{
+    const int n = (m_tiles + chunk_tiles - 1) / chunk_tiles;
+    const int h = n > 0 ? (m_tiles + n - 1) / n : 0;
+    *lo = min(m_tiles, c * h);
+    *hi = min(m_tiles, *lo + h);
+}
+
+// The chunk scratch holds, for each block of 32 rows and each 4 columns, the 32 rows'
+// z_s (16 bytes a row) and then their z_s - z_t: a warp of the epilogue, one row per
+// lane, stores 512 contiguous bytes at a time, and k_fused_g reads them the same way.
+__device__ __forceinline__ size_t z_index(int64_t vpad, int row_block, int64_t col4)
+{
+    return ((size_t)row_block * (size_t)(vpad / 4) + (size_t)col4) * 64;
+}
+
 // ----------------------------------------------------------------------------
-// Forward statistics (MODE 0) / backward logit gradient (MODE 1).
-// Work unit: one pair M tile x one vocabulary group of kTilesPerGroup
-// 256-wide tiles, folded into one partial per row.
+// Forward statistics (kForward; kForwardStore also leaves the chunk's logits in the
+// scratch) / backward logit gradient by recomputing the tiles (kRecompute).
+// Work unit: one pair M tile x one vocabulary group of pick_group() 256-wide tiles,
+// folded into one partial per row.
+enum { kForward = 0, kRecompute = 1, kForwardStore = 2 };
 template <int MODE>
 __global__ void __launch_bounds__(kThreads, 1)
 k_fused_lm(const __grid_constant__ CUtensorMap tHs, const __grid_constant__ CUtensorMap tWs,
@@ -262,9 +311,15 @@ k_fused_lm(const __grid_constant__ CUtensorMap tHs, const __grid_constant__ CUte
     const uint32_t rank = cluster_ctarank();
     const int pair = (int)cluster_id(), n_pairs = (int)cluster_count();
     const int nvalid = *a.nvalid;
-    const int m_tiles = (nvalid + BMP - 1) / BMP;
     const int n_tiles = (int)((a.vocab + BN - 1) / BN);
-    const int units = m_tiles * a.n_groups;
+    int mt_lo, mt_hi;
+    chunk_range((nvalid + BMP - 1) / BMP, a.chunk_tiles, a.chunk, &mt_lo, &mt_hi);
+    const int m_tiles = mt_hi - mt_lo;
+    if (m_tiles == 0)  // the same for every CTA of the grid
+        return;
+    const int gsize = pick_group(m_tiles, n_tiles, a.pairs, a.min_group);
+    const int n_groups = (n_tiles + gsize - 1) / gsize;
+    const int units = m_tiles * n_groups;
     const int kb_s = a.d_s / BK, kb_t = a.d_t / BK;
     const uint32_t tmem = pair_prologue(sm, &s_dead, 512);
 
@@ -279,9 +334,9 @@ k_fused_lm(const __grid_constant__ CUtensorMap tHs, const __grid_constant__ CUte
         uint32_t it = 0;
         for (int u = pair; u < units; u += n_pairs) {
             int mt, g;
-            unit_coords(u, m_tiles, a.n_groups, &mt, &g);
-            const int t0 = g * kTilesPerGroup, t1 = min(n_tiles, t0 + kTilesPerGroup);
-            const int ya = mt * BMP + (int)rank * BM;
+            unit_coords(u, m_tiles, n_groups, &mt, &g);
+            const int t0 = g * gsize, t1 = min(n_tiles, t0 + gsize);
+            const int ya = (mt_lo + mt) * BMP + (int)rank * BM;
             const int n_pos = (t1 - t0) * kb_tile;   // (tile, k-block) positions of this unit
             // L2 prefetch of this CTA's B rows at unit position p
             auto prefetch_b = [&](int p) {
@@ -337,8 +392,8 @@ k_fused_lm(const __grid_constant__ CUtensorMap tHs, const __grid_constant__ CUte
         };
         for (int u = pair; u < units; u += n_pairs) {
             int mt, g;
-            unit_coords(u, m_tiles, a.n_groups, &mt, &g);
-            const int t0 = g * kTilesPerGroup, t1 = min(n_tiles, t0 + kTilesPerGroup);
+            unit_coords(u, m_tiles, n_groups, &mt, &g);
+            const int t0 = g * gsize, t1 = min(n_tiles, t0 + gsize);
             for (int nt = t0; nt < t1; ++nt, ++tile) {
                 if (tile > 0)  // both epilogues hold Z_t of the previous tile in registers
                     wait_lim(sm.free_t, (tile - 1) & 1, a.status, &s_dead, true);
@@ -364,13 +419,14 @@ k_fused_lm(const __grid_constant__ CUtensorMap tHs, const __grid_constant__ CUte
         uint32_t tile = 0;
         for (int u = pair; u < units; u += n_pairs) {
             int mt, g;
-            unit_coords(u, m_tiles, a.n_groups, &mt, &g);
-            const int t0 = g * kTilesPerGroup, t1 = min(n_tiles, t0 + kTilesPerGroup);
-            const int row = mt * BMP + (int)rank * BM + q * 32 + lane;
+            unit_coords(u, m_tiles, n_groups, &mt, &g);
+            const int t0 = g * gsize, t1 = min(n_tiles, t0 + gsize);
+            const int lrow = mt * BMP + (int)rank * BM + q * 32 + lane;  // within the chunk
+            const int row = mt_lo * BMP + lrow;
             const bool valid_row = row < nvalid;
             float ms = -INFINITY, ss = 0.f, sa = 0.f, mt_ = -INFINITY, st = 0.f;
             float nl = 0.f, cp = 0.f, sg = 1.f;
-            if (MODE == 1 && valid_row) {
+            if (MODE == kRecompute && valid_row) {
                 const float4 c = reinterpret_cast<const float4 *>(a.rowc)[row];
                 nl = c.x, cp = c.y, sg = c.z;
             }
@@ -386,7 +442,7 @@ k_fused_lm(const __grid_constant__ CUtensorMap tHs, const __grid_constant__ CUte
                 tmem_ld32(tmem + lane_off + kColT + col0 + 32, *reinterpret_cast<float(*)[32]>(&zt[32]));
                 tmem_ld_wait();
                 release_cols(free_t0, lane);
-                if (MODE == 0 && nv > 0) {
+                if (MODE != kRecompute && nv > 0) {
                     float cmt = -INFINITY;
 #pragma unroll
                     for (int j = 0; j < kEpiCols; ++j)
@@ -405,7 +461,7 @@ k_fused_lm(const __grid_constant__ CUtensorMap tHs, const __grid_constant__ CUte
                 // G columns [vbase, vbase + 64) lie wholly inside or outside [0, vpad)
                 // (both multiples of 64); the staging buffer is free once the previous
                 // tile's store has read it
-                const bool in_g = MODE == 1 && vbase < a.vpad;
+                const bool in_g = MODE == kRecompute && vbase < a.vpad;
                 if (in_g) {
                     if (lane == 0)
                         bulk_wait_read0();
@@ -420,7 +476,16 @@ k_fused_lm(const __grid_constant__ CUtensorMap tHs, const __grid_constant__ CUte
                     tmem_ld16(tmem + lane_off + kColS + col0 + ch * 16, zs);
                     tmem_ld_wait();
                     const int c0 = ch * 16;
-                    if (MODE == 0) {
+                    if (MODE == kForwardStore && vbase < a.vpad) {
+                        float4 *zq = a.z + z_index(a.vpad, lrow / 32, (vbase + c0) / 4) + lane;
+#pragma unroll
+                        for (int j = 0; j < 16; j += 4) {
+                            __stcs(zq + 16 * j, make_float4(zs[j], zs[j + 1], zs[j + 2], zs[j + 3]));
+                            __stcs(zq + 16 * j + 32, make_float4(zs[j] - zt[c0 + j], zs[j + 1] - zt[c0 + j + 1],
+                                                                  zs[j + 2] - zt[c0 + j + 2], zs[j + 3] - zt[c0 + j + 3]));
+                        }
+                    }
+                    if (MODE != kRecompute) {
                         if (c0 < nv) {
                             float cmx = -INFINITY;
 #pragma unroll
@@ -466,22 +531,22 @@ k_fused_lm(const __grid_constant__ CUtensorMap tHs, const __grid_constant__ CUte
                     }
                 }
                 release_cols(free_s0, lane);
-                if (MODE == 1 && in_g) {
+                if (MODE == kRecompute && in_g) {
                     fence_proxy_async_smem();
                     __syncwarp();
                     if (lane == 0) {
-                        tma_store_2d(&tGst, (int)vbase, mt * BMP + (int)rank * BM + q * 32, stg);
+                        tma_store_2d(&tGst, (int)vbase, (mt_lo + mt) * BMP + (int)rank * BM + q * 32, stg);
                         bulk_commit();
                     }
                 }
             }
-            if (MODE == 0 && valid_row) {
-                float *pp = a.part + (((size_t)g * kColQuarters + cq) * a.cap + row) * 8;
+            if (MODE != kRecompute && valid_row) {
+                float *pp = a.part + (((size_t)g * kColQuarters + cq) * a.part_rows + lrow) * 8;
                 reinterpret_cast<float4 *>(pp)[0] = make_float4(ms, ss, sa, mt_);
                 reinterpret_cast<float4 *>(pp)[1] = make_float4(st, 0.f, 0.f, 0.f);
             }
         }
-        if (MODE == 1 && lane == 0)
+        if (MODE == kRecompute && lane == 0)
             bulk_wait0();
     }
     pair_epilogue(sm, tmem, 512, rank);
@@ -840,37 +905,123 @@ __global__ void k_gather_rows(const int4 *__restrict__ rows, const int32_t *__re
     }
 }
 
-// Per supervised row: merge the vocabulary-group partials into LSE_s, LSE_t,
-// KL; write l, w*l and the backward constants.
-__global__ void k_fused_merge(const int4 *__restrict__ rows, const int32_t *__restrict__ nvalid,
-                              const float *__restrict__ part, int n_groups, int64_t cap,
-                              float *__restrict__ token_loss, double *__restrict__ row_wl,
-                              float *__restrict__ rowc, int32_t *status)
+// Per supervised row of the chunk: merge the vocabulary-group partials into LSE_s,
+// LSE_t, KL; write l, w*l and the backward constants.  One warp per row, a record per
+// lane and step, then a fixed tree over the lanes.  (One thread per row walked its 240
+// records of V = 151,936 as one chain of loads and exponentials: 150 us whatever the
+// number of rows.)
+__global__ void __launch_bounds__(256)
+k_fused_merge(const int4 *__restrict__ rows, FusedArgs a, float *__restrict__ token_loss,
+              double *__restrict__ row_wl, float *__restrict__ rowc)
 {
-    const int n = *nvalid;
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
+    const int n = *a.nvalid, lane = threadIdx.x & 31;
+    const int n_tiles = (int)((a.vocab + BN - 1) / BN);
+    int mt_lo, mt_hi;
+    chunk_range((n + BMP - 1) / BMP, a.chunk_tiles, a.chunk, &mt_lo, &mt_hi);
+    if (mt_lo == mt_hi)
+        return;
+    const int gsize = pick_group(mt_hi - mt_lo, n_tiles, a.pairs, a.min_group);
+    const int recs = (n_tiles + gsize - 1) / gsize * kColQuarters;
+    const int row0 = mt_lo * BMP, row1 = min(n, mt_hi * BMP);
+    const int nwarp = gridDim.x * (blockDim.x / 32);
+    for (int j = row0 + (int)(blockIdx.x * blockDim.x + threadIdx.x) / 32; j < row1; j += nwarp) {
         Student S = student_empty();
         Teacher T = teacher_empty();
-        for (int gh = 0; gh < kColQuarters * n_groups; ++gh) {
-            const float *pp = part + ((size_t)gh * cap + j) * 8;
-            const float4 x = reinterpret_cast<const float4 *>(pp)[0];
-            const float4 y = reinterpret_cast<const float4 *>(pp)[1];
+        const float4 *pp = reinterpret_cast<const float4 *>(a.part) + (size_t)(j - row0) * 2;
+#pragma unroll 4
+        for (int gh = lane; gh < recs; gh += 32) {
+            const float4 x = pp[(size_t)gh * a.part_rows * 2];
+            const float4 y = pp[(size_t)gh * a.part_rows * 2 + 1];
             if (x.x != -INFINITY)
                 S = student_merge(S, Student{x.x, x.y, x.z, 0.f});
             if (x.w != -INFINITY)
                 T = teacher_merge(T, Teacher{x.w, y.x});
         }
-        const RowConst rc = row_const(S, T);
-        const int4 m = rows[j];
-        const float w = __int_as_float(m.w);
-        const float ell = rc.kl;
-        if (!isfinite(rc.lse_s) || !isfinite(rc.lse_t) || !isfinite(ell))
-            set_status(status, TURNOPD_ERR_NONFINITE);
-        token_loss[m.x] = ell;
-        row_wl[j] = (double)w * (double)ell;
-        // p |w| = 2^(z_s log2e - nl): nl = LSE_s log2e - log2 |w|
-        reinterpret_cast<float4 *>(rowc)[j] =
-            make_float4(rc.lse_s * kLog2e - log2f(fabsf(w)), rc.d + rc.cp, w < 0.f ? -1.f : 1.f, 0.f);
+        S = warp_merge(S);
+        T = warp_merge(T);
+        if (lane == 0) {
+            const RowConst rc = row_const(S, T);
+            const int4 m = rows[j];
+            const float w = __int_as_float(m.w);
+            const float ell = rc.kl;
+            if (!isfinite(rc.lse_s) || !isfinite(rc.lse_t) || !isfinite(ell))
+                set_status(a.status, TURNOPD_ERR_NONFINITE);
+            token_loss[m.x] = ell;
+            row_wl[j] = (double)w * (double)ell;
+            // p |w| = 2^(z_s log2e - nl): nl = LSE_s log2e - log2 |w|
+            reinterpret_cast<float4 *>(rowc)[j] =
+                make_float4(rc.lse_s * kLog2e - log2f(fabsf(w)), rc.d + rc.cp, w < 0.f ? -1.f : 1.f, 0.f);
+        }
+    }
+}
+
+// G of one chunk from its stored logits: a stream of 8 bytes read and 2 written per
+// logit, bound by HBM.  A warp takes 32 rows x 64 columns at a time: 16 KB of scratch in
+// whole 512-byte reads, one row per lane; the bf16 values cross the warp through shared
+// memory (128-byte rows, 16-byte pieces swizzled by row % 8) and leave as whole 128-byte
+// lines.  Columns past the vocabulary and rows past the supervised ones get zeros, as
+// the GEMMs that read G want them.
+constexpr int kGThreads = 256;
+__global__ void __launch_bounds__(kGThreads)
+k_fused_g(FusedArgs a)
+{
+    __shared__ __align__(128) uint8_t stage[kGThreads / 32][32 * 128];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int n = *a.nvalid;
+    int mt_lo, mt_hi;
+    chunk_range((n + BMP - 1) / BMP, a.chunk_tiles, a.chunk, &mt_lo, &mt_hi);
+    const int row_blocks = (mt_hi - mt_lo) * (BMP / 32);
+    const int col_blocks = (int)(a.vpad / 64);
+    const int64_t units = (int64_t)row_blocks * col_blocks;
+    uint8_t *stg = stage[warp];
+    const int64_t nw = (int64_t)gridDim.x * (kGThreads / 32);
+    for (int64_t u = (int64_t)blockIdx.x * (kGThreads / 32) + warp; u < units; u += nw) {
+        const int rb = (int)(u / col_blocks), cb = (int)(u % col_blocks);
+        const int row = mt_lo * BMP + rb * 32 + lane;
+        const bool valid = row < n;
+        float nl = 0.f, cp = 0.f, sg = 1.f;
+        if (valid) {
+            const float4 c = reinterpret_cast<const float4 *>(a.rowc)[row];
+            nl = c.x, cp = c.y, sg = c.z;
+        }
+        const int64_t left = a.vocab - (int64_t)cb * 64;
+        const int nv = left >= 64 ? 64 : (int)left;
+        const float4 *zq = a.z + z_index(a.vpad, rb, (int64_t)cb * 16) + lane;
+        __syncwarp();  // the stage's previous block has been read
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+            float4 zs[8], x[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                zs[j] = __ldcs(zq + (half * 8 + j) * 64);
+                x[j] = __ldcs(zq + (half * 8 + j) * 64 + 32);
+            }
+#pragma unroll
+            for (int j = 0; j < 8; j += 2) {
+                uint32_t pk[4];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int c0 = half * 32 + (j + h) * 4;
+                    const float zv[4] = {zs[j + h].x, zs[j + h].y, zs[j + h].z, zs[j + h].w};
+                    const float xv[4] = {x[j + h].x, x[j + h].y, x[j + h].z, x[j + h].w};
+                    float g[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        g[i] = valid && c0 + i < nv ? sg * ex2(fmaf(zv[i], kLog2e, -nl)) * (xv[i] - cp) : 0.f;
+                    pk[2 * h] = pack_bf16x2(g[0], g[1]);
+                    pk[2 * h + 1] = pack_bf16x2(g[2], g[3]);
+                }
+                const int piece = (half * 4 + j / 2) ^ (lane & 7);
+                *reinterpret_cast<uint4 *>(stg + lane * 128 + piece * 16) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+            }
+        }
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int r = i * 4 + lane / 8, c = lane % 8;
+            const uint4 v = *reinterpret_cast<const uint4 *>(stg + r * 128 + (c ^ (r & 7)) * 16);
+            *reinterpret_cast<uint4 *>(a.G + (size_t)(mt_lo * BMP + rb * 32 + r) * a.vpad + (size_t)cb * 64 + c * 8) = v;
+        }
     }
 }
 
@@ -913,11 +1064,27 @@ struct FusedLayout {
     double *row_wl;
     __nv_bfloat16 *hs, *ht, *G;
     float *part, *rowc, *dh_partial;
+    size_t base_bytes;   // without the chunk scratch: the least a call accepts
+    float *chunk_part;   // [groups of kMinTilesPerGroup][kColQuarters][chunk rows][8]
+    float4 *z;           // chunk logits
     size_t bytes;
 };
 
-FusedLayout fused_layout(void *ws, int64_t T, int64_t V, int64_t d_s, int64_t d_t, int n_groups, int sms)
+// Row tiles of a chunk, and so the size of its scratch: 8 bytes per logit, 2.5 GB at
+// V = 151,936.  A chunk is one launch, which reads both heads once.
+#ifndef TURNOPD_FUSED_CHUNK
+#define TURNOPD_FUSED_CHUNK 8
+#endif
+constexpr int kChunkTiles = TURNOPD_FUSED_CHUNK;
+
+int groups_for(int64_t V, int tiles_per_group)
 {
+    return (int)(((V + BN - 1) / BN + tiles_per_group - 1) / tiles_per_group);
+}
+
+FusedLayout fused_layout(void *ws, int64_t T, int64_t V, int64_t d_s, int64_t d_t, int sms)
+{
+    const int n_groups = groups_for(V, kTilesPerGroup);
     const int64_t vpad = (V + BK - 1) / BK * BK;
     const int64_t cap = (T + BMP - 1) / BMP * BMP;
     const int64_t nblk = (T + kCompactBlock - 1) / kCompactBlock;
@@ -939,11 +1106,14 @@ FusedLayout fused_layout(void *ws, int64_t T, int64_t V, int64_t d_s, int64_t d_
     L.rowc = reinterpret_cast<float *>(take(sizeof(float) * 4 * (size_t)cap));
     L.G = reinterpret_cast<__nv_bfloat16 *>(take(2 * (size_t)cap * vpad));
     L.dh_partial = reinterpret_cast<float *>(take(sizeof(float) * (size_t)max_pairs(sms) * 2 * BMP * BN));
+    L.base_bytes = off + 256;
+    const int64_t chunk = std::min<int64_t>(cap, (int64_t)kChunkTiles * BMP);
+    L.chunk_part = reinterpret_cast<float *>(
+        take(sizeof(float) * 8 * kColQuarters * (size_t)groups_for(V, kMinTilesPerGroup) * chunk));
+    L.z = reinterpret_cast<float4 *>(take(8 * (size_t)chunk * vpad));
     L.bytes = off + 256;
     return L;
 }
-
-int groups_for(int64_t V) { return (int)(((V + BN - 1) / BN + kTilesPerGroup - 1) / kTilesPerGroup); }
 
 // Launch `kern` on `pairs` 2-CTA clusters.
 template <class... KArgs, class... Args>
@@ -968,7 +1138,7 @@ cudaError_t launch_pairs(void (*kern)(KArgs...), int pairs, size_t smem, cudaStr
 template <class... KArgs>
 cudaError_t pairs_for(void (*kern)(KArgs...), size_t smem, int slot, int *pairs)
 {
-    static int cache[64][4] = {};
+    static int cache[64][5] = {};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess)
@@ -1008,14 +1178,18 @@ cudaError_t pairs_for(void (*kern)(KArgs...), size_t smem, int slot, int *pairs)
 
 size_t fused_workspace_bytes(int64_t T, int64_t V, int64_t d_s, int64_t d_t)
 {
-    return fused_layout(nullptr, T, V, d_s, d_t, groups_for(V), device_sm_count()).bytes;
+    return fused_layout(nullptr, T, V, d_s, d_t, device_sm_count()).bytes;
+}
+
+size_t fused_workspace_min_bytes(int64_t T, int64_t V, int64_t d_s, int64_t d_t)
+{
+    return fused_layout(nullptr, T, V, d_s, d_t, device_sm_count()).base_bytes;
 }
 
 cudaError_t launch_fused(const FusedCall &c, cudaStream_t stream)
 {
-    const int n_groups = groups_for(c.vocab);
     const int sms = device_sm_count();
-    FusedLayout L = fused_layout(c.workspace, c.T, c.vocab, c.d_s, c.d_t, n_groups, sms);
+    FusedLayout L = fused_layout(c.workspace, c.T, c.vocab, c.d_s, c.d_t, sms);
     const int64_t vpad = (c.vocab + BK - 1) / BK * BK;
     const int64_t cap = (c.T + BMP - 1) / BMP * BMP;
 
@@ -1050,11 +1224,13 @@ cudaError_t launch_fused(const FusedCall &c, cudaStream_t stream)
         !make_map(&tGmn, L.G, cap, vpad, BK, 64) || !make_map(&tHmn, L.hs, cap, c.d_s, BK, 64))
         return cudaErrorInvalidValue;
 
-    int p_lm0 = 0, p_lm1 = 0, p_dh = 0, p_dw = 0;
-    if ((e = pairs_for(k_fused_dw, kDhSmem, 3, &p_dw)) != cudaSuccess)
-        return e;
-    if ((e = pairs_for(k_fused_lm<0>, kFusedSmem, 0, &p_lm0)) != cudaSuccess ||
-        (e = pairs_for(k_fused_lm<1>, kFusedSmem, 1, &p_lm1)) != cudaSuccess ||
+    const bool backward = c.dh_s || c.dW_s;
+    const bool store = backward && c.workspace_bytes >= L.bytes;
+    int p_lm = 0, p_re = 0, p_dh = 0, p_dw = 0;
+    if ((e = pairs_for(k_fused_dw, kDhSmem, 3, &p_dw)) != cudaSuccess ||
+        (e = store ? pairs_for(k_fused_lm<kForwardStore>, kFusedSmem, 4, &p_lm)
+                   : pairs_for(k_fused_lm<kForward>, kFusedSmem, 0, &p_lm)) != cudaSuccess ||
+        (e = pairs_for(k_fused_lm<kRecompute>, kFusedSmem, 1, &p_re)) != cudaSuccess ||
         (e = pairs_for(k_fused_dh, kDhSmem, 2, &p_dh)) != cudaSuccess)
         return e;
 
@@ -1065,22 +1241,37 @@ cudaError_t launch_fused(const FusedCall &c, cudaStream_t stream)
     fa.d_t = (int)c.d_t;
     fa.rows = L.rows;
     fa.nvalid = L.nvalid;
-    fa.n_groups = n_groups;
-    fa.part = L.part;
-    fa.cap = cap;
+    fa.pairs = p_lm;
+    fa.chunk = 0;
+    fa.chunk_tiles = store ? kChunkTiles : (int)(cap / BMP);
+    fa.min_group = store ? kMinTilesPerGroup : kTilesPerGroup;
+    fa.part = store ? L.chunk_part : L.part;
+    fa.part_rows = store ? std::min<int64_t>(cap, (int64_t)kChunkTiles * BMP) : cap;
+    fa.z = store ? L.z : nullptr;
     fa.rowc = L.rowc;
     fa.G = L.G;
     fa.status = c.status;
 
-    if ((e = launch_pairs(k_fused_lm<0>, p_lm0, kFusedSmem, stream, tHs, tWs, tHt, tWt, tGst, fa)) != cudaSuccess)
-        return e;
-    k_fused_merge<<<(int)((cap + 255) / 256), 256, 0, stream>>>(L.rows, L.nvalid, L.part, n_groups, cap,
-                                                               c.token_loss, L.row_wl, L.rowc, c.status);
-    e = cudaGetLastError();
-    if (e != cudaSuccess)
-        return e;
-    if (c.dh_s || c.dW_s) {
-        if ((e = launch_pairs(k_fused_lm<1>, p_lm1, kFusedSmem, stream, tHs, tWs, tHt, tWt, tGst, fa)) != cudaSuccess)
+    // the number of supervised rows is known on the device alone: chunks past the last
+    // supervised row are empty launches
+    const int chunks = (int)((cap / BMP + fa.chunk_tiles - 1) / fa.chunk_tiles);
+    const int merge_grid = (int)std::min<int64_t>((fa.part_rows + 7) / 8, (int64_t)sms * 8);
+    for (fa.chunk = 0; fa.chunk < chunks; ++fa.chunk) {
+        e = store ? launch_pairs(k_fused_lm<kForwardStore>, p_lm, kFusedSmem, stream, tHs, tWs, tHt, tWt, tGst, fa)
+                  : launch_pairs(k_fused_lm<kForward>, p_lm, kFusedSmem, stream, tHs, tWs, tHt, tWt, tGst, fa);
+        if (e != cudaSuccess)
+            return e;
+        k_fused_merge<<<merge_grid, 256, 0, stream>>>(L.rows, fa, c.token_loss, L.row_wl, L.rowc);
+        if (store)
+            k_fused_g<<<sms * 4, kGThreads, 0, stream>>>(fa);
+        if ((e = cudaGetLastError()) != cudaSuccess)
+            return e;
+    }
+    if (backward && !store) {
+        fa.chunk = 0;
+        fa.pairs = p_re;
+        if ((e = launch_pairs(k_fused_lm<kRecompute>, p_re, kFusedSmem, stream, tHs, tWs, tHt, tWt, tGst, fa)) !=
+            cudaSuccess)
             return e;
     }
     if (c.dW_s) {

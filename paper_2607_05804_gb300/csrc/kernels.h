@@ -164,9 +164,13 @@ struct FusedCall {
     float *token_loss;
     double *loss;
     void *workspace;
+    size_t workspace_bytes;
     int32_t *status;
 };
+// With room for the chunk scratch (the forward pass's logits kept for the backward one),
+// and the least that a call accepts (the tiles are then computed twice).
 size_t fused_workspace_bytes(int64_t T, int64_t V, int64_t d_s, int64_t d_t);
+size_t fused_workspace_min_bytes(int64_t T, int64_t V, int64_t d_s, int64_t d_t);
 cudaError_t launch_fused(const FusedCall &c, cudaStream_t stream);
 
 // Cluster-resident kernel for aligned bf16 rows; sets *used = false (and

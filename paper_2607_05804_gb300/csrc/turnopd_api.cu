@@ -411,7 +411,7 @@ turnopd_status turnopd_fused_lmhead_fwd_bwd(const void *h_s, const void *W_s, in
         misaligned(loss_out, 8))
         return TURNOPD_ERR_SHAPE;
     if (!workspace || misaligned(workspace, 256) ||
-        workspace_bytes < fused_workspace_bytes(num_tokens, vocab, d_s, d_t))
+        workspace_bytes < fused_workspace_min_bytes(num_tokens, vocab, d_s, d_t))
         return TURNOPD_ERR_WORKSPACE;
     cudaStream_t s = (cudaStream_t)stream;
     if (num_tokens == 0) {
@@ -423,7 +423,7 @@ turnopd_status turnopd_fused_lmhead_fwd_bwd(const void *h_s, const void *W_s, in
         return cuda_status(cudaMemsetAsync(loss_out, 0, sizeof(double), s));
     }
     FusedCall c{h_s, W_s, h_t, W_t, d_s, d_t, vocab, num_tokens, loss_mask, w, dh_s_out, dW_s_out,
-                token_loss_out, loss_out, workspace, dev_status};
+                token_loss_out, loss_out, workspace, workspace_bytes, dev_status};
     return cuda_status(launch_fused(c, s));
 }
 

@@ -249,3 +249,42 @@ def test_fused_full_size_sampled_rows(P, oracle):
     assert (tl[b.loss_mask == 1] >= -1e-4).all()
     wl = float(np.dot(w.astype(np.float64), tl.astype(np.float64)))
     assert abs(loss - wl) <= 1e-9 * abs(wl)
+
+
+@pytest.mark.parametrize("traj_len,V", [(1700, 1000), (3700, 1000), (600, 8200)])
+def test_fused_chunk_scratch_and_recompute_agree(P, oracle, traj_len, V):
+    """A workspace of the reported size keeps the forward pass's logits chunk by chunk
+    (at most 8 pair row tiles: 1 to 3 chunks here, the last row tile ragged); one that
+    is smaller recomputes them.  Both against the oracle, and against each other: the
+    two differ by the order of the statistics' merges alone (~1e-6 of G before its
+    rounding to bf16, so single bf16 ulps, 2^-8 relative, of a few elements)."""
+    from paper_2607_05804_gb300.step import LossStep, to_device
+
+    b = W.packed(seed=41, num_traj=2, traj_len=traj_len)
+    d_s, d_t, T = 256, 192, b.num_tokens
+    heads = W.make_fused(T, d_s, d_t, V, seed=42, device="cuda")
+    tid, msk, off, _ = to_device(b, "cuda", compact=False)
+    step = LossStep(tid, msk, off, b.max_turns, V, alpha=1.0)
+    w = step.weights()
+    ws = torch.empty(P.turnopd_fused_workspace_bytes(T, V, d_s, d_t), dtype=torch.uint8, device="cuda")
+    out = []
+    for room in (ws, ws[:ws.numel() - 256]):
+        ws.fill_(255)  # NaN bit patterns: nothing may be read before it is written
+        dh = torch.full((T, d_s), 3.0, dtype=torch.float32, device="cuda")
+        dW = torch.full((V, d_s), 5.0, dtype=torch.float32, device="cuda")
+        tl = torch.full((T,), 7.0, dtype=torch.float32, device="cuda")
+        loss = torch.zeros(1, dtype=torch.float64, device="cuda")
+        P.turnopd_fused_lmhead_fwd_bwd(*heads, msk, w, 0, dh, tl, loss, room, step.dev_status, dW_s_out=dW)
+        torch.cuda.synchronize()
+        assert step.status() == 0
+        out.append((dh.cpu().numpy(), dW.cpu().numpy(), tl.cpu().numpy(), loss.item()))
+    bits = [W.bf16_bits(x) for x in heads]
+    dh_ref, tl_ref, loss_ref, dw_ref = oracle.fused_lmhead(*bits, b.loss_mask, w.cpu().numpy(), dW=True)
+    m = b.loss_mask == 1
+    for dh, dW, tl, loss in out:
+        assert_token_loss(tl, tl_ref, b.loss_mask)
+        assert_loss(loss, loss_ref)
+        assert (dh[~m] == 0).all()
+        assert_dh(dh[m], dh_ref[m])
+        assert_dh(dW, dw_ref)
+    assert_dh(out[0][0][m], out[1][0][m])
