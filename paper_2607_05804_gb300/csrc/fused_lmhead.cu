@@ -154,10 +154,12 @@ __device__ __forceinline__ FusedSmem carve(uint8_t *raw, int b_region, int stg_b
 
 constexpr int kLmBRegion = STAGES * B_BYTES;
 constexpr int kStgWarpBytes = 32 * kEpiCols * 2;             // 32 rows x 128 B
+static_assert(kStgWarpBytes == 32 * 32 * 4, "a 32 x 32 fp32 box of dW_s fits it");
 constexpr int kStgBytes = kEpiWarps * kStgWarpBytes;          // 64 KB
 // The dH kernel reads B as an MN-major operand; 16 KB of slack after the ring
 // keeps every address its descriptors can form inside the allocation.
 constexpr int kDhBRegion = STAGES * B_BYTES + 16384;
+static_assert(kStgBytes >= 16384, "the staging buffers stand in for the slack in k_fused_dw");
 constexpr size_t kFusedSmem = STAGES * A_BYTES + kLmBRegion + kStgBytes + 1024 + 256;
 static_assert(kFusedSmem <= 232448, "shared memory per CTA");
 constexpr size_t kDhSmem = STAGES * A_BYTES + kDhBRegion + 1024 + 256;
@@ -709,12 +711,17 @@ k_fused_dh(const __grid_constant__ CUtensorMap tG, const __grid_constant__ CUten
 }
 
 // ----------------------------------------------------------------------------
-// dW_s = G^T H_s: [V, d_s] fp32, K = the supervised tokens (padded to the pair
-// tile with zero rows of G and H_s).  A = G read as an MN-major operand (its
+// dW_s = G^T H_s: [V, d_s] fp32, K = the supervised tokens (padded to a k-block
+// with zero rows of G and H_s).  A = G read as an MN-major operand (its
 // columns are vocabulary ids), B = the gathered H_s read MN-major (columns are
 // d_s); two 256-column accumulators in tensor memory, so the epilogue's stores
 // of tile j overlap the MMAs of tile j+1.  Tiles: 256 vocabulary rows x 256
 // columns of d_s, column tile fastest (pairs in flight share the G panel).
+// With few tokens the kernel is bound by its 4 V d_s bytes of output: a warp copies
+// its 32 x 64 block to registers, hands the accumulator back, and sends the block out
+// through shared memory by TMA, whole 128-byte lines at a time (stores straight from
+// the registers, one row a lane, touched 32 lines each, 16 bytes of every one: 1,122
+// us for 308 tokens x 151,936 x 4,096; now 471, the output alone takes 366).
 struct DwArgs {
     const int32_t *nvalid;
     int64_t vocab;
@@ -724,16 +731,18 @@ struct DwArgs {
 };
 
 __global__ void __launch_bounds__(kThreads, 1)
-k_fused_dw(const __grid_constant__ CUtensorMap tGmn, const __grid_constant__ CUtensorMap tHmn, DwArgs a)
+k_fused_dw(const __grid_constant__ CUtensorMap tGmn, const __grid_constant__ CUtensorMap tHmn,
+           const __grid_constant__ CUtensorMap tDw, DwArgs a)
 {
     extern __shared__ uint8_t smem_raw[];
     __shared__ int s_dead;
-    FusedSmem sm = carve(smem_raw, kDhBRegion, 0);
+    // the staging buffers after the ring are also its slack (kDhBRegion)
+    FusedSmem sm = carve(smem_raw, kLmBRegion, kStgBytes);
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const uint32_t rank = cluster_ctarank();
     const int pair = (int)cluster_id(), n_pairs = (int)cluster_count();
     const int nvalid = *a.nvalid;
-    const int kbs = (nvalid + BMP - 1) / BMP * (BMP / BK);
+    const int kbs = (nvalid + BK - 1) / BK;
     const int v_tiles = (int)((a.vocab + BMP - 1) / BMP);
     const int d_tiles = a.d_s / BN;
     const int tiles = kbs > 0 ? v_tiles * d_tiles : 0;
@@ -792,6 +801,7 @@ k_fused_dw(const __grid_constant__ CUtensorMap tGmn, const __grid_constant__ CUt
         const int ew = warp - 2, q = warp % 4, cq = ew / 4;
         const uint32_t lane_off = (uint32_t)(q * 32) << 16;
         const int col0 = cq * kEpiCols;
+        uint8_t *stg = sm.stg + ew * kStgWarpBytes;
         const uint32_t acce0[2] = {mapa(smem_u32(acce[0]), 0), mapa(smem_u32(acce[1]), 0)};
         uint32_t tile = 0;
         if (kbs == 0) {  // no supervised token: dW_s = 0
@@ -807,24 +817,35 @@ k_fused_dw(const __grid_constant__ CUtensorMap tGmn, const __grid_constant__ CUt
         }
         for (int t = pair; t < tiles; t += n_pairs, ++tile) {
             const int mv = t / d_tiles, nd = t % d_tiles, buf = tile & 1;
-            const int64_t v = (int64_t)mv * BMP + (int)rank * BM + q * 32 + lane;
+            const int v0 = mv * BMP + (int)rank * BM + q * 32;  // this warp's first vocabulary row
             wait_lim(accf[buf], (tile >> 1) & 1, a.status, &s_dead);
             tc_fence_after();
-            float *dst = a.dw + v * a.d_s + nd * BN + col0;
-#pragma unroll 1
-            for (int ch = 0; ch < kEpiCols / 32; ++ch) {
-                float x[32];
-                tmem_ld32(tmem + lane_off + (uint32_t)buf * 256u + (uint32_t)(col0 + ch * 32), x);
-                tmem_ld_wait();
-                if (v < a.vocab) {
-                    float4 *d4 = reinterpret_cast<float4 *>(dst + ch * 32);
+            float x[kEpiCols];
+            tmem_ld32(tmem + lane_off + (uint32_t)buf * 256u + (uint32_t)col0, *reinterpret_cast<float(*)[32]>(&x[0]));
+            tmem_ld32(tmem + lane_off + (uint32_t)buf * 256u + (uint32_t)col0 + 32,
+                      *reinterpret_cast<float(*)[32]>(&x[32]));
+            tmem_ld_wait();
+            release_cols(acce0[buf], lane);
 #pragma unroll
-                    for (int jj = 0; jj < 8; ++jj)
-                        d4[jj] = make_float4(x[4 * jj], x[4 * jj + 1], x[4 * jj + 2], x[4 * jj + 3]);
+            for (int ch = 0; ch < kEpiCols / 32; ++ch) {
+                if (lane == 0)
+                    bulk_wait_read0();  // the staging buffer's previous box has left it
+                __syncwarp();
+#pragma unroll
+                for (int jj = 0; jj < 8; ++jj)
+                    *reinterpret_cast<float4 *>(stg + lane * 128 + (jj ^ (lane & 7)) * 16) =
+                        make_float4(x[ch * 32 + 4 * jj], x[ch * 32 + 4 * jj + 1], x[ch * 32 + 4 * jj + 2],
+                                    x[ch * 32 + 4 * jj + 3]);
+                fence_proxy_async_smem();
+                __syncwarp();
+                if (lane == 0 && v0 < a.vocab) {  // a box's rows past the vocabulary are clipped
+                    tma_store_2d(&tDw, nd * BN + col0 + ch * 32, v0, stg);
+                    bulk_commit();
                 }
             }
-            release_cols(acce0[buf], lane);
         }
+        if (lane == 0)
+            bulk_wait0();
     }
     pair_epilogue(sm, tmem, 512, rank);
 }
@@ -854,9 +875,14 @@ k_dh_fixup(const float *__restrict__ partial, const int4 *__restrict__ rows, con
             // pairs whose non-empty k-block range meets tile j's [lo, hi), in pair order
             const int64_t lo = (int64_t)j * kbs, hi = lo + kbs;
             int n = 0;
-            for (int c = 0; c < P; ++c) {
+            // pair c's range starts at floor(total c / P): none before lo P / total - 1
+            // reaches lo (walking all P pairs per job: 53 us for the 32 split tiles of 308
+            // rows, now 18)
+            for (int c = max(0, (int)(lo * P / total) - 1); c < P; ++c) {
                 const int64_t b = total * c / P, en = total * (c + 1) / P;
-                if (b >= en || en <= lo || b >= hi)
+                if (b >= hi)
+                    break;
+                if (b >= en || en <= lo)
                     continue;
                 s_src[n++] = c * 2 + ((b / kbs == j) ? 0 : 1);
             }
@@ -909,7 +935,7 @@ __global__ void k_gather_rows(const int4 *__restrict__ rows, const int32_t *__re
 // LSE_t, KL; write l, w*l and the backward constants.  One warp per row, a record per
 // lane and step, then a fixed tree over the lanes.  (One thread per row walked its 240
 // records of V = 151,936 as one chain of loads and exponentials: 150 us whatever the
-// number of rows.)
+// number of rows; now 12 us for 308 rows, 13 for a chunk of 2,048.)
 __global__ void __launch_bounds__(256)
 k_fused_merge(const int4 *__restrict__ rows, FusedArgs a, float *__restrict__ token_loss,
               double *__restrict__ row_wl, float *__restrict__ rowc)
@@ -956,7 +982,7 @@ k_fused_merge(const int4 *__restrict__ rows, FusedArgs a, float *__restrict__ to
 }
 
 // G of one chunk from its stored logits: a stream of 8 bytes read and 2 written per
-// logit, bound by HBM.  A warp takes 32 rows x 64 columns at a time: 16 KB of scratch in
+// logit, bound by HBM (2,048 rows x 151,936: 471 us, 6.6 TB/s).  A warp takes 32 rows x 64 columns at a time: 16 KB of scratch in
 // whole 512-byte reads, one row per lane; the bf16 values cross the warp through shared
 // memory (128-byte rows, 16-byte pieces swizzled by row % 8) and leave as whole 128-byte
 // lines.  Columns past the vocabulary and rows past the supervised ones get zeros, as
@@ -1042,18 +1068,20 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn()
     return fn;
 }
 
-// 2-D bf16 tensor map over a row-major [rows, cols] matrix, 128-byte swizzle,
+// 2-D bf16 (or fp32) tensor map over a row-major [rows, cols] matrix, 128-byte swizzle,
 // box of box_cols (128 B) x box_rows; rows beyond the matrix read as zero.
-bool make_map(CUtensorMap *m, const void *base, int64_t rows, int64_t cols, int box_rows, int box_cols)
+bool make_map(CUtensorMap *m, const void *base, int64_t rows, int64_t cols, int box_rows, int box_cols,
+              bool fp32 = false)
 {
     auto fn = encode_fn();
     if (!fn)
         return false;
     cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-    cuuint64_t strides[1] = {(cuuint64_t)cols * 2};
+    cuuint64_t strides[1] = {(cuuint64_t)cols * (fp32 ? 4 : 2)};
     cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
     cuuint32_t es[2] = {1, 1};
-    return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), dims, strides, box, es,
+    return fn(m, fp32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2,
+              const_cast<void *>(base), dims, strides, box, es,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
@@ -1214,20 +1242,21 @@ cudaError_t launch_fused(const FusedCall &c, cudaStream_t stream)
     if (e != cudaSuccess)
         return e;
 
-    alignas(64) CUtensorMap tHs, tWs, tHt, tWt, tG, tGst, tWmn, tGmn, tHmn;
+    alignas(64) CUtensorMap tHs, tWs, tHt, tWt, tG, tGst, tWmn, tGmn, tHmn, tDw;
     if (!make_map(&tHs, L.hs, cap, c.d_s, BM, BK) || !make_map(&tWs, c.W_s, c.vocab, c.d_s, BNH, BK) ||
         !make_map(&tHt, L.ht, cap, c.d_t, BM, BK) || !make_map(&tWt, c.W_t, c.vocab, c.d_t, BNH, BK) ||
         !make_map(&tG, L.G, cap, vpad, BM, BK) || !make_map(&tGst, L.G, cap, vpad, 32, kEpiCols) ||
         // W_s as the MN-major B of dH: boxes of 64 d-columns x BK vocabulary rows
         !make_map(&tWmn, c.W_s, c.vocab, c.d_s, BK, 64) ||
         // G and the gathered H_s as the MN-major operands of dW_s: 64 columns x BK token rows
-        !make_map(&tGmn, L.G, cap, vpad, BK, 64) || !make_map(&tHmn, L.hs, cap, c.d_s, BK, 64))
+        !make_map(&tGmn, L.G, cap, vpad, BK, 64) || !make_map(&tHmn, L.hs, cap, c.d_s, BK, 64) ||
+        (c.dW_s && !make_map(&tDw, c.dW_s, c.vocab, c.d_s, 32, 32, true)))
         return cudaErrorInvalidValue;
 
     const bool backward = c.dh_s || c.dW_s;
     const bool store = backward && c.workspace_bytes >= L.bytes;
     int p_lm = 0, p_re = 0, p_dh = 0, p_dw = 0;
-    if ((e = pairs_for(k_fused_dw, kDhSmem, 3, &p_dw)) != cudaSuccess ||
+    if ((e = pairs_for(k_fused_dw, kFusedSmem, 3, &p_dw)) != cudaSuccess ||
         (e = store ? pairs_for(k_fused_lm<kForwardStore>, kFusedSmem, 4, &p_lm)
                    : pairs_for(k_fused_lm<kForward>, kFusedSmem, 0, &p_lm)) != cudaSuccess ||
         (e = pairs_for(k_fused_lm<kRecompute>, kFusedSmem, 1, &p_re)) != cudaSuccess ||
@@ -1281,7 +1310,7 @@ cudaError_t launch_fused(const FusedCall &c, cudaStream_t stream)
         wa.d_s = (int)c.d_s;
         wa.dw = c.dW_s;
         wa.status = c.status;
-        if ((e = launch_pairs(k_fused_dw, p_dw, kDhSmem, stream, tGmn, tHmn, wa)) != cudaSuccess)
+        if ((e = launch_pairs(k_fused_dw, p_dw, kFusedSmem, stream, tGmn, tHmn, tDw, wa)) != cudaSuccess)
             return e;
     }
     if (c.dh_s) {
