@@ -153,8 +153,9 @@ size_t turnopd_weights_workspace_bytes(int32_t num_traj, int32_t max_turns);
  * Inputs:
  *   z_student, z_teacher  [num_rows, ld] row-major, in_dtype (F32 or BF16);
  *                          the values of columns [vocab, ld) never enter a result
- *                          (bf16 rows with ld a multiple of 8 read up to the next
- *                          multiple of 8 of vocab, inside the buffer, and mask it).
+ *                          (bf16 rows are read in whole 16-byte vectors, so up to 7
+ *                          elements beside a row are read and masked; nothing after
+ *                          the last row's column vocab - 1 is read).
  *   row_of_token           int32[num_tokens] or NULL (then num_rows >= num_tokens);
  *                          read only where loss_mask = 1, must lie in [0, num_rows).
  *   sampled_ids            int32[num_tokens], required for SAMPLED_TOKEN, in [0, vocab).
@@ -173,10 +174,11 @@ size_t turnopd_weights_workspace_bytes(int32_t num_traj, int32_t max_turns);
  *   l_i = 0), TURNOPD_ERR_NONFINITE (non-finite LSE or l_i).
  * Precision: fp32 arithmetic on exact fp32/bf16 inputs, fp64 loss sum.
  * Kernels (the results agree within the tolerances above whichever runs):
- *   bf16 logits, ld a multiple of 8, 16-byte aligned arrays: row clusters of
+ *   bf16 logits, 16-byte aligned arrays: row clusters of
  *     2 to 16 CTAs (the smallest whose slices fit three shared-memory stages)
  *     beside a helper grid on the remaining SMs, or the helper grid alone for
- *     short rows; a vocab that is not a multiple of 8 ends in a masked vector;
+ *     short rows; where vocab or ld is not a multiple of 8, a row's first and
+ *     last 16-byte vectors are masked;
  *   fp32 logits, vocab and ld multiples of 4, 16-byte aligned arrays: the
  *     split-row kernel (clusters of 8 CTAs per row, 4 for sampled-token rows)
  *     beside a helper grid on the remaining SMs; it marks its first read of

@@ -91,6 +91,7 @@ struct RowIn {
     // split_den > 0: the cluster kernel takes rows [0, nvalid split_num / split_den) of the
     // row list and the helper kernel the rest (set by launch_row_cluster)
     int32_t split_num, split_den;
+    int64_t elems;  // logits from the arrays' start to the last row's last column
 };
 
 int device_sm_count();
@@ -176,7 +177,7 @@ cudaError_t launch_fused(const FusedCall &c, cudaStream_t stream);
 // Cluster-resident kernel for aligned bf16 rows; sets *used = false (and
 // launches nothing) when the shape does not fit it.
 cudaError_t launch_row_cluster(const RowIn &p, bool fp32_grad, cudaStream_t stream, bool *used);
-// The same for a vocabulary that is not a multiple of 8 (a masked last vector).
+// The same for a vocabulary or stride that is not a multiple of 8 (masked end vectors).
 cudaError_t launch_row_cluster_tail(const RowIn &p, bool fp32_grad, cudaStream_t stream, bool *used);
 // Split-row kernel (clusters of CTAs share each row) for aligned fp32 rows; sets
 // *used = false (and launches nothing) when the shape does not fit it.

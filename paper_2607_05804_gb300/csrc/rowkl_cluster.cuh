@@ -58,26 +58,61 @@ struct GradConst {
     float gy;         // sampled: g_y = w l (1 - p_y)
 };
 
-// v with its bf16 lanes n..7 replaced by the lowest finite bf16 (the padding lanes of a
-// row's last vector when V % 8 != 0)
-__device__ __forceinline__ uint4 fill_from(uint4 v, int n)
+// What a lane that does not count reads as: -2^127.  It adds 0 beside any real logit, and
+// where a thread or a vector holds nothing else its maximum times log2 e is still finite
+// (the lowest finite bf16's is not: exp2(-inf + inf) made such a row NaN).
+constexpr uint32_t kFillLane = 0xff00u;
+
+// v with its bf16 lanes outside [lo, hi) replaced by kFillLane (the lanes
+// of a row's first and last vectors that belong to other rows or to padding)
+__device__ __forceinline__ uint4 keep_lanes(uint4 v, int lo, int hi)
 {
     uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-        if (2 * j >= n)
-            w[j] = 0xff7fff7fu;
-        else if (2 * j + 1 >= n)
-            w[j] = (w[j] & 0x0000ffffu) | 0xff7f0000u;
+        const bool in0 = 2 * j >= lo && 2 * j < hi, in1 = 2 * j + 1 >= lo && 2 * j + 1 < hi;
+        w[j] = (in0 ? w[j] & 0x0000ffffu : kFillLane) | (in1 ? w[j] & 0xffff0000u : kFillLane << 16);
     }
     return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-// v with its bf16 lane i (0..7) replaced by the lowest finite bf16
+// Lanes [lo, hi) of the vector at p read one element at a time (the others
+// kFillLane): the vector that would pass the end of the logits.
+__device__ __forceinline__ uint4 load_lanes(const __nv_bfloat16 *p, int lo, int hi)
+{
+    uint32_t w[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const uint32_t e0 = 2 * j >= lo && 2 * j < hi ? __bfloat16_as_ushort(p[2 * j]) : kFillLane;
+        const uint32_t e1 = 2 * j + 1 >= lo && 2 * j + 1 < hi ? __bfloat16_as_ushort(p[2 * j + 1]) : kFillLane;
+        w[j] = e0 | (e1 << 16);
+    }
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// Ragged rows (TL): the row stride or the vocabulary is no multiple of 8, so a row starts
+// `head` elements into a 16-byte vector and ends `tail` elements into one (tail 0: at its
+// end).  Its vectors are those of the 16-byte grid that hold any of its columns; the
+// first and the last may be partial.  (Rows of a stride that is no multiple of 8 took
+// the portable kernel's 2-byte loads before: dense 4 x 1024 tokens, V = 50,001, step
+// 1,075 us, now 216; 133 is its traffic at the copy bandwidth.)
+struct Ragged {
+    int head, nvec, tail;
+};
+__device__ __forceinline__ Ragged ragged(int row, int64_t ld, int64_t vocab)
+{
+    Ragged g;
+    g.head = ((row & 7) * (int)(ld & 7)) & 7;
+    g.nvec = (int)((g.head + vocab + 7) >> 3);
+    g.tail = (int)((g.head + vocab) & 7);
+    return g;
+}
+
+// v with its bf16 lane i (0..7) replaced by kFillLane
 __device__ __forceinline__ uint4 fill_lane(uint4 v, int i)
 {
     const uint32_t keep = (i & 1) ? 0x0000ffffu : 0xffff0000u;
-    const uint32_t fill = 0xff7fff7fu & ~keep;
+    const uint32_t fill = (kFillLane | kFillLane << 16) & ~keep;
     const int w = i >> 1;
     v.x = w == 0 ? (v.x & keep) | fill : v.x;
     v.y = w == 1 ? (v.y & keep) | fill : v.y;
@@ -111,16 +146,31 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
     const uint32_t stage_bytes = 2u * slice_bytes;
     const int v0 = (int)rank * slice_vec;  // first vector of my slice
     const int my_vec = max(0, min(slice_vec, nvec - v0));
-    const uint32_t my_bytes = (uint32_t)my_vec * 16u;
-    // TL (V % 8 != 0): the row's last vector (in the last slice) holds V % 8 columns.
-    // Its other lanes, row padding, read as the lowest finite bf16 in the statistics
-    // (set in shared memory by the thread that reads the vector) and are never
-    // written: the gradient loop stores gvec whole vectors, that thread the tail's
-    // columns.  Without TL all of this compiles away.
-    const int tail = TL ? (int)(p.vocab & 7) : 0;
-    const int tailq = TL && my_vec > 0 && v0 + my_vec == nvec ? my_vec - 1 : -1;
-    const int tailown = tailq >= 0 ? tailq % NT : -1;
-    const int gvec = TL && tailq >= 0 ? my_vec - 1 : my_vec;
+    // TL (ragged rows): the slice's vectors and the partial ones among them vary from row
+    // to row.  A partial vector's other lanes read as kFillLane in the
+    // statistics (set in shared memory by the thread that reads the vector) and are
+    // never written: the gradient loop stores whole vectors, that thread the partial
+    // one's columns.  Without TL all of this compiles away.
+    struct Slice {
+        int my_vec, head0, g0, gvec, tailq, tail;  // head0: of the row (every slice)
+        bool head;                                  // vector 0 is partial
+        bool cut;                                   // the last vector passes the end of the logits
+    };
+    auto slice_of = [&](int row) {
+        Slice g{my_vec, 0, 0, my_vec, -1, 0, false, false};
+        if (TL) {
+            const Ragged r = ragged(row, p.ld, p.vocab);
+            g.my_vec = max(0, min(slice_vec, r.nvec - v0));
+            g.head0 = r.head;
+            g.head = v0 == 0 && r.head > 0;
+            g.tail = r.tail;
+            g.tailq = r.tail && g.my_vec > 0 && v0 + g.my_vec == r.nvec ? g.my_vec - 1 : -1;
+            g.g0 = g.head ? 1 : 0;
+            g.gvec = g.tailq >= 0 ? g.my_vec - 1 : g.my_vec;
+            g.cut = g.tailq >= 0 && (int64_t)row * p.ld - r.head + (int64_t)r.nvec * 8 > p.elems;
+        }
+        return g;
+    };
 
     unsigned char *stage = smem;
     float *rec = reinterpret_cast<float *>(smem + kStages * stage_bytes);  // [kSlots][CS][8]
@@ -196,13 +246,15 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
     // previous row is done with it)
     auto issue = [&](int k, int4 m) {
         const int s = k % kStages;
+        const Slice g = slice_of(m.y);
         meta[s] = m;
         if (SM) {  // the thread that will read y's vector (sampled-token rows; see stats)
-            const int q = m.z >= 0 ? (m.z >> 3) - v0 : -1;
-            yown[s] = q >= 0 && q < my_vec ? q % NT : -1;
+            const int q = m.z >= 0 ? ((m.z + g.head0) >> 3) - v0 : -1;
+            yown[s] = q >= 0 && q < g.my_vec ? q % NT : -1;
         }
         *(volatile int *)&srow[s] = k;
-        const size_t off = (size_t)m.y * (size_t)p.ld + (size_t)v0 * 8;
+        const uint32_t my_bytes = (uint32_t)(TL && g.cut ? g.my_vec - 1 : g.my_vec) * 16u;
+        const size_t off = (size_t)m.y * (size_t)p.ld - (size_t)g.head0 + (size_t)v0 * 8;
         const char *gs = reinterpret_cast<const char *>(zs + off);
         const char *gt = reinterpret_cast<const char *>(zt + off);
         unsigned char *ds = stage + s * stage_bytes;
@@ -220,28 +272,43 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
         const int s = k % kStages;
         const uint4 *vs = reinterpret_cast<const uint4 *>(stage + s * stage_bytes);
         const uint4 *vt = reinterpret_cast<const uint4 *>(stage + s * stage_bytes + slice_bytes);
+        const Slice g = slice_of(meta[s].y);
+        const int my_vec = g.my_vec;
+        if (TL && ((g.tailq >= 0 && g.tailq % NT == gtid) || (g.head && gtid == 0))) {
+            // partial vectors: lanes of other rows and padding out of both models' statistics
+            uint4 *ws = reinterpret_cast<uint4 *>(stage + s * stage_bytes);
+            uint4 *wt = reinterpret_cast<uint4 *>(stage + s * stage_bytes + slice_bytes);
+            if (g.tailq >= 0 && g.tailq % NT == gtid) {
+                if (g.cut) {
+                    const size_t e = (size_t)meta[s].y * (size_t)p.ld - (size_t)g.head0 + (size_t)(v0 + g.tailq) * 8;
+                    ws[g.tailq] = load_lanes(zs + e, 0, g.tail);
+                    wt[g.tailq] = load_lanes(zt + e, 0, g.tail);
+                } else {
+                    ws[g.tailq] = keep_lanes(ws[g.tailq], 0, g.tail);
+                    wt[g.tailq] = keep_lanes(wt[g.tailq], 0, g.tail);
+                }
+            }
+            if (g.head && gtid == 0) {
+                ws[0] = keep_lanes(ws[0], g.head0, 8);
+                wt[0] = keep_lanes(wt[0], g.head0, 8);
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        }
         // A sampled-token row leaves y out of the student statistics (add_sampled_term
         // brings its term back at the merge): the thread that reads y's vector in both
-        // passes below (named at issue) keeps z_s[y] for the record and puts the lowest
-        // finite bf16 in its place, which is never the maximum and adds 0.  (The gradient
+        // passes below (named at issue) keeps z_s[y] for the record and puts kFillLane
+        // in its place, which adds 0.  (The gradient
         // pass replaces g_y; the proxy fence orders the store before the stage's next
         // bulk copy.)
         if (SM && yown[s] == gtid) {
-            const uint32_t ay = smem_u32(stage + s * stage_bytes) + 2u * (uint32_t)(meta[s].z - v0 * 8);
+            const uint32_t ay = smem_u32(stage + s * stage_bytes) + 2u * (uint32_t)(meta[s].z + g.head0 - v0 * 8);
             uint32_t old;
             asm volatile("ld.shared.u16 %0, [%1];\n\tst.shared.u16 [%1], %2;\n\t"
                          "fence.proxy.async.shared::cta;"
                          : "=r"(old)
-                         : "r"(ay), "r"(0xff7fu)
+                         : "r"(ay), "r"(kFillLane)
                          : "memory");
             rcs[group * 16 + 15] = __uint_as_float(old << 16);
-        }
-        if (TL && tailown == gtid) {  // the row's last vector: padding lanes out of both models' statistics
-            uint4 *ts = reinterpret_cast<uint4 *>(stage + s * stage_bytes) + tailq;
-            uint4 *tt = reinterpret_cast<uint4 *>(stage + s * stage_bytes + slice_bytes) + tailq;
-            *ts = fill_from(*ts, tail);
-            *tt = fill_from(*tt, tail);
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         }
         // max pass (packed bf16): running maxima, plus each vector's student
         // maximum kept packed so the argmax vector is found after the loop
@@ -328,9 +395,9 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
             B.s = __shfl_sync(0xffffffffu, B.s, 0);
             if (lane < CS) {
                 float ys = 0.f, yt = 0.f;  // sampled-token logits, from the CTA holding y
-                const int y = meta[s].z;
-                if (y >= 0 && y / 8 >= v0 && y / 8 < v0 + my_vec) {
-                    const int e = y - v0 * 8;
+                const int y = meta[s].z, yh = y + g.head0;
+                if (y >= 0 && yh / 8 >= v0 && yh / 8 < v0 + my_vec) {
+                    const int e = yh - v0 * 8;
                     ys = SM ? rcs[group * 16 + 15] : to_float(reinterpret_cast<const __nv_bfloat16 *>(vs)[e]);
                     yt = to_float(reinterpret_cast<const __nv_bfloat16 *>(vt)[e]);
                 }
@@ -363,7 +430,8 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
             lane_merge<CS, kUseD>(A, B);
             if (lane == 0) {
                 const int y = meta[k % kStages].z;
-                const int owner = SM ? (y / 8) / slice_vec : 0;
+                const int yh = TL ? y + ragged(meta[k % kStages].y, p.ld, p.vocab).head : y;
+                const int owner = SM ? (yh / 8) / slice_vec : 0;
                 float omp = 0.f;  // 1 - p_y (sampled)
                 if (SM)
                     omp = add_sampled_term(A, r[owner * 8 + 6]);
@@ -404,7 +472,9 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
         const uint4 *vt = reinterpret_cast<const uint4 *>(stage + s * stage_bytes + slice_bytes);
         const int y = m.z;
         const float gy = gc.gy;
-        const size_t row_off = (size_t)m.y * (size_t)p.ld + (size_t)v0 * 8;
+        const Slice sl = slice_of(m.y);
+        const int gvec = sl.gvec;
+        const size_t row_off = (size_t)m.y * (size_t)p.ld - (size_t)sl.head0 + (size_t)v0 * 8;
         // p |w| = 2^(z_s log2e - LSE_s log2e + log2 |w|); the sign of w enters through an
         // fma by (sg, sg), which is exact on z_s - z_t
         const float2 L2 = splat(kLog2e), NLW = splat(gc.nlw);
@@ -413,7 +483,7 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
 #pragma unroll
         for (int u = 0; u < VPT; ++u) {
             const int q = gtid + u * NT;
-            if (q < gvec) {
+            if (q < gvec && (!TL || q >= sl.g0)) {
                 float2 g[4];
                 // y < 0 exactly when !SM; the fp32-gradient instantiations keep the run-time
                 // test, which compiles to a loop 5 % faster there (and 2.4 % slower for bf16)
@@ -450,8 +520,9 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
                 }
             }
         }
-        if (TL && tailown == gtid) {  // the row's last vector, column by column (the loop's formulas)
-            const uint4 a = vs[tailq], b = vt[tailq];
+        // a partial vector, column by column (the loop's formulas)
+        auto store_lanes = [&](int q, int lo, int hi) {
+            const uint4 a = vs[q], b = vt[q];
             float gl[8];
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
@@ -462,16 +533,20 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
                 gl[2 * j] = gg.x;
                 gl[2 * j + 1] = gg.y;
             }
-            const size_t to = row_off + (size_t)tailq * 8;
+            const size_t to = row_off + (size_t)q * 8;
 #pragma unroll
             for (int i = 0; i < 8; ++i)
-                if (i < tail) {
+                if (i >= lo && i < hi) {
                     if (G32)
                         static_cast<float *>(p.grad)[to + i] = gl[i];
                     else
                         static_cast<__nv_bfloat16 *>(p.grad)[to + i] = __float2bfloat16_rn(gl[i]);
                 }
-        }
+        };
+        if (TL && sl.tailq >= 0 && sl.tailq % NT == gtid)
+            store_lanes(sl.tailq, 0, sl.tail);
+        if (TL && sl.head && gtid == 0)
+            store_lanes(0, sl.head0, 8);
         // sampled token: g_y = w l (1 - p_y), over the value the vector store wrote
         // (same thread, so the later store wins)
         if (SM && yown[s] == gtid) {
@@ -554,7 +629,7 @@ __global__ void __launch_bounds__(NTH, MINB) k_row_helper(RowIn p)
 {
     constexpr int kHelpThreads = NTH;
     constexpr int NW = kHelpThreads / 32;
-    constexpr uint32_t kFill = 0xff7fff7fu;  // lowest finite bf16 pair: adds 0, never the max
+    constexpr uint32_t kFill = kFillLane | kFillLane << 16;
     __shared__ float red[NW][8];
     __shared__ float bc[8];
     extern __shared__ uint4 hring[];  // [kHelpStages][2][kHelpU][NTH] (AS)
@@ -563,20 +638,24 @@ __global__ void __launch_bounds__(NTH, MINB) k_row_helper(RowIn p)
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nvalid = *p.nvalid;
     const int j0 = p.split_den ? (int)((int64_t)nvalid * p.split_num / p.split_den) : 0;
-    // TL (V % 8 != 0): the last vector holds `tail` columns (its padding lanes read as
-    // the lowest finite bf16 and are never written); the gradient loop stores nfull vectors
-    const int nvec = TL ? (int)((p.vocab + 7) / 8) : (int)(p.vocab / 8);
-    const int tail = TL ? (int)(p.vocab & 7) : 0;
-    const int nfull = TL ? nvec - 1 : nvec;
     const __nv_bfloat16 *zs = static_cast<const __nv_bfloat16 *>(p.zs);
     const __nv_bfloat16 *zt = static_cast<const __nv_bfloat16 *>(p.zt);
     const float2 L2 = splat(kLog2e);
     for (int j = j0 + (int)blockIdx.x; j < nvalid; j += gridDim.x) {
         const int4 m = p.rows[j];
         const size_t off = (size_t)m.y * (size_t)p.ld;
-        const uint4 *vs = reinterpret_cast<const uint4 *>(zs + off);
-        const uint4 *vt = reinterpret_cast<const uint4 *>(zt + off);
-        const int yvec = m.z >= 0 ? (m.z >> 3) : -1;     // the vector holding the sampled id
+        // TL (ragged rows): a partial first or last vector's other lanes read as kFillLane
+        // and are never written; the gradient loop stores vectors [g0, nfull)
+        const Ragged rg = TL ? ragged(m.y, p.ld, p.vocab) : Ragged{0, (int)(p.vocab / 8), 0};
+        const int head = rg.head, nvec = rg.nvec, tail = rg.tail;
+        const int g0 = TL && head ? 1 : 0, nfull = TL && tail ? nvec - 1 : nvec;
+        const size_t voff = off - (size_t)head;          // the row's first vector
+        const bool cut = TL && (int64_t)voff + (int64_t)nvec * 8 > p.elems;  // the last passes the end
+        auto lanes_lo = [&](int q) { return q == 0 ? head : 0; };
+        auto lanes_hi = [&](int q) { return q == nvec - 1 && tail ? tail : 8; };
+        const uint4 *vs = reinterpret_cast<const uint4 *>(zs + voff);
+        const uint4 *vt = reinterpret_cast<const uint4 *>(zt + voff);
+        const int yvec = m.z >= 0 ? ((m.z + head) >> 3) : -1;  // the vector holding the sampled id
         float ms = -INFINITY, mt = -INFINITY, dd = 0.f;  // dd: reference difference (fp32 gradient)
         float2 S2 = make_float2(0.f, 0.f), A2 = S2, T2 = S2;
         // this thread's batches of the row: kHelpU vectors of each model, kHelpThreads apart
@@ -588,7 +667,7 @@ __global__ void __launch_bounds__(NTH, MINB) k_row_helper(RowIn p)
 #pragma unroll
                 for (int u = 0; u < kHelpU; ++u) {
                     const int q = q0 + u * kHelpThreads;
-                    if (q < nvec) {
+                    if (q < nvec && !(TL && cut && q == nvec - 1)) {
                         cp_async16(&hring[slot(s, 0, u)], vs + q);
                         cp_async16(&hring[slot(s, 1, u)], vt + q);
                     }
@@ -609,7 +688,10 @@ __global__ void __launch_bounds__(NTH, MINB) k_row_helper(RowIn p)
 #pragma unroll
             for (int u = 0; u < kHelpU; ++u) {
                 const int q = q0 + u * kHelpThreads;
-                if (q < nvec) {
+                if (TL && cut && q == nvec - 1) {
+                    a[u] = load_lanes(zs + voff + (size_t)q * 8, lanes_lo(q), lanes_hi(q));
+                    b[u] = load_lanes(zt + voff + (size_t)q * 8, lanes_lo(q), lanes_hi(q));
+                } else if (q < nvec) {
                     if (AS) {
                         a[u] = hring[slot(bi % kHelpStages, 0, u)];
                         b[u] = hring[slot(bi % kHelpStages, 1, u)];
@@ -621,21 +703,23 @@ __global__ void __launch_bounds__(NTH, MINB) k_row_helper(RowIn p)
                     a[u] = b[u] = make_uint4(kFill, kFill, kFill, kFill);
                 }
             }
-            // a sampled-token row leaves y out of the student statistics (lowest finite
-            // bf16 in its place; add_sampled_term brings its term back at the merge)
+            if (TL && ((head && q0 == 0) || (tail && (unsigned)(nvec - 1 - q0) < (unsigned)(kHelpU * kHelpThreads)))) {
+#pragma unroll
+                for (int u = 0; u < kHelpU; ++u) {
+                    const int q = q0 + u * kHelpThreads;
+                    if ((head && q == 0) || (tail && q == nvec - 1)) {
+                        a[u] = keep_lanes(a[u], lanes_lo(q), lanes_hi(q));
+                        b[u] = keep_lanes(b[u], lanes_lo(q), lanes_hi(q));
+                    }
+                }
+            }
+            // a sampled-token row leaves y out of the student statistics (kFillLane
+            // in its place; add_sampled_term brings its term back at the merge)
             if (SM && (unsigned)(yvec - q0) < (unsigned)(kHelpU * kHelpThreads)) {
 #pragma unroll
                 for (int u = 0; u < kHelpU; ++u)
                     if (yvec == q0 + u * kHelpThreads)
-                        a[u] = fill_lane(a[u], m.z & 7);
-            }
-            if (TL && (unsigned)(nvec - 1 - q0) < (unsigned)(kHelpU * kHelpThreads)) {
-#pragma unroll
-                for (int u = 0; u < kHelpU; ++u)
-                    if (nvec - 1 == q0 + u * kHelpThreads) {
-                        a[u] = fill_from(a[u], tail);
-                        b[u] = fill_from(b[u], tail);
-                    }
+                        a[u] = fill_lane(a[u], (m.z + head) & 7);
             }
             uint32_t bs = hmax4(a[0]), bt = hmax4(b[0]);
 #pragma unroll
@@ -731,7 +815,7 @@ __global__ void __launch_bounds__(NTH, MINB) k_row_helper(RowIn p)
             const float2 ND = splat(bc[5]), NCP = splat(bc[6]);
             const float gy = bc[4];
             const int y = m.z;
-            for (int q0 = tid; q0 < nfull; q0 += kHelpU * kHelpThreads) {
+            for (int q0 = tid; q0 < nfull; q0 += kHelpU * kHelpThreads) {  // (a partial vector 0 is skipped below)
                 uint4 a[kHelpU], b[kHelpU];
 #pragma unroll
                 for (int u = 0; u < kHelpU; ++u) {
@@ -747,6 +831,8 @@ __global__ void __launch_bounds__(NTH, MINB) k_row_helper(RowIn p)
                     const int q = q0 + u * kHelpThreads;
                     if (q >= nfull)
                         break;
+                    if (TL && q < g0)
+                        continue;
                     float2 g[4];
                     if (!SM) {  // full vocabulary: g = w p ((z_s - z_t) - d - cp)
 #pragma unroll
@@ -761,7 +847,7 @@ __global__ void __launch_bounds__(NTH, MINB) k_row_helper(RowIn p)
                             g[w] = fmul2(ex2x2(ffma2(unpack2(word(a[u], w)), L2, NLW)), SGL);
                     }
                     if (G32) {
-                        float4 *dst = reinterpret_cast<float4 *>(static_cast<float *>(p.grad) + off) + 2 * (size_t)q;
+                        float4 *dst = reinterpret_cast<float4 *>(static_cast<float *>(p.grad) + voff) + 2 * (size_t)q;
                         __stcs(dst, make_float4(g[0].x, g[0].y, g[1].x, g[1].y));
                         __stcs(dst + 1, make_float4(g[2].x, g[2].y, g[3].x, g[3].y));
                     } else {
@@ -770,12 +856,15 @@ __global__ void __launch_bounds__(NTH, MINB) k_row_helper(RowIn p)
                         o.y = pack_bf16x2(g[1].x, g[1].y);
                         o.z = pack_bf16x2(g[2].x, g[2].y);
                         o.w = pack_bf16x2(g[3].x, g[3].y);
-                        __stcs(reinterpret_cast<uint4 *>(static_cast<__nv_bfloat16 *>(p.grad) + off) + q, o);
+                        __stcs(reinterpret_cast<uint4 *>(static_cast<__nv_bfloat16 *>(p.grad) + voff) + q, o);
                     }
                 }
             }
-            if (TL && (nvec - 1) % kHelpThreads == tid) {  // the last vector, column by column
-                const uint4 a = __ldg(vs + nvec - 1), b = __ldg(vt + nvec - 1);
+            // a partial vector, column by column
+            auto store_lanes = [&](int q) {
+                const int lo = lanes_lo(q), hi = lanes_hi(q);
+                const size_t to = voff + (size_t)q * 8;
+                const uint4 a = load_lanes(zs + to, lo, hi), b = load_lanes(zt + to, lo, hi);
                 float gl[8];
 #pragma unroll
                 for (int w = 0; w < 4; ++w) {
@@ -786,19 +875,22 @@ __global__ void __launch_bounds__(NTH, MINB) k_row_helper(RowIn p)
                     gl[2 * w] = gg.x;
                     gl[2 * w + 1] = gg.y;
                 }
-                const size_t to = off + (size_t)(nvec - 1) * 8;
 #pragma unroll
                 for (int i = 0; i < 8; ++i)
-                    if (i < tail) {
+                    if (i >= lo && i < hi) {
                         if (G32)
                             static_cast<float *>(p.grad)[to + i] = gl[i];
                         else
                             static_cast<__nv_bfloat16 *>(p.grad)[to + i] = __float2bfloat16_rn(gl[i]);
                     }
-            }
+            };
+            if (TL && tail && (nvec - 1) % kHelpThreads == tid)
+                store_lanes(nvec - 1);
+            if (TL && head && tid == 0 && !(tail && nvec == 1))
+                store_lanes(0);
             // sampled token: g_y = w l (1 - p_y), over the value the vector store wrote
             // (same thread, so the later store wins)
-            if (SM && (y >> 3) % kHelpThreads == tid) {
+            if (SM && ((y + head) >> 3) % kHelpThreads == tid) {
                 if (G32)
                     static_cast<float *>(p.grad)[off + y] = gy;
                 else
@@ -984,21 +1076,22 @@ void launch_helper_alone(const RowIn &p, int nvec, cudaStream_t stream)
         k_row_helper<G32, SM, TL, false><<<sms, kHelpThreads, 0, stream>>>(p);
 }
 
-// The row grids for bf16 logits; TL: V % 8 != 0 (a masked last vector).
+// The row grids for bf16 logits; TL: ragged rows (V or ld no multiple of 8).
 template <bool TL>
 cudaError_t launch_row_cluster_t(const RowIn &p, bool fp32_grad, cudaStream_t stream, bool *used)
 {
     *used = false;
     auto al16 = [](const void *q) { return (reinterpret_cast<uintptr_t>(q) & 15u) == 0; };
-    // rows 16-byte aligned; V % 8 != 0 takes a masked last vector (the row's padding up to
-    // the next multiple of 8 is read, never written)
-    if (p.ld % 8 != 0 || !al16(p.zs) || !al16(p.zt) || (p.grad && !al16(p.grad)))
+    // 16-byte aligned arrays; TL: any stride and vocabulary (a row's first and last vectors
+    // are masked; what they hold of other rows or of padding is read, never written)
+    if ((!TL && p.ld % 8 != 0) || !al16(p.zs) || !al16(p.zt) || (p.grad && !al16(p.grad)))
         return cudaSuccess;
     // the smallest cluster whose slices fit three stages (2, 3, 4, 5, 6, 8 or 16 CTAs;
     // 16 is a non-portable size)
-    if ((p.vocab + 7) / 8 > (int64_t)0x7fffffff)
+    if ((p.vocab + 14) / 8 > (int64_t)0x7fffffff)
         return cudaSuccess;
-    const int nvec = (int)((p.vocab + 7) / 8);
+    // the most vectors a row spans: 7 more elements where rows start anywhere in a vector
+    const int nvec = (int)((p.vocab + (p.ld % 8 != 0 ? 7 : 0) + 7) / 8);
     static const int kSizes[] = {2, 3, 4, 5, 6, 8, 16};
     int cs = 16;
     for (int c : kSizes)

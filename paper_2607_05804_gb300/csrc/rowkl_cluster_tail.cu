@@ -1,5 +1,6 @@
-// The bf16 row grids of rowkl_cluster.cuh for a vocabulary that is not a multiple of
-// 8: the row's last vector is masked in the statistics and written column by column.
+// The bf16 row grids of rowkl_cluster.cuh for a vocabulary or a row stride that is not
+// a multiple of 8: the row's first and last vectors are masked in the statistics and
+// written column by column.
 
 #include "rowkl_cluster.cuh"
 

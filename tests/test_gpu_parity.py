@@ -274,6 +274,62 @@ def test_masked_tail_vocab(P, oracle, V, mode, gdt):
         assert (y[r] == V - 1).all()
 
 
+@pytest.mark.parametrize("V,ld", [(2, 2), (3, 5), (9, 9), (4097, 4097), (8192, 8195), (27187, 27187),
+                                  (32007, 32009), (50001, 50001), (W.V_QWEN + 3, W.V_QWEN + 3)])
+@pytest.mark.parametrize("mode", [0, 1], ids=["full", "sampled"])
+@pytest.mark.parametrize("gdt", ["bf16", "f32", "none"])
+def test_ragged_rows_bf16(P, oracle, V, ld, mode, gdt):
+    """bf16 rows that start anywhere in a 16-byte vector (stride no multiple of 8): the
+    helper alone (up to V = 8,192, rows shorter than a vector among them, down to V = 2: at
+    V = 1 every l is 0 and a relative bound on the total loss is void), clusters of 2
+    (27,187 and 32,007), of 3 (50,001) and of 8.  The logits end with the last row's last
+    column: NaN behind it must not enter a result.  In sampled mode y is pushed into the
+    first and the last column of some rows, the partial vectors."""
+    b = W.packed(seed=61, num_traj=2, traj_len=128 if V > 60000 else 256)
+    R = b.num_valid
+    zs0, zt0 = W.make_logits(R, V, "agent" if V > 8 else "tiny", torch.bfloat16, seed=62, device="cuda")
+    if mode == 1 and V > 8:
+        r = torch.arange(R, device="cuda")
+        for k, col in ((0, 0), (1, V - 1)):
+            rows = r[r % 3 == k]
+            zs0[rows, col] = (zs0[rows].float().amax(dim=1) + 30.0).to(torch.bfloat16)
+
+    def strided(z):
+        buf = torch.full((R * ld + 64,), float("nan"), dtype=torch.bfloat16, device="cuda")
+        v = buf[:R * ld].view(R, ld)
+        v[:, :V] = z
+        buf[(R - 1) * ld + V:] = float("nan")
+        return v
+
+    zs, zt = strided(zs0), strided(zt0)
+    if gdt == "none":
+        y = per_token_ids(b, W.sample_ids(zs, 63, V), True) if mode == 1 else None
+        step = make_step(P, b, V, compact=True, mode=mode, y=y)
+        step.run(zs, zt, None)
+        torch.cuda.synchronize()
+        assert step.status() == 0
+        w = step.w[:b.num_tokens].cpu().numpy()
+        _, tl_ref, loss_ref = oracle.loss_fwd_bwd(
+            bits_or_f32(zs), bits_or_f32(zt), V, b.loss_mask, w, mode=mode, row_of_token=b.compact_rows(),
+            sampled_ids=y.cpu().numpy() if y is not None else None, grad=False)
+        assert_token_loss(step.token_loss[:b.num_tokens].cpu().numpy(), tl_ref, b.loss_mask)
+        return
+    _, grad = run_chain(P, oracle, b, V, zs, zt, mode=mode, alpha=0.5, compact=True, seed_y=63,
+                        grad_dtype=torch.bfloat16 if gdt == "bf16" else torch.float32)
+    if ld > V:
+        assert (grad[:, V:].float() == 7.0).all()
+
+
+def test_ragged_rows_dense_neighbours_untouched(P, oracle):
+    """One row per token, odd stride: the gradient rows of masked tokens share vectors
+    with supervised ones and stay as they were."""
+    b = W.packed(seed=64, num_traj=2, traj_len=128)
+    for V in (4099, 50001):
+        zs, zt = W.make_logits(b.num_tokens, V, "agent", torch.bfloat16, seed=65, device="cuda")
+        _, grad = run_chain(P, oracle, b, V, zs, zt, mode=0, alpha=0.5)
+        assert (grad[torch.from_numpy(b.loss_mask == 0).cuda()].float() == 7.0).all()
+
+
 @pytest.mark.parametrize("n_sup", [1, 5])
 def test_split_kernel_fewer_rows_than_clusters(P, oracle, n_sup):
     """fp32 rows at the full vocabulary with fewer rows than clusters: most clusters
