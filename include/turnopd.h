@@ -153,8 +153,8 @@ size_t turnopd_weights_workspace_bytes(int32_t num_traj, int32_t max_turns);
  * Inputs:
  *   z_student, z_teacher  [num_rows, ld] row-major, in_dtype (F32 or BF16);
  *                          the values of columns [vocab, ld) never enter a result
- *                          (bf16 rows are read in whole 16-byte vectors, so up to 7
- *                          elements beside a row are read and masked; nothing after
+ *                          (rows are read in whole 16-byte vectors, so a few elements
+ *                          beside a row are read and masked; nothing after
  *                          the last row's column vocab - 1 is read).
  *   row_of_token           int32[num_tokens] or NULL (then num_rows >= num_tokens);
  *                          read only where loss_mask = 1, must lie in [0, num_rows).
@@ -174,17 +174,16 @@ size_t turnopd_weights_workspace_bytes(int32_t num_traj, int32_t max_turns);
  *   l_i = 0), TURNOPD_ERR_NONFINITE (non-finite LSE or l_i).
  * Precision: fp32 arithmetic on exact fp32/bf16 inputs, fp64 loss sum.
  * Kernels (the results agree within the tolerances above whichever runs):
- *   bf16 logits, 16-byte aligned arrays: row clusters of
- *     2 to 16 CTAs (the smallest whose slices fit three shared-memory stages)
- *     beside a helper grid on the remaining SMs, or the helper grid alone for
- *     short rows; where vocab or ld is not a multiple of 8, a row's first and
- *     last 16-byte vectors are masked;
- *   fp32 logits, vocab and ld multiples of 4, 16-byte aligned arrays: the
- *     split-row kernel (clusters of 8 CTAs per row, 4 for sampled-token rows)
- *     beside a helper grid on the remaining SMs; it marks its first read of
- *     each logit chunk L2 evict-last and returns the lines to normal priority
- *     after the gradient's second read;
- *   any other shape: one CTA per row.
+ *   16-byte aligned arrays: a row held in the shared memory of one CTA, or of a
+ *     cluster of 2 to 16 (the smallest whose slices fit) beside a helper grid on
+ *     the remaining SMs; where vocab or ld is not a multiple of a 16-byte vector,
+ *     a row's first and last vectors are masked;
+ *   rows longer than a cluster of 16 holds (152,576 fp32 columns, 305,152 bf16
+ *     ones): fp32 with vocab and ld multiples of 4 on clusters of 8 CTAs (4 for
+ *     sampled-token rows) that stream each row twice, beside a helper grid, the
+ *     first read of each chunk marked L2 evict-last and its lines returned to
+ *     normal priority after the second; others one CTA per row;
+ *   other arrays: one CTA per row.
  */
 turnopd_status turnopd_loss_fwd_bwd(const void *z_student, const void *z_teacher,
                                     int32_t in_dtype, int64_t ld, int64_t vocab,

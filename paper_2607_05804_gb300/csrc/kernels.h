@@ -91,6 +91,7 @@ struct RowIn {
     // split_den > 0: the cluster kernel takes rows [0, nvalid split_num / split_den) of the
     // row list and the helper kernel the rest (set by launch_row_cluster)
     int32_t split_num, split_den;
+    int32_t split_ctas;  // CTAs of the helper grid (held-row kernels: its share comes in whole turns)
     int64_t elems;  // logits from the arrays' start to the last row's last column
 };
 
@@ -174,13 +175,17 @@ size_t fused_workspace_bytes(int64_t T, int64_t V, int64_t d_s, int64_t d_t);
 size_t fused_workspace_min_bytes(int64_t T, int64_t V, int64_t d_s, int64_t d_t);
 cudaError_t launch_fused(const FusedCall &c, cudaStream_t stream);
 
-// Cluster-resident kernel for aligned bf16 rows; sets *used = false (and
-// launches nothing) when the shape does not fit it.
-cudaError_t launch_row_cluster(const RowIn &p, bool fp32_grad, cudaStream_t stream, bool *used);
-// The same for a vocabulary or stride that is not a multiple of 8 (masked end vectors).
-cudaError_t launch_row_cluster_tail(const RowIn &p, bool fp32_grad, cudaStream_t stream, bool *used);
-// Split-row kernel (clusters of CTAs share each row) for aligned fp32 rows; sets
-// *used = false (and launches nothing) when the shape does not fit it.
-cudaError_t launch_row_split(const RowIn &p, bool fp32_grad, cudaStream_t stream, bool *used);
+// The row grids for 16-byte aligned arrays; sets *used = false (and launches nothing) for
+// others, which the portable kernel takes.
+cudaError_t launch_rows(const RowIn &p, bool bf16, bool fp32_grad, cudaStream_t stream, bool *used);
+// Its sets of kernels: rows held whole in the shared memory of a CTA or a cluster, by type,
+// and ragged (vocabulary or stride no multiple of a 16-byte vector: masked end vectors).
+cudaError_t launch_rows_bf16(const RowIn &p, bool fp32_grad, cudaStream_t stream);
+cudaError_t launch_rows_bf16_ragged(const RowIn &p, bool fp32_grad, cudaStream_t stream);
+cudaError_t launch_rows_f32(const RowIn &p, bool fp32_grad, cudaStream_t stream);
+cudaError_t launch_rows_f32_ragged(const RowIn &p, bool fp32_grad, cudaStream_t stream);
+// Split-row kernel (clusters of CTAs stream each row twice) for fp32 rows longer than a
+// cluster holds, vocab and ld multiples of 4.
+cudaError_t launch_row_split(const RowIn &p, bool fp32_grad, cudaStream_t stream);
 
 }  // namespace turnopd

@@ -1,17 +1,33 @@
-// The bf16 row path's entry: the row grids of rowkl_cluster.cuh for vocabularies and
-// row strides that are multiples of 8.  Others take the same kernels compiled with
-// masked first and last vectors, in their own translation unit
-// (rowkl_cluster_tail.cu), so that neither set slows the other's build or changes its code.
+// The row path's entry, and the row grids of rowkl_cluster.cuh for bf16 logits whose
+// vocabulary and row stride are multiples of 8.  The grids for other rows and for fp32
+// logits are the same kernels, each set in its own translation unit, so that none slows
+// another's build or changes its code.
 
 #include "rowkl_cluster.cuh"
 
 namespace turnopd {
 
-cudaError_t launch_row_cluster(const RowIn &p, bool fp32_grad, cudaStream_t stream, bool *used)
+cudaError_t launch_rows_bf16(const RowIn &p, bool fp32_grad, cudaStream_t stream)
 {
-    if (p.vocab % 8 != 0 || p.ld % 8 != 0)
-        return launch_row_cluster_tail(p, fp32_grad, stream, used);
-    return launch_row_cluster_t<false>(p, fp32_grad, stream, used);
+    return launch_rows_t<__nv_bfloat16, false>(p, fp32_grad, stream);
+}
+
+// *used = false (and nothing is launched) for arrays that are not 16-byte aligned.
+cudaError_t launch_rows(const RowIn &p, bool bf16, bool fp32_grad, cudaStream_t stream, bool *used)
+{
+    auto al16 = [](const void *q) { return (reinterpret_cast<uintptr_t>(q) & 15u) == 0; };
+    *used = al16(p.zs) && al16(p.zt) && (!p.grad || al16(p.grad)) && p.vocab <= (int64_t)INT32_MAX - 16;
+    if (!*used)
+        return cudaSuccess;
+    const int n = bf16 ? 8 : 4;
+    const bool whole = p.vocab % n == 0 && p.ld % n == 0;
+    if (bf16)
+        return whole ? launch_rows_bf16(p, fp32_grad, stream) : launch_rows_bf16_ragged(p, fp32_grad, stream);
+    // rows longer than 16 CTAs hold are streamed twice (V = 151,936 on clusters of 8: 5,400
+    // GB/s, held by clusters of 16: 6,020)
+    if (whole && cluster_size((int)(p.vocab / 4)) == 0)
+        return launch_row_split(p, fp32_grad, stream);
+    return whole ? launch_rows_f32(p, fp32_grad, stream) : launch_rows_f32_ragged(p, fp32_grad, stream);
 }
 
 }  // namespace turnopd

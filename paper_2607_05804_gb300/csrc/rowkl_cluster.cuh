@@ -1,29 +1,29 @@
-// Cluster-resident row kernel for the per-token OPD loss (sm_103a).
+// Held-row kernels for the per-token OPD loss (sm_103a): bf16 and fp32 logits, any
+// vocabulary and row stride.
 //
-// One logit row of V = 151,936 bf16 values is 303,872 bytes per model: the
-// student and teacher rows together (607 KB) do not fit one SM, and the
-// gradient needs both rows twice (statistics, then p_s and z_s - z_t).  A
-// cluster of CS CTAs therefore owns one row at a time: CTA c holds vector
-// slice c of both rows in shared memory, so HBM is read exactly once per row
-// and the gradient written once (911,616 algorithmic bytes per row in bf16).
+// The gradient needs both rows of a token twice (statistics, then p_s and z_s - z_t).  A
+// CTA, or a cluster of CTAs where the rows are longer than one's shared memory holds (V =
+// 151,936 bf16: 607 KB for the two, 8 CTAs; fp32: 16), therefore owns one row at a time:
+// CTA c of CS holds vector slice c of both in shared memory, so HBM is read exactly once per
+// row and the gradient written once (911,616 algorithmic bytes per row in bf16).
 //
 // Per CTA (persistent, one per SM, rows cid, cid + nclusters, ...):
-//   * thread 0 streams slices into a 3-stage ring with bulk asynchronous
-//     copies (cp.async.bulk, completion on a "full" mbarrier, L2 evict-first);
-//     a stage is refilled once every warp has arrived on its "empty" mbarrier;
-//   * stats(k+1): per thread a max pass (packed bf16x2 max) and a sum pass
+//   * slices stream into a ring of ST stages with bulk asynchronous copies
+//     (cp.async.bulk, completion on a "full" mbarrier, L2 evict-first); a stage is refilled
+//     once every warp of the group that used it has arrived on its "empty" mbarrier;
+//   * G groups of threads take the rows in turn: while one waits for its row's data or
+//     records, the others compute;
+//   * stats(k): per thread a max pass (packed bf16x2 max) and a sum pass
 //     (packed f32x2 arithmetic): S = sum exp(z - m) for both models and
 //     A = sum exp(z_s - m_s)((z_s - z_t) - d), d taken at the student's max.
 //     The CTA's partial is pushed to every CTA of the cluster with st.async
-//     into a 4-slot record ring; completion lands on the receiver's mbarrier
+//     into a record ring; completion lands on the receiver's mbarrier
 //     (32 bytes per sender), so no cluster-wide barrier runs per row;
-//   * grad(k) from the resident slice of the previous row, overlapping the
-//     record exchange of row k+1;
-//   * every warp merges the CS records by the same fixed 8-lane tree, so all
-//     CTAs use bit-identical LSE and KL (deterministic).
-// Each thread reads its vectors of a row from shared memory twice: once into
-// registers for the maxima and sums, once for the gradient (3 exponentials
-// per element in all).
+//   * the group's first warp merges the CS records by the same fixed lane tree, so all
+//     CTAs use bit-identical LSE and KL (deterministic);
+//   * grad(k) from the resident slice.
+// Each thread reads its vectors of a row from shared memory three times: for the maxima,
+// for the sums and for the gradient (3 exponentials per element in all).
 // Clusters of 8 fill 120 of the 152 SMs; a helper grid of one 512-thread CTA per
 // free SM takes the last share of the rows, each row read from HBM once (staged
 // through a cp.async ring) and again from L2 (k_row_helper below).
@@ -43,7 +43,6 @@
 namespace turnopd {
 namespace {
 
-constexpr int kStages = 3;
 constexpr uint32_t kCopyChunk = 65536;       // bytes per bulk copy instruction
 constexpr uint32_t kWaitLimit = 1u << 22;    // mbarrier polls before giving up
 
@@ -60,81 +59,207 @@ struct GradConst {
 
 // What a lane that does not count reads as: -2^127.  It adds 0 beside any real logit, and
 // where a thread or a vector holds nothing else its maximum times log2 e is still finite
-// (the lowest finite bf16's is not: exp2(-inf + inf) made such a row NaN).
-constexpr uint32_t kFillLane = 0xff00u;
+// (the lowest finite value's is not: exp2(-inf + inf) made such a row NaN).
+constexpr uint32_t kFillHi = 0xff00u;            // the upper 16 bits; as bf16 and, shifted, as fp32
 
-// v with its bf16 lanes outside [lo, hi) replaced by kFillLane (the lanes
-// of a row's first and last vectors that belong to other rows or to padding)
-__device__ __forceinline__ uint4 keep_lanes(uint4 v, int lo, int hi)
-{
-    uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const bool in0 = 2 * j >= lo && 2 * j < hi, in1 = 2 * j + 1 >= lo && 2 * j + 1 < hi;
-        w[j] = (in0 ? w[j] & 0x0000ffffu : kFillLane) | (in1 ? w[j] & 0xffff0000u : kFillLane << 16);
+// One 16-byte vector of logits: N elements, NP pairs of them, and the running maximum of
+// vectors (packed for bf16).
+template <typename T> struct Elem;
+template <> struct Elem<__nv_bfloat16> {
+    static constexpr int N = 8, NP = 4, LOG = 3;
+    static constexpr uint32_t kFillWord = kFillHi | kFillHi << 16;
+    using Max = uint32_t;  // two candidates
+    __device__ static Max max_empty() { return 0xff80ff80u; }  // (-inf, -inf)
+    __device__ static Max max_of(const uint4 &v) { return hmax4(v); }
+    __device__ static Max max2(Max a, Max b) { return hmax2u(a, b); }
+    __device__ static float value(Max m) { return fmaxf(bf16lo(m), bf16hi(m)); }
+    __device__ static bool has(Max m, float x) { return bf16lo(m) == x || bf16hi(m) == x; }
+    __device__ static float2 pair(const uint4 &v, int j) { return unpack2(word(v, j)); }
+    // v with lane i replaced by the fill
+    __device__ static uint4 fill_lane(uint4 v, int i)
+    {
+        const uint32_t keep = (i & 1) ? 0x0000ffffu : 0xffff0000u;
+        const uint32_t fill = kFillWord & ~keep;
+        const int w = i >> 1;
+        v.x = w == 0 ? (v.x & keep) | fill : v.x;
+        v.y = w == 1 ? (v.y & keep) | fill : v.y;
+        v.z = w == 2 ? (v.z & keep) | fill : v.z;
+        v.w = w == 3 ? (v.w & keep) | fill : v.w;
+        return v;
     }
-    return make_uint4(w[0], w[1], w[2], w[3]);
+    // v with its lanes outside [lo, hi) replaced by the fill (the lanes of a row's first
+    // and last vectors that belong to other rows or to padding)
+    __device__ static uint4 keep_lanes(uint4 v, int lo, int hi)
+    {
+        uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const bool in0 = 2 * j >= lo && 2 * j < hi, in1 = 2 * j + 1 >= lo && 2 * j + 1 < hi;
+            w[j] = (in0 ? w[j] & 0x0000ffffu : kFillHi) | (in1 ? w[j] & 0xffff0000u : kFillHi << 16);
+        }
+        return make_uint4(w[0], w[1], w[2], w[3]);
+    }
+    // lanes [lo, hi) of the vector at p read one element at a time, the others the fill: the
+    // vector that would pass the end of the logits
+    __device__ static uint4 load_lanes(const __nv_bfloat16 *p, int lo, int hi)
+    {
+        uint32_t w[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const uint32_t e0 = 2 * j >= lo && 2 * j < hi ? __bfloat16_as_ushort(p[2 * j]) : kFillHi;
+            const uint32_t e1 = 2 * j + 1 >= lo && 2 * j + 1 < hi ? __bfloat16_as_ushort(p[2 * j + 1]) : kFillHi;
+            w[j] = e0 | (e1 << 16);
+        }
+        return make_uint4(w[0], w[1], w[2], w[3]);
+    }
+    // the element at shared address `a` replaced by the fill; returns it
+    __device__ static float swap_shared(uint32_t a)
+    {
+        uint32_t old;
+        asm volatile("ld.shared.u16 %0, [%1];\n\tst.shared.u16 [%1], %2;\n\t" : "=r"(old) : "r"(a), "r"(kFillHi) : "memory");
+        return __uint_as_float(old << 16);
+    }
+};
+template <> struct Elem<float> {
+    static constexpr int N = 4, NP = 2, LOG = 2;
+    static constexpr uint32_t kFillWord = kFillHi << 16;
+    using Max = float;
+    __device__ static Max max_empty() { return -INFINITY; }
+    __device__ static Max max_of(const uint4 &v)
+    {
+        return fmaxf(fmaxf(__uint_as_float(v.x), __uint_as_float(v.y)), fmaxf(__uint_as_float(v.z), __uint_as_float(v.w)));
+    }
+    __device__ static Max max2(Max a, Max b) { return fmaxf(a, b); }
+    __device__ static float value(Max m) { return m; }
+    __device__ static bool has(Max m, float x) { return m == x; }
+    __device__ static float2 pair(const uint4 &v, int j)
+    {
+        return j == 0 ? make_float2(__uint_as_float(v.x), __uint_as_float(v.y))
+                      : make_float2(__uint_as_float(v.z), __uint_as_float(v.w));
+    }
+    __device__ static uint4 fill_lane(uint4 v, int i)
+    {
+        v.x = i == 0 ? kFillWord : v.x;
+        v.y = i == 1 ? kFillWord : v.y;
+        v.z = i == 2 ? kFillWord : v.z;
+        v.w = i == 3 ? kFillWord : v.w;
+        return v;
+    }
+    __device__ static uint4 keep_lanes(uint4 v, int lo, int hi)
+    {
+        v.x = lo <= 0 && hi > 0 ? v.x : kFillWord;
+        v.y = lo <= 1 && hi > 1 ? v.y : kFillWord;
+        v.z = lo <= 2 && hi > 2 ? v.z : kFillWord;
+        v.w = lo <= 3 && hi > 3 ? v.w : kFillWord;
+        return v;
+    }
+    __device__ static uint4 load_lanes(const float *p, int lo, int hi)
+    {
+        uint32_t w[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            w[j] = j >= lo && j < hi ? __float_as_uint(p[j]) : kFillWord;
+        return make_uint4(w[0], w[1], w[2], w[3]);
+    }
+    __device__ static float swap_shared(uint32_t a)
+    {
+        uint32_t old;
+        asm volatile("ld.shared.u32 %0, [%1];\n\tst.shared.u32 [%1], %2;\n\t" : "=r"(old) : "r"(a), "r"(kFillWord) : "memory");
+        return __uint_as_float(old);
+    }
+};
+
+// One vector of the gradient, g[NP] pairs, stored whole: vector q of the row at `off`.
+template <typename T, bool G32>
+__device__ __forceinline__ void store_grad(void *grad, size_t off, int q, const float2 *g)
+{
+    constexpr int N = Elem<T>::N, NP = Elem<T>::NP;
+    if (G32) {
+        float4 *dst = reinterpret_cast<float4 *>(static_cast<float *>(grad) + off + (size_t)q * N);
+        __stcs(dst, make_float4(g[0].x, g[0].y, g[1].x, g[1].y));
+        if (NP == 4)
+            __stcs(dst + 1, make_float4(g[NP - 2].x, g[NP - 2].y, g[NP - 1].x, g[NP - 1].y));
+    } else if (NP == 4) {
+        uint4 o;
+        o.x = pack_bf16x2(g[0].x, g[0].y);
+        o.y = pack_bf16x2(g[1].x, g[1].y);
+        o.z = pack_bf16x2(g[NP - 2].x, g[NP - 2].y);
+        o.w = pack_bf16x2(g[NP - 1].x, g[NP - 1].y);
+        __stcs(reinterpret_cast<uint4 *>(static_cast<__nv_bfloat16 *>(grad) + off + (size_t)q * N), o);
+    } else {
+        uint2 o;
+        o.x = pack_bf16x2(g[0].x, g[0].y);
+        o.y = pack_bf16x2(g[1].x, g[1].y);
+        __stcs(reinterpret_cast<uint2 *>(static_cast<__nv_bfloat16 *>(grad) + off + (size_t)q * N), o);
+    }
 }
 
-// Lanes [lo, hi) of the vector at p read one element at a time (the others
-// kFillLane): the vector that would pass the end of the logits.
-__device__ __forceinline__ uint4 load_lanes(const __nv_bfloat16 *p, int lo, int hi)
+// Columns [lo, hi) of one vector of the gradient, one at a time.
+template <typename T, bool G32>
+__device__ __forceinline__ void store_grad_lanes(void *grad, size_t e, const float2 *g, int lo, int hi)
 {
-    uint32_t w[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const uint32_t e0 = 2 * j >= lo && 2 * j < hi ? __bfloat16_as_ushort(p[2 * j]) : kFillLane;
-        const uint32_t e1 = 2 * j + 1 >= lo && 2 * j + 1 < hi ? __bfloat16_as_ushort(p[2 * j + 1]) : kFillLane;
-        w[j] = e0 | (e1 << 16);
-    }
-    return make_uint4(w[0], w[1], w[2], w[3]);
+    for (int i = 0; i < Elem<T>::N; ++i)
+        if (i >= lo && i < hi) {
+            const float x = i & 1 ? g[i / 2].y : g[i / 2].x;
+            if (G32)
+                static_cast<float *>(grad)[e + i] = x;
+            else
+                static_cast<__nv_bfloat16 *>(grad)[e + i] = __float2bfloat16_rn(x);
+        }
 }
 
-// Ragged rows (TL): the row stride or the vocabulary is no multiple of 8, so a row starts
-// `head` elements into a 16-byte vector and ends `tail` elements into one (tail 0: at its
-// end).  Its vectors are those of the 16-byte grid that hold any of its columns; the
-// first and the last may be partial.  (Rows of a stride that is no multiple of 8 took
-// the portable kernel's 2-byte loads before: dense 4 x 1024 tokens, V = 50,001, step
-// 1,075 us, now 216; 133 is its traffic at the copy bandwidth.)
+// Ragged rows (TL): the row stride or the vocabulary is no multiple of a vector's N
+// elements, so a row starts `head` elements into a 16-byte vector and ends `tail`
+// elements into one (tail 0: at its end).  Its vectors are those of the 16-byte grid that
+// hold any of its columns; the first and the last may be partial.  (Rows of a stride that
+// is no multiple of 8 took the portable kernel's 2-byte loads before: dense 4 x 1024
+// tokens, V = 50,001, bf16, step 1,075 us, now 216; 133 is its traffic at the copy
+// bandwidth.)
 struct Ragged {
     int head, nvec, tail;
 };
-__device__ __forceinline__ Ragged ragged(int row, int64_t ld, int64_t vocab)
+template <typename T> __device__ __forceinline__ Ragged ragged(int row, int64_t ld, int64_t vocab)
 {
+    constexpr int N = Elem<T>::N;
     Ragged g;
-    g.head = ((row & 7) * (int)(ld & 7)) & 7;
-    g.nvec = (int)((g.head + vocab + 7) >> 3);
-    g.tail = (int)((g.head + vocab) & 7);
+    g.head = ((row & (N - 1)) * (int)(ld & (N - 1))) & (N - 1);
+    g.nvec = (int)((g.head + vocab + N - 1) / N);
+    g.tail = (int)((g.head + vocab) & (N - 1));
     return g;
 }
 
-// v with its bf16 lane i (0..7) replaced by kFillLane
-__device__ __forceinline__ uint4 fill_lane(uint4 v, int i)
+// The clusters' share of nvalid rows: the host's ratio, with a helper grid of few rows a
+// CTA rounded down to whole turns (a helper CTA takes as long for a row as a cluster for
+// eight, so a last turn of a few CTAs holds up a small batch).
+__device__ __forceinline__ int split_rows(const RowIn &p, int nvalid)
 {
-    const uint32_t keep = (i & 1) ? 0x0000ffffu : 0xffff0000u;
-    const uint32_t fill = (kFillLane | kFillLane << 16) & ~keep;
-    const int w = i >> 1;
-    v.x = w == 0 ? (v.x & keep) | fill : v.x;
-    v.y = w == 1 ? (v.y & keep) | fill : v.y;
-    v.z = w == 2 ? (v.z & keep) | fill : v.z;
-    v.w = w == 3 ? (v.w & keep) | fill : v.w;
-    return v;
+    if (!p.split_den)
+        return nvalid;
+    const int h = nvalid - (int)((int64_t)nvalid * p.split_num / p.split_den);
+    return nvalid - (h >= p.split_ctas && h < 8 * p.split_ctas ? h - h % p.split_ctas : h);
 }
 
-// G groups of NT threads per CTA take the rows of the cluster in turn (row k
-// to group k % G).  Record slots: 2G, so a slot is reused by the same group
-// two rows later, after that group has read it (a peer can run at most G rows
-// ahead of the slowest CTA in sending records).  SM: a sampled-token call, where
-// every listed row carries its y in [0, V); otherwise the full vocabulary (y = -1).
-template <int CS, int NT, int VPT, int G, bool G32, bool SM, bool TL>
+// G groups of NT threads per CTA take the rows of the cluster in turn (row k to group
+// k % G), each thread VPT vectors of each model, from a ring of ST stages.  Record slots:
+// 2G, so a slot is reused by the same group two rows later, after that group has read it
+// (a peer can run at most G rows ahead of the slowest CTA in sending records).  SM: a
+// sampled-token call, where every listed row carries its y in [0, V); otherwise the full
+// vocabulary (y = -1).  TL: ragged rows.
+template <typename T, int CS, int NT, int VPT, int G, int ST, bool G32, bool SM, bool TL>
 __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_vec, int nvec)
 {
+    using E = Elem<T>;
+    constexpr int N = E::N, NP = E::NP;
+    constexpr int kStages = ST;
     constexpr int kSlots = 2 * G;
+    static_assert(G <= 15 || NT == 32, "one named barrier per group");
     // Reference difference d (A = sum e ((z_s - z_t) - d), d at the student's
     // max): it keeps gradients at a dominant token accurate to fp32 relative
     // precision.  A bf16 gradient needs no such care: without d the error of
-    // E_p[z_s - z_t] is ~1e-6 absolute, under a bf16 ulp of those gradients.
-    constexpr bool kUseD = G32;
+    // E_p[z_s - z_t] is ~1e-6 absolute, under a bf16 ulp of those gradients.  (fp32
+    // logits always keep it.)
+    constexpr bool kUseD = G32 || N == 4;
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ int s_dead;
     constexpr int NWG = NT / 32;  // warps per group
@@ -147,7 +272,7 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
     const int v0 = (int)rank * slice_vec;  // first vector of my slice
     const int my_vec = max(0, min(slice_vec, nvec - v0));
     // TL (ragged rows): the slice's vectors and the partial ones among them vary from row
-    // to row.  A partial vector's other lanes read as kFillLane in the
+    // to row.  A partial vector's other lanes read as the fill in the
     // statistics (set in shared memory by the thread that reads the vector) and are
     // never written: the gradient loop stores whole vectors, that thread the partial
     // one's columns.  Without TL all of this compiles away.
@@ -159,7 +284,7 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
     auto slice_of = [&](int row) {
         Slice g{my_vec, 0, 0, my_vec, -1, 0, false, false};
         if (TL) {
-            const Ragged r = ragged(row, p.ld, p.vocab);
+            const Ragged r = ragged<T>(row, p.ld, p.vocab);
             g.my_vec = max(0, min(slice_vec, r.nvec - v0));
             g.head0 = r.head;
             g.head = v0 == 0 && r.head > 0;
@@ -167,7 +292,7 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
             g.tailq = r.tail && g.my_vec > 0 && v0 + g.my_vec == r.nvec ? g.my_vec - 1 : -1;
             g.g0 = g.head ? 1 : 0;
             g.gvec = g.tailq >= 0 ? g.my_vec - 1 : g.my_vec;
-            g.cut = g.tailq >= 0 && (int64_t)row * p.ld - r.head + (int64_t)r.nvec * 8 > p.elems;
+            g.cut = g.tailq >= 0 && (int64_t)row * p.ld - r.head + (int64_t)r.nvec * N > p.elems;
         }
         return g;
     };
@@ -179,9 +304,9 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
     uint64_t *empty = full + kStages;                                      // [kStages]
     uint64_t *recv = empty + kStages;                                      // [kSlots]
     float *red = reinterpret_cast<float *>(recv + kSlots);                 // [G][NWG][8]
-    int *srow = reinterpret_cast<int *>(red + G * NWG * 8);                // [kStages] row in stage
-    int *yown = srow + 4;                                                  // [kStages] thread reading y, or -1
-    float *rcs = reinterpret_cast<float *>(srow + 8);                       // [G][16] row constants; [15]: z_s[y]
+    int *srow = reinterpret_cast<int *>(red + G * NWG * 8);            // [kStages] row in stage
+    int *yown = srow + (kStages + 3) / 4 * 4;                                            // [kStages] thread reading y, or -1
+    float *rcs = reinterpret_cast<float *>(yown + (kStages + 3) / 4 * 4);                 // [G][16] row constants; [15]: z_s[y]
 
     if (tid == 0) {
         s_dead = 0;
@@ -190,27 +315,30 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
             mbar_init(&empty[s], NWG);
             srow[s] = -1;
         }
-        for (int s = 0; s < kSlots; ++s)
-            mbar_init(&recv[s], 1);
+        if (CS > 1)
+            for (int s = 0; s < kSlots; ++s)
+                mbar_init(&recv[s], 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        for (int s = 0; s < kSlots; ++s)
-            mbar_arrive_expect_tx(&recv[s], CS * 32u);  // first record of each slot
+        if (CS > 1)
+            for (int s = 0; s < kSlots; ++s)
+                mbar_arrive_expect_tx(&recv[s], CS * 32u);  // first record of each slot
     }
     __syncthreads();
-    cluster_sync();  // peers' barriers are initialised before any record is sent
+    if (CS > 1)
+        cluster_sync();  // peers' barriers are initialised before any record is sent
     // Every CTA of this grid is resident: a helper grid launched after this one may
     // start now, on the SMs the clusters left free.
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     const int nv_all = *p.nvalid;
-    const int nvalid = p.split_den ? (int)((int64_t)nv_all * p.split_num / p.split_den) : nv_all;
+    const int nvalid = split_rows(p, nv_all);
     const int n = nvalid > cid ? (nvalid - cid + ncl - 1) / ncl : 0;  // same for the whole cluster
     if (n == 0)
         return;
 
-    const __nv_bfloat16 *zs = static_cast<const __nv_bfloat16 *>(p.zs);
-    const __nv_bfloat16 *zt = static_cast<const __nv_bfloat16 *>(p.zt);
+    const T *zs = static_cast<const T *>(p.zs);
+    const T *zt = static_cast<const T *>(p.zt);
 
     auto dead = [&]() { return *(volatile int *)&s_dead != 0; };
     auto wait_bar = [&](uint64_t *bar, uint32_t parity, bool cluster_scope) {
@@ -222,7 +350,12 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
         s_dead = 1;
         set_status(p.status, TURNOPD_ERR_TIMEOUT);
     };
-    auto group_sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "r"(NT) : "memory"); };
+    auto group_sync = [&]() {
+        if (NT == 32)
+            __syncwarp();
+        else
+            asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "r"(NT) : "memory");
+    };
 
     // Data of row k: wait until the stage has been armed for row k, then for
     // its phase.  (A parity wait alone would also accept the phase of the
@@ -249,12 +382,12 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
         const Slice g = slice_of(m.y);
         meta[s] = m;
         if (SM) {  // the thread that will read y's vector (sampled-token rows; see stats)
-            const int q = m.z >= 0 ? ((m.z + g.head0) >> 3) - v0 : -1;
+            const int q = m.z >= 0 ? (m.z + g.head0) / N - v0 : -1;
             yown[s] = q >= 0 && q < g.my_vec ? q % NT : -1;
         }
         *(volatile int *)&srow[s] = k;
         const uint32_t my_bytes = (uint32_t)(TL && g.cut ? g.my_vec - 1 : g.my_vec) * 16u;
-        const size_t off = (size_t)m.y * (size_t)p.ld - (size_t)g.head0 + (size_t)v0 * 8;
+        const size_t off = (size_t)m.y * (size_t)p.ld - (size_t)g.head0 + (size_t)v0 * N;
         const char *gs = reinterpret_cast<const char *>(zs + off);
         const char *gt = reinterpret_cast<const char *>(zt + off);
         unsigned char *ds = stage + s * stage_bytes;
@@ -267,7 +400,33 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
         }
     };
 
-    // statistics of row k: this CTA's record into slot k % kSlots of every CTA
+    // row k's constants for the gradient pass from its merged statistics and its sampled
+    // token's logits (one thread of the group)
+    auto row_constants = [&](int k, Student A, const Teacher &B, float ys, float yt) {
+        float *bc = rcs + group * 16;
+        float omp = 0.f;  // 1 - p_y (sampled)
+        if (SM)
+            omp = add_sampled_term(A, ys);
+        const RowConst rc = row_const(A, B);
+        float e = rc.kl;
+        if (SM)
+            e = (ys - yt) - rc.dl;
+        // gradient constants of the row (see grad): p w = 2^(z_s log2e + nlw),
+        // sign sg of w applied through fma by (sg, sg)
+        const float wi = __int_as_float(meta[k % kStages].w), wl = wi * e;
+        const float sg = wi < 0.f ? -1.f : 1.f;
+        bc[0] = rc.lse_s, bc[1] = rc.lse_t, bc[2] = rc.kl, bc[3] = e;
+        bc[4] = -rc.lse_s * kLog2e + log2f(fabsf(SM ? wl : wi));  // nlw
+        bc[5] = sg;
+        bc[6] = -sg * rc.d;
+        bc[7] = -sg * rc.cp;
+        bc[8] = -sg * (rc.d + rc.cp);     // bf16 output: one rounding of d + cp
+        bc[9] = wl > 0.f ? -1.f : 1.f;    // sampled: sign of -w l
+        bc[10] = wl * omp;                 // sampled: g_y = w l (1 - p_y)
+    };
+
+    // statistics of row k: this CTA's record into slot k % kSlots of every CTA (a cluster
+    // of one: the row's constants at once)
     auto stats = [&](int k) {
         const int s = k % kStages;
         const uint4 *vs = reinterpret_cast<const uint4 *>(stage + s * stage_bytes);
@@ -280,66 +439,60 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
             uint4 *wt = reinterpret_cast<uint4 *>(stage + s * stage_bytes + slice_bytes);
             if (g.tailq >= 0 && g.tailq % NT == gtid) {
                 if (g.cut) {
-                    const size_t e = (size_t)meta[s].y * (size_t)p.ld - (size_t)g.head0 + (size_t)(v0 + g.tailq) * 8;
-                    ws[g.tailq] = load_lanes(zs + e, 0, g.tail);
-                    wt[g.tailq] = load_lanes(zt + e, 0, g.tail);
+                    const size_t e = (size_t)meta[s].y * (size_t)p.ld - (size_t)g.head0 + (size_t)(v0 + g.tailq) * N;
+                    ws[g.tailq] = E::load_lanes(zs + e, 0, g.tail);
+                    wt[g.tailq] = E::load_lanes(zt + e, 0, g.tail);
                 } else {
-                    ws[g.tailq] = keep_lanes(ws[g.tailq], 0, g.tail);
-                    wt[g.tailq] = keep_lanes(wt[g.tailq], 0, g.tail);
+                    ws[g.tailq] = E::keep_lanes(ws[g.tailq], 0, g.tail);
+                    wt[g.tailq] = E::keep_lanes(wt[g.tailq], 0, g.tail);
                 }
             }
             if (g.head && gtid == 0) {
-                ws[0] = keep_lanes(ws[0], g.head0, 8);
-                wt[0] = keep_lanes(wt[0], g.head0, 8);
+                ws[0] = E::keep_lanes(ws[0], g.head0, N);
+                wt[0] = E::keep_lanes(wt[0], g.head0, N);
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         }
         // A sampled-token row leaves y out of the student statistics (add_sampled_term
         // brings its term back at the merge): the thread that reads y's vector in both
-        // passes below (named at issue) keeps z_s[y] for the record and puts kFillLane
+        // passes below (named at issue) keeps z_s[y] for the record and puts the fill
         // in its place, which adds 0.  (The gradient
         // pass replaces g_y; the proxy fence orders the store before the stage's next
         // bulk copy.)
         if (SM && yown[s] == gtid) {
-            const uint32_t ay = smem_u32(stage + s * stage_bytes) + 2u * (uint32_t)(meta[s].z + g.head0 - v0 * 8);
-            uint32_t old;
-            asm volatile("ld.shared.u16 %0, [%1];\n\tst.shared.u16 [%1], %2;\n\t"
-                         "fence.proxy.async.shared::cta;"
-                         : "=r"(old)
-                         : "r"(ay), "r"(kFillLane)
-                         : "memory");
-            rcs[group * 16 + 15] = __uint_as_float(old << 16);
+            rcs[group * 16 + 15] = E::swap_shared(smem_u32(stage + s * stage_bytes) +
+                                                  (uint32_t)sizeof(T) * (uint32_t)(meta[s].z + g.head0 - v0 * N));
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         }
-        // max pass (packed bf16): running maxima, plus each vector's student
-        // maximum kept packed so the argmax vector is found after the loop
-        uint32_t smax = 0xff80ff80u, tmax = 0xff80ff80u;  // (-inf, -inf)
-        uint32_t vmax[VPT];
+        // max pass (packed for bf16): running maxima, plus each vector's student
+        // maximum so the argmax vector is found after the loop
+        typename E::Max smax = E::max_empty(), tmax = E::max_empty();
+        typename E::Max vmax[VPT];
 #pragma unroll
         for (int u = 0; u < VPT; ++u) {
             const int q = gtid + u * NT;
-            vmax[u] = 0xff80ff80u;
+            vmax[u] = E::max_empty();
             if (q < my_vec) {
                 const uint4 a = vs[q], b = vt[q];
-                vmax[u] = hmax2u(hmax2u(a.x, a.y), hmax2u(a.z, a.w));
-                smax = hmax2u(smax, vmax[u]);
-                tmax = hmax2u(tmax, hmax2u(hmax2u(b.x, b.y), hmax2u(b.z, b.w)));
+                vmax[u] = E::max_of(a);
+                smax = E::max2(smax, vmax[u]);
+                tmax = E::max2(tmax, E::max_of(b));
             }
         }
-        const float ms = fmaxf(bf16lo(smax), bf16hi(smax)), mt = fmaxf(bf16lo(tmax), bf16hi(tmax));
-        // reference difference at the first element equal to the student max;
-        // only the fp32 gradient needs it (see kUseD)
+        const float ms = E::value(smax), mt = E::value(tmax);
+        // reference difference at the first element equal to the student max (see kUseD)
         float xd = 0.f;
         if (kUseD && ms != -INFINITY) {
             int bq = gtid;
 #pragma unroll
             for (int u = VPT - 1; u >= 0; --u)
-                if (bf16lo(vmax[u]) == ms || bf16hi(vmax[u]) == ms)
+                if (E::has(vmax[u], ms))
                     bq = gtid + u * NT;
             const uint4 a = vs[bq], b = vt[bq];
             bool found = false;
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const float2 x = unpack2(word(a, j)), y = unpack2(word(b, j));
+            for (int j = 0; j < NP; ++j) {
+                const float2 x = E::pair(a, j), y = E::pair(b, j);
                 if (!found && x.x == ms) {
                     xd = x.x - y.x;
                     found = true;
@@ -360,8 +513,8 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
             if (q < my_vec) {
                 const uint4 a = vs[q], b = vt[q];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const float2 a2 = unpack2(word(a, j)), b2 = unpack2(word(b, j));
+                for (int j = 0; j < NP; ++j) {
+                    const float2 a2 = E::pair(a, j), b2 = E::pair(b, j);
                     const float2 es = ex2x2(ffma2(a2, L2, NS));
                     S2 = fadd2(S2, es);
                     A2 = ffma2(es, kUseD ? fsub2(fsub2(a2, b2), D) : fsub2(a2, b2), A2);
@@ -387,6 +540,12 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
                 B = Teacher{r[4], r[5]};
             }
             lane_merge<NWG, kUseD>(A, B);
+            if (CS == 1) {  // the CTA's partial is the row's
+                if (lane == 0)
+                    row_constants(k, A, B, SM ? rcs[group * 16 + 15] : 0.f,
+                                  SM ? to_float(reinterpret_cast<const T *>(vt)[meta[s].z + g.head0]) : 0.f);
+                return;
+            }
             A.m = __shfl_sync(0xffffffffu, A.m, 0);
             A.s = __shfl_sync(0xffffffffu, A.s, 0);
             A.a = __shfl_sync(0xffffffffu, A.a, 0);
@@ -396,10 +555,10 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
             if (lane < CS) {
                 float ys = 0.f, yt = 0.f;  // sampled-token logits, from the CTA holding y
                 const int y = meta[s].z, yh = y + g.head0;
-                if (y >= 0 && yh / 8 >= v0 && yh / 8 < v0 + my_vec) {
-                    const int e = yh - v0 * 8;
-                    ys = SM ? rcs[group * 16 + 15] : to_float(reinterpret_cast<const __nv_bfloat16 *>(vs)[e]);
-                    yt = to_float(reinterpret_cast<const __nv_bfloat16 *>(vt)[e]);
+                if (y >= 0 && yh / N >= v0 && yh / N < v0 + my_vec) {
+                    const int e = yh - v0 * N;
+                    ys = SM ? rcs[group * 16 + 15] : to_float(reinterpret_cast<const T *>(vs)[e]);
+                    yt = to_float(reinterpret_cast<const T *>(vt)[e]);
                 }
                 const int slot = k % kSlots;
                 const uint32_t ra = mapa(smem_u32(rec + (slot * CS + (int)rank) * 8), (uint32_t)lane);
@@ -416,7 +575,7 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
     auto combine = [&](int k, float &ell) {
         const int slot = k % kSlots;
         float *bc = rcs + group * 16;
-        if (gwarp == 0) {
+        if (CS > 1 && gwarp == 0) {
             wait_bar(&recv[slot], (uint32_t)((k / kSlots) & 1), true);
             const float *r = rec + slot * CS * 8;
             Student A = student_empty();
@@ -430,27 +589,9 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
             lane_merge<CS, kUseD>(A, B);
             if (lane == 0) {
                 const int y = meta[k % kStages].z;
-                const int yh = TL ? y + ragged(meta[k % kStages].y, p.ld, p.vocab).head : y;
-                const int owner = SM ? (yh / 8) / slice_vec : 0;
-                float omp = 0.f;  // 1 - p_y (sampled)
-                if (SM)
-                    omp = add_sampled_term(A, r[owner * 8 + 6]);
-                const RowConst rc = row_const(A, B);
-                float e = rc.kl;
-                if (SM)
-                    e = (r[owner * 8 + 6] - r[owner * 8 + 7]) - rc.dl;
-                // gradient constants of the row (see grad): p w = 2^(z_s log2e + nlw),
-                // sign sg of w applied through fma by (sg, sg)
-                const float wi = __int_as_float(meta[k % kStages].w), wl = wi * e;
-                const float sg = wi < 0.f ? -1.f : 1.f;
-                bc[0] = rc.lse_s, bc[1] = rc.lse_t, bc[2] = rc.kl, bc[3] = e;
-                bc[4] = -rc.lse_s * kLog2e + log2f(fabsf(SM ? wl : wi));  // nlw
-                bc[5] = sg;
-                bc[6] = -sg * rc.d;
-                bc[7] = -sg * rc.cp;
-                bc[8] = -sg * (rc.d + rc.cp);     // bf16 output: one rounding of d + cp
-                bc[9] = wl > 0.f ? -1.f : 1.f;    // sampled: sign of -w l
-                bc[10] = wl * omp;                 // sampled: g_y = w l (1 - p_y)
+                const int yh = TL ? y + ragged<T>(meta[k % kStages].y, p.ld, p.vocab).head : y;
+                const int owner = SM ? (yh / N) / slice_vec : 0;
+                row_constants(k, A, B, r[owner * 8 + 6], r[owner * 8 + 7]);
                 mbar_arrive_expect_tx(&recv[slot], CS * 32u);  // re-arm for row k + kSlots
             }
         }
@@ -474,7 +615,7 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
         const float gy = gc.gy;
         const Slice sl = slice_of(m.y);
         const int gvec = sl.gvec;
-        const size_t row_off = (size_t)m.y * (size_t)p.ld - (size_t)sl.head0 + (size_t)v0 * 8;
+        const size_t row_off = (size_t)m.y * (size_t)p.ld - (size_t)sl.head0 + (size_t)v0 * N;
         // p |w| = 2^(z_s log2e - LSE_s log2e + log2 |w|); the sign of w enters through an
         // fma by (sg, sg), which is exact on z_s - z_t
         const float2 L2 = splat(kLog2e), NLW = splat(gc.nlw);
@@ -484,14 +625,15 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
         for (int u = 0; u < VPT; ++u) {
             const int q = gtid + u * NT;
             if (q < gvec && (!TL || q >= sl.g0)) {
-                float2 g[4];
-                // y < 0 exactly when !SM; the fp32-gradient instantiations keep the run-time
-                // test, which compiles to a loop 5 % faster there (and 2.4 % slower for bf16)
-                if (G32 ? y < 0 : !SM) {  // full vocabulary: g = w p ((z_s - z_t) - d - cp)
+                float2 g[NP];
+                // y < 0 exactly when !SM; the bf16 logits' fp32-gradient instantiations keep the
+                // run-time test, which compiles to a loop 5 % faster there (and 2.4 % slower for
+                // bf16 gradients)
+                if (G32 && N == 8 ? y < 0 : !SM) {  // full vocabulary: g = w p ((z_s - z_t) - d - cp)
                     const uint4 a = vs[q], b = vt[q];
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const float2 a2 = unpack2(word(a, j)), b2 = unpack2(word(b, j));
+                    for (int j = 0; j < NP; ++j) {
+                        const float2 a2 = E::pair(a, j), b2 = E::pair(b, j);
                         const float2 pw = ex2x2(ffma2(a2, L2, NLW));
                         // sg ((z_s - z_t) - c) with one rounding; sg (z_s - z_t) is exact
                         const float2 x = fsub2(a2, b2);
@@ -500,53 +642,29 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
                 } else {  // sampled token: g = -w l p (g_y is written after the loop)
                     const uint4 a = vs[q];
 #pragma unroll
-                    for (int j = 0; j < 4; ++j)
-                        g[j] = fmul2(ex2x2(ffma2(unpack2(word(a, j)), L2, NLW)), SGL);
+                    for (int j = 0; j < NP; ++j)
+                        g[j] = fmul2(ex2x2(ffma2(E::pair(a, j), L2, NLW)), SGL);
                 }
-                if (G32) {
-                    float4 *dst = reinterpret_cast<float4 *>(static_cast<float *>(p.grad) + row_off +
-                                                             (size_t)q * 8);
-                    __stcs(dst, make_float4(g[0].x, g[0].y, g[1].x, g[1].y));
-                    __stcs(dst + 1, make_float4(g[2].x, g[2].y, g[3].x, g[3].y));
-                } else {
-                    uint4 o;
-                    o.x = pack_bf16x2(g[0].x, g[0].y);
-                    o.y = pack_bf16x2(g[1].x, g[1].y);
-                    o.z = pack_bf16x2(g[2].x, g[2].y);
-                    o.w = pack_bf16x2(g[3].x, g[3].y);
-                    __stcs(reinterpret_cast<uint4 *>(static_cast<__nv_bfloat16 *>(p.grad) + row_off +
-                                                     (size_t)q * 8),
-                           o);
-                }
+                store_grad<T, G32>(p.grad, row_off, q, g);
             }
         }
         // a partial vector, column by column (the loop's formulas)
         auto store_lanes = [&](int q, int lo, int hi) {
             const uint4 a = vs[q], b = vt[q];
-            float gl[8];
+            float2 g[NP];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const float2 a2 = unpack2(word(a, j)), b2 = unpack2(word(b, j));
+            for (int j = 0; j < NP; ++j) {
+                const float2 a2 = E::pair(a, j), b2 = E::pair(b, j);
                 const float2 pw = ex2x2(ffma2(a2, L2, NLW)), x = fsub2(a2, b2);
-                const float2 gg = SM ? fmul2(pw, SGL)
-                                     : (G32 ? fmul2(pw, fadd2(ffma2(x, SG, ND), NCP)) : fmul2(pw, ffma2(x, SG, NC)));
-                gl[2 * j] = gg.x;
-                gl[2 * j + 1] = gg.y;
+                g[j] = SM ? fmul2(pw, SGL)
+                          : (G32 ? fmul2(pw, fadd2(ffma2(x, SG, ND), NCP)) : fmul2(pw, ffma2(x, SG, NC)));
             }
-            const size_t to = row_off + (size_t)q * 8;
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-                if (i >= lo && i < hi) {
-                    if (G32)
-                        static_cast<float *>(p.grad)[to + i] = gl[i];
-                    else
-                        static_cast<__nv_bfloat16 *>(p.grad)[to + i] = __float2bfloat16_rn(gl[i]);
-                }
+            store_grad_lanes<T, G32>(p.grad, row_off + (size_t)q * N, g, lo, hi);
         };
-        if (TL && sl.tailq >= 0 && sl.tailq % NT == gtid)
+        if (TL && sl.tailq > 0 && sl.tailq % NT == gtid)
             store_lanes(sl.tailq, 0, sl.tail);
-        if (TL && sl.head && gtid == 0)
-            store_lanes(0, sl.head0, 8);
+        if (TL && gtid == 0 && (sl.head || sl.tailq == 0))
+            store_lanes(0, sl.head ? sl.head0 : 0, sl.tailq == 0 ? sl.tail : N);
         // sampled token: g_y = w l (1 - p_y), over the value the vector store wrote
         // (same thread, so the later store wins)
         if (SM && yown[s] == gtid) {
@@ -560,9 +678,13 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
 
     // The groups take rows in turn: while one waits for its row's records or
     // data, the others compute.
-    if (tid == 0)
-        for (int k = 0; k < kStages && k < n; ++k)
-            issue(k, p.rows[cid + k * ncl]);
+    if (kStages <= 5) {  // (in parallel these few cost the steady state 0.3 to 3 %)
+        if (tid == 0)
+            for (int k = 0; k < kStages && k < n; ++k)
+                issue(k, p.rows[cid + k * ncl]);
+    } else if (tid < kStages && tid < n) {
+        issue(tid, p.rows[cid + tid * ncl]);
+    }
     for (int k = group; k < n; k += G) {
         int4 ahead = make_int4(0, 0, -1, 0);
         if (gtid == 0 && k + kStages < n)
@@ -597,7 +719,8 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
                 if (mbar_try_wait(&full[k % kStages], (uint32_t)((k / kStages) & 1)))
                     break;
     }
-    cluster_sync();  // no CTA leaves while a peer may still address its shared memory
+    if (CS > 1)
+        cluster_sync();  // no CTA leaves while a peer may still address its shared memory
 }
 
 // Helper for the SMs the clusters leave free (15 eight-CTA clusters cover 120 of
@@ -607,7 +730,7 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
 // ring, AS) with a running maximum per thread (one rescale per batch of kHelpU
 // vectors when the maximum moves); the gradient
 // pass reads them again from L2, where the pass before left them (the clusters'
-// own copies are evict-first).  bf16 logits; a bf16 or fp32 gradient or none.
+// own copies are evict-first).  A bf16 or fp32 gradient or none.
 // Like the cluster kernel, the fp32 gradient also keeps A relative to the
 // reference difference d at the thread's running student argmax (re-referenced,
 // A <- (A + S (d - d')) f, when the maximum moves).  Launched as a dependent
@@ -624,12 +747,15 @@ constexpr int kHelpU = 4;  // vectors of each model per thread and batch
 constexpr int kHelpStages = 3;
 constexpr size_t helper_smem_bytes(bool as, int nth) { return as ? (size_t)kHelpStages * 2 * kHelpU * nth * 16 : 0; }
 
-template <bool G32, bool SM, bool TL, bool AS, int NTH = kHelpThreads, int MINB = 1>
+template <typename T, bool G32, bool SM, bool TL, bool AS, int NTH = kHelpThreads, int MINB = 1>
 __global__ void __launch_bounds__(NTH, MINB) k_row_helper(RowIn p)
 {
     constexpr int kHelpThreads = NTH;
     constexpr int NW = kHelpThreads / 32;
-    constexpr uint32_t kFill = kFillLane | kFillLane << 16;
+    using E = Elem<T>;
+    constexpr int N = E::N, NP = E::NP;
+    constexpr uint32_t kFill = E::kFillWord;
+    constexpr bool kUseD = G32 || N == 4;  // as in the cluster kernel
     __shared__ float red[NW][8];
     __shared__ float bc[8];
     extern __shared__ uint4 hring[];  // [kHelpStages][2][kHelpU][NTH] (AS)
@@ -637,25 +763,25 @@ __global__ void __launch_bounds__(NTH, MINB) k_row_helper(RowIn p)
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nvalid = *p.nvalid;
-    const int j0 = p.split_den ? (int)((int64_t)nvalid * p.split_num / p.split_den) : 0;
-    const __nv_bfloat16 *zs = static_cast<const __nv_bfloat16 *>(p.zs);
-    const __nv_bfloat16 *zt = static_cast<const __nv_bfloat16 *>(p.zt);
+    const int j0 = p.split_den ? split_rows(p, nvalid) : 0;
+    const T *zs = static_cast<const T *>(p.zs);
+    const T *zt = static_cast<const T *>(p.zt);
     const float2 L2 = splat(kLog2e);
     for (int j = j0 + (int)blockIdx.x; j < nvalid; j += gridDim.x) {
         const int4 m = p.rows[j];
         const size_t off = (size_t)m.y * (size_t)p.ld;
-        // TL (ragged rows): a partial first or last vector's other lanes read as kFillLane
+        // TL (ragged rows): a partial first or last vector's other lanes read as the fill
         // and are never written; the gradient loop stores vectors [g0, nfull)
-        const Ragged rg = TL ? ragged(m.y, p.ld, p.vocab) : Ragged{0, (int)(p.vocab / 8), 0};
+        const Ragged rg = TL ? ragged<T>(m.y, p.ld, p.vocab) : Ragged{0, (int)(p.vocab / N), 0};
         const int head = rg.head, nvec = rg.nvec, tail = rg.tail;
         const int g0 = TL && head ? 1 : 0, nfull = TL && tail ? nvec - 1 : nvec;
         const size_t voff = off - (size_t)head;          // the row's first vector
-        const bool cut = TL && (int64_t)voff + (int64_t)nvec * 8 > p.elems;  // the last passes the end
+        const bool cut = TL && (int64_t)voff + (int64_t)nvec * N > p.elems;  // the last passes the end
         auto lanes_lo = [&](int q) { return q == 0 ? head : 0; };
-        auto lanes_hi = [&](int q) { return q == nvec - 1 && tail ? tail : 8; };
+        auto lanes_hi = [&](int q) { return q == nvec - 1 && tail ? tail : N; };
         const uint4 *vs = reinterpret_cast<const uint4 *>(zs + voff);
         const uint4 *vt = reinterpret_cast<const uint4 *>(zt + voff);
-        const int yvec = m.z >= 0 ? ((m.z + head) >> 3) : -1;  // the vector holding the sampled id
+        const int yvec = m.z >= 0 ? (m.z + head) / N : -1;  // the vector holding the sampled id
         float ms = -INFINITY, mt = -INFINITY, dd = 0.f;  // dd: reference difference (fp32 gradient)
         float2 S2 = make_float2(0.f, 0.f), A2 = S2, T2 = S2;
         // this thread's batches of the row: kHelpU vectors of each model, kHelpThreads apart
@@ -689,8 +815,8 @@ __global__ void __launch_bounds__(NTH, MINB) k_row_helper(RowIn p)
             for (int u = 0; u < kHelpU; ++u) {
                 const int q = q0 + u * kHelpThreads;
                 if (TL && cut && q == nvec - 1) {
-                    a[u] = load_lanes(zs + voff + (size_t)q * 8, lanes_lo(q), lanes_hi(q));
-                    b[u] = load_lanes(zt + voff + (size_t)q * 8, lanes_lo(q), lanes_hi(q));
+                    a[u] = E::load_lanes(zs + voff + (size_t)q * N, lanes_lo(q), lanes_hi(q));
+                    b[u] = E::load_lanes(zt + voff + (size_t)q * N, lanes_lo(q), lanes_hi(q));
                 } else if (q < nvec) {
                     if (AS) {
                         a[u] = hring[slot(bi % kHelpStages, 0, u)];
@@ -708,37 +834,37 @@ __global__ void __launch_bounds__(NTH, MINB) k_row_helper(RowIn p)
                 for (int u = 0; u < kHelpU; ++u) {
                     const int q = q0 + u * kHelpThreads;
                     if ((head && q == 0) || (tail && q == nvec - 1)) {
-                        a[u] = keep_lanes(a[u], lanes_lo(q), lanes_hi(q));
-                        b[u] = keep_lanes(b[u], lanes_lo(q), lanes_hi(q));
+                        a[u] = E::keep_lanes(a[u], lanes_lo(q), lanes_hi(q));
+                        b[u] = E::keep_lanes(b[u], lanes_lo(q), lanes_hi(q));
                     }
                 }
             }
-            // a sampled-token row leaves y out of the student statistics (kFillLane
+            // a sampled-token row leaves y out of the student statistics (the fill
             // in its place; add_sampled_term brings its term back at the merge)
             if (SM && (unsigned)(yvec - q0) < (unsigned)(kHelpU * kHelpThreads)) {
 #pragma unroll
                 for (int u = 0; u < kHelpU; ++u)
                     if (yvec == q0 + u * kHelpThreads)
-                        a[u] = fill_lane(a[u], (m.z + head) & 7);
+                        a[u] = E::fill_lane(a[u], (m.z + head) & (N - 1));
             }
-            uint32_t bs = hmax4(a[0]), bt = hmax4(b[0]);
+            typename E::Max bs = E::max_of(a[0]), bt = E::max_of(b[0]);
 #pragma unroll
             for (int u = 1; u < kHelpU; ++u) {
-                bs = hmax2u(bs, hmax4(a[u]));
-                bt = hmax2u(bt, hmax4(b[u]));
+                bs = E::max2(bs, E::max_of(a[u]));
+                bt = E::max2(bt, E::max_of(b[u]));
             }
-            const float nms = fmaxf(ms, fmaxf(bf16lo(bs), bf16hi(bs)));
-            const float nmt = fmaxf(mt, fmaxf(bf16lo(bt), bf16hi(bt)));
+            const float nms = fmaxf(ms, E::value(bs));
+            const float nmt = fmaxf(mt, E::value(bt));
             if (nms > ms) {
                 const float2 f = splat(ex2((ms - nms) * kLog2e));
-                if (G32) {  // d at the first element of the batch equal to the new maximum
+                if (kUseD) {  // d at the first element of the batch equal to the new maximum
                     float xd = 0.f;
                     bool found = false;
 #pragma unroll
                     for (int u = 0; u < kHelpU; ++u)
 #pragma unroll
-                        for (int w = 0; w < 4; ++w) {
-                            const float2 x = unpack2(word(a[u], w)), y = unpack2(word(b[u], w));
+                        for (int w = 0; w < NP; ++w) {
+                            const float2 x = E::pair(a[u], w), y = E::pair(b[u], w);
                             if (!found && x.x == nms) {
                                 xd = x.x - y.x;
                                 found = true;
@@ -764,17 +890,17 @@ __global__ void __launch_bounds__(NTH, MINB) k_row_helper(RowIn p)
 #pragma unroll
             for (int u = 0; u < kHelpU; ++u)
 #pragma unroll
-                for (int w = 0; w < 4; ++w) {
-                    const float2 a2 = unpack2(word(a[u], w)), b2 = unpack2(word(b[u], w));
+                for (int w = 0; w < NP; ++w) {
+                    const float2 a2 = E::pair(a[u], w), b2 = E::pair(b[u], w);
                     const float2 es = ex2x2(ffma2(a2, L2, NS));
                     S2 = fadd2(S2, es);
-                    A2 = ffma2(es, G32 ? fsub2(fsub2(a2, b2), D) : fsub2(a2, b2), A2);
+                    A2 = ffma2(es, kUseD ? fsub2(fsub2(a2, b2), D) : fsub2(a2, b2), A2);
                     T2 = fadd2(T2, ex2x2(ffma2(b2, L2, NTT)));
                 }
         }
         Student S = Student{ms, S2.x + S2.y, A2.x + A2.y, dd};
         Teacher U = Teacher{mt, T2.x + T2.y};
-        lane_merge<32, G32>(S, U);
+        lane_merge<32, kUseD>(S, U);
         if (lane == 0) {
             red[warp][0] = S.m, red[warp][1] = S.s, red[warp][2] = S.a;
             red[warp][3] = U.m, red[warp][4] = U.s, red[warp][5] = S.d;
@@ -787,7 +913,7 @@ __global__ void __launch_bounds__(NTH, MINB) k_row_helper(RowIn p)
                 A = Student{red[lane][0], red[lane][1], red[lane][2], red[lane][5]};
                 B = Teacher{red[lane][3], red[lane][4]};
             }
-            lane_merge<NW, G32>(A, B);
+            lane_merge<NW, kUseD>(A, B);
             if (lane == 0) {
                 const int y = m.z;  // SM: in [0, V) (the compaction drops ids out of range); else -1
                 const float omp = SM ? add_sampled_term(A, to_float(zs[off + y])) : 0.f;  // 1 - p_y
@@ -833,56 +959,36 @@ __global__ void __launch_bounds__(NTH, MINB) k_row_helper(RowIn p)
                         break;
                     if (TL && q < g0)
                         continue;
-                    float2 g[4];
+                    float2 g[NP];
                     if (!SM) {  // full vocabulary: g = w p ((z_s - z_t) - d - cp)
 #pragma unroll
-                        for (int w = 0; w < 4; ++w) {
-                            const float2 a2 = unpack2(word(a[u], w)), b2 = unpack2(word(b[u], w));
+                        for (int w = 0; w < NP; ++w) {
+                            const float2 a2 = E::pair(a[u], w), b2 = E::pair(b[u], w);
                             const float2 pw = ex2x2(ffma2(a2, L2, NLW)), x = fsub2(a2, b2);
                             g[w] = G32 ? fmul2(pw, fadd2(ffma2(x, SG, ND), NCP)) : fmul2(pw, ffma2(x, SG, NC));
                         }
                     } else {  // sampled token: g = -w l p (g_y is written after the loop)
 #pragma unroll
-                        for (int w = 0; w < 4; ++w)
-                            g[w] = fmul2(ex2x2(ffma2(unpack2(word(a[u], w)), L2, NLW)), SGL);
+                        for (int w = 0; w < NP; ++w)
+                            g[w] = fmul2(ex2x2(ffma2(E::pair(a[u], w), L2, NLW)), SGL);
                     }
-                    if (G32) {
-                        float4 *dst = reinterpret_cast<float4 *>(static_cast<float *>(p.grad) + voff) + 2 * (size_t)q;
-                        __stcs(dst, make_float4(g[0].x, g[0].y, g[1].x, g[1].y));
-                        __stcs(dst + 1, make_float4(g[2].x, g[2].y, g[3].x, g[3].y));
-                    } else {
-                        uint4 o;
-                        o.x = pack_bf16x2(g[0].x, g[0].y);
-                        o.y = pack_bf16x2(g[1].x, g[1].y);
-                        o.z = pack_bf16x2(g[2].x, g[2].y);
-                        o.w = pack_bf16x2(g[3].x, g[3].y);
-                        __stcs(reinterpret_cast<uint4 *>(static_cast<__nv_bfloat16 *>(p.grad) + voff) + q, o);
-                    }
+                    store_grad<T, G32>(p.grad, voff, q, g);
                 }
             }
             // a partial vector, column by column
             auto store_lanes = [&](int q) {
                 const int lo = lanes_lo(q), hi = lanes_hi(q);
-                const size_t to = voff + (size_t)q * 8;
-                const uint4 a = load_lanes(zs + to, lo, hi), b = load_lanes(zt + to, lo, hi);
-                float gl[8];
+                const size_t to = voff + (size_t)q * N;
+                const uint4 a = E::load_lanes(zs + to, lo, hi), b = E::load_lanes(zt + to, lo, hi);
+                float2 g[NP];
 #pragma unroll
-                for (int w = 0; w < 4; ++w) {
-                    const float2 a2 = unpack2(word(a, w)), b2 = unpack2(word(b, w));
+                for (int w = 0; w < NP; ++w) {
+                    const float2 a2 = E::pair(a, w), b2 = E::pair(b, w);
                     const float2 pw = ex2x2(ffma2(a2, L2, NLW)), x = fsub2(a2, b2);
-                    const float2 gg = SM ? fmul2(pw, SGL)
-                                         : (G32 ? fmul2(pw, fadd2(ffma2(x, SG, ND), NCP)) : fmul2(pw, ffma2(x, SG, NC)));
-                    gl[2 * w] = gg.x;
-                    gl[2 * w + 1] = gg.y;
+                    g[w] = SM ? fmul2(pw, SGL)
+                              : (G32 ? fmul2(pw, fadd2(ffma2(x, SG, ND), NCP)) : fmul2(pw, ffma2(x, SG, NC)));
                 }
-#pragma unroll
-                for (int i = 0; i < 8; ++i)
-                    if (i >= lo && i < hi) {
-                        if (G32)
-                            static_cast<float *>(p.grad)[to + i] = gl[i];
-                        else
-                            static_cast<__nv_bfloat16 *>(p.grad)[to + i] = __float2bfloat16_rn(gl[i]);
-                    }
+                store_grad_lanes<T, G32>(p.grad, to, g, lo, hi);
             };
             if (TL && tail && (nvec - 1) % kHelpThreads == tid)
                 store_lanes(nvec - 1);
@@ -890,7 +996,7 @@ __global__ void __launch_bounds__(NTH, MINB) k_row_helper(RowIn p)
                 store_lanes(0);
             // sampled token: g_y = w l (1 - p_y), over the value the vector store wrote
             // (same thread, so the later store wins)
-            if (SM && ((y + head) >> 3) % kHelpThreads == tid) {
+            if (SM && (y + head) / N % kHelpThreads == tid) {
                 if (G32)
                     static_cast<float *>(p.grad)[off + y] = gy;
                 else
@@ -902,103 +1008,131 @@ __global__ void __launch_bounds__(NTH, MINB) k_row_helper(RowIn p)
     asm volatile("griddepcontrol.wait;" ::: "memory");  // complete only after the cluster grid
 }
 
-// Threads per row group and groups per CTA (tuning knobs).
-#ifndef TURNOPD_ROW_THREADS
-#define TURNOPD_ROW_THREADS 512
-#endif
-#ifndef TURNOPD_ROW_GROUPS
-#define TURNOPD_ROW_GROUPS 2
-#endif
-constexpr int kNT = TURNOPD_ROW_THREADS;
-constexpr int kG = TURNOPD_ROW_GROUPS;
-constexpr int kMaxSlice = 2400;                      // vectors per CTA: 3 stages fit 227 KB
-constexpr int kVPT = (kMaxSlice + kNT - 1) / kNT;    // vectors per thread
-// The cluster size is the smallest of 2, 3, 4, 5, 6, 8 and 16 CTAs whose slices fit
-// three stages, which keeps the slices long (a short slice cannot hide the per-row
-// record exchange) and, for short rows, puts more SMs in clusters (76 pairs cover
-// all 152).  Below kMinSlice vectors per CTA the helper kernel alone, on every SM,
-// takes the rows (measured: slices of 2,000-2,400 vectors reach 0.87-0.93 of the
-// copy bandwidth, the helper alone on rows of up to 8,192 vectors about 0.73).
-// Clusters of 16 are exempt: the rows that need them are long, and the helper
-// alone streams those poorly (V = 200,000: 0.58 against 0.77 with clusters of 16
-// and 1,563-vector slices).
-#ifndef TURNOPD_CLUSTER_MIN_SLICE
-#define TURNOPD_CLUSTER_MIN_SLICE 1700
-#endif
-constexpr int kMinSlice = TURNOPD_CLUSTER_MIN_SLICE;
-constexpr int kSmallRowVec = 7168;  // up to this many vectors per row: 256-thread helpers, 2 per SM
+
+// Shapes of a CTA, by the longest slice they hold (kMax vectors).  A shorter slice takes
+// smaller groups and more of them, so that as many bytes are in flight and as many rows
+// in progress whatever the row's length.  GB/s of the whole step at 4e8 logits of V,
+// bf16 (fp32), with a gradient of the same type: Shape32 4,600 at V = 1,024, Shape12
+// 4,800 (5,670) at 2,048 (1,024), Shape8 5,400 (6,300) at 4,096, Shape4 5,700 (6,480) at
+// 8,192, ShapeMid 5,960 at 12,288, where ShapeBig gives 5,380; rows held in no shape (one
+// 256- or 512-thread CTA a row, the second read from L2) reached 820, 1,350, 2,380,
+// 3,920 and 3,930, and fp32 rows on clusters of 8 (k_row_split) 186, 370, 736 and 1,370.
+struct ShapeBig { static constexpr int NT = 512, G = 2, VPT = 5, ST = 3, kMax = 2384; };
+struct ShapeMid { static constexpr int NT = 320, G = 3, VPT = 6, ST = 4, kMax = 1780; };
+struct Shape4 { static constexpr int NT = 256, G = 4, VPT = 5, ST = 5, kMax = 1280; };
+struct Shape8 { static constexpr int NT = 128, G = 8, VPT = 5, ST = 10, kMax = 640; };
+struct Shape12 { static constexpr int NT = 64, G = 12, VPT = 5, ST = 20, kMax = 320; };
+struct Shape32 { static constexpr int NT = 32, G = 32, VPT = 5, ST = 40, kMax = 160; };
+
+// Cluster size for rows of nvec vectors: the smallest whose slices a CTA holds (0: none).
+// That keeps the slices long (a short slice cannot hide the per-row record exchange) and,
+// for short rows, puts more SMs in clusters: every SM for 1 and 2, then 36 clusters of 4
+// are co-resident, 28 of 5, 23 of 6, 15 of 8, 7 of 16.  7 is left out (only 15).
+inline int cluster_size(int nvec)
+{
+    static const int kSizes[] = {1, 2, 3, 4, 5, 6, 8, 16};
+    for (int c : kSizes)
+        if ((nvec + c - 1) / c <= ShapeBig::kMax)
+            return c;
+    return 0;
+}
+
 // The helper's rows per SM and second against the clusters', which decides the
 // split of the row list.  A cluster SM is less efficient on a shorter slice and in a
-// larger cluster (more records per row), so the rate rises with both.  Measured best
-// (packed 8 x 4096, the ring-fed helper): clusters of 8, 0.72 at 2,374 vectors
-// (V = 151,936) and 0.85 at 2,004 (128,256); clusters of 16, 0.80 at 2,048 (262,144)
-// and about 1.0 at 1,563 (200,000); clusters of 3 to 6 (few helper SMs, where an
-// overloaded helper decides the call), 0.60: V = 50,000 (3) 0.946 ms against 1.042 at
-// 0.70, 90,000 (5) 1.623 against 1.709, 110,000 (6) 1.968 against 2.017, 65,536 (4)
-// flat from 0.65 to 0.75.  Sampled-token rows, whose helper gradient pass reads the
-// student only, more: 0.03 with a bf16 gradient (0.75 at 2,374), 0.10 with an fp32 one
-// (0.82 at 2,374: 4.196 ms against 4.260 at 0.75 and 4.539 at 0.92), whose larger
-// gradient writes weigh more beside the skipped teacher read.
-double helper_rate(int slice_vec, int cs, bool sampled, bool g32)
+// larger cluster (more records per row), so the rate rises with both; where few SMs are
+// left (clusters of 3 to 6) an overloaded helper decides the call.  Measured best (GB/s of
+// the step at 4e8 to 1.5e9 logits, or us; slices in vectors):
+//   bf16, clusters of 8 at 2,374 (V = 151,936; 8 x 4096 packed tokens): 0.81 (2,724 us;
+//   2,759 at 0.72, 2,845 at 0.88), with an fp32 gradient 0.73 (16 x 8192 household tokens
+//   2,375; 2,400 at 0.68, 2,431 at 0.76), sampled tokens 0.86 (64 multihop 1,028; 1,049 at
+//   0.72); at 2,004 (128,256) 0.92 (6,232; 6,003 at 0.72) and 0.78 (5,865; 5,471 at 0.85);
+//   of 16: 0.8 at 2,048 and 1,563 (200,000: 5,487, 5,265 at 0.6), 0.6 at 1,758 (5,405, 5,097
+//   at 0.8), with an fp32 gradient 0.2 less; of 3 in ShapeMid 0.5 (39,000: 6,183, 5,222 at
+//   0.7); of 3 to 6 otherwise 0.7 (90,000: 6,335, 6,245 at 0.4), 0.62 with an fp32 gradient
+//   (49,152: 6,252 at 0.6, 5,978 at 0.7);
+//   fp32, clusters of 16: 0.69 at 2,374 (151,936: 4 x 4096 packed tokens 2,808 us; 2,833 at
+//   0.65, 2,873 at 0.76), 0.80 at 2,048 (6,035, 5,823 at 0.6), 0.65 at 1,719 in ShapeMid
+//   (6,361 at 0.6, 6,186 at 0.7), 0.9 at 1,536 (6,203, 5,909 at 0.5), 0.7 at 1,204 in Shape4
+//   (6,026, 5,747 at 0.9); of 8 0.70 at 2,350 (6,310, 6,143 at 0.85), more at 2,048 (65,536:
+//   6,375 at 0.7, 6,124 at 0.4); of 5 and 6 0.7 (49,152: 6,531, 6,460 at 0.4); of 3 and 4 0.60
+//   (28,000: 6,283, 5,562 at 0.75);
+//   sampled-token rows, whose helper gradient pass reads the student only: 0.05 more with a
+//   bf16 gradient, 0.10 with an fp32 one;
+//   forward-only rows, which the helper reads once: 1.0 (bf16 at 2,374: 4,743, 4,478 at 0.7;
+//   fp32, clusters of 8 at 2,350: 6,185, 5,836 at 0.7), 0.7 for bf16 in clusters of 3 and 4
+//   (57,000: 4,570, 3,443 at 1.0), 0.85 of 5 and 6, 0.9 for fp32 in clusters of 3.
+template <typename T> double helper_rate(int slice_vec, int cs, bool sampled, bool g32, bool forward)
 {
-#ifdef TURNOPD_HELPER_RATE
-    (void)slice_vec;
-    (void)cs;
-    (void)sampled;
-    (void)g32;
-    return TURNOPD_HELPER_RATE;
-#else
-    double r = 0.60;
-    if (cs == 8)
-        r = 0.72 + (2374 - slice_vec) * 0.00035;
-    else if (cs > 8)
-        r = 0.80 + (2048 - slice_vec) * 0.00041;
-    r = r < 0.60 ? 0.60 : (r > 1.1 ? 1.1 : r);
-    return sampled ? r + (g32 ? 0.10 : 0.03) : r;
-#endif
+    const bool bf16 = sizeof(T) == 2;
+    if (forward)
+        return cs >= 8 ? 1.0 : bf16 ? (cs <= 4 ? 0.7 : 0.85) : (cs == 3 ? 0.9 : 1.0);
+    double r;
+    if (bf16) {
+        if (cs == 3 && slice_vec <= ShapeMid::kMax)
+            return 0.50;
+        if (cs < 8)
+            return g32 ? 0.62 : 0.70;
+        if (cs == 8)
+            r = g32 ? 0.73 + (2374 - slice_vec) * 0.00014 : 0.81 + (2374 - slice_vec) * 0.0003;
+        else
+            r = (slice_vec > 1563 && slice_vec <= ShapeMid::kMax ? 0.80 - (slice_vec - 1563) * 0.001 : 0.80) -
+                (g32 ? 0.2 : 0.0);
+    } else {
+        if (cs < 8)
+            return cs <= 4 ? 0.60 : 0.70;
+        if (cs == 8)
+            r = 0.70 + (2350 - slice_vec) * 0.0002;
+        else
+            r = slice_vec <= Shape4::kMax ? 0.70
+                : slice_vec <= ShapeMid::kMax ? 0.90 + (1536 - slice_vec) * 0.0014
+                                              : 0.80 + (2048 - slice_vec) * 0.00034;
+        r = r > 0.9 ? 0.9 : r;
+    }
+    r = r < 0.60 ? 0.60 : r;
+    return sampled ? r + (g32 ? 0.10 : 0.05) : r;
 }
-// The helper grid beside the clusters: CTAs of kSideThreads threads, kSideBlocks per free SM.
-#ifndef TURNOPD_HELPER_THREADS
-#define TURNOPD_HELPER_THREADS 512
-#endif
-#ifndef TURNOPD_HELPER_BLOCKS
-#define TURNOPD_HELPER_BLOCKS 1
-#endif
-constexpr int kSideThreads = TURNOPD_HELPER_THREADS, kSideBlocks = TURNOPD_HELPER_BLOCKS;
 
-size_t cluster_smem_bytes(int slice_vec, int cs)
+template <class Shape> size_t cluster_smem_bytes(int slice_vec, int cs)
 {
-    return (size_t)kStages * 2 * slice_vec * 16 + 2 * kG * cs * 8 * sizeof(float) +
-           kStages * sizeof(int4) + (2 * kStages + 2 * kG) * sizeof(uint64_t) +
-           kG * (kNT / 32) * 8 * sizeof(float) +  // per-group warp partials
-           8 * sizeof(int) +                        // row held by each stage, thread reading y
-           kG * 16 * sizeof(float);                 // broadcast row constants
+    constexpr int ST = Shape::ST, G = Shape::G;
+    return (size_t)ST * 2 * slice_vec * 16 + 2 * G * cs * 8 * sizeof(float) +
+           ST * sizeof(int4) + (2 * ST + 2 * G) * sizeof(uint64_t) +
+           G * (Shape::NT / 32) * 8 * sizeof(float) +  // per-group warp partials
+           2 * ((ST + 3) / 4 * 4) * sizeof(int) +                       // row held by each stage, thread reading y
+           G * 16 * sizeof(float);                      // broadcast row constants
 }
 
 // The cluster grid (as many clusters as are co-resident, cached per device) and
 // the helper grid on the SMs the clusters leave free, with the row list split so
-// that both finish together.
-template <bool G32, int CS, bool SM, bool TL>
-cudaError_t launch_t(const RowIn &p, int slice_vec, int nvec, size_t smem, cudaStream_t stream)
+// that both finish together.  *used = false (and nothing is launched) where the slices
+// do not fit shared memory.
+template <typename T, bool G32, int CS, class Shape, bool SM, bool TL>
+cudaError_t launch_t(const RowIn &p, int nvec, cudaStream_t stream, bool *used)
 {
-    auto kern = k_row_cluster<CS, kNT, kVPT, kG, G32, SM, TL>;
-    int dev = 0;
+    auto kern = k_row_cluster<T, CS, Shape::NT, Shape::VPT, Shape::G, Shape::ST, G32, SM, TL>;
+    const int slice_vec = (nvec + CS - 1) / CS;
+    const size_t smem = cluster_smem_bytes<Shape>(slice_vec, CS);
+    int dev = 0, optin = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess)
         return e;
-    static int grid_cache[64][2];
-    static size_t smem_cache[64][2];
-    const int gi = G32 ? 1 : 0;  // (the statics are per instantiation: cluster size, gradient type, mode)
+    if ((e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess)
+        return e;
+    *used = smem + 128 <= (size_t)optin;  // room for the kernel's static shared memory and alignment
+    if (!*used)
+        return cudaSuccess;
+    static int grid_cache[64];  // (per instantiation)
+    static size_t smem_cache[64];
     if (dev >= 64)
         return cudaErrorInvalidDevice;
-    if (smem_cache[dev][gi] < smem) {
+    if (smem_cache[dev] < smem) {
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess)
             return e;
         if (CS > 8 && (e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess)
             return e;
-        smem_cache[dev][gi] = smem;
-        grid_cache[dev][gi] = 0;
+        smem_cache[dev] = smem;
+        grid_cache[dev] = 0;
     }
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
@@ -1008,10 +1142,10 @@ cudaError_t launch_t(const RowIn &p, int slice_vec, int nvec, size_t smem, cudaS
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cfg.blockDim = dim3(kG * kNT);
+    cfg.blockDim = dim3(Shape::G * Shape::NT);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
-    if (grid_cache[dev][gi] == 0) {
+    if (grid_cache[dev] == 0) {
         cfg.gridDim = dim3(CS);
         int ncl = 0;
         e = cudaOccupancyMaxActiveClusters(&ncl, kern, &cfg);
@@ -1019,16 +1153,17 @@ cudaError_t launch_t(const RowIn &p, int slice_vec, int nvec, size_t smem, cudaS
             return e;
         if (ncl < 1)
             return cudaErrorInvalidConfiguration;
-        grid_cache[dev][gi] = ncl;
+        grid_cache[dev] = ncl;
     }
     RowIn pl = p;
-    const int free_sm = device_sm_count() - grid_cache[dev][gi] * CS;
+    const int free_sm = device_sm_count() - grid_cache[dev] * CS;
     if (free_sm > 0) {
-        const double cl = (double)(grid_cache[dev][gi] * CS);
+        const double cl = (double)(grid_cache[dev] * CS);
         pl.split_den = 1 << 20;
-        pl.split_num = (int32_t)(pl.split_den * cl / (cl + helper_rate(slice_vec, CS, SM, G32) * free_sm) + 0.5);
+        pl.split_ctas = free_sm;
+        pl.split_num = (int32_t)(pl.split_den * cl / (cl + helper_rate<T>(slice_vec, CS, SM, G32, !p.grad) * free_sm) + 0.5);
     }
-    cfg.gridDim = dim3(grid_cache[dev][gi] * CS);
+    cfg.gridDim = dim3(grid_cache[dev] * CS);
     e = cudaLaunchKernelEx(&cfg, kern, pl, slice_vec, nvec);
     if (e != cudaSuccess || pl.split_den == 0)
         return e;
@@ -1039,95 +1174,89 @@ cudaError_t launch_t(const RowIn &p, int slice_vec, int nvec, size_t smem, cudaS
     ha[0].val.programmaticStreamSerializationAllowed = 1;
     hc.attrs = ha;
     hc.numAttrs = 1;
-    hc.gridDim = dim3(free_sm * kSideBlocks);
-    hc.blockDim = dim3(kSideThreads);
-    hc.dynamicSmemBytes = helper_smem_bytes(true, kSideThreads);
+    hc.gridDim = dim3(free_sm);
+    hc.blockDim = dim3(kHelpThreads);
+    hc.dynamicSmemBytes = helper_smem_bytes(true, kHelpThreads);
     hc.stream = stream;
-    auto helper = k_row_helper<G32, SM, TL, true, kSideThreads, kSideBlocks>;
+    auto helper = k_row_helper<T, G32, SM, TL, true>;
     if ((e = cudaFuncSetAttribute(helper, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)helper_smem_bytes(true, kSideThreads))) != cudaSuccess)
+                                  (int)helper_smem_bytes(true, kHelpThreads))) != cudaSuccess)
         return e;
     return cudaLaunchKernelEx(&hc, helper, pl);
 }
 
-// Cluster sizes offered: 7 is left out (only 15 clusters of 7 are co-resident, 105 SMs).
-template <bool G32, bool SM, bool TL>
-cudaError_t launch_cs(int cs, const RowIn &p, int slice_vec, int nvec, size_t smem, cudaStream_t stream)
+template <typename T, bool G32, bool SM, bool TL>
+cudaError_t launch_cs(const RowIn &p, int nvec, cudaStream_t stream, bool *used)
 {
+    const int cs = cluster_size(nvec);
+    const int slice = cs ? (nvec + cs - 1) / cs : 0;
+    const int shape = slice <= Shape32::kMax  ? 5
+                : slice <= Shape12::kMax  ? 4
+                : slice <= Shape8::kMax   ? 3
+                : slice <= Shape4::kMax   ? 2
+                : slice <= ShapeMid::kMax ? 1
+                                          : 0;
+    *used = false;
+#define TURNOPD_ROWS(CSIZE, SHAPE) launch_t<T, G32, CSIZE, SHAPE, SM, TL>(p, nvec, stream, used)
     switch (cs) {
-    case 2: return launch_t<G32, 2, SM, TL>(p, slice_vec, nvec, smem, stream);
-    case 3: return launch_t<G32, 3, SM, TL>(p, slice_vec, nvec, smem, stream);
-    case 4: return launch_t<G32, 4, SM, TL>(p, slice_vec, nvec, smem, stream);
-    case 5: return launch_t<G32, 5, SM, TL>(p, slice_vec, nvec, smem, stream);
-    case 6: return launch_t<G32, 6, SM, TL>(p, slice_vec, nvec, smem, stream);
-    case 8: return launch_t<G32, 8, SM, TL>(p, slice_vec, nvec, smem, stream);
-    default: return launch_t<G32, 16, SM, TL>(p, slice_vec, nvec, smem, stream);
+    case 1:
+        switch (shape) {
+        case 5: return TURNOPD_ROWS(1, Shape32);
+        case 4: return TURNOPD_ROWS(1, Shape12);
+        case 3: return TURNOPD_ROWS(1, Shape8);
+        case 2: return TURNOPD_ROWS(1, Shape4);
+        case 1: return TURNOPD_ROWS(1, ShapeMid);
+        default: return TURNOPD_ROWS(1, ShapeBig);
+        }
+    case 2:
+        switch (shape) {
+        case 2: return TURNOPD_ROWS(2, Shape4);
+        case 1: return TURNOPD_ROWS(2, ShapeMid);
+        default: return TURNOPD_ROWS(2, ShapeBig);
+        }
+    // slices of clusters of 3 to 8 have 1,584 vectors or more, of 16 1,188 or more
+    case 3: return shape ? TURNOPD_ROWS(3, ShapeMid) : TURNOPD_ROWS(3, ShapeBig);
+    case 4: return TURNOPD_ROWS(4, ShapeBig);
+    case 5: return TURNOPD_ROWS(5, ShapeBig);
+    case 6: return TURNOPD_ROWS(6, ShapeBig);
+    case 8: return TURNOPD_ROWS(8, ShapeBig);
+    case 16: return shape == 2 ? TURNOPD_ROWS(16, Shape4) : shape == 1 ? TURNOPD_ROWS(16, ShapeMid) : TURNOPD_ROWS(16, ShapeBig);
     }
+#undef TURNOPD_ROWS
+    return cudaSuccess;
 }
 
 // The helper kernel alone, every row, every SM.
-template <bool G32, bool SM, bool TL>
-void launch_helper_alone(const RowIn &p, int nvec, cudaStream_t stream)
+template <typename T, bool G32, bool SM, bool TL>
+void launch_helper_alone(const RowIn &p, cudaStream_t stream)
 {
-    const int sms = device_sm_count();
-    if (nvec <= kSmallRowVec)
-        k_row_helper<G32, SM, TL, false, 256, 2><<<sms * 2, 256, 0, stream>>>(p);
-    else
-        k_row_helper<G32, SM, TL, false><<<sms, kHelpThreads, 0, stream>>>(p);
+    RowIn pl = p;
+    pl.split_den = 0;
+    k_row_helper<T, G32, SM, TL, false><<<device_sm_count(), kHelpThreads, 0, stream>>>(pl);
 }
 
-// The row grids for bf16 logits; TL: ragged rows (V or ld no multiple of 8).
-template <bool TL>
-cudaError_t launch_row_cluster_t(const RowIn &p, bool fp32_grad, cudaStream_t stream, bool *used)
+template <typename T, bool G32, bool SM, bool TL>
+cudaError_t launch_rows_m(const RowIn &p, int nvec, cudaStream_t stream)
 {
-    *used = false;
-    auto al16 = [](const void *q) { return (reinterpret_cast<uintptr_t>(q) & 15u) == 0; };
-    // 16-byte aligned arrays; TL: any stride and vocabulary (a row's first and last vectors
-    // are masked; what they hold of other rows or of padding is read, never written)
-    if ((!TL && p.ld % 8 != 0) || !al16(p.zs) || !al16(p.zt) || (p.grad && !al16(p.grad)))
-        return cudaSuccess;
-    // the smallest cluster whose slices fit three stages (2, 3, 4, 5, 6, 8 or 16 CTAs;
-    // 16 is a non-portable size)
-    if ((p.vocab + 14) / 8 > (int64_t)0x7fffffff)
-        return cudaSuccess;
-    // the most vectors a row spans: 7 more elements where rows start anywhere in a vector
-    const int nvec = (int)((p.vocab + (p.ld % 8 != 0 ? 7 : 0) + 7) / 8);
-    static const int kSizes[] = {2, 3, 4, 5, 6, 8, 16};
-    int cs = 16;
-    for (int c : kSizes)
-        if ((nvec + c - 1) / c <= kMaxSlice) {
-            cs = c;
-            break;
-        }
-    const int slice_vec = (nvec + cs - 1) / cs;
+    bool used = false;
+    const cudaError_t e = launch_cs<T, G32, SM, TL>(p, nvec, stream, &used);
+    if (e != cudaSuccess || used)
+        return e;
+    launch_helper_alone<T, G32, SM, TL>(p, stream);
+    return cudaGetLastError();
+}
+
+// The row grids for logits of T; TL: ragged rows (V or ld no multiple of a vector).
+template <typename T, bool TL>
+cudaError_t launch_rows_t(const RowIn &p, bool fp32_grad, cudaStream_t stream)
+{
+    constexpr int N = 16 / (int)sizeof(T);
+    // the most vectors a row spans: N - 1 more elements where rows start anywhere in a vector
+    const int nvec = (int)((p.vocab + (p.ld % N != 0 ? N - 1 : 0) + N - 1) / N);
     const bool sm = p.mode == TURNOPD_SAMPLED_TOKEN;
-    // short rows, or a slice too long even for clusters of 16: the helper kernel alone, every row, every SM
-    if ((slice_vec < kMinSlice && cs < 16) || slice_vec > kMaxSlice) {
-        RowIn pl = p;
-        pl.split_den = 0;
-        *used = true;
-        if (fp32_grad)
-            sm ? launch_helper_alone<true, true, TL>(pl, nvec, stream) : launch_helper_alone<true, false, TL>(pl, nvec, stream);
-        else
-            sm ? launch_helper_alone<false, true, TL>(pl, nvec, stream) : launch_helper_alone<false, false, TL>(pl, nvec, stream);
-        return cudaGetLastError();
-    }
-    const size_t smem = cluster_smem_bytes(slice_vec, cs);
-    int dev = 0, optin = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess)
-        return e;
-    e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    if (e != cudaSuccess)
-        return e;
-    if (smem + 64 > (size_t)optin)  // room for the kernel's static shared memory
-        return cudaSuccess;
-    *used = true;
     if (fp32_grad)
-        return sm ? launch_cs<true, true, TL>(cs, p, slice_vec, nvec, smem, stream)
-                  : launch_cs<true, false, TL>(cs, p, slice_vec, nvec, smem, stream);
-    return sm ? launch_cs<false, true, TL>(cs, p, slice_vec, nvec, smem, stream)
-              : launch_cs<false, false, TL>(cs, p, slice_vec, nvec, smem, stream);
+        return sm ? launch_rows_m<T, true, true, TL>(p, nvec, stream) : launch_rows_m<T, true, false, TL>(p, nvec, stream);
+    return sm ? launch_rows_m<T, false, true, TL>(p, nvec, stream) : launch_rows_m<T, false, false, TL>(p, nvec, stream);
 }
 
 }  // namespace

@@ -825,19 +825,11 @@ cudaError_t launch_split_t(const RowIn &p, bool fp32_grad, int nvec, double rate
 
 }  // namespace
 
-// fp32 logits, 16-byte aligned rows (V and ld multiples of 4): the split-row
-// kernel on as many clusters as are co-resident, the helper kernel beside it.
-// *used = false leaves the row to the portable kernel.
-cudaError_t launch_row_split(const RowIn &p, bool fp32_grad, cudaStream_t stream, bool *used)
+// fp32 logits, 16-byte aligned arrays, V and ld multiples of 4: the split-row kernel on as
+// many clusters as are co-resident, the helper kernel beside it.
+cudaError_t launch_row_split(const RowIn &p, bool fp32_grad, cudaStream_t stream)
 {
-    *used = false;
-    auto al16 = [](const void *q) { return (reinterpret_cast<uintptr_t>(q) & 15u) == 0; };
-    if (p.vocab % 4 != 0 || p.ld % 4 != 0 || !al16(p.zs) || !al16(p.zt) || (p.grad && !al16(p.grad)))
-        return cudaSuccess;
-    if (p.vocab / 4 > (int64_t)0x7fffffff)
-        return cudaSuccess;
     const int nvec = (int)(p.vocab / 4);
-    *used = true;
     // every listed row of a sampled-token call carries y in [0, V)
     if (p.mode == TURNOPD_SAMPLED_TOKEN)
         return launch_split_t<kCSSampled, true>(p, fp32_grad, nvec, kRateSampled, stream);

@@ -320,6 +320,54 @@ def test_ragged_rows_bf16(P, oracle, V, ld, mode, gdt):
         assert (grad[:, V:].float() == 7.0).all()
 
 
+# Longest rows of each shape of the held-row kernels, in 16-byte vectors of one CTA, and the
+# cluster sizes whose slices reach them: (vectors, cluster)
+SHAPE_EDGES = [(160, 1), (320, 1), (640, 1), (1280, 1), (1780, 1), (2384, 1), (1280, 2), (1780, 2), (1780, 3)]
+
+
+@pytest.mark.parametrize("vec,cs", SHAPE_EDGES)
+@pytest.mark.parametrize("step", [0, 1], ids=["last", "next"])
+@pytest.mark.parametrize("idt", ["bf16", "f32"])
+def test_held_row_shape_edges(P, oracle, vec, cs, step, idt):
+    """The longest row of a shape and the shortest of the next (one vector more per CTA), in
+    both modes and gradient types, on more rows than a CTA's groups and ring hold at once."""
+    n = 8 if idt == "bf16" else 4
+    V = n * cs * (vec + step)
+    dt = torch.bfloat16 if idt == "bf16" else torch.float32
+    rows = 152 * 48 if vec <= 320 else 152 * 12 if vec <= 640 else 500
+    b = W.packed(seed=71, num_traj=2, traj_len=int(rows / 1.2))
+    zs, zt = W.make_logits(b.num_valid, V, "agent", dt, seed=72, device="cuda")
+    for mode in (0, 1):
+        for gdt in (torch.bfloat16, torch.float32):
+            run_chain(P, oracle, b, V, zs, zt, mode=mode, alpha=0.5, compact=True, grad_dtype=gdt, seed_y=73)
+
+
+@pytest.mark.parametrize("V,ld", [(2, 2), (3, 5), (1027, 1027), (4099, 4101), (9537, 9537), (38150, 38151),
+                                  (76293, 76293), (W.V_QWEN + 3, W.V_QWEN + 3)])
+@pytest.mark.parametrize("mode", [0, 1], ids=["full", "sampled"])
+@pytest.mark.parametrize("gdt", ["bf16", "f32"])
+def test_ragged_rows_fp32(P, oracle, V, ld, mode, gdt):
+    """fp32 rows that start anywhere in a 16-byte vector: a CTA alone (to 9,536), clusters of
+    2 to 8 (38,150) and of 16; NaN behind the last row's last column, y in a partial vector."""
+    b = W.packed(seed=75, num_traj=2, traj_len=96 if V > 30000 else 256)
+    R = b.num_valid
+    zs0, zt0 = W.make_logits(R, V, "agent" if V > 8 else "tiny", torch.float32, seed=76, device="cuda")
+    if mode == 1 and V > 8:
+        r = torch.arange(R, device="cuda")
+        for k, col in ((0, 0), (1, V - 1)):
+            zs0[r[r % 3 == k], col] = zs0[r % 3 == k].amax(dim=1) + 30.0
+    z = []
+    for src in (zs0, zt0):
+        buf = torch.full((R * ld + 64,), float("nan"), dtype=torch.float32, device="cuda")
+        buf[:R * ld].view(R, ld)[:, :V] = src
+        buf[(R - 1) * ld + V:] = float("nan")
+        z.append(buf[:R * ld].view(R, ld))
+    _, grad = run_chain(P, oracle, b, V, *z, mode=mode, alpha=0.5, compact=True, seed_y=77,
+                        grad_dtype=torch.bfloat16 if gdt == "bf16" else torch.float32)
+    if ld > V:
+        assert (grad[:, V:].float() == 7.0).all()
+
+
 def test_ragged_rows_dense_neighbours_untouched(P, oracle):
     """One row per token, odd stride: the gradient rows of masked tokens share vectors
     with supervised ones and stay as they were."""
