@@ -18,9 +18,11 @@
 //   bound    (streaming warps) for K <= 64, tau = the K-th largest of the 8
 //            largest lane maxima of every streaming warp: K-th largest of
 //            distinct elements of the row, so a lower bound of the row's K-th
-//            largest logit; above, the K-th largest group bucket (K groups each
-//            hold an element that large), by binary search on its value; then
-//            the groups whose bucket reaches tau's are listed;
+//            largest logit; above, the K-th largest thread maximum, or (K above
+//            288, or rows of few groups) the K-th largest group bucket (K groups
+//            each hold an element that large), by binary search on its value;
+//            then the groups whose bucket reaches tau's are listed (and above K =
+//            192 the bound is refined to the K-th largest bucket of the listed);
 //   collect  (selector warps) only the listed groups are read again, in step
 //            across the lanes (a few dozen per row at K = 50), and their
 //            elements >= tau go to a shared-memory candidate buffer (1,024
@@ -29,8 +31,9 @@
 //            tau, one key byte per pass, raises tau until the keys above it fit
 //            the buffer, then collects again (at most 6 passes for bf16 keys,
 //            8 for fp32);
-//   select   up to 256 candidates: the exact K-th largest by radix select, then
-//            each selected key's rank among the candidates is its position;
+//   select   up to 320 candidates: the exact K-th largest by radix select (buffers
+//            over 2 K), then each selected key's rank among the candidates is its
+//            position;
 //            more: a bitonic sort of the buffer.
 // The KL over S is evaluated by one warp in fp32 with
 // l = E_p[z_s - z_t] - (LSE_s - LSE_t) and g_v = w p_v ((z_s - z_t)_v - E_p[.]).
@@ -56,14 +59,15 @@ namespace {
 #define TURNOPD_TOPK_MINB 2
 #endif
 constexpr int kTkStreamWarps = TURNOPD_TOPK_STREAM_WARPS;  // pass A, row after row
-#ifndef TURNOPD_TOPK_SEL_WARPS
-#define TURNOPD_TOPK_SEL_WARPS 2
+// Selector warps (the later phases, a row behind): SW is a template parameter of what they
+// run, 2 up to K = 96 and 4 above, where they set the pace (their collect, sort and KL grow
+// with K; sort_desc needs n >= 2 x 32 SW and n >= 256, so at most 4).  9,870 rows of V =
+// 151,936, bf16: K = 256 sparse 863 us with 4, 1,115 with 2; K = 128 642, 641.
+#ifndef TURNOPD_TOPK_SEL_LARGE
+#define TURNOPD_TOPK_SEL_LARGE 4
 #endif
-constexpr int kTkSelWarps = TURNOPD_TOPK_SEL_WARPS;         // the later phases, a row behind
-constexpr int kTkSelThreads = kTkSelWarps * 32;
-static_assert(kTkSelWarps >= 1 && kTkSelWarps <= 4, "sort_desc needs n >= 2 kTkSelThreads, n >= 256");
+constexpr int kTkSelSmall = 2, kTkSelLarge = TURNOPD_TOPK_SEL_LARGE;
 constexpr int kTkStreamThreads = kTkStreamWarps * 32;
-constexpr int kTkThreads = kTkStreamThreads + kTkSelThreads;
 constexpr int kTkMinBlocks = TURNOPD_TOPK_MINB;  // CTAs (rows in flight) per SM
 // named barriers: buffer b full (1 + b), buffer b free (3 + b), selectors only (5),
 // streaming warps only (6)
@@ -77,9 +81,12 @@ __host__ __device__ constexpr int topk_cap(int K) { return K <= 512 ? 1024 : 204
 constexpr int kTkLaneTop = 8;
 constexpr int kTkLaneBoundMaxK = kTkStreamWarps * kTkLaneTop;
 // candidates above which the selection sorts the buffer instead of ranking
-constexpr int kTkRankMax = 256;
+constexpr int kTkRankMax = 320;
 constexpr uint32_t kTkQueue = 64;  // ring of group indices per selector warp (at most 63 held)
 constexpr int kTkGroup = 16;      // ids per recorded bucket
+constexpr int kRefine = 2;        // listed groups per streaming thread that the bound is refined on
+// (K = 256 at V = 151,936: 863 us with it, 883 without; K = 128: 728 and 642)
+constexpr int kRefineMinK = 192;
 static_assert(kTkQueue >= 64 && (kTkQueue & (kTkQueue - 1)) == 0, "group ring");
 static_assert(TURNOPD_TOPK_MAX_VOCAB / kTkGroup <= 65536, "group indices are 16-bit");
 static_assert(TURNOPD_TOPK_MAX_VOCAB <= (1 << 20) && topk_cap(TURNOPD_TOPK_MAX) <= 2048,
@@ -241,9 +248,11 @@ __device__ __forceinline__ void pick_bin(SelScratch &sc, int need, int lane)
 // Returns 0 when fewer than K keys are present.  Stops early once the chosen
 // bin holds exactly the remaining count.  Every selector thread (stid =
 // 0 .. kTkSelThreads-1) calls it; it synchronises them on kBarSel.
+template <int SW>
 __device__ uint64_t sel_kth_largest(const uint64_t *keys, int n, int K, int hi_byte, int lo_byte,
                                     SelScratch &sc, int stid)
 {
+    constexpr int kTkSelThreads = 32 * SW;
     uint64_t prefix = 0, mask = 0;
     int need = K;
     for (int byte = hi_byte; byte >= lo_byte; --byte) {
@@ -283,9 +292,10 @@ __device__ __forceinline__ int count_ge2(uint32_t x, uint32_t m)
 // padding) in descending order: bitonic network over the selector threads, each
 // thread loading U pairs before it compares and stores any, synchronised on
 // kBarSel after every step.
-template <int U>
+template <int U, int SW>
 __device__ void sort_desc(uint64_t *keys, int n, int stid)
 {
+    constexpr int kTkSelThreads = 32 * SW;
     const int np = n / 2;  // pairs per step
     for (int k = 2; k <= n; k <<= 1)
         for (int j = k >> 1; j > 0; j >>= 1) {
@@ -351,9 +361,11 @@ size_t topk_smem_bytes(int64_t V, int K) { return topk_fixed_bytes(K) + 2 * topk
 // bound of row i + 1 (into bucket buffer (i + 1) % 2) while its two selector
 // warps run collect, select and the KL of row i from buffer i % 2, so the SM's
 // teacher stream does not pause for the latency-bound phases.
-template <bool BF16>
-__global__ void __launch_bounds__(kTkThreads, kTkMinBlocks) k_topk_rows(TopkArgs a)
+// DN: a dense gradient row is written.
+template <bool BF16, int SW, bool DN>
+__global__ void __launch_bounds__(kTkStreamThreads + 32 * SW, kTkMinBlocks) k_topk_rows(TopkArgs a)
 {
+    constexpr int kTkSelWarps = SW, kTkSelThreads = 32 * SW, kTkThreads = kTkStreamThreads + kTkSelThreads;
     // the loss sum after this grid may take the first SM it frees (it waits for the grid)
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     extern __shared__ __align__(128) uint64_t tk_smem[];
@@ -411,6 +423,47 @@ __global__ void __launch_bounds__(kTkThreads, kTkMinBlocks) k_topk_rows(TopkArgs
         auto row_vectors = [&](const int4 &mr) {
             return reinterpret_cast<const uint4 *>(static_cast<const char *>(a.zt) + (size_t)mr.y * (size_t)a.ld * esz);
         };
+        auto zero_row = [&](int row, int t0) {
+            const size_t gesz = a.grad_dtype == TURNOPD_BF16 ? 2 : 4;
+            char *grow = static_cast<char *>(a.grad) + (size_t)row * (size_t)a.ld * gesz;
+            const int64_t bytes = a.vocab * (int64_t)gesz;
+            // 16-byte stores between a head up to the first 16-byte boundary and a tail
+            const int64_t head = min(bytes, (int64_t)((16u - (reinterpret_cast<uintptr_t>(grow) & 15u)) & 15u));
+            const int64_t nv16 = (bytes - head) / 16;
+            uint4 *body = reinterpret_cast<uint4 *>(grow + head);
+            for (int64_t q = t0; q < nv16; q += kTkStreamThreads)
+                __stcs(body + q, make_uint4(0, 0, 0, 0));
+            for (int64_t q = t0; q < head / 2; q += kTkStreamThreads)
+                reinterpret_cast<uint16_t *>(grow)[q] = 0;
+            for (int64_t q = (head + nv16 * 16) / 2 + t0; q < bytes / 2; q += kTkStreamThreads)
+                reinterpret_cast<uint16_t *>(grow)[q] = 0;
+        };
+        // The largest value x <= hi with at least K counted at or above it (0: none), by binary
+        // search; warp_count(x) is a warp's count.  The first pass probes 255 below hi (where
+        // the K-th largest bucket of a row with a few hundred large logits lies), and only when
+        // fewer than K reach that does the search span the rest.  The warps' counts alternate
+        // between two rows of s_scnt, so one barrier a pass suffices: a pass's reads finish
+        // before any thread passes the next barrier.
+        auto kth_bucket = [&](uint32_t hi, auto &&warp_count) {
+            uint32_t lo = 0;  // count(>= lo) >= K or lo = 0; the answer is in [lo, hi]
+            const uint32_t probe = hi > 255u ? hi - 255u : 0u;
+            for (int par = 0, first = 1; lo < hi; par ^= 1, first = 0) {
+                const uint32_t mid = first && probe > lo ? probe : (lo + hi + 1) >> 1;
+                const int c = warp_count(mid);
+                if (lane == 0)
+                    s_scnt[par][warp] = c;
+                named_sync(kBarStream, kTkStreamThreads);
+                int tot = 0;
+#pragma unroll
+                for (int w = 0; w < kTkStreamWarps; ++w)
+                    tot += s_scnt[par][w];
+                if (tot >= K)
+                    lo = mid;
+                else
+                    hi = mid - 1;
+            }
+            return lo;
+        };
         int4 m_next = n_it > 0 ? a.rows[blockIdx.x] : make_int4(0, 0, -1, 0);
         if (n_it > 0)
             load_batch(row_vectors(m_next), tid);  // the first batch of each row is loaded a row ahead
@@ -427,6 +480,7 @@ __global__ void __launch_bounds__(kTkThreads, kTkMinBlocks) k_topk_rows(TopkArgs
             }
             const char *zt_row = static_cast<const char *>(a.zt) + (size_t)m.y * (size_t)a.ld * esz;
             uint16_t *s_bucket = s_bucket0 + b * bucket_elems;
+            bool refine = false;  // the bound came from the thread maxima (below)
             // group buckets and the thread's largest logit; whole groups of a 16-byte
             // aligned row are read as vectors, a batch at a time
             uint32_t tmax = 0;
@@ -455,6 +509,10 @@ __global__ void __launch_bounds__(kTkThreads, kTkMinBlocks) k_topk_rows(TopkArgs
                     tmax = max(tmax, o);
                 }
             }
+            // the dense gradient row's zeros (the selectors write the K values over them once
+            // this row's buffer is full)
+            if (DN)
+                zero_row(m.y, tid);
             // groups left: the partial last group, or every group of a misaligned row
             for (int g = ngv + tid; g < (int)ng; g += kTkStreamThreads) {
                 const uint32_t o = group_max_ord_scalar<BF16>(zt_row, a.vocab, g);
@@ -501,9 +559,6 @@ __global__ void __launch_bounds__(kTkThreads, kTkMinBlocks) k_topk_rows(TopkArgs
                 // bound, tau = 0, when the row has fewer than K groups)
                 const uint4 *b4 = reinterpret_cast<const uint4 *>(s_bucket);
                 const int n4 = (int)ng / 8;
-                // The answer is at most the row's largest bucket; the first pass probes 255 below
-                // it (where the K-th largest bucket of a row with a few hundred large logits lies),
-                // and only when fewer than K buckets reach that does the search span the rest.
                 const uint32_t wmax = __reduce_max_sync(0xffffffffu, bucket<BF16>(tmax));
                 if (lane == 0)
                     s_smax[warp] = wmax;
@@ -512,12 +567,17 @@ __global__ void __launch_bounds__(kTkThreads, kTkMinBlocks) k_topk_rows(TopkArgs
 #pragma unroll
                 for (int w = 0; w < kTkStreamWarps; ++w)
                     hi = max(hi, s_smax[w]);
-                uint32_t lo = 0;  // count(>= lo) >= K or lo = 0; the answer is in [lo, hi]
-                const uint32_t probe = hi > 255u ? hi - 255u : 0u;
-                // the warps' counts alternate between two rows of s_scnt, so one barrier a pass
-                // suffices: a pass's reads finish before any thread passes the next barrier
-                for (int par = 0, first = 1; lo < hi; par ^= 1, first = 0) {
-                    const uint32_t mid = first && probe > lo ? probe : (lo + hi + 1) >> 1;
+                // Up to three quarters of the threads the K-th largest thread maximum stands in for
+                // the K-th largest bucket: also K distinct elements, at most n ln 4 = 1.4 n elements
+                // of a row reach it (n threads), and its passes count registers where the others
+                // walk the row's buckets.
+                const int n_thr = min((int)ng, kTkStreamThreads);
+                const bool by_thread = K <= n_thr / 4 * 3;
+                refine = by_thread && K > kRefineMinK;
+                const uint32_t tb = bucket<BF16>(tmax);
+                const uint32_t lo = kth_bucket(hi, [&](uint32_t mid) {
+                    if (by_thread)
+                        return __popc(__ballot_sync(0xffffffffu, tb >= mid));
                     int c = 0;
                     for (int i = tid; i < n4; i += kTkStreamThreads) {
                         const uint4 q = b4[i];
@@ -525,26 +585,15 @@ __global__ void __launch_bounds__(kTkThreads, kTkMinBlocks) k_topk_rows(TopkArgs
                     }
                     for (int g = n4 * 8 + tid; g < (int)ng; g += kTkStreamThreads)
                         c += (uint32_t)s_bucket[g] >= mid;
-                    c = __reduce_add_sync(0xffffffffu, c);
-                    if (lane == 0)
-                        s_scnt[par][warp] = c;
-                    named_sync(kBarStream, kTkStreamThreads);
-                    int tot = 0;
-#pragma unroll
-                    for (int w = 0; w < kTkStreamWarps; ++w)
-                        tot += s_scnt[par][w];
-                    if (tot >= K)
-                        lo = mid;
-                    else
-                        hi = mid - 1;
-                }
+                    return (int)__reduce_add_sync(0xffffffffu, c);
+                });
                 if (tid == 0)
                     s_tau[b] = BF16 ? lo : lo << 16;
             }
             named_sync(kBarStream, kTkStreamThreads);
             // the whole groups that can hold an element >= tau: their bucket reaches tau's
             // (eight buckets a load; the list's order does not matter)
-            const uint32_t tb = bucket<BF16>(s_tau[b]);
+            const uint32_t taub = bucket<BF16>(s_tau[b]);
             auto list = [&](int g) {
                 const int p = atomicAdd(&s_ng[b], 1);
                 if (p < kTkGroupCap)
@@ -557,12 +606,55 @@ __global__ void __launch_bounds__(kTkThreads, kTkMinBlocks) k_topk_rows(TopkArgs
                 const uint32_t w4[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
                 for (int e = 0; e < 8; ++e)
-                    if (((w4[e >> 1] >> (16 * (e & 1))) & 0xFFFFu) >= tb)
+                    if (((w4[e >> 1] >> (16 * (e & 1))) & 0xFFFFu) >= taub)
                         list(i * 8 + e);
             }
             for (int g = n8 * 8 + tid; g < ngv; g += kTkStreamThreads)
-                if (s_bucket[g] >= tb)
+                if (s_bucket[g] >= taub)
                     list(g);
+            if (refine) {
+                // The list (about 1.6 K groups) holds every group whose bucket reaches the bound,
+                // so the K-th largest bucket among the listed is the row's: K groups are at or
+                // above it, and the list shrinks to those and its ties.
+                named_sync(kBarStream, kTkStreamThreads);
+                const int nl = s_ng[b];
+                if (nl > K && nl <= kRefine * kTkStreamThreads && nl <= kTkGroupCap) {
+                    uint16_t lg[kRefine];
+                    uint32_t lb[kRefine];
+                    uint32_t mx = 0;
+#pragma unroll
+                    for (int e = 0; e < kRefine; ++e) {
+                        const int i = tid + e * kTkStreamThreads;
+                        lg[e] = i < nl ? s_glist[b][i] : 0;
+                        lb[e] = i < nl ? s_bucket[lg[e]] : 0u;
+                        mx = max(mx, lb[e]);
+                    }
+                    mx = __reduce_max_sync(0xffffffffu, mx);
+                    if (lane == 0)
+                        s_smax[warp] = mx;
+                    named_sync(kBarStream, kTkStreamThreads);
+                    uint32_t hi = 0;
+#pragma unroll
+                    for (int w = 0; w < kTkStreamWarps; ++w)
+                        hi = max(hi, s_smax[w]);
+                    const uint32_t kth = kth_bucket(hi, [&](uint32_t mid) {
+                        int c = 0;
+#pragma unroll
+                        for (int e = 0; e < kRefine; ++e)
+                            c += __popc(__ballot_sync(0xffffffffu, lb[e] >= mid));
+                        return c;
+                    });
+                    if (tid == 0) {
+                        s_tau[b] = max(s_tau[b], BF16 ? kth : kth << 16);
+                        s_ng[b] = 0;
+                    }
+                    named_sync(kBarStream, kTkStreamThreads);
+#pragma unroll
+                    for (int e = 0; e < kRefine; ++e)
+                        if (tid + e * kTkStreamThreads < nl && lb[e] >= kth)
+                            list(lg[e]);
+                }
+            }
             named_arrive(kBarFull + b, kTkThreads);  // row it is in buffer b
         }
         return;
@@ -772,7 +864,7 @@ __global__ void __launch_bounds__(kTkThreads, kTkMinBlocks) k_topk_rows(TopkArgs
                 // of two, at most the buffer's size) and take the first K
                 // Each key carries its buffer position in its low 11 bits, below the id's 20:
                 // ids are below 2^20, so ~id's upper 12 bits are ones and the order is kept.
-                int n2 = kTkRankMax;
+                int n2 = 512;
                 while (n2 < nc)
                     n2 <<= 1;
                 for (int i = stid; i < n2; i += kTkSelThreads) {
@@ -780,7 +872,7 @@ __global__ void __launch_bounds__(kTkThreads, kTkMinBlocks) k_topk_rows(TopkArgs
                     s_cand[i] = i < nc ? (k & 0xFFFFFFFF00000000ull) | ((k & 0xFFFFFull) << 11) | (uint64_t)i : 0ull;
                 }
                 named_sync(kBarSel, kTkSelThreads);
-                sort_desc<BF16 ? 4 : 2>(s_cand, n2, stid);
+                sort_desc<BF16 ? 4 : 2, SW>(s_cand, n2, stid);
                 for (int r = stid; r < K; r += kTkSelThreads) {
                     const uint64_t p = s_cand[r];
                     s_top[r] = (p & 0xFFFFFFFF00000000ull) | 0xFFF00000ull | ((p >> 11) & 0xFFFFFull);
@@ -788,19 +880,24 @@ __global__ void __launch_bounds__(kTkThreads, kTkMinBlocks) k_topk_rows(TopkArgs
                 }
             } else {
                 // ---- the K largest: each candidate's rank among the candidates is its position
-                // (keys are unique); a buffer larger than the selector threads is first cut to the
-                // K largest by radix select
-                const uint64_t kth = nc <= kTkSelThreads ? 0 : sel_kth_largest(s_cand, nc, K, hi_val, 0, s_sel, stid);
+                // (keys are unique).  A buffer of more than twice K is first cut to the K largest by
+                // radix select; below that its passes cost more than the ranks they save.  Two keys
+                // of the buffer are read a load.
+                const uint64_t kth = nc <= 2 * K ? 0 : sel_kth_largest<SW>(s_cand, nc, K, hi_val, 0, s_sel, stid);
+                if (stid == 0 && (nc & 1))
+                    s_cand[nc] = 0;  // the last pair's second key
+                named_sync(kBarSel, kTkSelThreads);
+                const ulonglong2 *pairs = reinterpret_cast<const ulonglong2 *>(s_cand);
                 for (int i = stid; i < nc; i += kTkSelThreads) {
                     const uint64_t k = s_cand[i];
                     if (k < kth)
                         continue;
                     int rank = 0;
-                    int i2 = 0;
-                    for (; i2 + 4 <= nc; i2 += 4)
-                        rank += (s_cand[i2] > k) + (s_cand[i2 + 1] > k) + (s_cand[i2 + 2] > k) + (s_cand[i2 + 3] > k);
-                    for (; i2 < nc; ++i2)
-                        rank += s_cand[i2] > k;
+#pragma unroll 2
+                    for (int q = 0; q < (nc + 1) / 2; ++q) {
+                        const ulonglong2 x = pairs[q];
+                        rank += (int)(x.x > k) + (int)(x.y > k);
+                    }
                     if (rank < K) {
                         s_top[rank] = k;
                         s_g[rank] = s_cz[i];
@@ -851,18 +948,11 @@ __global__ void __launch_bounds__(kTkThreads, kTkMinBlocks) k_topk_rows(TopkArgs
                     a.row_wl[j] = (double)w * (double)ell;
                 }
             }
-            // ---- dense gradient row: zeros, then the K entries
-            if (a.grad) {
+            // ---- dense gradient row: the K entries, over the streaming warps' zeros
+            if (DN) {
                 const size_t gesz = a.grad_dtype == TURNOPD_BF16 ? 2 : 4;
                 char *grow = static_cast<char *>(a.grad) + (size_t)m.y * (size_t)a.ld * gesz;
-                const int64_t bytes = a.vocab * (int64_t)gesz;
-                const bool g_ok = ((reinterpret_cast<uintptr_t>(grow)) & 15u) == 0;
-                const int64_t nv16 = g_ok ? bytes / 16 : 0;
-                for (int64_t q = stid; q < nv16; q += kTkSelThreads)
-                    reinterpret_cast<uint4 *>(grow)[q] = make_uint4(0, 0, 0, 0);
-                for (int64_t q = nv16 * 16 + stid; q < bytes; q += kTkSelThreads)
-                    grow[q] = 0;
-                named_sync(kBarSel, kTkSelThreads);
+                named_sync(kBarSel, kTkSelThreads);  // every entry of s_g is written
                 for (int r = stid; r < K; r += kTkSelThreads) {
                     const uint32_t id = key_id(s_top[r]);
                     if (a.grad_dtype == TURNOPD_BF16)
@@ -922,10 +1012,18 @@ cudaError_t launch_topk(const TopkCall &c, cudaStream_t stream)
     int dev = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess)
         return e;
-    const int ti = c.in_dtype == TURNOPD_BF16 ? 0 : 1;
-    auto kern = c.in_dtype == TURNOPD_BF16 ? k_topk_rows<true> : k_topk_rows<false>;
+    const bool large = c.K > kTkLaneBoundMaxK;
+    const int ti = (c.in_dtype == TURNOPD_BF16 ? 0 : 1) + (large ? 2 : 0) + (c.grad ? 4 : 0);
+    using Kern = void (*)(TopkArgs);
+    static const Kern kerns[8] = {
+        k_topk_rows<true, kTkSelSmall, false>, k_topk_rows<false, kTkSelSmall, false>,
+        k_topk_rows<true, kTkSelLarge, false>, k_topk_rows<false, kTkSelLarge, false>,
+        k_topk_rows<true, kTkSelSmall, true>,  k_topk_rows<false, kTkSelSmall, true>,
+        k_topk_rows<true, kTkSelLarge, true>,  k_topk_rows<false, kTkSelLarge, true>};
+    const Kern kern = kerns[ti];
+    const int kTkThreads = kTkStreamThreads + 32 * (large ? kTkSelLarge : kTkSelSmall);
     const size_t smem = topk_smem_bytes(c.vocab, c.K);
-    static size_t attr_smem[64][2] = {};
+    static size_t attr_smem[64][8] = {};
     const int di = dev < 64 ? dev : 0;
     if (attr_smem[di][ti] < smem) {
         if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
