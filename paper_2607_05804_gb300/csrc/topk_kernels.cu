@@ -6,7 +6,8 @@
 //   l   = sum_{v in S} ps_v (log ps_v - log pt_v)
 //   g_v = w ps_v (log ps_v - log pt_v - l)  on S, 0 elsewhere (= w dl/dz_s).
 //
-// Persistent CTAs, each with two rows in flight: streaming warps run pass A
+// Short rows and rows of any other alignment: k_topk_short, one CTA a row.  Others:
+// persistent CTAs, each with two rows in flight: streaming warps run pass A
 // of a row while two selector warps run the later phases of the previous row
 // (double-buffered buckets, named barriers).  Selection with 64-bit keys
 // (order-preserving logit bits << 32 | ~id, so larger key = larger logit,
@@ -41,6 +42,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <cmath>
 
 #include "common.cuh"
 #include "kernels.h"
@@ -968,6 +970,323 @@ __global__ void __launch_bounds__(kTkStreamThreads + 32 * SW, kTkMinBlocks) k_to
     }
 }
 
+// ---------------------------------------------------------------- short rows
+
+// The loss of a row from its K selected: l, ids and sparse gradient out, s_g (the student
+// logits) replaced by the gradient.  One warp, fp32.
+template <bool BF16>
+__device__ __forceinline__ void short_kl(const TopkArgs &a, const int4 &m, int j, const uint64_t *s_top, float *s_g,
+                                         int lane)
+{
+    const int K = a.K, tok = m.x;
+    const float w = __int_as_float(m.w);
+    float m_s = -INFINITY, m_t = -INFINITY;
+    for (int r = lane; r < K; r += 32) {
+        m_s = fmaxf(m_s, s_g[r]);
+        m_t = fmaxf(m_t, key_value<BF16>(s_top[r]));
+    }
+    m_s = warp_max_f(m_s);
+    m_t = warp_max_f(m_t);
+    float s_s = 0.f, s_t = 0.f, a_sd = 0.f;
+    for (int r = lane; r < K; r += 32) {
+        const float zs_v = s_g[r], zt_v = key_value<BF16>(s_top[r]);
+        const float es = expf(zs_v - m_s);
+        s_s += es;
+        s_t += expf(zt_v - m_t);
+        a_sd = fmaf(es, zs_v - zt_v, a_sd);
+    }
+    s_s = warp_sum_f(s_s);
+    s_t = warp_sum_f(s_t);
+    a_sd = warp_sum_f(a_sd);
+    const float ep = a_sd / s_s;                    // E_p[z_s - z_t]
+    const float c = (m_s - m_t) + logf(s_s / s_t);  // LSE_s - LSE_t
+    const float ell = ep - c;
+    for (int r = lane; r < K; r += 32) {
+        const float zs_v = s_g[r], zt_v = key_value<BF16>(s_top[r]);
+        const float g = w * (expf(zs_v - m_s) / s_s) * ((zs_v - zt_v) - ep);
+        s_g[r] = g;
+        if (a.topk_ids)
+            a.topk_ids[(size_t)tok * K + r] = (int32_t)key_id(s_top[r]);
+        if (a.topk_grad)
+            a.topk_grad[(size_t)tok * K + r] = g;
+    }
+    if (lane == 0) {
+        if (!isfinite(ell))
+            set_status(a.status, TURNOPD_ERR_NONFINITE);
+        a.token_loss[tok] = ell;
+        a.row_wl[j] = (double)w * (double)ell;
+    }
+}
+
+// Candidates a short row's CTA holds: the K selected and the ties of the last bucket.
+__host__ __device__ constexpr int short_cap(int K) { return K <= 128 ? 256 : K <= 256 ? 512 : K <= 512 ? 1024 : 2048; }
+__host__ __device__ __forceinline__ size_t short_smem(int K)
+{
+    return (sizeof(uint64_t) + sizeof(float) + sizeof(int32_t)) * (size_t)short_cap(K) +
+           (sizeof(uint64_t) + sizeof(float)) * (size_t)K + 16;
+}
+constexpr int kShortPerThread = 64;  // elements of a row per thread
+// Aligned rows up to here (K above kTkLaneBoundMaxK: the second) take the kernel below; the
+// streaming kernel reads longer ones faster (bf16, K = 50, GB/s of the step at 4e8 logits:
+// V = 6,144 1,096 here and 773 there, 12,288 1,099 and 1,402; K = 256: 12,288 709 and 435,
+// 24,576 785 and 784).  Rows that are not 16-byte aligned, which the streaming kernel reads
+// element by element, take it at every length it holds (32,700: 1,248 and 448).
+constexpr int kShortMaxV = 7168, kShortMaxVLarge = 16384;
+
+// Rows of up to 64 NT elements, one CTA of NT threads a row, any alignment: the row's
+// 16-bit buckets (the logit itself for bf16) stay in registers, 2 to a word, from the only
+// read of the teacher.  The K-th largest bucket comes from a binary search on its value, a
+// compare and an add per pair and pass (bf16x2); the elements at or above it, K and the
+// ties of the last bucket, are ranked by their full keys.  k_topk_rows spends 10 us and
+// more a row on its two roles' hand-over and selection, whatever the row's length, with 608
+// rows in flight, and its bound fails where a row has fewer groups than K; here a short row
+// holds one to sixteen warps, up to 4,864 are in flight.  Bound by issue (3,200 warp
+// instructions a row of 2,034 at K = 50, IPC 1.9).  GB/s of the step at 4e8 logits, bf16, in
+// k_topk_rows and here: K = 50, V = 1,024 47 and 653, 2,034 47 and 988, 4,096 437 and 788;
+// K = 256 82 and 265, 65 and 368, 101 and 463.
+template <bool BF16, int NT>
+__global__ void __launch_bounds__(NT, 1024 / NT) k_topk_short(TopkArgs a)
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    constexpr int NW = NT / 32;
+    constexpr int ESZ = BF16 ? 2 : 4;
+    extern __shared__ __align__(16) uint64_t tk_smem[];
+    const int K = a.K, cap = short_cap(K);
+    uint64_t *s_key = tk_smem;                                 // [cap] candidates
+    uint64_t *s_top = s_key + cap;                             // [K] selected
+    float *s_cz = reinterpret_cast<float *>(s_top + K);        // [cap] their student logits
+    float *s_g = s_cz + cap;                                   // [K]
+    int32_t *s_id = reinterpret_cast<int32_t *>(s_g + K);      // [cap]
+    __shared__ int s_cnt[2][NW];
+    __shared__ float s_max[NW];
+    __shared__ int s_n;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int V = (int)a.vocab;
+    const int n_rows = *a.nvalid;
+    auto sync = [&]() {
+        if (NT == 32)
+            __syncwarp();
+        else
+            __syncthreads();
+    };
+    int par = 0;  // the warps' counts alternate between two rows of s_cnt: one barrier a count
+    auto block_count = [&](int c) {  // c: this thread's
+        c = __reduce_add_sync(0xffffffffu, c);
+        if (NT == 32)
+            return c;
+        if (lane == 0)
+            s_cnt[par][warp] = c;
+        __syncthreads();
+        int tot = 0;
+#pragma unroll
+        for (int w = 0; w < NW; ++w)
+            tot += s_cnt[par][w];
+        par ^= 1;
+        return tot;
+    };
+    auto bits_of = [](uint32_t o) { return (o & 0x8000u) ? o & 0x7FFFu : ~o & 0xFFFFu; };
+    auto splat2 = [](uint32_t bits) {
+        const uint32_t w = bits | bits << 16;
+        return *reinterpret_cast<const __nv_bfloat162 *>(&w);
+    };
+
+    for (int j = blockIdx.x; j < n_rows; j += gridDim.x) {
+        const int4 m = a.rows[j];
+        const char *zt_row = static_cast<const char *>(a.zt) + (size_t)m.y * (size_t)a.ld * ESZ;
+        const char *zs_row = static_cast<const char *>(a.zs) + (size_t)m.y * (size_t)a.ld * ESZ;
+        // the row starts `head` elements into a 16-byte vector; octet q holds ids 8 q - head ..
+        const int head = (int)(reinterpret_cast<uintptr_t>(zt_row) & 15u) / ESZ;
+        const int octets = (head + V + 7) / 8;
+        __nv_bfloat162 bk[kShortPerThread / 2];
+        const char *vec = zt_row - head * ESZ;
+#pragma unroll
+        for (int u = 0; u < kShortPerThread / 8; ++u) {
+            const int q = tid + u * NT, i0 = q * 8 - head;
+            uint32_t w[4] = {0xff80ff80u, 0xff80ff80u, 0xff80ff80u, 0xff80ff80u};  // -inf: no element
+            if (q < octets) {
+                if (i0 >= 0 && i0 + 8 <= V) {
+                    const uint4 x = __ldg(reinterpret_cast<const uint4 *>(vec) + q * (ESZ / 2));
+                    if (BF16) {
+                        w[0] = x.x, w[1] = x.y, w[2] = x.z, w[3] = x.w;
+                    } else {
+                        const uint4 y = __ldg(reinterpret_cast<const uint4 *>(vec) + q * 2 + 1);
+                        w[0] = __byte_perm(x.x, x.y, 0x7632), w[1] = __byte_perm(x.z, x.w, 0x7632);
+                        w[2] = __byte_perm(y.x, y.y, 0x7632), w[3] = __byte_perm(y.z, y.w, 0x7632);
+                    }
+                } else {  // the first or the last octet: element by element
+#pragma unroll
+                    for (int e = 0; e < 8; ++e)
+                        if (i0 + e >= 0 && i0 + e < V) {
+                            const uint32_t b = BF16 ? reinterpret_cast<const uint16_t *>(zt_row)[i0 + e]
+                                                    : reinterpret_cast<const uint32_t *>(zt_row)[i0 + e] >> 16;
+                            w[e / 2] = e & 1 ? (w[e / 2] & 0xFFFFu) | b << 16 : (w[e / 2] & 0xFFFF0000u) | b;
+                        }
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k)  // + 0: -0 and +0 are the same logit
+                bk[u * 4 + k] = __hadd2(*reinterpret_cast<const __nv_bfloat162 *>(&w[k]), splat2(0));
+        }
+        if (a.grad) {  // the dense gradient row's zeros
+            const size_t gesz = a.grad_dtype == TURNOPD_BF16 ? 2 : 4;
+            char *grow = static_cast<char *>(a.grad) + (size_t)m.y * (size_t)a.ld * gesz;
+            const int64_t bytes = (int64_t)V * (int64_t)gesz;
+            const int64_t gh = min(bytes, (int64_t)((16u - (reinterpret_cast<uintptr_t>(grow) & 15u)) & 15u));
+            const int64_t nv16 = (bytes - gh) / 16;
+            uint4 *body = reinterpret_cast<uint4 *>(grow + gh);
+            for (int64_t q = tid; q < nv16; q += NT)
+                __stcs(body + q, make_uint4(0, 0, 0, 0));
+            for (int64_t q = tid; q < gh / 2; q += NT)
+                reinterpret_cast<uint16_t *>(grow)[q] = 0;
+            for (int64_t q = (gh + nv16 * 16) / 2 + tid; q < bytes / 2; q += NT)
+                reinterpret_cast<uint16_t *>(grow)[q] = 0;
+        }
+        // the row's largest bucket, NaN if one is
+        __nv_bfloat162 mx = bk[0];
+#pragma unroll
+        for (int k = 1; k < kShortPerThread / 2; ++k)
+            mx = __hmax2_nan(mx, bk[k]);
+        auto max_nan = [](float x, float y) { return x != x || y != y ? NAN : fmaxf(x, y); };
+        float top = max_nan(__bfloat162float(mx.x), __bfloat162float(mx.y));
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            top = max_nan(top, __shfl_xor_sync(0xffffffffu, top, o));
+        if (NT > 32) {
+            if (lane == 0)
+                s_max[warp] = top;
+            __syncthreads();
+#pragma unroll
+            for (int w = 0; w < NW; ++w)
+                top = max_nan(top, s_max[w]);
+        }
+        auto count = [&](const __nv_bfloat162 &x) {  // this thread's elements >= x (at most 32 in a half: exact)
+            __nv_bfloat162 c = splat2(0);
+#pragma unroll
+            for (int k = 0; k < kShortPerThread / 2; ++k)
+                c = __hadd2(c, __hge2(bk[k], x));
+            return (int)(__bfloat162float(c.x) + __bfloat162float(c.y));
+        };
+        // the K-th largest bucket: the largest x with at least K elements >= x.  The first probe
+        // is 255 below the maximum (where the K-th largest of a row of a few thousand lies)
+        uint32_t hi = ord16(__float_as_uint(top) >> 16), lo = 0x0080u;  // the lowest finite value: V >= K elements
+        const uint32_t probe = hi > 255u + lo ? hi - 255u : lo;
+        for (bool first = true; lo < hi; first = false) {
+            const uint32_t mid = first && probe > lo ? probe : (lo + hi + 1) >> 1;
+            if (block_count(count(splat2(bits_of(mid)))) >= K)
+                lo = mid;
+            else
+                hi = mid - 1;
+        }
+        // the elements at or above it, in a fixed order
+        const __nv_bfloat162 T = splat2(bits_of(lo));
+        const int mine = __reduce_add_sync(0xffffffffu, count(T));
+        int base = 0, n = mine;
+        if (NT > 32) {
+            if (lane == 0)
+                s_cnt[par][warp] = mine;
+            __syncthreads();
+            n = 0;
+#pragma unroll
+            for (int w = 0; w < NW; ++w) {
+                base += w < warp ? s_cnt[par][w] : 0;
+                n += s_cnt[par][w];
+            }
+            par ^= 1;
+        }
+        auto full_key = [&](int id) {
+            const uint32_t o = BF16 ? ord16(reinterpret_cast<const uint16_t *>(zt_row)[id])
+                                    : ord32(reinterpret_cast<const uint32_t *>(zt_row)[id]);
+            return mkkey(o, (uint32_t)id);
+        };
+        auto student = [&](int id) {
+            return BF16 ? __bfloat162float(reinterpret_cast<const __nv_bfloat16 *>(zs_row)[id])
+                        : reinterpret_cast<const float *>(zs_row)[id];
+        };
+        if (n <= cap && n >= K && top == top) {
+            const uint32_t below = (1u << lane) - 1u;
+#pragma unroll
+            for (int k = 0; k < kShortPerThread / 2; ++k) {
+                const unsigned hit = __hge2_mask(bk[k], T);
+                if (!__any_sync(0xffffffffu, hit))
+                    continue;
+                const int id = (tid + k / 4 * NT) * 8 - head + k % 4 * 2;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const bool in = h ? hit >> 16 : hit & 0xFFFFu;
+                    const unsigned who = __ballot_sync(0xffffffffu, in);
+                    if (in)
+                        s_id[base + __popc(who & below)] = id + h;
+                    base += __popc(who);
+                }
+            }
+            sync();
+            for (int i = tid; i < n; i += NT) {
+                const int id = s_id[i];
+                s_key[i] = full_key(id);
+                s_cz[i] = student(id);
+            }
+        } else {
+            // more ties than the buffer holds (rows of many equal logits), fewer than K finite
+            // logits, or a NaN: the K-th largest full key, bit by bit, then exactly K elements
+            uint64_t kth = 0;
+            for (int bit = BF16 ? 47 : 63; bit >= 0; --bit) {
+                const uint64_t x = kth | 1ull << bit;
+                int c = 0;
+                for (int id = tid; id < V; id += NT)
+                    c += full_key(id) >= x;
+                if (block_count(c) >= K)
+                    kth = x;
+            }
+            if (tid == 0)
+                s_n = 0;
+            sync();
+            for (int id = tid; id < V; id += NT) {
+                const uint64_t k = full_key(id);
+                if (k >= kth) {
+                    const int p = atomicAdd(&s_n, 1);
+                    s_key[p] = k;
+                    s_cz[p] = student(id);
+                }
+            }
+            n = K;
+        }
+        if (tid == 0 && (n & 1))
+            s_key[n] = 0;  // the last pair's second key
+        sync();
+        // each candidate's rank among the candidates is its position
+        const ulonglong2 *pairs = reinterpret_cast<const ulonglong2 *>(s_key);
+        for (int i = tid; i < n; i += NT) {
+            const uint64_t k = s_key[i];
+            int rank = 0;
+#pragma unroll 4
+            for (int q = 0; q < (n + 1) / 2; ++q) {
+                const ulonglong2 x = pairs[q];
+                rank += (int)(x.x > k) + (int)(x.y > k);
+            }
+            if (rank < K) {
+                s_top[rank] = k;
+                s_g[rank] = s_cz[i];
+            }
+        }
+        sync();
+        if (warp == 0)
+            short_kl<BF16>(a, m, j, s_top, s_g, lane);
+        if (a.grad) {
+            sync();
+            const size_t gesz = a.grad_dtype == TURNOPD_BF16 ? 2 : 4;
+            char *grow = static_cast<char *>(a.grad) + (size_t)m.y * (size_t)a.ld * gesz;
+            for (int r = tid; r < K; r += NT) {
+                const uint32_t id = key_id(s_top[r]);
+                if (a.grad_dtype == TURNOPD_BF16)
+                    reinterpret_cast<__nv_bfloat16 *>(grow)[id] = __float2bfloat16_rn(s_g[r]);
+                else
+                    reinterpret_cast<float *>(grow)[id] = s_g[r];
+            }
+        }
+        sync();  // the shared arrays are free
+    }
+}
+
 // Masked tokens' sparse rows: ids -1, gradients 0.
 __global__ void k_topk_zero_masked(const uint8_t *mask, int64_t T, int32_t K, int32_t *ids, float *g)
 {
@@ -1012,33 +1331,49 @@ cudaError_t launch_topk(const TopkCall &c, cudaStream_t stream)
     int dev = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess)
         return e;
+    using Kern = void (*)(TopkArgs);
+    static size_t attr_smem[64][16] = {};
+    const int di = dev < 64 ? dev : 0;
+    auto launch = [&](Kern kern, int slot, int threads, size_t smem) {
+        cudaError_t e = cudaSuccess;
+        if (attr_smem[di][slot] < smem) {
+            if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+                return e;
+            attr_smem[di][slot] = smem;
+        }
+        int nb = 0;
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, threads, smem)) != cudaSuccess)
+            return e;
+        if (nb < 1)
+            return cudaErrorInvalidConfiguration;
+        kern<<<sms * nb, threads, smem, stream>>>(a);
+        return cudaGetLastError();
+    };
+    const bool bf16 = c.in_dtype == TURNOPD_BF16;
+    // rows that a CTA holds in registers, with up to 7 elements before the first (kShortMaxV)
+    const int64_t span = c.vocab + 7;
+    const size_t esz = bf16 ? 2 : 4;
+    const bool aligned = ((reinterpret_cast<uintptr_t>(c.zt) | reinterpret_cast<uintptr_t>(c.zs) | (uintptr_t)(c.ld * esz)) & 15u) == 0;
+    if (span <= (int64_t)kShortPerThread * 512 && (!aligned || c.vocab <= (c.K <= kTkLaneBoundMaxK ? kShortMaxV : kShortMaxVLarge))) {
+        const int s4 = span <= kShortPerThread * 32 ? 0 : span <= kShortPerThread * 128 ? 1 : span <= kShortPerThread * 256 ? 2 : 3;
+        static const Kern shorts[2][4] = {
+            {k_topk_short<false, 32>, k_topk_short<false, 128>, k_topk_short<false, 256>, k_topk_short<false, 512>},
+            {k_topk_short<true, 32>, k_topk_short<true, 128>, k_topk_short<true, 256>, k_topk_short<true, 512>}};
+        static const int threads[4] = {32, 128, 256, 512};
+        if ((e = launch(shorts[bf16][s4], 8 + bf16 * 4 + s4, threads[s4], short_smem(c.K))) != cudaSuccess)
+            return e;
+        launch_loss_sum(ws.row_wl, ws.nvalid, c.loss, c.status, stream);
+        return cudaGetLastError();
+    }
     const bool large = c.K > kTkLaneBoundMaxK;
     const int ti = (c.in_dtype == TURNOPD_BF16 ? 0 : 1) + (large ? 2 : 0) + (c.grad ? 4 : 0);
-    using Kern = void (*)(TopkArgs);
     static const Kern kerns[8] = {
         k_topk_rows<true, kTkSelSmall, false>, k_topk_rows<false, kTkSelSmall, false>,
         k_topk_rows<true, kTkSelLarge, false>, k_topk_rows<false, kTkSelLarge, false>,
         k_topk_rows<true, kTkSelSmall, true>,  k_topk_rows<false, kTkSelSmall, true>,
         k_topk_rows<true, kTkSelLarge, true>,  k_topk_rows<false, kTkSelLarge, true>};
-    const Kern kern = kerns[ti];
-    const int kTkThreads = kTkStreamThreads + 32 * (large ? kTkSelLarge : kTkSelSmall);
-    const size_t smem = topk_smem_bytes(c.vocab, c.K);
-    static size_t attr_smem[64][8] = {};
-    const int di = dev < 64 ? dev : 0;
-    if (attr_smem[di][ti] < smem) {
-        if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
-            cudaSuccess)
-            return e;
-        attr_smem[di][ti] = smem;
-    }
-    int nb = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, kTkThreads, smem)) != cudaSuccess)
-        return e;
-    if (nb < 1)
-        return cudaErrorInvalidConfiguration;
-    kern<<<sms * nb, kTkThreads, smem, stream>>>(a);
-    e = cudaGetLastError();
-    if (e != cudaSuccess)
+    if ((e = launch(kerns[ti], ti, kTkStreamThreads + 32 * (large ? kTkSelLarge : kTkSelSmall),
+                    topk_smem_bytes(c.vocab, c.K))) != cudaSuccess)
         return e;
     launch_loss_sum(ws.row_wl, ws.nvalid, c.loss, c.status, stream);
     return cudaGetLastError();

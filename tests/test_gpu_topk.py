@@ -260,3 +260,52 @@ def test_empty_and_all_masked(P):
     ids, gk, tl, loss, st = run_topk(P, e, e, V, torch.zeros(0, dtype=torch.uint8, device="cuda"),
                                      torch.zeros(0, dtype=torch.float32, device="cuda"), K)
     assert st == 0 and loss == 0.0
+
+
+# Longest rows of the register-held selection, 64 elements a thread less 7 for the alignment,
+# for CTAs of 32, 128, 256 and 512 threads, and one more (the last: the streaming kernel).
+SHORT_EDGES = [64 * nt - 7 for nt in (32, 128, 256, 512)]
+
+
+@pytest.mark.parametrize("V", [3, 9, 100] + [e + d for e in SHORT_EDGES for d in (0, 1)])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_short_rows_at_the_edges(P, oracle, V, dtype):
+    """Odd strides (rows start anywhere in a vector; the logits end with the last row's last
+    column, NaN behind it), K = 1, 50 and 256, every row against the oracle; some rows hold
+    many equal largest logits (more ties than the candidate buffer), signed zeros, and the
+    type's lowest value outside their first ids; the dense gradient holds the sparse one and zeros."""
+    T, ld = 24, V + 2
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(V)
+    base = torch.randn((T, V), generator=gen, device="cuda") * 3
+    zs0 = (base + torch.randn((T, V), generator=gen, device="cuda")).to(dtype)
+    zt0 = base.to(dtype)
+    zt0[1] = 1.5                               # all equal
+    zt0[2, V // 3:] = 4.25                     # two thirds tied
+    zt0[3, ::2], zt0[3, 1::2] = 0.0, -0.0      # signed zeros are one logit
+    if V >= 600:
+        zt0[4, 600:] = torch.finfo(dtype).min  # a masked vocabulary
+    z = []
+    for src in (zs0, zt0):
+        buf = torch.full((T * ld + 64,), float("nan"), dtype=dtype, device="cuda")
+        v = buf[3:3 + T * ld].view(T, ld)      # a base that is not 16-byte aligned
+        v[:, :V] = src
+        z.append(v)
+    mask = torch.ones(T, dtype=torch.uint8, device="cuda")
+    mask[7] = 0
+    w = torch.rand(T, generator=gen, device="cuda")
+    for K in sorted({1, min(50, V), min(256, V)}):
+        if V >= 600 and K > 600:
+            continue
+        dense = torch.full((T, ld), 6.0, dtype=torch.float32, device="cuda")
+        ids, gk, tl, loss, st = run_topk(P, z[0], z[1], V, mask, w, K, dense=dense)
+        assert st == 0
+        check_against_oracle(oracle, z[0].contiguous()[:, :V].contiguous(), z[1].contiguous()[:, :V].contiguous(), V,
+                             mask, w, K, ids, gk, tl, loss)
+        d = dense.cpu().numpy()
+        assert (d[:, V:] == 6.0).all() and (d[7] == 6.0).all()
+        for t in range(T):
+            if t != 7:
+                want = np.zeros(V, np.float32)
+                want[ids[t]] = gk[t]
+                np.testing.assert_array_equal(d[t, :V], want)
