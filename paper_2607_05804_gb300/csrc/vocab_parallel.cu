@@ -38,6 +38,31 @@ struct ShardIn {
     int32_t *status;
 };
 
+// How the rows are read: element by element, in vectors with every row aligned, in vectors from
+// each row's first boundary.  fp32 rows that are all aligned have a form of their own: with the
+// offset a run-time value the compiler pipelines their loads less (statistics + gradient at
+// 4e8 logits, V = 2,048: 6,105 -> 5,750-5,929 GB/s).
+enum RowForm { kSingles, kAligned, kAnyOffset };
+
+// Elements of row r before its first 16-byte boundary (the arrays start at one): read
+// alone, as the last ones are.
+template <typename TIn> __device__ __forceinline__ int row_head(int64_t r, int64_t ld, int64_t V)
+{
+    constexpr int N = Vec<TIn>::N;
+    const int h = (N - ((int)(r & (N - 1)) * (int)(ld & (N - 1)) & (N - 1))) & (N - 1);
+    return h < V ? h : (int)V;
+}
+
+// The elements of a row outside its whole vectors [head, head + nvec N), one at a time.
+// (Loading them ahead of the vectors instead costs aligned bf16 rows 2-4 %.)
+template <typename TIn, typename F> __device__ __forceinline__ void each_single(int64_t V, int head, int64_t nvec, F &&f)
+{
+    const int64_t whole = nvec * Vec<TIn>::N;
+    for (int64_t k = threadIdx.x; k < V - whole; k += kVpThreads)
+        f(k < head ? k : k + whole);
+}
+
+// A row read element by element, or an aligned one in vectors.
 template <typename TIn, bool VEC>
 __device__ __forceinline__ void fold_row(const TIn *rs, const TIn *rt, int64_t V, Student &s, Teacher &t)
 {
@@ -57,7 +82,7 @@ __device__ __forceinline__ void fold_row(const TIn *rs, const TIn *rt, int64_t V
     }
 }
 
-// The same statistics for an aligned bf16 row in 16-byte vectors, kVpU vectors of
+// The statistics of a bf16 row's whole 16-byte vectors, kVpU vectors of
 // each model in flight per thread: a running maximum rescaled once per batch when it
 // moves, A kept relative to d at the thread's running student argmax (re-referenced,
 // A <- (A + S (d - d')) f, with the maximum), packed f32x2 sums.
@@ -152,7 +177,7 @@ __device__ __forceinline__ void block_merge(Student &s, Teacher &t, Student *red
     }
 }
 
-template <typename TIn, bool VEC>
+template <typename TIn, RowForm FORM>
 __global__ void __launch_bounds__(kVpThreads) k_shard_stats(ShardIn p, const int4 *__restrict__ rows,
                                                              const int32_t *__restrict__ nvalid, float *__restrict__ stats)
 {
@@ -171,16 +196,40 @@ __global__ void __launch_bounds__(kVpThreads) k_shard_stats(ShardIn p, const int
         const int64_t i = m.x, r = m.y;
         Student s = student_empty();
         Teacher t = teacher_empty();
-        if constexpr (VEC && std::is_same<TIn, __nv_bfloat16>::value) {
-            const int64_t nvec = p.vocab / 8;
-            fold_row_bf16(reinterpret_cast<const uint4 *>(zs + r * p.ld), reinterpret_cast<const uint4 *>(zt + r * p.ld),
-                          nvec, s, t);
-            for (int64_t v = nvec * 8 + threadIdx.x; v < p.vocab; v += kVpThreads) {  // ragged tail
-                float a = to_float(zs[r * p.ld + v]), b = to_float(zt[r * p.ld + v]);
-                accumulate<1>(s, t, &a, &b);
-            }
+        const TIn *rs = zs + r * p.ld, *rt = zt + r * p.ld;
+        if constexpr (FORM != kAnyOffset) {
+            fold_row<TIn, FORM == kAligned>(rs, rt, p.vocab, s, t);
         } else {
-            fold_row<TIn, VEC>(zs + r * p.ld, zt + r * p.ld, p.vocab, s, t);
+            constexpr int N = Vec<TIn>::N;
+            const int head = row_head<TIn>(r, p.ld, p.vocab);
+            const int64_t nvec = (p.vocab - head) / N;
+            if constexpr (std::is_same<TIn, __nv_bfloat16>::value) {
+                fold_row_bf16(reinterpret_cast<const uint4 *>(rs + head), reinterpret_cast<const uint4 *>(rt + head),
+                              nvec, s, t);
+            } else {
+                int64_t q = threadIdx.x;
+                for (; q + kVpThreads < nvec; q += 2 * kVpThreads) {  // two pairs in flight: V = 151,939 5,208 -> 5,839 GB/s
+                    float a[2][N], b[2][N];
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        Vec<TIn>::load(rs + head + (q + u * kVpThreads) * N, a[u]);
+                        Vec<TIn>::load(rt + head + (q + u * kVpThreads) * N, b[u]);
+                    }
+#pragma unroll
+                    for (int u = 0; u < 2; ++u)
+                        accumulate<N>(s, t, a[u], b[u]);
+                }
+                if (q < nvec) {
+                    float a[N], b[N];
+                    Vec<TIn>::load(rs + head + q * N, a);
+                    Vec<TIn>::load(rt + head + q * N, b);
+                    accumulate<N>(s, t, a, b);
+                }
+            }
+            each_single<TIn>(p.vocab, head, nvec, [&](int64_t v) {
+                float a = to_float(rs[v]), b = to_float(rt[v]);
+                accumulate<1>(s, t, &a, &b);
+            });
         }
         block_merge(s, t, red_s[par], red_t[par]);
         if (threadIdx.x == 0) {
@@ -208,7 +257,7 @@ __global__ void k_stats_merge(const float *__restrict__ parts, int n_shards, con
     }
 }
 
-template <typename TIn, typename TOut, bool VEC>
+template <typename TIn, typename TOut, RowForm FORM>
 __global__ void __launch_bounds__(kVpThreads)
 k_shard_grad(ShardIn p, const int4 *__restrict__ rows, const int32_t *__restrict__ nvalid,
              const float *__restrict__ merged, TOut *grad, float *token_loss, double *wl)
@@ -218,7 +267,6 @@ k_shard_grad(ShardIn p, const int4 *__restrict__ rows, const int32_t *__restrict
     const TIn *zs = static_cast<const TIn *>(p.zs);
     const TIn *zt = static_cast<const TIn *>(p.zt);
     const int64_t V = p.vocab;
-    const int64_t nvec = VEC ? V / N : 0;
     const int n = *nvalid;
     int4 m_next = (int)blockIdx.x < n ? rows[blockIdx.x] : make_int4(0, 0, 0, 0);
     for (int j = blockIdx.x, par = 0; j < n; j += gridDim.x, par ^= 1) {
@@ -243,10 +291,13 @@ k_shard_grad(ShardIn p, const int4 *__restrict__ rows, const int32_t *__restrict
         __syncthreads();
         if (grad) {
             const float nl = -bc[0] * kLog2e, d = bc[1], cp = bc[2], wi = bc[3];
-            const TIn *rs = zs + r * p.ld;
-            const TIn *rt = zt + r * p.ld;
-            TOut *gr = grad + r * p.ld;
-            if constexpr (VEC && std::is_same<TIn, __nv_bfloat16>::value) {
+            const int head = FORM == kAnyOffset ? row_head<TIn>(r, p.ld, V) : 0;
+            const int64_t nvec = FORM != kSingles ? (V - head) / N : 0;
+            // the row from its first 16-byte boundary
+            const TIn *rs = zs + r * p.ld + head;
+            const TIn *rt = zt + r * p.ld + head;
+            TOut *gr = grad + r * p.ld + head;
+            if constexpr (FORM != kSingles && std::is_same<TIn, __nv_bfloat16>::value) {
                 // kVpU vector pairs in flight per thread, packed arithmetic
                 const uint4 *vs = reinterpret_cast<const uint4 *>(rs), *vt = reinterpret_cast<const uint4 *>(rt);
                 const float2 L2 = splat(kLog2e), NL = splat(nl), D = splat(d), CP = splat(cp), WI = splat(wi);
@@ -277,7 +328,7 @@ k_shard_grad(ShardIn p, const int4 *__restrict__ rows, const int32_t *__restrict
                         store_vec<TOut, 8>(gr + q * 8, g);
                     }
                 }
-            } else if (VEC) {
+            } else if (FORM != kSingles) {
                 for (int64_t qv = threadIdx.x; qv < nvec; qv += kVpThreads) {
                     float a[N], b[N], g[N];
                     Vec<TIn>::load(rs + qv * N, a);
@@ -288,15 +339,38 @@ k_shard_grad(ShardIn p, const int4 *__restrict__ rows, const int32_t *__restrict
                     store_vec<TOut, N>(gr + qv * N, g);
                 }
             }
-            for (int64_t v = nvec * N + threadIdx.x; v < V; v += kVpThreads) {
+            const auto single = [&](int64_t v) {  // from the first boundary
                 const float a = to_float(rs[v]), b = to_float(rt[v]);
                 gr[v] = from_float<TOut>(wi * ex2(fmaf(a, kLog2e, nl)) * (((a - b) - d) - cp));
-            }
+            };
+            if constexpr (FORM == kAnyOffset)
+                each_single<TIn>(V, head, nvec, [&](int64_t v) { single(v - head); });
+            else
+                for (int64_t v = nvec * N + threadIdx.x; v < V; v += kVpThreads)
+                    single(v);
         }
     }
 }
 
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
+
+// Shards of at least this many columns are read in 16-byte vectors from each row's first
+// boundary whatever the stride.  GB/s of statistics + gradient at 4e8 logits, read element by
+// element -> in vectors: bf16, V = 1,027 1,854 -> 1,705 (the two singles loops of a short row
+// cost more than its vectors save), 1,283 1,997 -> 2,092, 2,051 2,271 -> 3,109, 16,387 2,411 ->
+// 5,864, 151,939 1,449 -> 5,775; fp32, V = 1,027 3,432 -> 4,636, 16,387 4,320 -> 6,461.
+constexpr int64_t kVpVecMinBf16 = 1200;
+
+RowForm row_form(const VocabShardCall &c)
+{
+    const bool bf16 = c.in_dtype == TURNOPD_BF16;
+    if (!aligned16(c.zs) || !aligned16(c.zt))
+        return kSingles;
+    const bool rows_aligned = c.ld % (bf16 ? 8 : 4) == 0;
+    if (bf16)  // aligned rows too: 5,704 -> 5,980 GB/s at V = 151,936
+        return rows_aligned || c.vocab >= kVpVecMinBf16 ? kAnyOffset : kSingles;
+    return rows_aligned ? kAligned : kAnyOffset;
+}
 
 // The grids are persistent (each CTA strides over the rows), so they are sized to
 // the CTAs that are co-resident: a larger grid would run its surplus as a late
@@ -343,10 +417,12 @@ cudaError_t launch_vocab_shard_stats(const VocabShardCall &c, float *stats, cuda
     if (e != cudaSuccess)
         return e;
     ShardIn p{c.zs, c.zt, c.ld, c.vocab, c.num_rows, c.row_of_token, c.mask, c.T, c.status};
-    const size_t esz = c.in_dtype == TURNOPD_BF16 ? 2 : 4;
-    const bool vec = aligned16(c.zs) && aligned16(c.zt) && (c.ld * esz) % 16 == 0;
-    auto kern = c.in_dtype == TURNOPD_BF16 ? (vec ? k_shard_stats<__nv_bfloat16, true> : k_shard_stats<__nv_bfloat16, false>)
-                                           : (vec ? k_shard_stats<float, true> : k_shard_stats<float, false>);
+    const RowForm form = row_form(c);
+    auto kern = c.in_dtype == TURNOPD_BF16
+                    ? (form == kSingles ? k_shard_stats<__nv_bfloat16, kSingles> : k_shard_stats<__nv_bfloat16, kAnyOffset>)
+                : form == kSingles ? k_shard_stats<float, kSingles>
+                : form == kAligned ? k_shard_stats<float, kAligned>
+                                   : k_shard_stats<float, kAnyOffset>;
     kern<<<resident_grid(kern, c.T), kVpThreads, 0, stream>>>(p, ws.rows, ws.nvalid, stats);
     return cudaGetLastError();
 }
@@ -360,10 +436,14 @@ cudaError_t launch_vocab_stats_merge(const float *parts, int n_shards, const uin
 }
 
 template <typename TIn, typename TOut>
-static void shard_grad_kernel(const ShardIn &p, bool vec, const LossWorkspace &ws, const float *merged, void *grad,
+static void shard_grad_kernel(const ShardIn &p, RowForm form, const LossWorkspace &ws, const float *merged, void *grad,
                               float *tl, cudaStream_t stream)
 {
-    auto kern = vec ? k_shard_grad<TIn, TOut, true> : k_shard_grad<TIn, TOut, false>;
+    auto kern = form == kSingles ? k_shard_grad<TIn, TOut, kSingles> : k_shard_grad<TIn, TOut, kAnyOffset>;
+    if constexpr (std::is_same<TIn, float>::value) {
+        if (form == kAligned)
+            kern = k_shard_grad<TIn, TOut, kAligned>;
+    }
     kern<<<resident_grid(kern, p.T), kVpThreads, 0, stream>>>(p, ws.rows, ws.nvalid, merged,
                                                                   static_cast<TOut *>(grad), tl, ws.row_wl);
 }
@@ -372,10 +452,9 @@ cudaError_t launch_vocab_shard_grad(const VocabShardCall &c, const float *merged
 {
     LossWorkspace ws = loss_workspace_layout(c.workspace, c.T);
     ShardIn p{c.zs, c.zt, c.ld, c.vocab, c.num_rows, c.row_of_token, c.mask, c.T, c.status};
-    const size_t esz = c.in_dtype == TURNOPD_BF16 ? 2 : 4;
-    const size_t gesz = c.grad_dtype == TURNOPD_BF16 ? 2 : 4;
-    const bool vec = aligned16(c.zs) && aligned16(c.zt) && (c.ld * esz) % 16 == 0 &&
-                     (!c.grad || (aligned16(c.grad) && (c.ld * gesz) % 16 == 0));
+    // (a vector of the row starts at an element that is a multiple of N, so the gradient's
+    // vectors are as aligned as the array: 16 bytes, 8 for fp32 logits with a bf16 one)
+    const RowForm form = c.grad && !aligned16(c.grad) ? kSingles : row_form(c);
     cudaError_t e = compact_rows(c, c.w, c.token_loss, ws, stream);
     if (e != cudaSuccess)
         return e;
@@ -383,13 +462,13 @@ cudaError_t launch_vocab_shard_grad(const VocabShardCall &c, const float *merged
         launch_zero_masked_grad(c.mask, c.row_of_token, c.T, c.num_rows, c.ld, c.vocab, c.grad, c.grad_dtype, stream);
     const bool bf_in = c.in_dtype == TURNOPD_BF16, bf_out = c.grad_dtype == TURNOPD_BF16;
     if (bf_in && bf_out)
-        shard_grad_kernel<__nv_bfloat16, __nv_bfloat16>(p, vec, ws, merged, c.grad, c.token_loss, stream);
+        shard_grad_kernel<__nv_bfloat16, __nv_bfloat16>(p, form, ws, merged, c.grad, c.token_loss, stream);
     else if (bf_in)
-        shard_grad_kernel<__nv_bfloat16, float>(p, vec, ws, merged, c.grad, c.token_loss, stream);
+        shard_grad_kernel<__nv_bfloat16, float>(p, form, ws, merged, c.grad, c.token_loss, stream);
     else if (bf_out)
-        shard_grad_kernel<float, __nv_bfloat16>(p, vec, ws, merged, c.grad, c.token_loss, stream);
+        shard_grad_kernel<float, __nv_bfloat16>(p, form, ws, merged, c.grad, c.token_loss, stream);
     else
-        shard_grad_kernel<float, float>(p, vec, ws, merged, c.grad, c.token_loss, stream);
+        shard_grad_kernel<float, float>(p, form, ws, merged, c.grad, c.token_loss, stream);
     e = cudaGetLastError();
     if (e != cudaSuccess)
         return e;

@@ -152,3 +152,39 @@ def test_bad_row_index_sets_status_and_skips_the_token(P, oracle):
     assert (g[bad] == 7.0).all()  # no token maps to this row
     ok = m2 == 1
     assert_grad_rows(g[ok], g_ref[ok], bf16=False)
+
+
+@pytest.mark.parametrize("V,ld", [(2, 3), (7, 9), (12, 12), (1199, 1201), (1200, 1203), (8211, 8211)])
+@pytest.mark.parametrize("dt,gdt", [("bf16", "bf16"), ("bf16", "f32"), ("f32", "bf16"), ("f32", "f32")])
+def test_rows_at_any_offset(P, oracle, V, ld, dt, gdt):
+    """Rows that start anywhere in a 16-byte vector, from shorter than the head to several
+    rounds of vectors, and both sides of the bf16 line (1,200) below which elements are read
+    singly; the last row ends the array and the gradient's padding stays as it was."""
+    b = W.packed(seed=9, num_traj=2, traj_len=48)
+    tdt = {"bf16": torch.bfloat16, "f32": torch.float32}
+    T = b.num_tokens
+    z = []
+    for src in W.make_logits(T, V, "agent" if V > 16 else "tiny", tdt[dt], seed=43, device="cuda"):
+        buf = torch.full((T * ld,), float("nan"), dtype=tdt[dt], device="cuda")
+        z.append(buf.as_strided((T, V), (ld, 1)))
+        z[-1].copy_(src)
+    mask = torch.from_numpy(b.loss_mask).cuda()
+    w = torch.rand(T, generator=torch.Generator().manual_seed(8)).cuda()
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    ws = torch.empty(max(P.turnopd_loss_workspace_bytes(T), 256), dtype=torch.uint8, device="cuda")
+    stats = torch.empty((T, 6), dtype=torch.float32, device="cuda")
+    P.turnopd_vocab_shard_stats(z[0], z[1], None, mask, stats, ws, st)
+    whole = torch.full((T, ld), 7.0, dtype=tdt[gdt], device="cuda")
+    tl = torch.empty(T, dtype=torch.float32, device="cuda")
+    loss = torch.zeros(1, dtype=torch.float64, device="cuda")
+    P.turnopd_vocab_shard_loss_grad(z[0], z[1], None, mask, w, stats, whole[:, :V], 0, tl, loss, ws, st)
+    torch.cuda.synchronize()
+    assert st.item() == 0
+    g_ref, tl_ref, loss_ref = oracle.loss_fwd_bwd(z[0].float().cpu().numpy(), z[1].float().cpu().numpy(), V,
+                                                  b.loss_mask, w.cpu().numpy())
+    m = b.loss_mask == 1
+    assert_token_loss(tl.cpu().numpy(), tl_ref, b.loss_mask)
+    assert_loss(loss.item(), loss_ref)
+    assert_grad_rows(whole[:, :V].float().cpu().numpy()[m], g_ref[m], bf16=gdt == "bf16",
+                     zs=z[0][torch.from_numpy(m).cuda()].float(), w=w.cpu().numpy()[m], ell=tl_ref[m])
+    assert (whole[torch.from_numpy(~m).cuda()].float() == 7.0).all() and (whole[:, V:].float() == 7.0).all()
