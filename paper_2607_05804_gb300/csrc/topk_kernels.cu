@@ -1026,12 +1026,16 @@ __host__ __device__ __forceinline__ size_t short_smem(int K)
            (sizeof(uint64_t) + sizeof(float)) * (size_t)K + 16;
 }
 constexpr int kShortPerThread = 64;  // elements of a row per thread
-// Aligned rows up to here (K above kTkLaneBoundMaxK: the second) take the kernel below; the
-// streaming kernel reads longer ones faster (bf16, K = 50, GB/s of the step at 4e8 logits:
-// V = 6,144 1,096 here and 773 there, 12,288 1,099 and 1,402; K = 256: 12,288 709 and 435,
-// 24,576 785 and 784).  Rows that are not 16-byte aligned, which the streaming kernel reads
-// element by element, take it at every length it holds (32,700: 1,248 and 448).
-constexpr int kShortMaxV = 7168, kShortMaxVLarge = 16384;
+// Aligned rows up to here take the kernel below: what 128 threads hold, and what 256 hold from
+// K = kShortLargeK.  The streaming kernel reads longer rows faster.  us of a step of 2e8 bf16
+// logits, here and there: V = 8,184, K = 8 275 and 386, 50 316 and 501, 96 356 and 1,890;
+// V = 8,192 (256 threads), K = 64 551 and 676; 12,288, K = 32 370 and 300, 50 392 and 329, 64
+// 394 and 453; 16,376, K = 64 322 and 376, 256 516 and 879; 24,576 (512 threads), K = 80 434 and
+// 301, 128 459 and 354, 256 557 and 595.  fp32 rows cross at the same places.  Rows that are not
+// 16-byte aligned, which the streaming kernel reads element by element, take it at every length
+// it holds (32,700, K = 50: 1,248 GB/s and 448).
+constexpr int kShortMaxV = kShortPerThread * 128 - 7, kShortMaxVLarge = kShortPerThread * 256 - 7;
+constexpr int kShortLargeK = 64;
 
 // Rows of up to 64 NT elements, one CTA of NT threads a row, any alignment: the row's
 // 16-bit buckets (the logit itself for bf16) stay in registers, 2 to a word, from the only
@@ -1354,7 +1358,7 @@ cudaError_t launch_topk(const TopkCall &c, cudaStream_t stream)
     const int64_t span = c.vocab + 7;
     const size_t esz = bf16 ? 2 : 4;
     const bool aligned = ((reinterpret_cast<uintptr_t>(c.zt) | reinterpret_cast<uintptr_t>(c.zs) | (uintptr_t)(c.ld * esz)) & 15u) == 0;
-    if (span <= (int64_t)kShortPerThread * 512 && (!aligned || c.vocab <= (c.K <= kTkLaneBoundMaxK ? kShortMaxV : kShortMaxVLarge))) {
+    if (span <= (int64_t)kShortPerThread * 512 && (!aligned || c.vocab <= (c.K < kShortLargeK ? kShortMaxV : kShortMaxVLarge))) {
         const int s4 = span <= kShortPerThread * 32 ? 0 : span <= kShortPerThread * 128 ? 1 : span <= kShortPerThread * 256 ? 2 : 3;
         static const Kern shorts[2][4] = {
             {k_topk_short<false, 32>, k_topk_short<false, 128>, k_topk_short<false, 256>, k_topk_short<false, 512>},

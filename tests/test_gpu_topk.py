@@ -309,3 +309,21 @@ def test_short_rows_at_the_edges(P, oracle, V, dtype):
                 want = np.zeros(V, np.float32)
                 want[ids[t]] = gk[t]
                 np.testing.assert_array_equal(d[t, :V], want)
+
+
+@pytest.mark.parametrize("V", [e // 8 * 8 + d for e in SHORT_EDGES[1:3] for d in (0, 8)])
+@pytest.mark.parametrize("K", [1, 63, 64, 256])
+def test_aligned_rows_at_the_selection_lines(P, oracle, V, K):
+    """Aligned rows on both sides of the lengths and the K from which they are streamed."""
+    T = 12
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(V + K)
+    zt = torch.randn((T, V), generator=gen, device="cuda") * 3
+    zs = (zt + torch.randn((T, V), generator=gen, device="cuda")).to(torch.bfloat16)
+    zt = zt.to(torch.bfloat16)
+    mask = torch.ones(T, dtype=torch.uint8, device="cuda")
+    mask[5] = 0
+    w = torch.rand(T, generator=gen, device="cuda")
+    ids, gk, tl, loss, st = run_topk(P, zs, zt, V, mask, w, K)
+    assert st == 0
+    check_against_oracle(oracle, zs, zt, V, mask, w, K, ids, gk, tl, loss)
