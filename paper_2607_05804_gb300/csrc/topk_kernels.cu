@@ -884,21 +884,34 @@ __global__ void __launch_bounds__(kTkStreamThreads + 32 * SW, kTkMinBlocks) k_to
                 // ---- the K largest: each candidate's rank among the candidates is its position
                 // (keys are unique).  A buffer of more than twice K is first cut to the K largest by
                 // radix select; below that its passes cost more than the ranks they save.  Two keys
-                // of the buffer are read a load.
-                const uint64_t kth = nc <= 2 * K ? 0 : sel_kth_largest<SW>(s_cand, nc, K, hi_val, 0, s_sel, stid);
-                if (stid == 0 && (nc & 1))
-                    s_cand[nc] = 0;  // the last pair's second key
-                named_sync(kBarSel, kTkSelThreads);
+                // of the buffer are read a load, but for two warps, K > 16 and short rows (us of a
+                // step of 2e8 bf16 logits, pairs and singles: V = 16,384 with a dense row, K = 8 258
+                // and 264, 30 286 and 279, 50 302 and 296, 80 457 and 428; 151,936, K = 50 115, 117).
+                const uint64_t kth = nc <= max(2 * K, kTkSelThreads) ? 0 : sel_kth_largest<SW>(s_cand, nc, K, hi_val, 0, s_sel, stid);
+                const bool singles = SW == kTkSelSmall && K > 16 && a.vocab <= 32768;
+                if (!singles) {
+                    if (stid == 0 && (nc & 1))
+                        s_cand[nc] = 0;  // the last pair's second key
+                    named_sync(kBarSel, kTkSelThreads);
+                }
                 const ulonglong2 *pairs = reinterpret_cast<const ulonglong2 *>(s_cand);
                 for (int i = stid; i < nc; i += kTkSelThreads) {
                     const uint64_t k = s_cand[i];
                     if (k < kth)
                         continue;
                     int rank = 0;
+                    if (singles) {
+                        int q = 0;
+                        for (; q + 4 <= nc; q += 4)
+                            rank += (s_cand[q] > k) + (s_cand[q + 1] > k) + (s_cand[q + 2] > k) + (s_cand[q + 3] > k);
+                        for (; q < nc; ++q)
+                            rank += s_cand[q] > k;
+                    } else {
 #pragma unroll 2
-                    for (int q = 0; q < (nc + 1) / 2; ++q) {
-                        const ulonglong2 x = pairs[q];
-                        rank += (int)(x.x > k) + (int)(x.y > k);
+                        for (int q = 0; q < (nc + 1) / 2; ++q) {
+                            const ulonglong2 x = pairs[q];
+                            rank += (int)(x.x > k) + (int)(x.y > k);
+                        }
                     }
                     if (rank < K) {
                         s_top[rank] = k;
@@ -1026,16 +1039,20 @@ __host__ __device__ __forceinline__ size_t short_smem(int K)
            (sizeof(uint64_t) + sizeof(float)) * (size_t)K + 16;
 }
 constexpr int kShortPerThread = 64;  // elements of a row per thread
-// Aligned rows up to here take the kernel below: what 128 threads hold, and what 256 hold from
-// K = kShortLargeK.  The streaming kernel reads longer rows faster.  us of a step of 2e8 bf16
+// Aligned rows up to here take the kernel below: what 128 threads hold, 256 from K = 64, 512
+// for K = 240-288 (where the streaming kernel's bound, the K-th of 384 thread maxima, is loosest).
+// That kernel reads the other rows faster.  us of a step of 2e8 bf16
 // logits, here and there: V = 8,184, K = 8 275 and 386, 50 316 and 501, 96 356 and 1,890;
 // V = 8,192 (256 threads), K = 64 551 and 676; 12,288, K = 32 370 and 300, 50 392 and 329, 64
 // 394 and 453; 16,376, K = 64 322 and 376, 256 516 and 879; 24,576 (512 threads), K = 80 434 and
-// 301, 128 459 and 354, 256 557 and 595.  fp32 rows cross at the same places.  Rows that are not
-// 16-byte aligned, which the streaming kernel reads element by element, take it at every length
-// it holds (32,700, K = 50: 1,248 GB/s and 448).
-constexpr int kShortMaxV = kShortPerThread * 128 - 7, kShortMaxVLarge = kShortPerThread * 256 - 7;
-constexpr int kShortLargeK = 64;
+// 301, 128 459 and 354, 224 523 and 476, 240 541 and 563, 256 558 and 595, 320 611 and 566;
+// 32,744, K = 512 720 and 609.  fp32 rows cross at the same places.  Rows that are not 16-byte aligned, which the streaming kernel reads element by
+// element, take it at every length it holds (32,700, K = 50: 1,248 GB/s and 448).
+int short_max_vocab(int K)
+{
+    const int threads = K < 64 ? 128 : K < 240 || K > 288 ? 256 : 512;
+    return kShortPerThread * threads - 7;
+}
 
 // Rows of up to 64 NT elements, one CTA of NT threads a row, any alignment: the row's
 // 16-bit buckets (the logit itself for bf16) stay in registers, 2 to a word, from the only
@@ -1358,7 +1375,7 @@ cudaError_t launch_topk(const TopkCall &c, cudaStream_t stream)
     const int64_t span = c.vocab + 7;
     const size_t esz = bf16 ? 2 : 4;
     const bool aligned = ((reinterpret_cast<uintptr_t>(c.zt) | reinterpret_cast<uintptr_t>(c.zs) | (uintptr_t)(c.ld * esz)) & 15u) == 0;
-    if (span <= (int64_t)kShortPerThread * 512 && (!aligned || c.vocab <= (c.K < kShortLargeK ? kShortMaxV : kShortMaxVLarge))) {
+    if (span <= (int64_t)kShortPerThread * 512 && (!aligned || c.vocab <= short_max_vocab(c.K))) {
         const int s4 = span <= kShortPerThread * 32 ? 0 : span <= kShortPerThread * 128 ? 1 : span <= kShortPerThread * 256 ? 2 : 3;
         static const Kern shorts[2][4] = {
             {k_topk_short<false, 32>, k_topk_short<false, 128>, k_topk_short<false, 256>, k_topk_short<false, 512>},

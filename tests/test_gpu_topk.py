@@ -311,8 +311,8 @@ def test_short_rows_at_the_edges(P, oracle, V, dtype):
                 np.testing.assert_array_equal(d[t, :V], want)
 
 
-@pytest.mark.parametrize("V", [e // 8 * 8 + d for e in SHORT_EDGES[1:3] for d in (0, 8)])
-@pytest.mark.parametrize("K", [1, 63, 64, 256])
+@pytest.mark.parametrize("V", [e // 8 * 8 + d for e in SHORT_EDGES[1:] for d in (0, 8)])
+@pytest.mark.parametrize("K", [1, 63, 64, 239, 240, 289])
 def test_aligned_rows_at_the_selection_lines(P, oracle, V, K):
     """Aligned rows on both sides of the lengths and the K from which they are streamed."""
     T = 12
