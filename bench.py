@@ -37,8 +37,7 @@ METRIC = "loss fwd+bwd tokens/s at V=151936 bf16 on 1 GB300; achieved HBM GB/s v
 UNIT = "tokens/s"
 V_QWEN = 151_936  # the workloads' vocabulary (a --vocab run has no committed traffic record)
 # counts(2) + weights(1) + compaction(2) + row kernel + loss sum + stats(2); the full and
-# sampled modes add the helper grid that runs beside the cluster grid (k_row_helper for
-# bf16 logits, k_split_helper for fp32)
+# sampled modes add the helper grid that runs beside the cluster grid (k_row_helper)
 KERNELS_PER_STEP = 9
 ROW_KERNEL_SOURCES = ["paper_2607_05804_gb300/csrc/rowkl_cluster.cuh",
                       "paper_2607_05804_gb300/csrc/rowkl_cluster.cu",
@@ -69,7 +68,7 @@ def parse():
     p.add_argument("--vocab", type=int, default=0,
                    help="full/sampled/top-K modes: vocabulary size (0 = the workload's 151,936)")
     p.add_argument("--fp32-logits", action="store_true",
-                   help="full/sampled modes: fp32 logits instead of bf16 (the split-row kernel)")
+                   help="full/sampled modes: fp32 logits instead of bf16")
     p.add_argument("--alpha", type=float, default=0.5)
     p.add_argument("--no-e2e", action="store_true")
     p.add_argument("--no-cpu-baseline", action="store_true")
@@ -344,9 +343,12 @@ def reference_arm(args, world, rank):
     print(json.dumps(out), flush=True)
 
 
-# weights (3) + fused call (compaction 2, gathers 2, statistics pass, merge, gradient
-# pass, masked-row zeroing, dL/dh_s, dL/dh_s fix-up, loss sum) + turn statistics (2)
-FUSED_KERNELS_PER_STEP = 16
+def fused_kernels_per_step(tokens, dw):
+    """weights (3) + fused call (compaction 2, gathers 2; statistics pass, merge and G for each
+    chunk of up to 8 tiles of 256 token rows, sized for every token; masked-row zeroing, dL/dh_s,
+    its fix-up, loss sum, and dL/dW_s if asked for) + turn statistics (2)"""
+    tiles = (tokens + 255) // 256
+    return 13 + 3 * ((tiles + 7) // 8) + (1 if dw else 0)
 
 
 def fused_cpu_baseline(b, heads, w, budget_s=12.0):
@@ -448,7 +450,8 @@ def fused_bench(args, world, rank, local):
         n = torch.tensor([Tv], device=device, dtype=torch.int64)
         dist.all_reduce(n)
         tot_valid = int(n.item())
-    flops = 2.0 * Tv * V * (d_s + d_t) * 2 + 2.0 * Tv * V * d_s  # forward, recompute, dH
+    # forward and dH: the call's workspace holds the logits' scratch, so no tile is computed twice
+    flops = 2.0 * Tv * V * (d_s + d_t) + 2.0 * Tv * V * d_s
     if args.dw:
         flops += 2.0 * Tv * V * d_s  # dW_s
     peak = 1715.8
@@ -473,7 +476,7 @@ def fused_bench(args, world, rank, local):
                         "frac": tflops / peak, "peak_kind": peak_kind,
                         "kernel": "turnopd_fused_lmhead_fwd_bwd launch sequence", "launch_ms": call_ms,
                         "traffic": None},
-           "gpu_launches": (FUSED_KERNELS_PER_STEP + (1 if args.dw else 0)) * args.steps, "clocks": clocks,
+           "gpu_launches": fused_kernels_per_step(T, args.dw) * args.steps, "clocks": clocks,
            "e2e": None,
            "cpu_baseline": cpu}
     if rank == 0:
@@ -606,9 +609,6 @@ def main():
                            if args.mode == "topk" else
                            f"vocabulary-parallel path, {args.vocab_shards} shards of one GPU "
                            "(shard stats + merge + shard gradients)" if args.vocab_shards else
-                           "turnopd_loss_fwd_bwd launch sequence (split-row kernel on clusters of "
-                           f"{4 if args.mode == 'sampled' else 8} beside the fp32 helper grid + compaction "
-                           "+ loss sum)" if args.fp32_logits else
                            "turnopd_loss_fwd_bwd launch sequence (cluster row kernel beside the helper grid "
                            "+ compaction + loss sum)"),
                 "algorithmic_bytes_per_launch": alg_bytes,
