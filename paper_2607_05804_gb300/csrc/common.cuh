@@ -27,6 +27,13 @@ __device__ __forceinline__ float ex2(float x)
     return y;
 }
 
+// exp(z - m) is formed as 2^(z log2e + scale_of(m)), m a running maximum.  Below
+// -FLT_MAX / log2e the product would overflow, and a thread or vector that holds nothing but
+// the type's lowest value (a masked vocabulary) would make its row NaN: exp2(-inf + inf).
+// The reference stays there instead, and such values add 0 beside any real logit.
+constexpr float kLowestRef = -0x1.62e42ep+127f;  // the lowest float whose product is finite
+__device__ __forceinline__ float scale_of(float m) { return -fmaxf(m, kLowestRef) * kLog2e; }
+
 __device__ __forceinline__ float to_float(float x) { return x; }
 __device__ __forceinline__ float to_float(__nv_bfloat16 x) { return __bfloat162float(x); }
 

@@ -116,7 +116,7 @@ __device__ __forceinline__ void accumulate(Student &s, Teacher &t, const float *
         t.s *= ex2((t.m - my) * kLog2e);
         t.m = my;
     }
-    const float ns = -s.m * kLog2e, nt = -t.m * kLog2e;
+    const float ns = scale_of(s.m), nt = scale_of(t.m);
 #pragma unroll
     for (int k = 0; k < N; ++k) {
         const float e = ex2(fmaf(a[k], kLog2e, ns));
@@ -134,7 +134,7 @@ __device__ __forceinline__ void accumulate_teacher(Teacher &t, float b)
         t.s *= ex2((t.m - b) * kLog2e);
         t.m = b;
     }
-    t.s += ex2(fmaf(b, kLog2e, -t.m * kLog2e));
+    t.s += ex2(fmaf(b, kLog2e, scale_of(t.m)));
 }
 
 // Sampled-token row (Eq. opd-rkl's one-token estimator): the student statistics leave y

@@ -57,10 +57,9 @@ struct GradConst {
     float gy;         // sampled: g_y = w l (1 - p_y)
 };
 
-// What a lane that does not count reads as: -2^127.  It adds 0 beside any real logit, and
-// where a thread or a vector holds nothing else its maximum times log2 e is still finite
-// (the lowest finite value's is not: exp2(-inf + inf) made such a row NaN).
-constexpr uint32_t kFillHi = 0xff00u;            // the upper 16 bits; as bf16 and, shifted, as fp32
+// What a lane that does not count reads as: bf16's lowest finite value.  It adds 0 to every
+// sum, also where a thread or a vector holds nothing else (scale_of).
+constexpr uint32_t kFillHi = 0xff7fu;            // the upper 16 bits; as bf16 and, shifted, as fp32
 
 // One 16-byte vector of logits: N elements, NP pairs of them, and the running maximum of
 // vectors (packed for bf16).
@@ -504,7 +503,7 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
             }
         }
         // sum pass (packed pairs)
-        const float2 L2 = splat(kLog2e), NS = splat(-ms * kLog2e), NTT = splat(-mt * kLog2e);
+        const float2 L2 = splat(kLog2e), NS = splat(scale_of(ms)), NTT = splat(scale_of(mt));
         const float2 D = splat(xd);
         float2 S2 = make_float2(0.f, 0.f), A2 = S2, T2 = S2;
 #pragma unroll
@@ -886,7 +885,7 @@ __global__ void __launch_bounds__(NTH, MINB) k_row_helper(RowIn p)
                 T2 = fmul2(T2, splat(ex2((mt - nmt) * kLog2e)));
                 mt = nmt;
             }
-            const float2 NS = splat(-ms * kLog2e), NTT = splat(-mt * kLog2e), D = splat(dd);
+            const float2 NS = splat(scale_of(ms)), NTT = splat(scale_of(mt)), D = splat(dd);
 #pragma unroll
             for (int u = 0; u < kHelpU; ++u)
 #pragma unroll

@@ -404,7 +404,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_row_split(RowIn p, int slice_ve
                         T2 = fmul2(T2, splat(ex2((mt - cmt) * kLog2e)));
                         mt = cmt;
                     }
-                    const float2 L2 = splat(kLog2e), NS = splat(-ms * kLog2e), NTT = splat(-mt * kLog2e);
+                    const float2 L2 = splat(kLog2e), NS = splat(scale_of(ms)), NTT = splat(scale_of(mt));
                     const float2 D = splat(dd);
                     const float4 xs[2] = {x0, x1}, zz[2] = {z0, z1};
 #pragma unroll
@@ -656,7 +656,7 @@ __global__ void __launch_bounds__(NTH, 1) k_split_helper(RowIn p)
                 T2 = fmul2(T2, splat(ex2((mt - cmt) * kLog2e)));
                 mt = cmt;
             }
-            const float2 NS = splat(-ms * kLog2e), NTT = splat(-mt * kLog2e), D = splat(dd);
+            const float2 NS = splat(scale_of(ms)), NTT = splat(scale_of(mt)), D = splat(dd);
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 const float2 a01 = make_float2(a[u].x, a[u].y), a23 = make_float2(a[u].z, a[u].w);

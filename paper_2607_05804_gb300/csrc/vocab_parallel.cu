@@ -140,7 +140,7 @@ __device__ __forceinline__ void fold_row_bf16(const uint4 *vs, const uint4 *vt, 
             T2 = fmul2(T2, splat(ex2((mt - nmt) * kLog2e)));
             mt = nmt;
         }
-        const float2 NS = splat(-ms * kLog2e), NTT = splat(-mt * kLog2e), D = splat(dd);
+        const float2 NS = splat(scale_of(ms)), NTT = splat(scale_of(mt)), D = splat(dd);
 #pragma unroll
         for (int u = 0; u < kVpU; ++u)
 #pragma unroll

@@ -368,6 +368,27 @@ def test_ragged_rows_fp32(P, oracle, V, ld, mode, gdt):
         assert (grad[:, V:].float() == 7.0).all()
 
 
+@pytest.mark.parametrize("V,ld,flags", [(8195, 8195, 0), (8192, 8192, 0), (50001, 50001, 0), (W.V_QWEN, W.V_QWEN, 0),
+                                        (160004, 160004, 0), (8195, 8195, FORCE_PORTABLE),
+                                        (8192, 8192, FORCE_PORTABLE)])
+@pytest.mark.parametrize("mode", [0, 1], ids=["full", "sampled"])
+@pytest.mark.parametrize("idt", ["bf16", "f32"])
+def test_vocabulary_masked_with_the_lowest_value(P, oracle, V, ld, flags, mode, idt):
+    """Columns 600 and up hold the type's lowest finite value in both models, so that whole
+    vectors, threads and slices hold nothing else: the row is that of its live columns.  Some
+    rows mask the student or the teacher further (there the difference of the two is as large
+    as the type)."""
+    b = W.packed(seed=11, num_traj=1, traj_len=128)
+    dt = torch.bfloat16 if idt == "bf16" else torch.float32
+    zs, zt = W.make_logits(b.num_valid, V, "agent", dt, seed=44, device="cuda", ld=ld)
+    lowest = torch.finfo(dt).min
+    zs[:, 600:V] = lowest
+    zt[:, 600:V] = lowest
+    zs[::3, 300:600] = lowest  # p = 0 there; the teacher keeps a share
+    for gdt in (torch.bfloat16, torch.float32):
+        run_chain(P, oracle, b, V, zs, zt, mode=mode, alpha=0.5, flags=flags, compact=True, grad_dtype=gdt, seed_y=45)
+
+
 def test_ragged_rows_dense_neighbours_untouched(P, oracle):
     """One row per token, odd stride: the gradient rows of masked tokens share vectors
     with supervised ones and stay as they were."""

@@ -188,3 +188,26 @@ def test_rows_at_any_offset(P, oracle, V, ld, dt, gdt):
     assert_grad_rows(whole[:, :V].float().cpu().numpy()[m], g_ref[m], bf16=gdt == "bf16",
                      zs=z[0][torch.from_numpy(m).cuda()].float(), w=w.cpu().numpy()[m], ell=tl_ref[m])
     assert (whole[torch.from_numpy(~m).cuda()].float() == 7.0).all() and (whole[:, V:].float() == 7.0).all()
+
+
+@pytest.mark.parametrize("V,ld", [(2400, 2400), (2400, 2403)])
+@pytest.mark.parametrize("dt", ["bf16", "f32"])
+def test_vocabulary_masked_with_the_lowest_value(P, oracle, V, ld, dt):
+    """The type's lowest finite value from column 600 on, in both models: most threads of the
+    first shard, and the whole second one, hold nothing else."""
+    b = W.packed(seed=9, num_traj=2, traj_len=48)
+    tdt = torch.bfloat16 if dt == "bf16" else torch.float32
+    T = b.num_tokens
+    zs, zt = W.make_logits(T, V, "agent", tdt, seed=46, device="cuda", ld=ld)
+    zs[:, 600:] = torch.finfo(tdt).min
+    zt[:, 600:] = torch.finfo(tdt).min
+    mask = torch.from_numpy(b.loss_mask).cuda()
+    w = torch.rand(T, generator=torch.Generator().manual_seed(8)).cuda()
+    grad, tls, losses = run_split(P, zs, zt, None, mask, w, [0, 1200, V], torch.float32)
+    g_ref, tl_ref, loss_ref = oracle.loss_fwd_bwd(zs[:, :V].float().cpu().numpy(), zt[:, :V].float().cpu().numpy(), V,
+                                                  b.loss_mask, w.cpu().numpy())
+    m = b.loss_mask == 1
+    for tl, loss in zip(tls, losses):
+        assert_token_loss(tl, tl_ref, b.loss_mask)
+        assert_loss(loss, loss_ref)
+    assert_grad_rows(grad[:, :V].cpu().numpy()[m], g_ref[m], bf16=False)
