@@ -179,8 +179,10 @@ cudaError_t launch_fused(const FusedCall &c, cudaStream_t stream);
 // others, which the portable kernel takes.
 cudaError_t launch_rows(const RowIn &p, bool bf16, bool fp32_grad, cudaStream_t stream, bool *used);
 // Its sets of kernels: rows held whole in the shared memory of a CTA or a cluster, by type,
-// and ragged (vocabulary or stride no multiple of a 16-byte vector: masked end vectors).
+// ragged (no whole number of 16-byte vectors: masked end vectors), and for bf16 ragged at the
+// end alone (an aligned stride).
 cudaError_t launch_rows_bf16(const RowIn &p, bool fp32_grad, cudaStream_t stream);
+cudaError_t launch_rows_bf16_tail(const RowIn &p, bool fp32_grad, cudaStream_t stream);
 cudaError_t launch_rows_bf16_ragged(const RowIn &p, bool fp32_grad, cudaStream_t stream);
 cudaError_t launch_rows_f32(const RowIn &p, bool fp32_grad, cudaStream_t stream);
 cudaError_t launch_rows_f32_ragged(const RowIn &p, bool fp32_grad, cudaStream_t stream);

@@ -9,7 +9,7 @@ namespace turnopd {
 
 cudaError_t launch_rows_bf16(const RowIn &p, bool fp32_grad, cudaStream_t stream)
 {
-    return launch_rows_t<__nv_bfloat16, false>(p, fp32_grad, stream);
+    return launch_rows_t<__nv_bfloat16, kWhole>(p, fp32_grad, stream);
 }
 
 // *used = false (and nothing is launched) for arrays that are not 16-byte aligned.
@@ -22,7 +22,9 @@ cudaError_t launch_rows(const RowIn &p, bool bf16, bool fp32_grad, cudaStream_t 
     const int n = bf16 ? 8 : 4;
     const bool whole = p.vocab % n == 0 && p.ld % n == 0;
     if (bf16)
-        return whole ? launch_rows_bf16(p, fp32_grad, stream) : launch_rows_bf16_ragged(p, fp32_grad, stream);
+        return whole ? launch_rows_bf16(p, fp32_grad, stream)
+               : p.ld % n == 0 ? launch_rows_bf16_tail(p, fp32_grad, stream)
+                               : launch_rows_bf16_ragged(p, fp32_grad, stream);
     // rows longer than 16 CTAs hold are streamed twice (V = 151,936 on clusters of 8: 5,400
     // GB/s, held by clusters of 16: 6,020)
     if (whole && cluster_size((int)(p.vocab / 4)) == 0)

@@ -208,21 +208,24 @@ __device__ __forceinline__ void store_grad_lanes(void *grad, size_t e, const flo
         }
 }
 
-// Ragged rows (TL): the row stride or the vocabulary is no multiple of a vector's N
-// elements, so a row starts `head` elements into a 16-byte vector and ends `tail`
-// elements into one (tail 0: at its end).  Its vectors are those of the 16-byte grid that
-// hold any of its columns; the first and the last may be partial.  (Rows of a stride that
-// is no multiple of 8 took the portable kernel's 2-byte loads before: dense 4 x 1024
-// tokens, V = 50,001, bf16, step 1,075 us, now 216; 133 is its traffic at the copy
-// bandwidth.)
+// How rows lie in the 16-byte grid: whole vectors, a partial last vector alone (the stride is
+// a multiple of a vector's N elements, the vocabulary is not), or any stride.
+enum RowForm { kWhole = 0, kTail = 1, kAny = 2 };
+
+// Rows that are not whole (TL > kWhole): a row starts `head` elements into a 16-byte vector
+// and ends `tail` elements into one (tail 0: at its end; head 0 in kTail).  Its vectors are
+// those of the 16-byte grid that hold any of its columns; the first and the last may be
+// partial.  (Rows of a stride that is no multiple of 8 took the portable kernel's 2-byte loads
+// before: dense 4 x 1024 tokens, V = 50,001, bf16, step 1,075 us, now 230; 133 is its traffic
+// at the copy bandwidth.  kTail apart from kAny: V = 33,001 of stride 33,008 641 -> 606 us.)
 struct Ragged {
     int head, nvec, tail;
 };
-template <typename T> __device__ __forceinline__ Ragged ragged(int row, int64_t ld, int64_t vocab)
+template <typename T, int TL> __device__ __forceinline__ Ragged ragged(int row, int64_t ld, int64_t vocab)
 {
     constexpr int N = Elem<T>::N;
     Ragged g;
-    g.head = ((row & (N - 1)) * (int)(ld & (N - 1))) & (N - 1);
+    g.head = TL == kAny ? ((row & (N - 1)) * (int)(ld & (N - 1))) & (N - 1) : 0;
     g.nvec = (int)((g.head + vocab + N - 1) / N);
     g.tail = (int)((g.head + vocab) & (N - 1));
     return g;
@@ -244,8 +247,8 @@ __device__ __forceinline__ int split_rows(const RowIn &p, int nvalid)
 // 2G, so a slot is reused by the same group two rows later, after that group has read it
 // (a peer can run at most G rows ahead of the slowest CTA in sending records).  SM: a
 // sampled-token call, where every listed row carries its y in [0, V); otherwise the full
-// vocabulary (y = -1).  TL: ragged rows.
-template <typename T, int CS, int NT, int VPT, int G, int ST, bool G32, bool SM, bool TL>
+// vocabulary (y = -1).  TL: a RowForm.
+template <typename T, int CS, int NT, int VPT, int G, int ST, bool G32, bool SM, int TL>
 __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_vec, int nvec)
 {
     using E = Elem<T>;
@@ -255,10 +258,13 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
     static_assert(G <= 15 || NT == 32, "one named barrier per group");
     // Reference difference d (A = sum e ((z_s - z_t) - d), d at the student's
     // max): it keeps gradients at a dominant token accurate to fp32 relative
-    // precision.  A bf16 gradient needs no such care: without d the error of
-    // E_p[z_s - z_t] is ~1e-6 absolute, under a bf16 ulp of those gradients.  (fp32
-    // logits always keep it.)
-    constexpr bool kUseD = G32 || N == 4;
+    // precision.  bf16 rows of an aligned stride with a bf16 gradient leave it out: the error of
+    // E_p[z_s - z_t] is then ~1e-6 absolute, under a bf16 ulp of nearly all of those
+    // gradients.  Rows of any other stride keep it whatever the types, as do fp32 logits.
+    // (Relative error of g at a token 10, 12, 14 and 16 above the rest of its row, V = 50,001,
+    // bf16: without it 0.3, 2, 12 and 18 %, with it the rounding's 0.4 % at each.)
+    constexpr bool kUseD = G32 || N == 4 || (TL == kAny && !SM);
+    constexpr bool kGradD = G32 || TL == kAny;  // the gradient subtracts d and cp one after the other
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ int s_dead;
     constexpr int NWG = NT / 32;  // warps per group
@@ -270,20 +276,23 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
     const uint32_t stage_bytes = 2u * slice_bytes;
     const int v0 = (int)rank * slice_vec;  // first vector of my slice
     const int my_vec = max(0, min(slice_vec, nvec - v0));
-    // TL (ragged rows): the slice's vectors and the partial ones among them vary from row
-    // to row.  A partial vector's other lanes read as the fill in the
+    // TL: in kAny the slice's vectors and the partial ones among them vary from row to row.
+    // A partial vector's other lanes read as the fill in the
     // statistics (set in shared memory by the thread that reads the vector) and are
     // never written: the gradient loop stores whole vectors, that thread the partial
     // one's columns.  Without TL all of this compiles away.
     struct Slice {
         int my_vec, head0, g0, gvec, tailq, tail;  // head0: of the row (every slice)
         bool head;                                  // vector 0 is partial
-        bool cut;                                   // the last vector passes the end of the logits
     };
     auto slice_of = [&](int row) {
-        Slice g{my_vec, 0, 0, my_vec, -1, 0, false, false};
-        if (TL) {
-            const Ragged r = ragged<T>(row, p.ld, p.vocab);
+        Slice g{my_vec, 0, 0, my_vec, -1, 0, false};
+        if (TL == kTail) {
+            g.tail = (int)(p.vocab & (N - 1));
+            g.tailq = my_vec > 0 && v0 + my_vec == nvec ? my_vec - 1 : -1;
+            g.gvec = g.tailq >= 0 ? my_vec - 1 : my_vec;
+        } else if (TL == kAny) {
+            const Ragged r = ragged<T, TL>(row, p.ld, p.vocab);
             g.my_vec = max(0, min(slice_vec, r.nvec - v0));
             g.head0 = r.head;
             g.head = v0 == 0 && r.head > 0;
@@ -291,9 +300,15 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
             g.tailq = r.tail && g.my_vec > 0 && v0 + g.my_vec == r.nvec ? g.my_vec - 1 : -1;
             g.g0 = g.head ? 1 : 0;
             g.gvec = g.tailq >= 0 ? g.my_vec - 1 : g.my_vec;
-            g.cut = g.tailq >= 0 && (int64_t)row * p.ld - r.head + (int64_t)r.nvec * N > p.elems;
         }
         return g;
+    };
+    // the slice's last vector passes the end of the logits (kTail: only the last row's can)
+    const int last_row = TL == kTail ? (int)((p.elems - p.vocab) / p.ld) : 0;
+    auto cut = [&](const Slice &g, int row) {
+        if (TL == kTail)
+            return g.tailq >= 0 && row == last_row;
+        return TL && g.tailq >= 0 && (int64_t)row * p.ld - g.head0 + (int64_t)(v0 + g.my_vec) * N > p.elems;
     };
 
     unsigned char *stage = smem;
@@ -385,7 +400,7 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
             yown[s] = q >= 0 && q < g.my_vec ? q % NT : -1;
         }
         *(volatile int *)&srow[s] = k;
-        const uint32_t my_bytes = (uint32_t)(TL && g.cut ? g.my_vec - 1 : g.my_vec) * 16u;
+        const uint32_t my_bytes = (uint32_t)(cut(g, m.y) ? g.my_vec - 1 : g.my_vec) * 16u;
         const size_t off = (size_t)m.y * (size_t)p.ld - (size_t)g.head0 + (size_t)v0 * N;
         const char *gs = reinterpret_cast<const char *>(zs + off);
         const char *gt = reinterpret_cast<const char *>(zt + off);
@@ -437,7 +452,7 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
             uint4 *ws = reinterpret_cast<uint4 *>(stage + s * stage_bytes);
             uint4 *wt = reinterpret_cast<uint4 *>(stage + s * stage_bytes + slice_bytes);
             if (g.tailq >= 0 && g.tailq % NT == gtid) {
-                if (g.cut) {
+                if (cut(g, meta[s].y)) {
                     const size_t e = (size_t)meta[s].y * (size_t)p.ld - (size_t)g.head0 + (size_t)(v0 + g.tailq) * N;
                     ws[g.tailq] = E::load_lanes(zs + e, 0, g.tail);
                     wt[g.tailq] = E::load_lanes(zt + e, 0, g.tail);
@@ -588,7 +603,7 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
             lane_merge<CS, kUseD>(A, B);
             if (lane == 0) {
                 const int y = meta[k % kStages].z;
-                const int yh = TL ? y + ragged<T>(meta[k % kStages].y, p.ld, p.vocab).head : y;
+                const int yh = TL ? y + ragged<T, TL>(meta[k % kStages].y, p.ld, p.vocab).head : y;
                 const int owner = SM ? (yh / N) / slice_vec : 0;
                 row_constants(k, A, B, r[owner * 8 + 6], r[owner * 8 + 7]);
                 mbar_arrive_expect_tx(&recv[slot], CS * 32u);  // re-arm for row k + kSlots
@@ -623,7 +638,7 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
 #pragma unroll
         for (int u = 0; u < VPT; ++u) {
             const int q = gtid + u * NT;
-            if (q < gvec && (!TL || q >= sl.g0)) {
+            if (q < gvec && (TL != kAny || q >= sl.g0)) {
                 float2 g[NP];
                 // y < 0 exactly when !SM; the bf16 logits' fp32-gradient instantiations keep the
                 // run-time test, which compiles to a loop 5 % faster there (and 2.4 % slower for
@@ -636,7 +651,7 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
                         const float2 pw = ex2x2(ffma2(a2, L2, NLW));
                         // sg ((z_s - z_t) - c) with one rounding; sg (z_s - z_t) is exact
                         const float2 x = fsub2(a2, b2);
-                        g[j] = G32 ? fmul2(pw, fadd2(ffma2(x, SG, ND), NCP)) : fmul2(pw, ffma2(x, SG, NC));
+                        g[j] = kGradD ? fmul2(pw, fadd2(ffma2(x, SG, ND), NCP)) : fmul2(pw, ffma2(x, SG, NC));
                     }
                 } else {  // sampled token: g = -w l p (g_y is written after the loop)
                     const uint4 a = vs[q];
@@ -656,7 +671,7 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
                 const float2 a2 = E::pair(a, j), b2 = E::pair(b, j);
                 const float2 pw = ex2x2(ffma2(a2, L2, NLW)), x = fsub2(a2, b2);
                 g[j] = SM ? fmul2(pw, SGL)
-                          : (G32 ? fmul2(pw, fadd2(ffma2(x, SG, ND), NCP)) : fmul2(pw, ffma2(x, SG, NC)));
+                          : (kGradD ? fmul2(pw, fadd2(ffma2(x, SG, ND), NCP)) : fmul2(pw, ffma2(x, SG, NC)));
             }
             store_grad_lanes<T, G32>(p.grad, row_off + (size_t)q * N, g, lo, hi);
         };
@@ -746,7 +761,7 @@ constexpr int kHelpU = 4;  // vectors of each model per thread and batch
 constexpr int kHelpStages = 3;
 constexpr size_t helper_smem_bytes(bool as, int nth) { return as ? (size_t)kHelpStages * 2 * kHelpU * nth * 16 : 0; }
 
-template <typename T, bool G32, bool SM, bool TL, bool AS, int NTH = kHelpThreads, int MINB = 1>
+template <typename T, bool G32, bool SM, int TL, bool AS, int NTH = kHelpThreads, int MINB = 1>
 __global__ void __launch_bounds__(NTH, MINB) k_row_helper(RowIn p)
 {
     constexpr int kHelpThreads = NTH;
@@ -754,7 +769,7 @@ __global__ void __launch_bounds__(NTH, MINB) k_row_helper(RowIn p)
     using E = Elem<T>;
     constexpr int N = E::N, NP = E::NP;
     constexpr uint32_t kFill = E::kFillWord;
-    constexpr bool kUseD = G32 || N == 4;  // as in the cluster kernel
+    constexpr bool kUseD = G32 || N == 4 || (TL == kAny && !SM), kGradD = G32 || TL == kAny;  // as in the cluster kernel
     __shared__ float red[NW][8];
     __shared__ float bc[8];
     extern __shared__ uint4 hring[];  // [kHelpStages][2][kHelpU][NTH] (AS)
@@ -769,9 +784,9 @@ __global__ void __launch_bounds__(NTH, MINB) k_row_helper(RowIn p)
     for (int j = j0 + (int)blockIdx.x; j < nvalid; j += gridDim.x) {
         const int4 m = p.rows[j];
         const size_t off = (size_t)m.y * (size_t)p.ld;
-        // TL (ragged rows): a partial first or last vector's other lanes read as the fill
+        // TL: a partial first or last vector's other lanes read as the fill
         // and are never written; the gradient loop stores vectors [g0, nfull)
-        const Ragged rg = TL ? ragged<T>(m.y, p.ld, p.vocab) : Ragged{0, (int)(p.vocab / N), 0};
+        const Ragged rg = TL ? ragged<T, TL>(m.y, p.ld, p.vocab) : Ragged{0, (int)(p.vocab / N), 0};
         const int head = rg.head, nvec = rg.nvec, tail = rg.tail;
         const int g0 = TL && head ? 1 : 0, nfull = TL && tail ? nvec - 1 : nvec;
         const size_t voff = off - (size_t)head;          // the row's first vector
@@ -930,7 +945,7 @@ __global__ void __launch_bounds__(NTH, MINB) k_row_helper(RowIn p)
                 bc[2] = -sg * (rc.d + rc.cp);  // bf16 output: one rounding of d + cp
                 bc[3] = wl > 0.f ? -1.f : 1.f;
                 bc[4] = wl * omp;              // sampled: g_y = w l (1 - p_y)
-                bc[5] = -sg * rc.d;            // fp32 output
+                bc[5] = -sg * rc.d;            // kGradD
                 bc[6] = -sg * rc.cp;
             }
         }
@@ -964,7 +979,7 @@ __global__ void __launch_bounds__(NTH, MINB) k_row_helper(RowIn p)
                         for (int w = 0; w < NP; ++w) {
                             const float2 a2 = E::pair(a[u], w), b2 = E::pair(b[u], w);
                             const float2 pw = ex2x2(ffma2(a2, L2, NLW)), x = fsub2(a2, b2);
-                            g[w] = G32 ? fmul2(pw, fadd2(ffma2(x, SG, ND), NCP)) : fmul2(pw, ffma2(x, SG, NC));
+                            g[w] = kGradD ? fmul2(pw, fadd2(ffma2(x, SG, ND), NCP)) : fmul2(pw, ffma2(x, SG, NC));
                         }
                     } else {  // sampled token: g = -w l p (g_y is written after the loop)
 #pragma unroll
@@ -985,7 +1000,7 @@ __global__ void __launch_bounds__(NTH, MINB) k_row_helper(RowIn p)
                     const float2 a2 = E::pair(a, w), b2 = E::pair(b, w);
                     const float2 pw = ex2x2(ffma2(a2, L2, NLW)), x = fsub2(a2, b2);
                     g[w] = SM ? fmul2(pw, SGL)
-                              : (G32 ? fmul2(pw, fadd2(ffma2(x, SG, ND), NCP)) : fmul2(pw, ffma2(x, SG, NC)));
+                              : (kGradD ? fmul2(pw, fadd2(ffma2(x, SG, ND), NCP)) : fmul2(pw, ffma2(x, SG, NC)));
                 }
                 store_grad_lanes<T, G32>(p.grad, to, g, lo, hi);
             };
@@ -1105,7 +1120,7 @@ template <class Shape> size_t cluster_smem_bytes(int slice_vec, int cs)
 // the helper grid on the SMs the clusters leave free, with the row list split so
 // that both finish together.  *used = false (and nothing is launched) where the slices
 // do not fit shared memory.
-template <typename T, bool G32, int CS, class Shape, bool SM, bool TL>
+template <typename T, bool G32, int CS, class Shape, bool SM, int TL>
 cudaError_t launch_t(const RowIn &p, int nvec, cudaStream_t stream, bool *used)
 {
     auto kern = k_row_cluster<T, CS, Shape::NT, Shape::VPT, Shape::G, Shape::ST, G32, SM, TL>;
@@ -1184,7 +1199,7 @@ cudaError_t launch_t(const RowIn &p, int nvec, cudaStream_t stream, bool *used)
     return cudaLaunchKernelEx(&hc, helper, pl);
 }
 
-template <typename T, bool G32, bool SM, bool TL>
+template <typename T, bool G32, bool SM, int TL>
 cudaError_t launch_cs(const RowIn &p, int nvec, cudaStream_t stream, bool *used)
 {
     const int cs = cluster_size(nvec);
@@ -1226,7 +1241,7 @@ cudaError_t launch_cs(const RowIn &p, int nvec, cudaStream_t stream, bool *used)
 }
 
 // The helper kernel alone, every row, every SM.
-template <typename T, bool G32, bool SM, bool TL>
+template <typename T, bool G32, bool SM, int TL>
 void launch_helper_alone(const RowIn &p, cudaStream_t stream)
 {
     RowIn pl = p;
@@ -1234,7 +1249,7 @@ void launch_helper_alone(const RowIn &p, cudaStream_t stream)
     k_row_helper<T, G32, SM, TL, false><<<device_sm_count(), kHelpThreads, 0, stream>>>(pl);
 }
 
-template <typename T, bool G32, bool SM, bool TL>
+template <typename T, bool G32, bool SM, int TL>
 cudaError_t launch_rows_m(const RowIn &p, int nvec, cudaStream_t stream)
 {
     bool used = false;
@@ -1245,8 +1260,8 @@ cudaError_t launch_rows_m(const RowIn &p, int nvec, cudaStream_t stream)
     return cudaGetLastError();
 }
 
-// The row grids for logits of T; TL: ragged rows (V or ld no multiple of a vector).
-template <typename T, bool TL>
+// The row grids for logits of T in rows of form TL.
+template <typename T, int TL>
 cudaError_t launch_rows_t(const RowIn &p, bool fp32_grad, cudaStream_t stream)
 {
     constexpr int N = 16 / (int)sizeof(T);

@@ -7,7 +7,7 @@ namespace turnopd {
 
 cudaError_t launch_rows_f32(const RowIn &p, bool fp32_grad, cudaStream_t stream)
 {
-    return launch_rows_t<float, false>(p, fp32_grad, stream);
+    return launch_rows_t<float, kWhole>(p, fp32_grad, stream);
 }
 
 }  // namespace turnopd

@@ -8,7 +8,7 @@ namespace turnopd {
 
 cudaError_t launch_rows_f32_ragged(const RowIn &p, bool fp32_grad, cudaStream_t stream)
 {
-    return launch_rows_t<float, true>(p, fp32_grad, stream);
+    return launch_rows_t<float, kAny>(p, fp32_grad, stream);
 }
 
 }  // namespace turnopd

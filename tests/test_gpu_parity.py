@@ -389,6 +389,31 @@ def test_vocabulary_masked_with_the_lowest_value(P, oracle, V, ld, flags, mode, 
         run_chain(P, oracle, b, V, zs, zt, mode=mode, alpha=0.5, flags=flags, compact=True, grad_dtype=gdt, seed_y=45)
 
 
+@pytest.mark.parametrize("V", [4099, 50001, W.V_QWEN + 1])
+@pytest.mark.parametrize("idt", ["bf16", "f32"])
+def test_dominant_token_of_ragged_rows(P, oracle, V, idt):
+    """Rows of odd stride with one token 10 to 24 above the rest and a bf16 gradient: at that
+    token ls - lt and KL cancel, and its gradient is still the oracle's to 2 bf16 ulps (2^-7)
+    with no allowance for the KL's own error."""
+    b = W.packed(seed=11, num_traj=2, traj_len=256)
+    R = b.num_valid
+    dt = torch.bfloat16 if idt == "bf16" else torch.float32
+    zs, zt = W.make_logits(R, V, "agent", dt, seed=4, device="cuda")
+    r = torch.arange(R, device="cuda")
+    y = torch.randint(V, (R,), generator=torch.Generator().manual_seed(5)).cuda()
+    zs[r, y] = (zs.float().amax(dim=1) + 10.0 + 2.0 * (r % 8)).to(dt)
+    step = make_step(P, b, V, compact=True)
+    grad = torch.empty(zs.shape, dtype=torch.bfloat16, device="cuda")
+    step.run(zs, zt, grad)
+    torch.cuda.synchronize()
+    assert step.status() == 0
+    g_ref, _, _ = oracle.loss_fwd_bwd(bits_or_f32(zs), bits_or_f32(zt), V, b.loss_mask,
+                                      step.w[:b.num_tokens].cpu().numpy(), row_of_token=b.compact_rows())
+    k = np.arange(R), y.cpu().numpy()
+    ref, got = g_ref[k], grad.double().cpu().numpy()[k]
+    assert (np.abs(got - ref) <= 2.0 ** -7 * np.abs(ref)).all(), np.abs(got / ref - 1).max()
+
+
 def test_ragged_rows_dense_neighbours_untouched(P, oracle):
     """One row per token, odd stride: the gradient rows of masked tokens share vectors
     with supervised ones and stay as they were."""
