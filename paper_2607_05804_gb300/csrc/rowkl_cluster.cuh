@@ -1060,8 +1060,10 @@ inline int cluster_size(int nvec)
 //   2,759 at 0.72, 2,845 at 0.88), with an fp32 gradient 0.73 (16 x 8192 household tokens
 //   2,375; 2,400 at 0.68, 2,431 at 0.76), sampled tokens 0.86 (64 multihop 1,028; 1,049 at
 //   0.72); at 2,004 (128,256) 0.92 (6,232; 6,003 at 0.72) and 0.78 (5,865; 5,471 at 0.85);
-//   of 16: 0.8 at 2,048 and 1,563 (200,000: 5,487, 5,265 at 0.6), 0.6 at 1,758 (5,405, 5,097
-//   at 0.8), with an fp32 gradient 0.2 less; of 3 in ShapeMid 0.5 (39,000: 6,183, 5,222 at
+//   of 16: 0.8 at 1,563 (200,000: 5,487, 5,265 at 0.6), 0.6 at 1,758 (5,405, 5,097 at 0.8), with an
+//   fp32 gradient 0.2 less; in ShapeBig (us at 6e8 logits) 0.95 at 1,875 (240,000: 610, 633 at
+//   0.8), 0.84 at 2,048 (262,144: 603, 616 at 0.75), 0.65 at 2,344 (300,000: 605, 685 at 0.8), with
+//   an fp32 gradient 0.85 (907, 958 at 0.65), 0.8 (826, 868 at 0.6) and 0.7 (825, 964 at 0.8); of 3 in ShapeMid 0.5 (39,000: 6,183, 5,222 at
 //   0.7); of 3 to 6 otherwise 0.7 (90,000: 6,335, 6,245 at 0.4), 0.62 with an fp32 gradient
 //   (49,152: 6,252 at 0.6, 5,978 at 0.7);
 //   fp32, clusters of 16: 0.69 at 2,374 (151,936: 4 x 4096 packed tokens 2,808 us; 2,833 at
@@ -1075,22 +1077,33 @@ inline int cluster_size(int nvec)
 //   forward-only rows, which the helper reads once: 1.0 (bf16 at 2,374: 4,743, 4,478 at 0.7;
 //   fp32, clusters of 8 at 2,350: 6,185, 5,836 at 0.7), 0.7 for bf16 in clusters of 3 and 4
 //   (57,000: 4,570, 3,443 at 1.0), 0.85 of 5 and 6, 0.9 for fp32 in clusters of 3.
-template <typename T> double helper_rate(int slice_vec, int cs, bool sampled, bool g32, bool forward)
+//   bf16 rows that do not all start on a 32-byte sector, which cost the helper's own loads more
+//   than the clusters' bulk copies: clusters of 8 0.13 less with a bf16 gradient (V = 151,944: 579
+//   us at 0.68, 636 at 0.81), 0.07 less with an fp32 one (820, 880), 0.9 forward (473, 495 at 1.0);
+//   of any stride 0.06, 0.04, 0.9 (151,937: 673, 692; 890, 905; 500, 524); of 3 and 4 0.63 (50,008:
+//   590, 625 at 0.70; 70,008: 573, 597); of 16 in ShapeBig 0.15, 0.05 (240,008: 631 at 0.8, 670 at
+//   0.85; 909, 938).  The other sizes peak where aligned rows do.
+template <typename T, int TL>
+double helper_rate(int slice_vec, int cs, bool sampled, bool g32, bool forward, bool sectors)
 {
     const bool bf16 = sizeof(T) == 2;
     if (forward)
-        return cs >= 8 ? 1.0 : bf16 ? (cs <= 4 ? 0.7 : 0.85) : (cs == 3 ? 0.9 : 1.0);
+        return cs == 8 && bf16 && !sectors ? 0.9
+               : cs >= 8 ? 1.0 : bf16 ? (cs <= 4 ? 0.7 : 0.85) : (cs == 3 ? 0.9 : 1.0);
     double r;
     if (bf16) {
         if (cs == 3 && slice_vec <= ShapeMid::kMax)
             return 0.50;
         if (cs < 8)
-            return g32 ? 0.62 : 0.70;
+            return g32 ? 0.62 : cs <= 4 && !sectors && TL != kAny ? 0.63 : 0.70;
         if (cs == 8)
-            r = g32 ? 0.73 + (2374 - slice_vec) * 0.00014 : 0.81 + (2374 - slice_vec) * 0.0003;
+            r = (g32 ? 0.73 + (2374 - slice_vec) * 0.00014 : 0.81 + (2374 - slice_vec) * 0.0003) -
+                (sectors ? 0.0 : TL == kAny ? (g32 ? 0.04 : 0.06) : (g32 ? 0.07 : 0.13));
+        else if (slice_vec > ShapeMid::kMax)
+            r = g32 ? 0.85 - (slice_vec - 1875) * 0.00032 - (sectors ? 0.0 : 0.05)
+                    : 0.95 - (slice_vec - 1875) * 0.00064 - (sectors ? 0.0 : 0.15);
         else
-            r = (slice_vec > 1563 && slice_vec <= ShapeMid::kMax ? 0.80 - (slice_vec - 1563) * 0.001 : 0.80) -
-                (g32 ? 0.2 : 0.0);
+            r = (slice_vec > 1563 ? 0.80 - (slice_vec - 1563) * 0.001 : 0.80) - (g32 ? 0.2 : 0.0);
     } else {
         if (cs < 8)
             return cs <= 4 ? 0.60 : 0.70;
@@ -1175,7 +1188,7 @@ cudaError_t launch_t(const RowIn &p, int nvec, cudaStream_t stream, bool *used)
         const double cl = (double)(grid_cache[dev] * CS);
         pl.split_den = 1 << 20;
         pl.split_ctas = free_sm;
-        pl.split_num = (int32_t)(pl.split_den * cl / (cl + helper_rate<T>(slice_vec, CS, SM, G32, !p.grad) * free_sm) + 0.5);
+        pl.split_num = (int32_t)(pl.split_den * cl / (cl + helper_rate<T, TL>(slice_vec, CS, SM, G32, !p.grad, p.ld * (int64_t)sizeof(T) % 32 == 0) * free_sm) + 0.5);
     }
     cfg.gridDim = dim3(grid_cache[dev] * CS);
     e = cudaLaunchKernelEx(&cfg, kern, pl, slice_vec, nvec);
