@@ -46,16 +46,44 @@ namespace {
 constexpr uint32_t kCopyChunk = 65536;       // bytes per bulk copy instruction
 constexpr uint32_t kWaitLimit = 1u << 22;    // mbarrier polls before giving up
 
-// Per-row constants the gradient pass needs (computed once per row).
+// Per-row constants the gradient pass needs (computed once per row): p |w| (full) or p |w l|
+// (sampled) is 2^(z_s log2e + nlw) |sg| (|sgl|).
 struct GradConst {
     float lse_s, lse_t, kl;
-    float nlw;        // -LSE_s log2e + log2 |w| (full) or log2 |w l| (sampled)
-    float sg;         // sign of w
-    float nd, ncp;    // -sg d, -sg cp
+    float nlw;        // -LSE_s log2e + log2 |w| or log2 |w l|; row_scale's hi where it is used
+    float sg;         // sign of w; row_scale's c
+    float nd, ncp;    // -sg d, -sg cp; with row_scale -d, -c cp
     float nc;         // -sg (d + cp)
-    float sgl;        // sign of -w l (sampled)
+    float sgl;        // sign of -w l (sampled); row_scale's c
     float gy;         // sampled: g_y = w l (1 - p_y)
 };
+
+// t 2^((z - m) log2e) as 2^(z log2e + hi) c, |c| <= 1 with the sign of t.  hi is -m log2e rounded
+// up, plus the power of two taken out of a t above 1; c holds t and what the rounding added.  A
+// constant -LSE log2e + log2 |w| rounded to one float instead is off by up to half an ulp of a
+// number as large as the logits, in every element of the row at once (2-norm error of the fp32
+// gradient, packed 4 x 4096, V = 151,936: 0.9-1.1e-6, with the two parts 1.4-1.9e-7; 2,803 and
+// 2,817 us).  |c| <= 1 keeps c ((z_s - z_t) - d) finite where the student alone is masked with the
+// type's lowest value.
+struct Scale {
+    float hi, c;
+};
+__device__ __forceinline__ Scale row_scale(float m, float t)
+{
+    const float M = fmaxf(m, kLowestRef);
+    int k = 0;
+    const float f = fabsf(t) > 1.f ? frexpf(t, &k) : t;
+    const float h0 = __fmul_rn(-M, kLog2e), kf = (float)k;
+    float h = __fadd_rn(h0, kf);
+    const float kb = __fsub_rn(h, h0);  // h + lo = -M log2e + k, exactly
+    float lo = __fadd_rn(__fmaf_rn(-M, kLog2e, -h0), __fadd_rn(__fsub_rn(h0, __fsub_rn(h, kb)), __fsub_rn(kf, kb)));
+    if (lo > 0.f) {
+        const float up = __int_as_float(__float_as_int(h) + (h < 0.f ? -1 : 1));  // the next float
+        lo -= __fsub_rn(up, h);
+        h = up;
+    }
+    return Scale{h, f * (lo > -0x1p-12f ? fmaf(lo, kLn2, 1.f) : exp2f(lo))};
+}
 
 // What a lane that does not count reads as: bf16's lowest finite value.  It adds 0 to every
 // sum, also where a thread or a vector holds nothing else (scale_of).
@@ -168,6 +196,16 @@ template <> struct Elem<float> {
     }
 };
 
+// Full-vocabulary gradient of a pair from p |w| (pw) and x = z_s - z_t: w p (x - d - cp), d and cp
+// subtracted one after the other (D) or as one constant; SC: the constants are row_scale's.
+template <bool D, bool SC>
+__device__ __forceinline__ float2 full_grad(float2 pw, float2 x, float2 SG, float2 ND, float2 NCP, float2 NC)
+{
+    if (SC)
+        return fmul2(pw, ffma2(fadd2(x, ND), SG, NCP));
+    return D ? fmul2(pw, fadd2(ffma2(x, SG, ND), NCP)) : fmul2(pw, ffma2(x, SG, NC));
+}
+
 // One vector of the gradient, g[NP] pairs, stored whole: vector q of the row at `off`.
 template <typename T, bool G32>
 __device__ __forceinline__ void store_grad(void *grad, size_t off, int q, const float2 *g)
@@ -265,6 +303,7 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
     // bf16: without it 0.3, 2, 12 and 18 %, with it the rounding's 0.4 % at each.)
     constexpr bool kUseD = G32 || N == 4 || (TL == kAny && !SM);
     constexpr bool kGradD = G32 || TL == kAny;  // the gradient subtracts d and cp one after the other
+    constexpr bool kScale = kGradD && N == 4;    // the row's constant in two parts (row_scale)
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ int s_dead;
     constexpr int NWG = NT / 32;  // warps per group
@@ -425,17 +464,26 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
         float e = rc.kl;
         if (SM)
             e = (ys - yt) - rc.dl;
-        // gradient constants of the row (see grad): p w = 2^(z_s log2e + nlw),
-        // sign sg of w applied through fma by (sg, sg)
+        // gradient constants of the row (see grad)
         const float wi = __int_as_float(meta[k % kStages].w), wl = wi * e;
         const float sg = wi < 0.f ? -1.f : 1.f;
         bc[0] = rc.lse_s, bc[1] = rc.lse_t, bc[2] = rc.kl, bc[3] = e;
-        bc[4] = -rc.lse_s * kLog2e + log2f(fabsf(SM ? wl : wi));  // nlw
-        bc[5] = sg;
-        bc[6] = -sg * rc.d;
-        bc[7] = -sg * rc.cp;
-        bc[8] = -sg * (rc.d + rc.cp);     // bf16 output: one rounding of d + cp
-        bc[9] = wl > 0.f ? -1.f : 1.f;    // sampled: sign of -w l
+        if (kScale) {
+            if (p.grad) {
+                const Scale q = row_scale(A.m, (SM ? -wl : wi) / A.s);
+                bc[4] = q.hi;
+                bc[5] = bc[9] = q.c;
+                bc[6] = -rc.d;
+                bc[7] = -q.c * rc.cp;
+            }
+        } else {
+            bc[4] = -rc.lse_s * kLog2e + log2f(fabsf(SM ? wl : wi));  // nlw
+            bc[5] = sg;
+            bc[6] = -sg * rc.d;
+            bc[7] = -sg * rc.cp;
+            bc[8] = -sg * (rc.d + rc.cp);     // one rounding of d + cp
+            bc[9] = wl > 0.f ? -1.f : 1.f;    // sampled: sign of -w l
+        }
         bc[10] = wl * omp;                 // sampled: g_y = w l (1 - p_y)
     };
 
@@ -630,8 +678,8 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
         const Slice sl = slice_of(m.y);
         const int gvec = sl.gvec;
         const size_t row_off = (size_t)m.y * (size_t)p.ld - (size_t)sl.head0 + (size_t)v0 * N;
-        // p |w| = 2^(z_s log2e - LSE_s log2e + log2 |w|); the sign of w enters through an
-        // fma by (sg, sg), which is exact on z_s - z_t
+        // the sign of w (and row_scale's c) enters through an fma by (sg, sg), which is exact on
+        // z_s - z_t for a sign alone
         const float2 L2 = splat(kLog2e), NLW = splat(gc.nlw);
         const float2 SG = splat(gc.sg), ND = splat(gc.nd), NCP = splat(gc.ncp), NC = splat(gc.nc);
         const float2 SGL = splat(gc.sgl);
@@ -649,9 +697,8 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
                     for (int j = 0; j < NP; ++j) {
                         const float2 a2 = E::pair(a, j), b2 = E::pair(b, j);
                         const float2 pw = ex2x2(ffma2(a2, L2, NLW));
-                        // sg ((z_s - z_t) - c) with one rounding; sg (z_s - z_t) is exact
                         const float2 x = fsub2(a2, b2);
-                        g[j] = kGradD ? fmul2(pw, fadd2(ffma2(x, SG, ND), NCP)) : fmul2(pw, ffma2(x, SG, NC));
+                        g[j] = full_grad<kGradD, kScale>(pw, x, SG, ND, NCP, NC);
                     }
                 } else {  // sampled token: g = -w l p (g_y is written after the loop)
                     const uint4 a = vs[q];
@@ -671,7 +718,7 @@ __global__ void __launch_bounds__(G * NT, 1) k_row_cluster(RowIn p, int slice_ve
                 const float2 a2 = E::pair(a, j), b2 = E::pair(b, j);
                 const float2 pw = ex2x2(ffma2(a2, L2, NLW)), x = fsub2(a2, b2);
                 g[j] = SM ? fmul2(pw, SGL)
-                          : (kGradD ? fmul2(pw, fadd2(ffma2(x, SG, ND), NCP)) : fmul2(pw, ffma2(x, SG, NC)));
+                          : full_grad<kGradD, kScale>(pw, x, SG, ND, NCP, NC);
             }
             store_grad_lanes<T, G32>(p.grad, row_off + (size_t)q * N, g, lo, hi);
         };
@@ -769,7 +816,7 @@ __global__ void __launch_bounds__(NTH, MINB) k_row_helper(RowIn p)
     using E = Elem<T>;
     constexpr int N = E::N, NP = E::NP;
     constexpr uint32_t kFill = E::kFillWord;
-    constexpr bool kUseD = G32 || N == 4 || (TL == kAny && !SM), kGradD = G32 || TL == kAny;  // as in the cluster kernel
+    constexpr bool kUseD = G32 || N == 4 || (TL == kAny && !SM), kGradD = G32 || TL == kAny, kScale = kGradD && N == 4;  // as in the cluster kernel
     __shared__ float red[NW][8];
     __shared__ float bc[8];
     extern __shared__ uint4 hring[];  // [kHelpStages][2][kHelpU][NTH] (AS)
@@ -940,13 +987,23 @@ __global__ void __launch_bounds__(NTH, MINB) k_row_helper(RowIn p)
                 p.token_loss[m.x] = e;
                 p.row_wl[j] = (double)wi * (double)e;
                 // the gradient constants of the cluster kernel
-                bc[0] = -rc.lse_s * kLog2e + log2f(fabsf(SM ? wl : wi));  // nlw
-                bc[1] = sg;
-                bc[2] = -sg * (rc.d + rc.cp);  // bf16 output: one rounding of d + cp
-                bc[3] = wl > 0.f ? -1.f : 1.f;
+                if (kScale) {
+                    if (p.grad) {
+                        const Scale q = row_scale(A.m, (SM ? -wl : wi) / A.s);
+                        bc[0] = q.hi;
+                        bc[1] = bc[3] = q.c;
+                        bc[5] = -rc.d;
+                        bc[6] = -q.c * rc.cp;
+                    }
+                } else {
+                    bc[0] = -rc.lse_s * kLog2e + log2f(fabsf(SM ? wl : wi));  // nlw
+                    bc[1] = sg;
+                    bc[2] = -sg * (rc.d + rc.cp);  // one rounding of d + cp
+                    bc[3] = wl > 0.f ? -1.f : 1.f;
+                    bc[5] = -sg * rc.d;            // kGradD
+                    bc[6] = -sg * rc.cp;
+                }
                 bc[4] = wl * omp;              // sampled: g_y = w l (1 - p_y)
-                bc[5] = -sg * rc.d;            // kGradD
-                bc[6] = -sg * rc.cp;
             }
         }
         __syncthreads();
@@ -979,7 +1036,7 @@ __global__ void __launch_bounds__(NTH, MINB) k_row_helper(RowIn p)
                         for (int w = 0; w < NP; ++w) {
                             const float2 a2 = E::pair(a[u], w), b2 = E::pair(b[u], w);
                             const float2 pw = ex2x2(ffma2(a2, L2, NLW)), x = fsub2(a2, b2);
-                            g[w] = kGradD ? fmul2(pw, fadd2(ffma2(x, SG, ND), NCP)) : fmul2(pw, ffma2(x, SG, NC));
+                            g[w] = full_grad<kGradD, kScale>(pw, x, SG, ND, NCP, NC);
                         }
                     } else {  // sampled token: g = -w l p (g_y is written after the loop)
 #pragma unroll
@@ -1000,7 +1057,7 @@ __global__ void __launch_bounds__(NTH, MINB) k_row_helper(RowIn p)
                     const float2 a2 = E::pair(a, w), b2 = E::pair(b, w);
                     const float2 pw = ex2x2(ffma2(a2, L2, NLW)), x = fsub2(a2, b2);
                     g[w] = SM ? fmul2(pw, SGL)
-                              : (kGradD ? fmul2(pw, fadd2(ffma2(x, SG, ND), NCP)) : fmul2(pw, ffma2(x, SG, NC)));
+                              : full_grad<kGradD, kScale>(pw, x, SG, ND, NCP, NC);
                 }
                 store_grad_lanes<T, G32>(p.grad, to, g, lo, hi);
             };

@@ -414,6 +414,33 @@ def test_dominant_token_of_ragged_rows(P, oracle, V, idt):
     assert (np.abs(got - ref) <= 2.0 ** -7 * np.abs(ref)).all(), np.abs(got / ref - 1).max()
 
 
+@pytest.mark.parametrize("V", [4100, 50001, W.V_QWEN])
+@pytest.mark.parametrize("mode", [0, 1], ids=["full", "sampled"])
+def test_fp32_gradient_rows_in_fp32(P, oracle, V, mode):
+    """fp32 logits and gradient: the median row's relative 2-norm error against fp64 is below 3e-7, an
+    exponential's 2^-22 and half an ulp of an exponent below 1, where most of a row's gradient lies.
+    (A row constant of LSE's size rounded to one float moves every element of a row at once by up to
+    1.3e-6: medians of 4 to 6e-7.)  A sampled-token row is compared at the GPU's own loss."""
+    b = W.packed(seed=81, num_traj=2, traj_len=256)
+    R = b.num_valid
+    zs, zt = W.make_logits(R, V, "agent", torch.float32, seed=82, device="cuda")
+    y = per_token_ids(b, W.sample_ids(zs, 83, V), True) if mode == 1 else None
+    step = make_step(P, b, V, compact=True, mode=mode, y=y)
+    grad = torch.empty_like(zs)
+    step.run(zs, zt, grad)
+    torch.cuda.synchronize()
+    assert step.status() == 0
+    g_ref, tl_ref, _ = oracle.loss_fwd_bwd(zs.cpu().numpy(), zt.cpu().numpy(), V, b.loss_mask,
+                                           step.w[:b.num_tokens].cpu().numpy(), mode=mode, row_of_token=b.compact_rows(),
+                                           sampled_ids=None if y is None else y.cpu().numpy())
+    ref, got = np.asarray(g_ref)[:R], grad.double().cpu().numpy()
+    if mode == 1:
+        m = b.loss_mask == 1
+        ref = ref * (step.token_loss[:b.num_tokens].cpu().numpy()[m] / tl_ref[m])[:, None]
+    err = np.linalg.norm(got - ref, axis=1) / np.linalg.norm(ref, axis=1)
+    assert np.median(err) <= 3e-7, np.median(err)
+
+
 def test_ragged_rows_dense_neighbours_untouched(P, oracle):
     """One row per token, odd stride: the gradient rows of masked tokens share vectors
     with supervised ones and stay as they were."""
