@@ -24,6 +24,7 @@ __all__ = [
     "turnopd_alpha_schedule", "turnopd_turn_floor", "turnopd_status_string", "turnopd_loss_fwd_bwd_static",
     "turnopd_selftest_wait_timeout",
     "TURNOPD_STATIC_MAX_TOKENS", "turnopd_fused_lmhead_fwd_bwd", "turnopd_fused_workspace_bytes",
+    "turnopd_fused_workspace_min_bytes",
     "turnopd_topk_loss_fwd_bwd", "TURNOPD_TOPK_MAX", "TURNOPD_TOPK_MAX_VOCAB",
     "turnopd_depth_params", "turnopd_depth_state", "turnopd_depth_default_params",
     "turnopd_depth_init", "turnopd_depth_plan", "turnopd_depth_update", "turnopd_depth_efficiency",
@@ -116,6 +117,8 @@ def load():
     lib.turnopd_loss_workspace_bytes.restype = sz
     lib.turnopd_fused_workspace_bytes.argtypes = [i64, i64, i64, i64]
     lib.turnopd_fused_workspace_bytes.restype = sz
+    lib.turnopd_fused_workspace_min_bytes.argtypes = [i64, i64, i64, i64]
+    lib.turnopd_fused_workspace_min_bytes.restype = sz
     lib.turnopd_alpha_schedule.argtypes = [i64, i64, f64, f64]
     lib.turnopd_alpha_schedule.restype = f64
     lib.turnopd_turn_floor.argtypes = [i64, i32, f64]
@@ -213,6 +216,12 @@ def turnopd_loss_workspace_bytes(num_tokens: int) -> int:
 
 def turnopd_fused_workspace_bytes(num_tokens: int, vocab: int, d_s: int, d_t: int) -> int:
     return int(load().turnopd_fused_workspace_bytes(int(num_tokens), int(vocab), int(d_s), int(d_t)))
+
+
+def turnopd_fused_workspace_min_bytes(num_tokens: int, vocab: int, d_s: int, d_t: int) -> int:
+    """The least a call accepts: without room for a chunk's logits, which the backward pass then
+    computes a second time."""
+    return int(load().turnopd_fused_workspace_min_bytes(int(num_tokens), int(vocab), int(d_s), int(d_t)))
 
 
 def turnopd_fused_lmhead_fwd_bwd(h_s, W_s, h_t, W_t, loss_mask, w, mode, dh_s_out, token_loss_out,

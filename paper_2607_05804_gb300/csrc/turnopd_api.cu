@@ -387,6 +387,13 @@ size_t turnopd_fused_workspace_bytes(int64_t num_tokens, int64_t vocab, int64_t 
     return fused_workspace_bytes(num_tokens, vocab, d_s, d_t);
 }
 
+size_t turnopd_fused_workspace_min_bytes(int64_t num_tokens, int64_t vocab, int64_t d_s, int64_t d_t)
+{
+    if (num_tokens < 0 || vocab < 1 || d_s < 1 || d_t < 1)
+        return 0;
+    return fused_workspace_min_bytes(num_tokens, vocab, d_s, d_t);
+}
+
 turnopd_status turnopd_fused_lmhead_fwd_bwd(const void *h_s, const void *W_s, int64_t d_s,
                                             const void *h_t, const void *W_t, int64_t d_t,
                                             int64_t vocab, const uint8_t *loss_mask,

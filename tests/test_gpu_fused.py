@@ -288,3 +288,32 @@ def test_fused_chunk_scratch_and_recompute_agree(P, oracle, traj_len, V):
         assert_dh(dh[m], dh_ref[m])
         assert_dh(dW, dw_ref)
     assert_dh(out[0][0][m], out[1][0][m])
+
+
+def test_fused_least_workspace(P, oracle):
+    """The reported least workspace is accepted and gives the same results; one byte less is
+    refused.  It leaves out the chunk's logits: 8 bytes for each of 2,048 rows' columns here."""
+    b = W.packed(seed=43, num_traj=2, traj_len=1500)
+    V, d_s, d_t, T = 1000, 256, 192, b.num_tokens
+    hs, Ws, ht, Wt = W.make_fused(T, d_s, d_t, V, seed=44, device="cuda")
+    msk = torch.from_numpy(b.loss_mask).cuda()
+    w = torch.rand(T, generator=torch.Generator().manual_seed(4)).cuda()
+    least, full = (f(T, V, d_s, d_t) for f in (P.turnopd_fused_workspace_min_bytes, P.turnopd_fused_workspace_bytes))
+    assert full - least >= 8 * 2048 * V
+    ws = torch.empty(least, dtype=torch.uint8, device="cuda")
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    dh = torch.zeros((T, d_s), dtype=torch.float32, device="cuda")
+    tl = torch.zeros(T, dtype=torch.float32, device="cuda")
+    loss = torch.zeros(1, dtype=torch.float64, device="cuda")
+    P.turnopd_fused_lmhead_fwd_bwd(hs, Ws, ht, Wt, msk, w, 0, dh, tl, loss, ws, st)
+    torch.cuda.synchronize()
+    assert st.item() == 0
+    dh_ref, tl_ref, loss_ref = oracle.fused_lmhead(*(W.bf16_bits(x) for x in (hs, Ws, ht, Wt)), b.loss_mask,
+                                                   w.cpu().numpy())[:3]
+    m = b.loss_mask == 1
+    assert_token_loss(tl.cpu().numpy(), tl_ref, b.loss_mask)
+    assert_loss(loss.item(), loss_ref)
+    assert_dh(dh.cpu().numpy()[m], dh_ref[m])
+    with pytest.raises(P.TurnopdError) as e:
+        P.turnopd_fused_lmhead_fwd_bwd(hs, Ws, ht, Wt, msk, w, 0, dh, tl, loss, ws[:least - 1], st)
+    assert e.value.code == 10  # TURNOPD_ERR_WORKSPACE
