@@ -25,10 +25,6 @@ cudaError_t launch_rows(const RowIn &p, bool bf16, bool fp32_grad, cudaStream_t 
         return whole ? launch_rows_bf16(p, fp32_grad, stream)
                : p.ld % n == 0 ? launch_rows_bf16_tail(p, fp32_grad, stream)
                                : launch_rows_bf16_ragged(p, fp32_grad, stream);
-    // rows longer than 16 CTAs hold are streamed twice (V = 151,936 on clusters of 8: 5,400
-    // GB/s, held by clusters of 16: 6,020)
-    if (whole && cluster_size((int)(p.vocab / 4)) == 0)
-        return launch_row_split(p, fp32_grad, stream);
     return whole ? launch_rows_f32(p, fp32_grad, stream) : launch_rows_f32_ragged(p, fp32_grad, stream);
 }
 

@@ -33,6 +33,7 @@
 #pragma once
 
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 #include "kernels.h"
@@ -1189,7 +1190,8 @@ template <class Shape> size_t cluster_smem_bytes(int slice_vec, int cs)
 // The cluster grid (as many clusters as are co-resident, cached per device) and
 // the helper grid on the SMs the clusters leave free, with the row list split so
 // that both finish together.  *used = false (and nothing is launched) where the slices
-// do not fit shared memory.
+// do not fit shared memory, or where the device places no cluster of this size (16 is not a
+// portable size; a partition of the device may have no room for it).
 template <typename T, bool G32, int CS, class Shape, bool SM, int TL>
 cudaError_t launch_t(const RowIn &p, int nvec, cudaStream_t stream, bool *used)
 {
@@ -1233,10 +1235,13 @@ cudaError_t launch_t(const RowIn &p, int nvec, cudaStream_t stream, bool *used)
         cfg.gridDim = dim3(CS);
         int ncl = 0;
         e = cudaOccupancyMaxActiveClusters(&ncl, kern, &cfg);
-        if (e != cudaSuccess)
+        if (e != cudaSuccess && e != cudaErrorInvalidClusterSize)
             return e;
-        if (ncl < 1)
-            return cudaErrorInvalidConfiguration;
+        if (e != cudaSuccess)
+            cudaGetLastError();  // answered below: nothing was launched
+        *used = e == cudaSuccess && ncl > 0;
+        if (!*used)
+            return cudaSuccess;
         grid_cache[dev] = ncl;
     }
     RowIn pl = p;
@@ -1326,8 +1331,14 @@ cudaError_t launch_rows_m(const RowIn &p, int nvec, cudaStream_t stream)
     const cudaError_t e = launch_cs<T, G32, SM, TL>(p, nvec, stream, &used);
     if (e != cudaSuccess || used)
         return e;
-    launch_helper_alone<T, G32, SM, TL>(p, stream);
-    return cudaGetLastError();
+    // rows that no cluster holds, or whose cluster size the device cannot place: whole fp32 ones are
+    // streamed twice by clusters of 8 (V = 151,936: 5,400 GB/s, held by clusters of 16 6,020)
+    if constexpr (std::is_same<T, float>::value && TL == kWhole) {
+        return launch_row_split(p, G32, stream);
+    } else {
+        launch_helper_alone<T, G32, SM, TL>(p, stream);
+        return cudaGetLastError();
+    }
 }
 
 // The row grids for logits of T in rows of form TL.
