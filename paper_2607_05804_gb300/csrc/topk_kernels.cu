@@ -8,7 +8,7 @@
 //
 // Short rows and rows of any other alignment: k_topk_short, one CTA a row.  Others:
 // persistent CTAs, each with two rows in flight: streaming warps run pass A
-// of a row while two selector warps run the later phases of the previous row
+// of a row while two or four selector warps run the later phases of the previous row
 // (double-buffered buckets, named barriers).  Selection with 64-bit keys
 // (order-preserving logit bits << 32 | ~id, so larger key = larger logit,
 // then lower id):
@@ -16,14 +16,14 @@
 //            consecutive ids the largest logit is recorded in shared memory as
 //            a 16-bit ordered bucket (the top 16 bits of the order-preserving
 //            bits), and every thread keeps the largest logit it saw;
-//   bound    (streaming warps) for K <= 64, tau = the K-th largest of the 8
+//   bound    (streaming warps) for K <= 96, tau = the K-th largest of the 8
 //            largest lane maxima of every streaming warp: K-th largest of
 //            distinct elements of the row, so a lower bound of the row's K-th
 //            largest logit; above, the K-th largest thread maximum, or (K above
 //            288, or rows of few groups) the K-th largest group bucket (K groups
 //            each hold an element that large), by binary search on its value;
 //            then the groups whose bucket reaches tau's are listed (and above K =
-//            192 the bound is refined to the K-th largest bucket of the listed);
+//            192, 160 for fp32, it is refined to the K-th largest bucket listed);
 //   collect  (selector warps) only the listed groups are read again, in step
 //            across the lanes (a few dozen per row at K = 50), and their
 //            elements >= tau go to a shared-memory candidate buffer (1,024
@@ -32,7 +32,7 @@
 //            tau, one key byte per pass, raises tau until the keys above it fit
 //            the buffer, then collects again (at most 6 passes for bf16 keys,
 //            8 for fp32);
-//   select   up to 320 candidates: the exact K-th largest by radix select (buffers
+//   select   up to 256 candidates: the exact K-th largest by radix select (buffers
 //            over 2 K), then each selected key's rank among the candidates is its
 //            position;
 //            more: a bitonic sort of the buffer.
@@ -83,12 +83,13 @@ __host__ __device__ constexpr int topk_cap(int K) { return K <= 512 ? 1024 : 204
 constexpr int kTkLaneTop = 8;
 constexpr int kTkLaneBoundMaxK = kTkStreamWarps * kTkLaneTop;
 // candidates above which the selection sorts the buffer instead of ranking
-constexpr int kTkRankMax = 320;
+constexpr int kTkRankMax = 256;
 constexpr uint32_t kTkQueue = 64;  // ring of group indices per selector warp (at most 63 held)
 constexpr int kTkGroup = 16;      // ids per recorded bucket
 constexpr int kRefine = 2;        // listed groups per streaming thread that the bound is refined on
-// (K = 256 at V = 151,936: 863 us with it, 883 without; K = 128: 728 and 642)
-constexpr int kRefineMinK = 192;
+// (K = 256 at V = 151,936: 863 us with it, 883 without; K = 128: 728 and 642; fp32, where the
+// listed groups' second read weighs double, K = 192 at V = 98,304 207 and 235, K = 160 200 and 192)
+constexpr int kRefineMinK = 192, kRefineMinKF32 = 160;
 static_assert(kTkQueue >= 64 && (kTkQueue & (kTkQueue - 1)) == 0, "group ring");
 static_assert(TURNOPD_TOPK_MAX_VOCAB / kTkGroup <= 65536, "group indices are 16-bit");
 static_assert(TURNOPD_TOPK_MAX_VOCAB <= (1 << 20) && topk_cap(TURNOPD_TOPK_MAX) <= 2048,
@@ -359,12 +360,17 @@ __host__ __device__ __forceinline__ size_t topk_bucket_bytes(int64_t V)
 
 size_t topk_smem_bytes(int64_t V, int K) { return topk_fixed_bytes(K) + 2 * topk_bucket_bytes(V); }
 
+// Who writes a dense gradient row's zeros: the selector warps, but on fp32 rows of 14,336 to 65,536
+// ids the streaming warps (us of a step of 2e8 logits, by the selectors and by the stream: bf16 V =
+// 16,384, K = 30 244 and 255; 151,936, K = 256 206 and 214; fp32, K = 30, 8,192 470 and 491, 16,384
+// 320 and 304, 32,768 285 and 272, 151,936 275 and 281; K = 320, 32,768 543 and 522, 98,304 340 and 354).
+enum DenseRow { kNoDense = 0, kZerosBySelectors = 1, kZerosByStream = 2 };
+
 // One CTA holds two rows at a time: its streaming warps run pass A and the
-// bound of row i + 1 (into bucket buffer (i + 1) % 2) while its two selector
+// bound of row i + 1 (into bucket buffer (i + 1) % 2) while its SW selector
 // warps run collect, select and the KL of row i from buffer i % 2, so the SM's
 // teacher stream does not pause for the latency-bound phases.
-// DN: a dense gradient row is written.
-template <bool BF16, int SW, bool DN>
+template <bool BF16, int SW, int DN>
 __global__ void __launch_bounds__(kTkStreamThreads + 32 * SW, kTkMinBlocks) k_topk_rows(TopkArgs a)
 {
     constexpr int kTkSelWarps = SW, kTkSelThreads = 32 * SW, kTkThreads = kTkStreamThreads + kTkSelThreads;
@@ -401,11 +407,31 @@ __global__ void __launch_bounds__(kTkStreamThreads + 32 * SW, kTkMinBlocks) k_to
     const int ngv = vec_ok ? (int)(a.vocab / kTkGroup) : 0;  // whole groups read as vectors
     const size_t bucket_elems = topk_bucket_bytes(a.vocab) / sizeof(uint16_t);
     constexpr int VPG = BF16 ? 2 : 4;  // 16-byte vectors per group
-    // lower bound of the K-th largest logit: for K <= 64 every streaming warp contributes
+    // lower bound of the K-th largest logit: up to K = 96 every streaming warp contributes
     // the 8 largest of its lanes' maxima, and the K-th largest of these distinct elements
     // cannot exceed the row's K-th largest; above, the streaming warps take the K-th
-    // largest group bucket.
-    const bool lane_bound = K <= kTkLaneBoundMaxK;
+    // largest thread maximum or group bucket.  SW tells which at compile time, but for fp32 rows on
+    // two selector warps, which launch_topk also gives some K above 96.  (Tested at run time, bf16
+    // rows of few K took 3-7 % longer: V = 12,288, K = 20, dense row, 314 us, now 295.)
+    constexpr bool kOneBound = SW != kTkSelSmall || BF16;
+    const bool lane_bound = kOneBound ? SW == kTkSelSmall : K <= kTkLaneBoundMaxK;
+
+    // the dense gradient row's zeros, by nt threads
+    auto zero_row = [&](int row, int t0, int nt) {
+        const size_t gesz = a.grad_dtype == TURNOPD_BF16 ? 2 : 4;
+        char *grow = static_cast<char *>(a.grad) + (size_t)row * (size_t)a.ld * gesz;
+        const int64_t bytes = a.vocab * (int64_t)gesz;
+        // 16-byte stores between a head up to the first 16-byte boundary and a tail
+        const int64_t head = min(bytes, (int64_t)((16u - (reinterpret_cast<uintptr_t>(grow) & 15u)) & 15u));
+        const int64_t nv16 = (bytes - head) / 16;
+        uint4 *body = reinterpret_cast<uint4 *>(grow + head);
+        for (int64_t q = t0; q < nv16; q += nt)
+            __stcs(body + q, make_uint4(0, 0, 0, 0));
+        for (int64_t q = t0; q < head / 2; q += nt)
+            reinterpret_cast<uint16_t *>(grow)[q] = 0;
+        for (int64_t q = (head + nv16 * 16) / 2 + t0; q < bytes / 2; q += nt)
+            reinterpret_cast<uint16_t *>(grow)[q] = 0;
+    };
 
     if (warp < kTkStreamWarps) {
         // ---- streaming warps: pass A, one row after another
@@ -424,21 +450,6 @@ __global__ void __launch_bounds__(kTkStreamThreads + 32 * SW, kTkMinBlocks) k_to
         };
         auto row_vectors = [&](const int4 &mr) {
             return reinterpret_cast<const uint4 *>(static_cast<const char *>(a.zt) + (size_t)mr.y * (size_t)a.ld * esz);
-        };
-        auto zero_row = [&](int row, int t0) {
-            const size_t gesz = a.grad_dtype == TURNOPD_BF16 ? 2 : 4;
-            char *grow = static_cast<char *>(a.grad) + (size_t)row * (size_t)a.ld * gesz;
-            const int64_t bytes = a.vocab * (int64_t)gesz;
-            // 16-byte stores between a head up to the first 16-byte boundary and a tail
-            const int64_t head = min(bytes, (int64_t)((16u - (reinterpret_cast<uintptr_t>(grow) & 15u)) & 15u));
-            const int64_t nv16 = (bytes - head) / 16;
-            uint4 *body = reinterpret_cast<uint4 *>(grow + head);
-            for (int64_t q = t0; q < nv16; q += kTkStreamThreads)
-                __stcs(body + q, make_uint4(0, 0, 0, 0));
-            for (int64_t q = t0; q < head / 2; q += kTkStreamThreads)
-                reinterpret_cast<uint16_t *>(grow)[q] = 0;
-            for (int64_t q = (head + nv16 * 16) / 2 + t0; q < bytes / 2; q += kTkStreamThreads)
-                reinterpret_cast<uint16_t *>(grow)[q] = 0;
         };
         // The largest value x <= hi with at least K counted at or above it (0: none), by binary
         // search; warp_count(x) is a warp's count.  The first pass probes 255 below hi (where
@@ -511,10 +522,9 @@ __global__ void __launch_bounds__(kTkStreamThreads + 32 * SW, kTkMinBlocks) k_to
                     tmax = max(tmax, o);
                 }
             }
-            // the dense gradient row's zeros (the selectors write the K values over them once
-            // this row's buffer is full)
-            if (DN)
-                zero_row(m.y, tid);
+            // the selectors write the K values over the zeros once this row's buffer is full
+            if (DN == kZerosByStream)
+                zero_row(m.y, tid, kTkStreamThreads);
             // groups left: the partial last group, or every group of a misaligned row
             for (int g = ngv + tid; g < (int)ng; g += kTkStreamThreads) {
                 const uint32_t o = group_max_ord_scalar<BF16>(zt_row, a.vocab, g);
@@ -555,7 +565,7 @@ __global__ void __launch_bounds__(kTkStreamThreads + 32 * SW, kTkMinBlocks) k_to
                     if (v != 0 && gt < K && ge >= K)
                         s_tau[b] = v;  // every such thread writes the same value
                 }
-            } else if (a.vocab > cap) {
+            } else if (!(kOneBound && SW == kTkSelSmall) && a.vocab > cap) {
                 // the K-th largest group bucket, by binary search on its value with counts of
                 // the buckets at or above it: K groups each hold an element that large (no
                 // bound, tau = 0, when the row has fewer than K groups)
@@ -575,20 +585,22 @@ __global__ void __launch_bounds__(kTkStreamThreads + 32 * SW, kTkMinBlocks) k_to
                 // walk the row's buckets.
                 const int n_thr = min((int)ng, kTkStreamThreads);
                 const bool by_thread = K <= n_thr / 4 * 3;
-                refine = by_thread && K > kRefineMinK;
+                refine = by_thread && K > (BF16 ? kRefineMinK : kRefineMinKF32);
                 const uint32_t tb = bucket<BF16>(tmax);
-                const uint32_t lo = kth_bucket(hi, [&](uint32_t mid) {
-                    if (by_thread)
-                        return __popc(__ballot_sync(0xffffffffu, tb >= mid));
-                    int c = 0;
-                    for (int i = tid; i < n4; i += kTkStreamThreads) {
-                        const uint4 q = b4[i];
-                        c += count_ge2(q.x, mid) + count_ge2(q.y, mid) + count_ge2(q.z, mid) + count_ge2(q.w, mid);
-                    }
-                    for (int g = n4 * 8 + tid; g < (int)ng; g += kTkStreamThreads)
-                        c += (uint32_t)s_bucket[g] >= mid;
-                    return (int)__reduce_add_sync(0xffffffffu, c);
-                });
+                uint32_t lo;
+                if (by_thread)
+                    lo = kth_bucket(hi, [&](uint32_t mid) { return __popc(__ballot_sync(0xffffffffu, tb >= mid)); });
+                else
+                    lo = kth_bucket(hi, [&](uint32_t mid) {
+                        int c = 0;
+                        for (int i = tid; i < n4; i += kTkStreamThreads) {
+                            const uint4 q = b4[i];
+                            c += count_ge2(q.x, mid) + count_ge2(q.y, mid) + count_ge2(q.z, mid) + count_ge2(q.w, mid);
+                        }
+                        for (int g = n4 * 8 + tid; g < (int)ng; g += kTkStreamThreads)
+                            c += (uint32_t)s_bucket[g] >= mid;
+                        return (int)__reduce_add_sync(0xffffffffu, c);
+                    });
                 if (tid == 0)
                     s_tau[b] = BF16 ? lo : lo << 16;
             }
@@ -614,7 +626,7 @@ __global__ void __launch_bounds__(kTkStreamThreads + 32 * SW, kTkMinBlocks) k_to
             for (int g = n8 * 8 + tid; g < ngv; g += kTkStreamThreads)
                 if (s_bucket[g] >= taub)
                     list(g);
-            if (refine) {
+            if (!(kOneBound && SW == kTkSelSmall) && refine) {
                 // The list (about 1.6 K groups) holds every group whose bucket reaches the bound,
                 // so the K-th largest bucket among the listed is the row's: K groups are at or
                 // above it, and the list shrinks to those and its ties.
@@ -884,11 +896,11 @@ __global__ void __launch_bounds__(kTkStreamThreads + 32 * SW, kTkMinBlocks) k_to
                 // ---- the K largest: each candidate's rank among the candidates is its position
                 // (keys are unique).  A buffer of more than twice K is first cut to the K largest by
                 // radix select; below that its passes cost more than the ranks they save.  Two keys
-                // of the buffer are read a load, but for two warps, K > 16 and short rows (us of a
-                // step of 2e8 bf16 logits, pairs and singles: V = 16,384 with a dense row, K = 8 258
-                // and 264, 30 286 and 279, 50 302 and 296, 80 457 and 428; 151,936, K = 50 115, 117).
+                // of the buffer are read a load, but for two warps and K > 16 (us of a step of 2e8
+                // bf16 logits, pairs and singles: V = 8,192, K = 8 327 and 344, 30 383 and 378;
+                // 151,936, K = 96 161 and 140).
                 const uint64_t kth = nc <= max(2 * K, kTkSelThreads) ? 0 : sel_kth_largest<SW>(s_cand, nc, K, hi_val, 0, s_sel, stid);
-                const bool singles = SW == kTkSelSmall && K > 16 && a.vocab <= 32768;
+                const bool singles = SW == kTkSelSmall && K > 16;
                 if (!singles) {
                     if (stid == 0 && (nc & 1))
                         s_cand[nc] = 0;  // the last pair's second key
@@ -963,11 +975,13 @@ __global__ void __launch_bounds__(kTkStreamThreads + 32 * SW, kTkMinBlocks) k_to
                     a.row_wl[j] = (double)w * (double)ell;
                 }
             }
-            // ---- dense gradient row: the K entries, over the streaming warps' zeros
+            // ---- dense gradient row: zeros, then the K entries
             if (DN) {
                 const size_t gesz = a.grad_dtype == TURNOPD_BF16 ? 2 : 4;
                 char *grow = static_cast<char *>(a.grad) + (size_t)m.y * (size_t)a.ld * gesz;
-                named_sync(kBarSel, kTkSelThreads);  // every entry of s_g is written
+                if (DN == kZerosBySelectors)
+                    zero_row(m.y, stid, kTkSelThreads);
+                named_sync(kBarSel, kTkSelThreads);  // zeros and every entry of s_g are written
                 for (int r = stid; r < K; r += kTkSelThreads) {
                     const uint32_t id = key_id(s_top[r]);
                     if (a.grad_dtype == TURNOPD_BF16)
@@ -1039,20 +1053,14 @@ __host__ __device__ __forceinline__ size_t short_smem(int K)
            (sizeof(uint64_t) + sizeof(float)) * (size_t)K + 16;
 }
 constexpr int kShortPerThread = 64;  // elements of a row per thread
-// Aligned rows up to here take the kernel below: what 128 threads hold, 256 from K = 64, 512
-// for K = 240-288 (where the streaming kernel's bound, the K-th of 384 thread maxima, is loosest).
-// That kernel reads the other rows faster.  us of a step of 2e8 bf16
-// logits, here and there: V = 8,184, K = 8 275 and 386, 50 316 and 501, 96 356 and 1,890;
-// V = 8,192 (256 threads), K = 64 551 and 676; 12,288, K = 32 370 and 300, 50 392 and 329, 64
-// 394 and 453; 16,376, K = 64 322 and 376, 256 516 and 879; 24,576 (512 threads), K = 80 434 and
-// 301, 128 459 and 354, 224 523 and 476, 240 541 and 563, 256 558 and 595, 320 611 and 566;
-// 32,744, K = 512 720 and 609.  fp32 rows cross at the same places.  Rows that are not 16-byte aligned, which the streaming kernel reads element by
-// element, take it at every length it holds (32,700, K = 50: 1,248 GB/s and 448).
-int short_max_vocab(int K)
-{
-    const int threads = K < 64 ? 128 : K < 240 || K > 288 ? 256 : 512;
-    return kShortPerThread * threads - 7;
-}
+// Aligned rows up to here take the kernel below: what 128 threads hold, 256 from K = 64.
+// k_topk_rows reads the other rows faster.  us of a step of 2e8 bf16 logits, here and there: V =
+// 8,184, K = 8 275 and 386, 50 316 and 501, 96 356 and 1,890; V = 8,192 (256 threads), K = 64 551
+// and 676; 12,288, K = 32 370 and 290, 50 392 and 322, 64 394 and 453; 16,376, K = 64 322 and 376,
+// 256 516 and 879; 24,576 (512 threads), K = 80 434 and 284, 256 576 and 540, 288 606 and 576.
+// fp32 rows cross at the same places.  Rows that are not 16-byte aligned, which k_topk_rows reads
+// element by element, take it at every length it holds (32,700, K = 50: 1,248 GB/s and 448).
+int short_max_vocab(int K) { return kShortPerThread * (K < 64 ? 128 : 256) - 7; }
 
 // Rows of up to 64 NT elements, one CTA of NT threads a row, any alignment: the row's
 // 16-bit buckets (the logit itself for bf16) stay in registers, 2 to a word, from the only
@@ -1071,7 +1079,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_topk_short(TopkArgs a)
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     constexpr int NW = NT / 32;
     constexpr int ESZ = BF16 ? 2 : 4;
-    extern __shared__ __align__(16) uint64_t tk_smem[];
+    extern __shared__ __align__(128) uint64_t tk_smem[];
     const int K = a.K, cap = short_cap(K);
     uint64_t *s_key = tk_smem;                                 // [cap] candidates
     uint64_t *s_top = s_key + cap;                             // [K] selected
@@ -1353,7 +1361,7 @@ cudaError_t launch_topk(const TopkCall &c, cudaStream_t stream)
     if ((e = cudaGetDevice(&dev)) != cudaSuccess)
         return e;
     using Kern = void (*)(TopkArgs);
-    static size_t attr_smem[64][16] = {};
+    static size_t attr_smem[64][20] = {};
     const int di = dev < 64 ? dev : 0;
     auto launch = [&](Kern kern, int slot, int threads, size_t smem) {
         cudaError_t e = cudaSuccess;
@@ -1371,7 +1379,7 @@ cudaError_t launch_topk(const TopkCall &c, cudaStream_t stream)
         return cudaGetLastError();
     };
     const bool bf16 = c.in_dtype == TURNOPD_BF16;
-    // rows that a CTA holds in registers, with up to 7 elements before the first (kShortMaxV)
+    // rows that a CTA holds in registers, with up to 7 elements before the first
     const int64_t span = c.vocab + 7;
     const size_t esz = bf16 ? 2 : 4;
     const bool aligned = ((reinterpret_cast<uintptr_t>(c.zt) | reinterpret_cast<uintptr_t>(c.zs) | (uintptr_t)(c.ld * esz)) & 15u) == 0;
@@ -1381,19 +1389,28 @@ cudaError_t launch_topk(const TopkCall &c, cudaStream_t stream)
             {k_topk_short<false, 32>, k_topk_short<false, 128>, k_topk_short<false, 256>, k_topk_short<false, 512>},
             {k_topk_short<true, 32>, k_topk_short<true, 128>, k_topk_short<true, 256>, k_topk_short<true, 512>}};
         static const int threads[4] = {32, 128, 256, 512};
-        if ((e = launch(shorts[bf16][s4], 8 + bf16 * 4 + s4, threads[s4], short_smem(c.K))) != cudaSuccess)
+        if ((e = launch(shorts[bf16][s4], 12 + bf16 * 4 + s4, threads[s4], short_smem(c.K))) != cudaSuccess)
             return e;
         launch_loss_sum(ws.row_wl, ws.nvalid, c.loss, c.status, stream);
         return cudaGetLastError();
     }
-    const bool large = c.K > kTkLaneBoundMaxK;
-    const int ti = (c.in_dtype == TURNOPD_BF16 ? 0 : 1) + (large ? 2 : 0) + (c.grad ? 4 : 0);
-    static const Kern kerns[8] = {
-        k_topk_rows<true, kTkSelSmall, false>, k_topk_rows<false, kTkSelSmall, false>,
-        k_topk_rows<true, kTkSelLarge, false>, k_topk_rows<false, kTkSelLarge, false>,
-        k_topk_rows<true, kTkSelSmall, true>,  k_topk_rows<false, kTkSelSmall, true>,
-        k_topk_rows<true, kTkSelLarge, true>,  k_topk_rows<false, kTkSelLarge, true>};
-    if ((e = launch(kerns[ti], ti, kTkStreamThreads + 32 * (large ? kTkSelLarge : kTkSelSmall),
+    // four selector warps above K = 96.  fp32 rows above 131,072 ids without a dense row keep two for
+    // K = 289-448: their bound walks the row's buckets, which the streaming warps do faster with 72
+    // registers than with 64 (us of a step of 2e8 logits, two and four: V = 151,936, K = 290 222 and
+    // 238, 320 224 and 238, 384 233 and 247, 448 247 and 251; 128,256, K = 320 238 and 238).
+    const bool walk = !bf16 && !c.grad && c.K > 288 && c.K <= 448 && c.vocab > 131072;
+    const bool large = c.K > kTkLaneBoundMaxK && !walk;
+    const DenseRow dn = !c.grad ? kNoDense
+                        : !bf16 && c.vocab > 14336 && c.vocab <= 65536 ? kZerosByStream : kZerosBySelectors;
+    const int ti = (bf16 ? 0 : 1) + (large ? 2 : 0);
+    static const Kern kerns[4][3] = {
+        {k_topk_rows<true, kTkSelSmall, kNoDense>, k_topk_rows<true, kTkSelSmall, kZerosBySelectors>, nullptr},
+        {k_topk_rows<false, kTkSelSmall, kNoDense>, k_topk_rows<false, kTkSelSmall, kZerosBySelectors>,
+         k_topk_rows<false, kTkSelSmall, kZerosByStream>},
+        {k_topk_rows<true, kTkSelLarge, kNoDense>, k_topk_rows<true, kTkSelLarge, kZerosBySelectors>, nullptr},
+        {k_topk_rows<false, kTkSelLarge, kNoDense>, k_topk_rows<false, kTkSelLarge, kZerosBySelectors>,
+         k_topk_rows<false, kTkSelLarge, kZerosByStream>}};
+    if ((e = launch(kerns[ti][dn], ti * 3 + dn, kTkStreamThreads + 32 * (large ? kTkSelLarge : kTkSelSmall),
                     topk_smem_bytes(c.vocab, c.K))) != cudaSuccess)
         return e;
     launch_loss_sum(ws.row_wl, ws.nvalid, c.loss, c.status, stream);

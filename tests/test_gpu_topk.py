@@ -327,3 +327,32 @@ def test_aligned_rows_at_the_selection_lines(P, oracle, V, K):
     ids, gk, tl, loss, st = run_topk(P, zs, zt, V, mask, w, K)
     assert st == 0
     check_against_oracle(oracle, zs, zt, V, mask, w, K, ids, gk, tl, loss)
+
+
+@pytest.mark.parametrize("V,K,dense", [(131072, 320, False), (131088, 288, False), (131088, 289, False),
+                                       (131088, 448, False), (131088, 449, False), (131088, 320, True),
+                                       (14336, 50, True), (14352, 50, True), (14352, 128, True), (65536, 128, True),
+                                       (65552, 50, True), (65552, 128, True)])
+def test_fp32_rows_at_the_streaming_lines(P, oracle, V, K, dense):
+    """fp32 rows on both sides of the lines between two and four selector warps, and between a dense
+    row's zeros by the selector and by the streaming warps; more rows than CTAs at the short ones, so
+    that a CTA's buffers come round."""
+    T = 700 if V < 20000 else 12
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(V + K)
+    zt = torch.randn((T, V), generator=gen, device="cuda") * 3
+    zs = zt + torch.randn((T, V), generator=gen, device="cuda")
+    zt[1] = 1.5
+    mask = torch.ones(T, dtype=torch.uint8, device="cuda")
+    mask[5] = 0
+    w = torch.rand(T, generator=gen, device="cuda")
+    d = torch.full((T, V), 6.0, dtype=torch.float32, device="cuda") if dense else None
+    ids, gk, tl, loss, st = run_topk(P, zs, zt, V, mask, w, K, dense=d)
+    assert st == 0
+    sub = np.arange(0, T, 7) if T > 12 else None
+    check_against_oracle(oracle, zs, zt, V, mask, w, K, ids, gk, tl, loss, subset=sub)
+    if dense:
+        want = torch.zeros((T, V), dtype=torch.float32, device="cuda")
+        want.scatter_(1, torch.from_numpy(ids).cuda().long().clamp(min=0), torch.from_numpy(gk).cuda())
+        want[5] = 6.0
+        assert torch.equal(d, want)
