@@ -1047,10 +1047,12 @@ __device__ __forceinline__ void short_kl(const TopkArgs &a, const int4 &m, int j
 
 // Candidates a short row's CTA holds: the K selected and the ties of the last bucket.
 __host__ __device__ constexpr int short_cap(int K) { return K <= 128 ? 256 : K <= 256 ? 512 : K <= 512 ? 1024 : 2048; }
-__host__ __device__ __forceinline__ size_t short_smem(int K)
+// Ids it lists: where the last bucket holds more than the candidates, the K-th key is found among
+// these.  (One-warp CTAs, 32 on an SM, keep the shared memory for the cache.)
+__host__ __device__ constexpr int short_list(int K, int nt) { return nt == 32 || K > 512 ? short_cap(K) : 1024; }
+__host__ __device__ __forceinline__ size_t short_smem(int K, int nt)
 {
-    return (sizeof(uint64_t) + sizeof(float) + sizeof(int32_t)) * (size_t)short_cap(K) +
-           (sizeof(uint64_t) + sizeof(float)) * (size_t)K + 16;
+    return (sizeof(uint64_t) + sizeof(float)) * (size_t)(short_cap(K) + K) + sizeof(int32_t) * (size_t)short_list(K, nt) + 16;
 }
 constexpr int kShortPerThread = 64;  // elements of a row per thread
 // Aligned rows up to here take the kernel below: what 128 threads hold, 256 from K = 64.
@@ -1061,6 +1063,86 @@ constexpr int kShortPerThread = 64;  // elements of a row per thread
 // fp32 rows cross at the same places.  Rows that are not 16-byte aligned, which k_topk_rows reads
 // element by element, take it at every length it holds (32,700, K = 50: 1,248 GB/s and 448).
 int short_max_vocab(int K) { return kShortPerThread * (K < 64 ? 128 : 256) - 7; }
+
+template <bool BF16>
+__device__ __forceinline__ uint64_t row_key(const char *zt_row, int id)
+{
+    return mkkey(elem_ord<BF16>(zt_row, id), (uint32_t)id);
+}
+
+// The K elements of largest key among `total` ids (listed in ids, or all of a row's), in any order,
+// into key and cz: radix select of the K-th key, a byte a pass (ids are below 65,536, so ~id's upper
+// bytes are all ones), then every key at or above it.  Lanes of equal digit add up before the
+// histogram, which a row of equal logits would serialise.  For rows with more ties than a short row's
+// CTA holds, fewer than K finite logits, or a NaN.  (Bit by bit over the whole row, 48 or 64
+// passes, before.  us of a step of 1e8 logits, K = 50: fp32 V = 4,096 with 1,000 added to every logit
+// 3,604 and 418, with multiples of 3 3,395 and 464; bf16 8,176, multiples of 3, 1,809 and 247.)
+template <bool BF16, int NT>
+__device__ __forceinline__ void short_ties(const char *zt_row, const char *zs_row, const int32_t *ids, int total, int K,
+                                           uint64_t *key, float *cz, int *n)
+{
+    static_assert(sizeof(SelScratch) <= 256 * sizeof(uint64_t), "key is free until the keys are collected");
+    SelScratch &sc = *reinterpret_cast<SelScratch *>(key);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    auto sync = [&]() {
+        if (NT == 32)
+            __syncwarp();
+        else
+            __syncthreads();
+    };
+    uint64_t prefix = 0xFFFF0000ull, mask = 0xFFFF0000ull;
+    int need = K;
+    for (int byte = BF16 ? 5 : 7; byte >= 0; byte -= byte == 4 ? 3 : 1) {
+        for (int i = tid; i < 256; i += NT)
+            sc.hist[i] = 0;
+        sync();
+        for (int i0 = warp * 32; i0 < total; i0 += NT) {
+            const int i = i0 + lane;
+            uint32_t digit = 256;
+            if (i < total) {
+                const uint64_t k = row_key<BF16>(zt_row, ids ? ids[i] : i);
+                if ((k & mask) == (prefix & mask))
+                    digit = (uint32_t)(k >> (8 * byte)) & 255u;
+            }
+            const unsigned same = __match_any_sync(0xffffffffu, digit);
+            if (digit < 256 && lane == __ffs(same) - 1)
+                atomicAdd(&sc.hist[digit], (uint32_t)__popc(same));
+        }
+        sync();
+        if (warp == 0)
+            pick_bin(sc, need, lane);
+        sync();
+        const int bin = sc.bin, nd = sc.need;
+        sync();
+        prefix |= (uint64_t)bin << (8 * byte);
+        mask |= 255ull << (8 * byte);
+        if (nd < 0)  // every key of this prefix is among the K
+            break;
+        need = nd;
+    }
+    if (tid == 0)
+        *n = 0;
+    sync();
+    for (int i = tid; i < total; i += NT) {
+        const int id = ids ? ids[i] : i;
+        const uint64_t k = row_key<BF16>(zt_row, id);
+        if (k >= prefix) {
+            const int p = atomicAdd(n, 1);
+            key[p] = k;
+            cz[p] = BF16 ? __bfloat162float(reinterpret_cast<const __nv_bfloat16 *>(zs_row)[id])
+                         : reinterpret_cast<const float *>(zs_row)[id];
+        }
+    }
+}
+
+// The same as a call, for the one-warp CTA, whose registers are all in use (inlined there it cost the
+// ordinary rows 2-6 %, as a call in the larger CTAs 8-12 %).
+template <bool BF16>
+__device__ __noinline__ void short_ties_call(const char *zt_row, const char *zs_row, const int32_t *ids, int total,
+                                             int K, uint64_t *key, float *cz, int *n)
+{
+    short_ties<BF16, 32>(zt_row, zs_row, ids, total, K, key, cz, n);
+}
 
 // Rows of up to 64 NT elements, one CTA of NT threads a row, any alignment: the row's
 // 16-bit buckets (the logit itself for bf16) stay in registers, 2 to a word, from the only
@@ -1080,12 +1162,12 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_topk_short(TopkArgs a)
     constexpr int NW = NT / 32;
     constexpr int ESZ = BF16 ? 2 : 4;
     extern __shared__ __align__(128) uint64_t tk_smem[];
-    const int K = a.K, cap = short_cap(K);
+    const int K = a.K, cap = short_cap(K), listed = short_list(K, NT);
     uint64_t *s_key = tk_smem;                                 // [cap] candidates
     uint64_t *s_top = s_key + cap;                             // [K] selected
     float *s_cz = reinterpret_cast<float *>(s_top + K);        // [cap] their student logits
     float *s_g = s_cz + cap;                                   // [K]
-    int32_t *s_id = reinterpret_cast<int32_t *>(s_g + K);      // [cap]
+    int32_t *s_id = reinterpret_cast<int32_t *>(s_g + K);      // [listed]
     __shared__ int s_cnt[2][NW];
     __shared__ float s_max[NW];
     __shared__ int s_n;
@@ -1222,16 +1304,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_topk_short(TopkArgs a)
             }
             par ^= 1;
         }
-        auto full_key = [&](int id) {
-            const uint32_t o = BF16 ? ord16(reinterpret_cast<const uint16_t *>(zt_row)[id])
-                                    : ord32(reinterpret_cast<const uint32_t *>(zt_row)[id]);
-            return mkkey(o, (uint32_t)id);
-        };
-        auto student = [&](int id) {
-            return BF16 ? __bfloat162float(reinterpret_cast<const __nv_bfloat16 *>(zs_row)[id])
-                        : reinterpret_cast<const float *>(zs_row)[id];
-        };
-        if (n <= cap && n >= K && top == top) {
+        if (n <= listed && n >= K && top == top) {
             const uint32_t below = (1u << lane) - 1u;
 #pragma unroll
             for (int k = 0; k < kShortPerThread / 2; ++k) {
@@ -1249,34 +1322,21 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_topk_short(TopkArgs a)
                 }
             }
             sync();
-            for (int i = tid; i < n; i += NT) {
-                const int id = s_id[i];
-                s_key[i] = full_key(id);
-                s_cz[i] = student(id);
-            }
-        } else {
-            // more ties than the buffer holds (rows of many equal logits), fewer than K finite
-            // logits, or a NaN: the K-th largest full key, bit by bit, then exactly K elements
-            uint64_t kth = 0;
-            for (int bit = BF16 ? 47 : 63; bit >= 0; --bit) {
-                const uint64_t x = kth | 1ull << bit;
-                int c = 0;
-                for (int id = tid; id < V; id += NT)
-                    c += full_key(id) >= x;
-                if (block_count(c) >= K)
-                    kth = x;
-            }
-            if (tid == 0)
-                s_n = 0;
-            sync();
-            for (int id = tid; id < V; id += NT) {
-                const uint64_t k = full_key(id);
-                if (k >= kth) {
-                    const int p = atomicAdd(&s_n, 1);
-                    s_key[p] = k;
-                    s_cz[p] = student(id);
+            if (n <= cap)
+                for (int i = tid; i < n; i += NT) {
+                    const int id = s_id[i];
+                    s_key[i] = row_key<BF16>(zt_row, id);
+                    s_cz[i] = BF16 ? __bfloat162float(reinterpret_cast<const __nv_bfloat16 *>(zs_row)[id])
+                                   : reinterpret_cast<const float *>(zs_row)[id];
                 }
-            }
+        }
+        if (n > cap || n < K || top != top) {
+            const bool from_list = n <= listed && n >= K && top == top;
+            const int32_t *ids = from_list ? s_id : nullptr;
+            if (NT == 32)
+                short_ties_call<BF16>(zt_row, zs_row, ids, from_list ? n : V, K, s_key, s_cz, &s_n);
+            else
+                short_ties<BF16, NT>(zt_row, zs_row, ids, from_list ? n : V, K, s_key, s_cz, &s_n);
             n = K;
         }
         if (tid == 0 && (n & 1))
@@ -1389,7 +1449,7 @@ cudaError_t launch_topk(const TopkCall &c, cudaStream_t stream)
             {k_topk_short<false, 32>, k_topk_short<false, 128>, k_topk_short<false, 256>, k_topk_short<false, 512>},
             {k_topk_short<true, 32>, k_topk_short<true, 128>, k_topk_short<true, 256>, k_topk_short<true, 512>}};
         static const int threads[4] = {32, 128, 256, 512};
-        if ((e = launch(shorts[bf16][s4], 12 + bf16 * 4 + s4, threads[s4], short_smem(c.K))) != cudaSuccess)
+        if ((e = launch(shorts[bf16][s4], 12 + bf16 * 4 + s4, threads[s4], short_smem(c.K, threads[s4]))) != cudaSuccess)
             return e;
         launch_loss_sum(ws.row_wl, ws.nvalid, c.loss, c.status, stream);
         return cudaGetLastError();

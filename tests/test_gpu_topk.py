@@ -356,3 +356,43 @@ def test_fp32_rows_at_the_streaming_lines(P, oracle, V, K, dense):
         want.scatter_(1, torch.from_numpy(ids).cuda().long().clamp(min=0), torch.from_numpy(gk).cuda())
         want[5] = 6.0
         assert torch.equal(d, want)
+
+
+@pytest.mark.parametrize("V,ld,K,threads", [(64, 64, 8, 32), (2042, 2042, 8, 128), (8186, 8187, 64, 256),
+                                            (16378, 16379, 20, 512)])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_short_rows_many_to_a_cta(P, oracle, V, ld, K, threads, dtype):
+    """Three rounds and more of the CTAs that an SM holds (32 of 32 threads, 1,024 threads' worth of
+    the larger ones), so that a CTA takes several rows, their kinds in a varying order: ordinary,
+    all equal, two thirds equal, more ties than the candidates or the list hold, masked by the
+    lowest value, and rows without loss.  What a row leaves behind must not enter the next."""
+    T = 152 * (32 if threads == 32 else 1024 // threads) * 3 + 77
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(V)
+    zs = torch.empty((T, ld), dtype=dtype, device="cuda")
+    zt = torch.empty((T, ld), dtype=dtype, device="cuda")
+    kind = torch.randint(7, (T,), generator=gen, device="cuda")
+    for r in range(0, T, 512):
+        n = min(512, T - r)
+        t = torch.randn((n, ld), generator=gen, device="cuda") * 3
+        k = kind[r:r + n, None]
+        s = 0.2 * t + 0.3 * torch.randn((n, ld), generator=gen, device="cuda")  # no token near p = 1, where g cancels
+        zs[r:r + n] = torch.where(k == 4, s + 1000.0, s).to(dtype)
+        col = torch.arange(ld, device="cuda")[None]
+        t = torch.where(k == 1, 1.5, t)
+        t = torch.where((k == 2) & (col >= V // 3), 4.25, t)
+        t = torch.where((k == 3) & (col % 8 == 5), 9.0, t)          # an eighth of the ids tied at the top
+        t = torch.where(k == 4, t + 1000.0, t)                      # few distinct leading bits
+        t = torch.where((k == 5) & (col >= K + 9), torch.finfo(dtype).min, t)
+        zt[r:r + n] = t.to(dtype)
+    mask = (torch.rand(T, generator=gen, device="cuda") < 0.9).to(torch.uint8)
+    w = torch.rand(T, generator=gen, device="cuda")
+    dense = torch.full((T, ld), 6.0, dtype=torch.float32, device="cuda")
+    ids, gk, tl, loss, st = run_topk(P, zs, zt, V, mask, w, K, dense=dense)
+    assert st == 0
+    check_against_oracle(oracle, zs, zt, V, mask, w, K, ids, gk, tl, loss)
+    m = mask.bool()
+    want = torch.zeros((T, ld), dtype=torch.float32, device="cuda")
+    want.scatter_(1, torch.from_numpy(ids).cuda().long().clamp(min=0), torch.from_numpy(gk).cuda())
+    assert torch.equal(dense[m][:, :V], want[m][:, :V])
+    assert (dense[~m] == 6.0).all() and (dense[:, V:] == 6.0).all()
