@@ -291,23 +291,21 @@ __device__ __forceinline__ int count_ge2(uint32_t x, uint32_t m)
     return (int)((x & 0xFFFFu) >= m) + (int)((x >> 16) >= m);
 }
 
-// Sorts keys[0, n) (n a power of two >= 2 kTkSelThreads, distinct keys but for 0
-// padding) in descending order: bitonic network over the selector threads, each
-// thread loading U pairs before it compares and stores any, synchronised on
-// kBarSel after every step.
-template <int U, int SW>
-__device__ void sort_desc(uint64_t *keys, int n, int stid)
+// Sorts keys[0, n) (n a power of two, distinct keys but for 0 padding) in
+// descending order: bitonic network over NT threads, each thread loading U pairs
+// before it compares and stores any, synchronised by sync() after every step.
+template <int U, int NT, class Sync>
+__device__ __forceinline__ void sort_desc(uint64_t *keys, int n, int tid, Sync &&sync)
 {
-    constexpr int kTkSelThreads = 32 * SW;
     const int np = n / 2;  // pairs per step
     for (int k = 2; k <= n; k <<= 1)
         for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int i0 = stid; i0 < np; i0 += U * kTkSelThreads) {
+            for (int i0 = tid; i0 < np; i0 += U * NT) {
                 uint64_t x[U], y[U];
                 int l[U];
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
-                    const int i = i0 + u * kTkSelThreads;
+                    const int i = i0 + u * NT;
                     l[u] = 2 * i - (i & (j - 1));
                     if (i < np) {
                         x[u] = keys[l[u]];
@@ -318,13 +316,13 @@ __device__ void sort_desc(uint64_t *keys, int n, int stid)
                 for (int u = 0; u < U; ++u) {
                     // blocks with (l & k) == 0 descending, the others ascending; the last merge
                     // (k = n) is descending throughout
-                    if (i0 + u * kTkSelThreads < np && (x[u] < y[u]) == ((l[u] & k) == 0)) {
+                    if (i0 + u * NT < np && (x[u] < y[u]) == ((l[u] & k) == 0)) {
                         keys[l[u]] = y[u];
                         keys[l[u] + j] = x[u];
                     }
                 }
             }
-            named_sync(kBarSel, kTkSelThreads);
+            sync();
         }
 }
 
@@ -886,7 +884,7 @@ __global__ void __launch_bounds__(kTkStreamThreads + 32 * SW, kTkMinBlocks) k_to
                     s_cand[i] = i < nc ? (k & 0xFFFFFFFF00000000ull) | ((k & 0xFFFFFull) << 11) | (uint64_t)i : 0ull;
                 }
                 named_sync(kBarSel, kTkSelThreads);
-                sort_desc<BF16 ? 4 : 2, SW>(s_cand, n2, stid);
+                sort_desc<BF16 ? 4 : 2, kTkSelThreads>(s_cand, n2, stid, [&]() { named_sync(kBarSel, kTkSelThreads); });
                 for (int r = stid; r < K; r += kTkSelThreads) {
                     const uint64_t p = s_cand[r];
                     s_top[r] = (p & 0xFFFFFFFF00000000ull) | 0xFFF00000ull | ((p >> 11) & 0xFFFFFull);
@@ -1144,6 +1142,33 @@ __device__ __noinline__ void short_ties_call(const char *zt_row, const char *zs_
     short_ties<BF16, 32>(zt_row, zs_row, ids, total, K, key, cz, n);
 }
 
+// The K largest of n candidates (a power of two above n fits the buffer) in order: a bitonic sort, as in
+// k_topk_rows, each key carrying its buffer position below the id's 20 bits.
+template <int NT>
+__device__ __forceinline__ void short_sort(uint64_t *key, const float *cz, int n, int K, uint64_t *top, float *g)
+{
+    const int tid = threadIdx.x;
+    auto sync = [&]() {
+        if (NT == 32)
+            __syncwarp();
+        else
+            __syncthreads();
+    };
+    int n2 = 512;
+    while (n2 < n)
+        n2 <<= 1;
+    for (int i = tid; i < n2; i += NT) {
+        const uint64_t k = key[i];
+        key[i] = i < n ? (k & 0xFFFFFFFF00000000ull) | ((k & 0xFFFFFull) << 11) | (uint64_t)i : 0ull;
+    }
+    sync();
+    sort_desc<2, NT>(key, n2, tid, sync);
+    for (int r = tid; r < K; r += NT) {
+        const uint64_t p = key[r];
+        top[r] = (p & 0xFFFFFFFF00000000ull) | 0xFFF00000ull | ((p >> 11) & 0xFFFFFull);
+        g[r] = cz[p & 0x7FFu];
+    }
+}
 // Rows of up to 64 NT elements, one CTA of NT threads a row, any alignment: the row's
 // 16-bit buckets (the logit itself for bf16) stay in registers, 2 to a word, from the only
 // read of the teacher.  The K-th largest bucket comes from a binary search on its value, a
@@ -1155,7 +1180,13 @@ __device__ __noinline__ void short_ties_call(const char *zt_row, const char *zs_
 // instructions a row of 2,034 at K = 50, IPC 1.9).  GB/s of the step at 4e8 logits, bf16, in
 // k_topk_rows and here: K = 50, V = 1,024 47 and 653, 2,034 47 and 988, 4,096 437 and 788;
 // K = 256 82 and 265, 65 and 368, 101 and 463.
-template <bool BF16, int NT>
+// SORT: the candidates are sorted, for K from 320 (kShortSortK), where ranks, whose cost grows with the
+// square, take longer (us of a step of 1e8 bf16 logits, ranks and sort: V = 1,040, K = 320 2,950 and
+// 2,154, 1,024 34,733 and 7,752; 4,096, K = 512 1,381 and 986, 1,024 4,790 and 2,149; 12,288, K = 256 319
+// and 361, 288 346 and 369, 320 367 and 371).  Kernels of their own: in one, the sort's registers cost
+// the other rows 4-8 %.
+constexpr int kShortSortK = 320;
+template <bool BF16, int NT, bool SORT>
 __global__ void __launch_bounds__(NT, 1024 / NT) k_topk_short(TopkArgs a)
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -1339,22 +1370,27 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_topk_short(TopkArgs a)
                 short_ties<BF16, NT>(zt_row, zs_row, ids, from_list ? n : V, K, s_key, s_cz, &s_n);
             n = K;
         }
-        if (tid == 0 && (n & 1))
-            s_key[n] = 0;  // the last pair's second key
-        sync();
-        // each candidate's rank among the candidates is its position
-        const ulonglong2 *pairs = reinterpret_cast<const ulonglong2 *>(s_key);
-        for (int i = tid; i < n; i += NT) {
-            const uint64_t k = s_key[i];
-            int rank = 0;
+        if (SORT) {
+            sync();
+            short_sort<NT>(s_key, s_cz, n, K, s_top, s_g);
+        } else {
+            if (tid == 0 && (n & 1))
+                s_key[n] = 0;  // the last pair's second key
+            sync();
+            // each candidate's rank among the candidates is its position
+            const ulonglong2 *pairs = reinterpret_cast<const ulonglong2 *>(s_key);
+            for (int i = tid; i < n; i += NT) {
+                const uint64_t k = s_key[i];
+                int rank = 0;
 #pragma unroll 4
-            for (int q = 0; q < (n + 1) / 2; ++q) {
-                const ulonglong2 x = pairs[q];
-                rank += (int)(x.x > k) + (int)(x.y > k);
-            }
-            if (rank < K) {
-                s_top[rank] = k;
-                s_g[rank] = s_cz[i];
+                for (int q = 0; q < (n + 1) / 2; ++q) {
+                    const ulonglong2 x = pairs[q];
+                    rank += (int)(x.x > k) + (int)(x.y > k);
+                }
+                if (rank < K) {
+                    s_top[rank] = k;
+                    s_g[rank] = s_cz[i];
+                }
             }
         }
         sync();
@@ -1421,7 +1457,7 @@ cudaError_t launch_topk(const TopkCall &c, cudaStream_t stream)
     if ((e = cudaGetDevice(&dev)) != cudaSuccess)
         return e;
     using Kern = void (*)(TopkArgs);
-    static size_t attr_smem[64][20] = {};
+    static size_t attr_smem[64][28] = {};
     const int di = dev < 64 ? dev : 0;
     auto launch = [&](Kern kern, int slot, int threads, size_t smem) {
         cudaError_t e = cudaSuccess;
@@ -1445,11 +1481,18 @@ cudaError_t launch_topk(const TopkCall &c, cudaStream_t stream)
     const bool aligned = ((reinterpret_cast<uintptr_t>(c.zt) | reinterpret_cast<uintptr_t>(c.zs) | (uintptr_t)(c.ld * esz)) & 15u) == 0;
     if (span <= (int64_t)kShortPerThread * 512 && (!aligned || c.vocab <= short_max_vocab(c.K))) {
         const int s4 = span <= kShortPerThread * 32 ? 0 : span <= kShortPerThread * 128 ? 1 : span <= kShortPerThread * 256 ? 2 : 3;
-        static const Kern shorts[2][4] = {
-            {k_topk_short<false, 32>, k_topk_short<false, 128>, k_topk_short<false, 256>, k_topk_short<false, 512>},
-            {k_topk_short<true, 32>, k_topk_short<true, 128>, k_topk_short<true, 256>, k_topk_short<true, 512>}};
+        static const Kern shorts[2][2][4] = {
+            {{k_topk_short<false, 32, false>, k_topk_short<false, 128, false>, k_topk_short<false, 256, false>,
+              k_topk_short<false, 512, false>},
+             {k_topk_short<true, 32, false>, k_topk_short<true, 128, false>, k_topk_short<true, 256, false>,
+              k_topk_short<true, 512, false>}},
+            {{k_topk_short<false, 32, true>, k_topk_short<false, 128, true>, k_topk_short<false, 256, true>,
+              k_topk_short<false, 512, true>},
+             {k_topk_short<true, 32, true>, k_topk_short<true, 128, true>, k_topk_short<true, 256, true>,
+              k_topk_short<true, 512, true>}}};
+        const int sort = c.K >= kShortSortK;
         static const int threads[4] = {32, 128, 256, 512};
-        if ((e = launch(shorts[bf16][s4], 12 + bf16 * 4 + s4, threads[s4], short_smem(c.K, threads[s4]))) != cudaSuccess)
+        if ((e = launch(shorts[sort][bf16][s4], 12 + sort * 8 + bf16 * 4 + s4, threads[s4], short_smem(c.K, threads[s4]))) != cudaSuccess)
             return e;
         launch_loss_sum(ws.row_wl, ws.nvalid, c.loss, c.status, stream);
         return cudaGetLastError();

@@ -358,8 +358,8 @@ def test_fp32_rows_at_the_streaming_lines(P, oracle, V, K, dense):
         assert torch.equal(d, want)
 
 
-@pytest.mark.parametrize("V,ld,K,threads", [(64, 64, 8, 32), (2042, 2042, 8, 128), (8186, 8187, 64, 256),
-                                            (16378, 16379, 20, 512)])
+@pytest.mark.parametrize("V,ld,K,threads", [(64, 64, 8, 32), (1040, 1041, 1024, 32), (2042, 2042, 8, 128),
+                                            (2042, 2042, 320, 128), (8186, 8187, 64, 256), (16378, 16379, 20, 512)])
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
 def test_short_rows_many_to_a_cta(P, oracle, V, ld, K, threads, dtype):
     """Three rounds and more of the CTAs that an SM holds (32 of 32 threads, 1,024 threads' worth of
