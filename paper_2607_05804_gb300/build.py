@@ -23,7 +23,7 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-ffp-contract=off",
          "--expt-relaxed-constexpr",
          "-Xptxas", "-warn-spills"]
-# Extra nvcc flags (e.g. tuning macros such as -DTURNOPD_ROW_THREADS=384) for experiments.
+# Extra nvcc flags (e.g. tuning macros such as -DTURNOPD_TOPK_MINB=1) for experiments.
 EXTRA = os.environ.get("TURNOPD_NVCC_FLAGS", "").split()
 
 

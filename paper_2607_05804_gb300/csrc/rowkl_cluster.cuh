@@ -807,12 +807,11 @@ constexpr int kHelpU = 4;  // vectors of each model per thread and batch
 // 2.743 ms per loss call with the split rate raised to 0.7); the helper alone on every
 // SM keeps the register path (V = 16,384: 0.405 against 0.433 ms).
 constexpr int kHelpStages = 3;
-constexpr size_t helper_smem_bytes(bool as, int nth) { return as ? (size_t)kHelpStages * 2 * kHelpU * nth * 16 : 0; }
+constexpr size_t kHelperSmem = (size_t)kHelpStages * 2 * kHelpU * kHelpThreads * 16;  // AS
 
-template <typename T, bool G32, bool SM, int TL, bool AS, int NTH = kHelpThreads, int MINB = 1>
-__global__ void __launch_bounds__(NTH, MINB) k_row_helper(RowIn p)
+template <typename T, bool G32, bool SM, int TL, bool AS>
+__global__ void __launch_bounds__(kHelpThreads, 1) k_row_helper(RowIn p)
 {
-    constexpr int kHelpThreads = NTH;
     constexpr int NW = kHelpThreads / 32;
     using E = Elem<T>;
     constexpr int N = E::N, NP = E::NP;
@@ -820,7 +819,7 @@ __global__ void __launch_bounds__(NTH, MINB) k_row_helper(RowIn p)
     constexpr bool kUseD = G32 || N == 4 || (TL == kAny && !SM), kGradD = G32 || TL == kAny, kScale = kGradD && N == 4;  // as in the cluster kernel
     __shared__ float red[NW][8];
     __shared__ float bc[8];
-    extern __shared__ uint4 hring[];  // [kHelpStages][2][kHelpU][NTH] (AS)
+    extern __shared__ uint4 hring[];  // [kHelpStages][2][kHelpU][kHelpThreads] (AS)
     // the loss sum after this grid may take the first SM it frees (it waits for the grid)
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1265,11 +1264,11 @@ cudaError_t launch_t(const RowIn &p, int nvec, cudaStream_t stream, bool *used)
     hc.numAttrs = 1;
     hc.gridDim = dim3(free_sm);
     hc.blockDim = dim3(kHelpThreads);
-    hc.dynamicSmemBytes = helper_smem_bytes(true, kHelpThreads);
+    hc.dynamicSmemBytes = kHelperSmem;
     hc.stream = stream;
     auto helper = k_row_helper<T, G32, SM, TL, true>;
     if ((e = cudaFuncSetAttribute(helper, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)helper_smem_bytes(true, kHelpThreads))) != cudaSuccess)
+                                  (int)kHelperSmem)) != cudaSuccess)
         return e;
     return cudaLaunchKernelEx(&hc, helper, pl);
 }
