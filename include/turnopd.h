@@ -178,7 +178,7 @@ size_t turnopd_weights_workspace_bytes(int32_t num_traj, int32_t max_turns);
  *     cluster of 2 to 16 (the smallest whose slices fit) beside a helper grid on
  *     the remaining SMs; where vocab or ld is not a multiple of a 16-byte vector,
  *     a row's first and last vectors are masked;
- *   rows longer than a cluster of 16 holds (152,576 fp32 columns, 305,152 bf16
+ *   rows longer than a cluster of 16 holds (152,640 fp32 columns, 305,280 bf16
  *     ones): fp32 with vocab and ld multiples of 4 on clusters of 8 CTAs (4 for
  *     sampled-token rows) that stream each row twice, beside a helper grid, the
  *     first read of each chunk marked L2 evict-last and its lines returned to

@@ -1088,22 +1088,35 @@ __global__ void __launch_bounds__(kHelpThreads, 1) k_row_helper(RowIn p)
 // 8,192, ShapeMid 5,960 at 12,288, where ShapeBig gives 5,380; rows held in no shape (one
 // 256- or 512-thread CTA a row, the second read from L2) reached 820, 1,350, 2,380,
 // 3,920 and 3,930, and fp32 rows on clusters of 8 (k_row_split) 186, 370, 736 and 1,370.
-struct ShapeBig { static constexpr int NT = 512, G = 2, VPT = 5, ST = 3, kMax = 2384; };
+struct ShapeBig { static constexpr int NT = 512, G = 2, VPT = 5, ST = 3, kMax = 2405; };  // less in clusters
 struct ShapeMid { static constexpr int NT = 320, G = 3, VPT = 6, ST = 4, kMax = 1780; };
 struct Shape4 { static constexpr int NT = 256, G = 4, VPT = 5, ST = 5, kMax = 1280; };
 struct Shape8 { static constexpr int NT = 128, G = 8, VPT = 5, ST = 10, kMax = 640; };
 struct Shape12 { static constexpr int NT = 64, G = 12, VPT = 5, ST = 20, kMax = 320; };
 struct Shape32 { static constexpr int NT = 32, G = 32, VPT = 5, ST = 40, kMax = 160; };
 
+template <class Shape> constexpr size_t cluster_smem_bytes(int slice_vec, int cs)
+{
+    constexpr int ST = Shape::ST, G = Shape::G;
+    return (size_t)ST * 2 * slice_vec * 16 + 2 * G * cs * 8 * sizeof(float) +
+           ST * sizeof(int4) + (2 * ST + 2 * G) * sizeof(uint64_t) +
+           G * (Shape::NT / 32) * 8 * sizeof(float) +  // per-group warp partials
+           2 * ((ST + 3) / 4 * 4) * sizeof(int) +                       // row held by each stage, thread reading y
+           G * 16 * sizeof(float);                      // broadcast row constants
+}
+// of the 227 KB a CTA may have, less the static part and alignment
+constexpr size_t kMaxClusterSmem = 232448 - 128;
+
 // Cluster size for rows of nvec vectors: the smallest whose slices a CTA holds (0: none).
 // That keeps the slices long (a short slice cannot hide the per-row record exchange) and,
 // for short rows, puts more SMs in clusters: every SM for 1 and 2, then 36 clusters of 4
-// are co-resident, 28 of 5, 23 of 6, 15 of 8, 7 of 16.  7 is left out (only 15).
+// are co-resident, 28 of 5, 23 of 6, 15 of 8, 7 of 16.  7 is left out (only 15).  A CTA holds 2,405
+// vectors alone, 2,403 in a cluster of 2, 2,395 of 8 and 2,385 of 16, whose records take more.
 inline int cluster_size(int nvec)
 {
     static const int kSizes[] = {1, 2, 3, 4, 5, 6, 8, 16};
     for (int c : kSizes)
-        if ((nvec + c - 1) / c <= ShapeBig::kMax)
+        if (cluster_smem_bytes<ShapeBig>((nvec + c - 1) / c, c) <= kMaxClusterSmem)
             return c;
     return 0;
 }
@@ -1122,7 +1135,8 @@ inline int cluster_size(int nvec)
 //   0.8), 0.84 at 2,048 (262,144: 603, 616 at 0.75), 0.65 at 2,344 (300,000: 605, 685 at 0.8), with
 //   an fp32 gradient 0.85 (907, 958 at 0.65), 0.8 (826, 868 at 0.6) and 0.7 (825, 964 at 0.8); of 3 in ShapeMid 0.5 (39,000: 6,183, 5,222 at
 //   0.7); of 3 to 6 otherwise 0.7 (90,000: 6,335, 6,245 at 0.4), 0.62 with an fp32 gradient
-//   (49,152: 6,252 at 0.6, 5,978 at 0.7);
+//   (49,152: 6,252 at 0.6, 5,978 at 0.7), of 3 above 2,250 0.6 (57,408: 559 us at 6e8 logits, 590
+//   at 0.7);
 //   fp32, clusters of 16: 0.69 at 2,374 (151,936: 4 x 4096 packed tokens 2,808 us; 2,833 at
 //   0.65, 2,873 at 0.76), 0.80 at 2,048 (6,035, 5,823 at 0.6), 0.65 at 1,719 in ShapeMid
 //   (6,361 at 0.6, 6,186 at 0.7), 0.9 at 1,536 (6,203, 5,909 at 0.5), 0.7 at 1,204 in Shape4
@@ -1151,6 +1165,8 @@ double helper_rate(int slice_vec, int cs, bool sampled, bool g32, bool forward, 
     if (bf16) {
         if (cs == 3 && slice_vec <= ShapeMid::kMax)
             return 0.50;
+        if (cs == 3 && slice_vec > 2250)
+            return 0.60;
         if (cs < 8)
             return g32 ? 0.62 : cs <= 4 && !sectors && TL != kAny ? 0.63 : 0.70;
         if (cs == 8)
@@ -1174,16 +1190,6 @@ double helper_rate(int slice_vec, int cs, bool sampled, bool g32, bool forward, 
     }
     r = r < 0.60 ? 0.60 : r;
     return sampled ? r + (g32 ? 0.10 : 0.05) : r;
-}
-
-template <class Shape> size_t cluster_smem_bytes(int slice_vec, int cs)
-{
-    constexpr int ST = Shape::ST, G = Shape::G;
-    return (size_t)ST * 2 * slice_vec * 16 + 2 * G * cs * 8 * sizeof(float) +
-           ST * sizeof(int4) + (2 * ST + 2 * G) * sizeof(uint64_t) +
-           G * (Shape::NT / 32) * 8 * sizeof(float) +  // per-group warp partials
-           2 * ((ST + 3) / 4 * 4) * sizeof(int) +                       // row held by each stage, thread reading y
-           G * 16 * sizeof(float);                      // broadcast row constants
 }
 
 // The cluster grid (as many clusters as are co-resident, cached per device) and

@@ -322,7 +322,8 @@ def test_ragged_rows_bf16(P, oracle, V, ld, mode, gdt):
 
 # Longest rows of each shape of the held-row kernels, in 16-byte vectors of one CTA, and the
 # cluster sizes whose slices reach them: (vectors, cluster)
-SHAPE_EDGES = [(160, 1), (320, 1), (640, 1), (1280, 1), (1780, 1), (2384, 1), (1280, 2), (1780, 2), (1780, 3)]
+SHAPE_EDGES = [(160, 1), (320, 1), (640, 1), (1280, 1), (1780, 1), (2405, 1), (1280, 2), (1780, 2), (2403, 2), (1780, 3),
+               (2395, 8), (2385, 16)]
 
 
 @pytest.mark.parametrize("vec,cs", SHAPE_EDGES)
@@ -334,7 +335,7 @@ def test_held_row_shape_edges(P, oracle, vec, cs, step, idt):
     n = 8 if idt == "bf16" else 4
     V = n * cs * (vec + step)
     dt = torch.bfloat16 if idt == "bf16" else torch.float32
-    rows = 152 * 48 if vec <= 320 else 152 * 12 if vec <= 640 else 500
+    rows = 152 * 48 if vec <= 320 else 152 * 12 if vec <= 640 else 500 if cs < 8 else 120
     b = W.packed(seed=71, num_traj=2, traj_len=int(rows / 1.2))
     zs, zt = W.make_logits(b.num_valid, V, "agent", dt, seed=72, device="cuda")
     for mode in (0, 1):
