@@ -179,8 +179,8 @@ def test_paper_turn_floor_on_household(P, oracle):
 @pytest.mark.parametrize("mode", [0, 1], ids=["full", "sampled"])
 @pytest.mark.parametrize("gdt", ["bf16", "f32"])
 def test_cluster_kernel_all_rows(P, oracle, V, mode, gdt):
-    """The bf16 row path on every row (vocabulary a multiple of 8): V = 8,192 takes the
-    helper kernel alone, V = 32,000 clusters of 2 on every SM, V = 50,000 clusters of 3
+    """The bf16 row path on every row (vocabulary a multiple of 8): V = 8,192 takes one
+    CTA a row, V = 32,000 clusters of 2 on every SM, V = 50,000 clusters of 3
     beside the helper (ragged last slice), V = 151,936 clusters of 8 beside it, and
     V = 200,000 and 262,144 clusters of 16 beside it (200,000: slices of 1,563 vectors,
     the shortest the clusters of 16 take)."""
@@ -191,9 +191,10 @@ def test_cluster_kernel_all_rows(P, oracle, V, mode, gdt):
 
 
 @pytest.mark.parametrize("kernel,V,idt,flags", [
-    ("helper alone", 8192, "bf16", 0), ("clusters of 2", 32000, "bf16", 0),
-    ("clusters of 8 + helper", W.V_QWEN, "bf16", 0), ("split rows", 4100, "f32", 0),
-    ("split rows", W.V_QWEN, "f32", 0), ("portable", 4099, "bf16", FORCE_PORTABLE),
+    ("one CTA", 8192, "bf16", 0), ("clusters of 2", 32000, "bf16", 0),
+    ("clusters of 8 + helper", W.V_QWEN, "bf16", 0), ("one CTA", 4100, "f32", 0),
+    ("clusters of 16 + helper", W.V_QWEN, "f32", 0), ("split rows + helper", 160004, "f32", 0),
+    ("portable", 4099, "bf16", FORCE_PORTABLE),
     ("portable", 4100, "f32", FORCE_PORTABLE)])
 @pytest.mark.parametrize("gdt", ["bf16", "f32"])
 def test_sampled_peaked_rows(P, oracle, kernel, V, idt, flags, gdt):
@@ -219,11 +220,10 @@ def test_sampled_peaked_rows(P, oracle, kernel, V, idt, flags, gdt):
 @pytest.mark.parametrize("V,ld", [(4100, 4100), (4100, 4104), (W.V_QWEN, W.V_QWEN), (262144, 262144)])
 @pytest.mark.parametrize("mode", [0, 1], ids=["full", "sampled"])
 @pytest.mark.parametrize("gdt", ["bf16", "f32"])
-def test_split_kernel_fp32_all_rows(P, oracle, V, ld, mode, gdt):
-    """fp32 logits through the split-row kernel on every row: clusters of 4 CTAs
-    share each row (ragged last slice at V = 4100, a ragged last chunk at
-    V = 151,936, whole chunks at 262,144), about 8 rows per cluster so the chunk
-    ring wraps across rows, and padding columns beyond V never read."""
+def test_fp32_all_rows(P, oracle, V, ld, mode, gdt):
+    """fp32 logits on every row: one CTA a row (V = 4,100, padding columns beyond V never
+    read), clusters of 16 (151,936), and the split-row kernel's clusters of 8 (4 for
+    sampled-token rows) at 262,144, whose chunk ring wraps across the rows of a cluster."""
     b = W.packed(seed=11, num_traj=2, traj_len=256)
     zs, zt = W.make_logits(b.num_valid, V, "agent", torch.float32, seed=12, device="cuda", ld=ld)
     _, grad = run_chain(P, oracle, b, V, zs, zt, mode=mode, alpha=0.5, compact=True,
@@ -253,7 +253,7 @@ def test_odd_vocabulary_full_size(P, oracle, ld, idt):
 @pytest.mark.parametrize("gdt", ["bf16", "f32"])
 def test_masked_tail_vocab(P, oracle, V, mode, gdt):
     """bf16 rows with V % 8 != 0 and the stride padded to a multiple of 8 take the row
-    grids with a masked last vector: V = 8,193 the helper alone, 32,007 clusters of 2,
+    grids with a masked last vector: V = 8,193 one CTA a row, 32,007 clusters of 2,
     50,005 clusters of 3 beside the helper, 151,937 and 151,943 clusters of 8 beside it.
     NaN and inf fill the padding; its gradient columns stay untouched.  In sampled mode
     every third row's y is pushed into the masked vector (its student logit 30 above the
@@ -279,8 +279,8 @@ def test_masked_tail_vocab(P, oracle, V, mode, gdt):
 @pytest.mark.parametrize("mode", [0, 1], ids=["full", "sampled"])
 @pytest.mark.parametrize("gdt", ["bf16", "f32", "none"])
 def test_ragged_rows_bf16(P, oracle, V, ld, mode, gdt):
-    """bf16 rows that start anywhere in a 16-byte vector (stride no multiple of 8): the
-    helper alone (up to V = 8,192, rows shorter than a vector among them, down to V = 2: at
+    """bf16 rows that start anywhere in a 16-byte vector (stride no multiple of 8): one CTA
+    a row (up to V = 8,192, rows shorter than a vector among them, down to V = 2: at
     V = 1 every l is 0 and a relative bound on the total loss is void), clusters of 2
     (27,187 and 32,007), of 3 (50,001) and of 8.  The logits end with the last row's last
     column: NaN behind it must not enter a result.  In sampled mode y is pushed into the
@@ -453,7 +453,7 @@ def test_ragged_rows_dense_neighbours_untouched(P, oracle):
 
 
 @pytest.mark.parametrize("n_sup", [1, 5])
-def test_split_kernel_fewer_rows_than_clusters(P, oracle, n_sup):
+def test_fp32_fewer_rows_than_clusters(P, oracle, n_sup):
     """fp32 rows at the full vocabulary with fewer rows than clusters: most clusters
     have no row and leave at once."""
     T = 40
@@ -525,6 +525,69 @@ def test_cluster_matches_portable(P, oracle):
     assert ((t0 - t1).abs() <= 2e-4 * t0.abs().clamp(min=1)).all()
     rowmax = g0.abs().amax(dim=1, keepdim=True)
     assert ((g0 - g1).abs() <= 2e-4 * rowmax).all()
+
+
+# Rows that no cluster holds: fp32 above 152,640 columns in k_row_split and k_split_helper where
+# they are whole vectors, the other fp32 ones and bf16 above 305,280 in k_row_helper alone.
+
+@pytest.mark.parametrize("V", [152644, 160004])
+@pytest.mark.parametrize("mode", [0, 1], ids=["full", "sampled"])
+@pytest.mark.parametrize("gdt", ["bf16", "f32"])
+def test_split_rows_ragged_last_chunk(P, oracle, V, mode, gdt):
+    """A last chunk and a last slice that are not full, on several rows to a cluster."""
+    b = W.packed(seed=11, num_traj=2, traj_len=192)
+    zs, zt = W.make_logits(b.num_valid, V, "agent", torch.float32, seed=12, device="cuda")
+    run_chain(P, oracle, b, V, zs, zt, mode=mode, alpha=0.5, compact=True,
+              grad_dtype=torch.bfloat16 if gdt == "bf16" else torch.float32)
+
+
+@pytest.mark.parametrize("n_sup", [1, 5])
+def test_split_rows_fewer_than_clusters(P, oracle, n_sup):
+    T, V = 40, 160004
+    turn_id = np.full(T, -1, np.int32)
+    mask = np.zeros(T, np.uint8)
+    idx = np.linspace(3, T - 2, n_sup).astype(int)
+    mask[idx] = 1
+    turn_id[idx] = np.arange(n_sup) % 3
+    b = W.Batch("few", turn_id, mask, np.array([0, T], np.int64), 3)
+    zs, zt = W.make_logits(b.num_valid, V, "agent", torch.float32, seed=60 + n_sup, device="cuda")
+    for mode in (0, 1):
+        run_chain(P, oracle, b, V, zs, zt, mode=mode, alpha=0.5, compact=True, grad_dtype=torch.float32)
+
+
+def test_split_rows_deterministic(P, oracle):
+    """Two calls on the same inputs give the same bits."""
+    b = W.packed(seed=1, num_traj=2, traj_len=512)
+    V = 160004
+    zs, zt = W.make_logits(b.num_valid, V, "agent", torch.float32, seed=1, device="cuda")
+    outs = []
+    for _ in range(2):
+        step = make_step(P, b, V, compact=True)
+        grad = torch.empty_like(zs)
+        step.run(zs, zt, grad)
+        torch.cuda.synchronize()
+        outs.append((grad, step.token_loss.clone(), step.loss.item()))
+    assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1])
+    assert outs[0][2] == outs[1][2]
+
+
+@pytest.mark.parametrize("idt,V,ld", [("bf16", 305288, 305288), ("bf16", 305289, 305296), ("bf16", 305289, 305289),
+                                      ("f32", 152645, 152645), ("f32", 152645, 152648)])
+@pytest.mark.parametrize("mode", [0, 1], ids=["full", "sampled"])
+def test_helper_alone(P, oracle, idt, V, ld, mode):
+    """Every row on k_row_helper's register path, whole, with a partial last vector and of any
+    stride; NaN behind the last row's last column."""
+    b = W.packed(seed=13, num_traj=1, traj_len=300)
+    R = b.num_valid
+    dt = torch.bfloat16 if idt == "bf16" else torch.float32
+    z = []
+    for src in W.make_logits(R, V, "agent", dt, seed=14, device="cuda"):
+        buf = torch.full((R * ld + 64,), float("nan"), dtype=dt, device="cuda")
+        z.append(buf[:R * ld].view(R, ld))
+        z[-1][:, :V] = src
+    for gdt in (torch.bfloat16, torch.float32):
+        _, grad = run_chain(P, oracle, b, V, *z, mode=mode, alpha=0.5, compact=True, grad_dtype=gdt, seed_y=15)
+        assert (grad[:, V:].float() == 7.0).all()
 
 
 # ---------------------------------------------------------------- full vocabulary, sampled rows
@@ -709,7 +772,7 @@ def test_padding_never_read(P, oracle):
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])
 def test_deterministic(P, oracle, dtype):
     """Two calls on the same inputs give the same bits (fixed merge orders in the
-    cluster kernel and helper grid for bf16, in the split-row clusters for fp32)."""
+    cluster kernel, of 8 CTAs for bf16 and 16 for fp32, and in the helper grid)."""
     b = W.packed(seed=1, num_traj=4, traj_len=2048)
     V = FULL_V
     zs, zt = W.make_logits(b.num_valid, V, "agent", torch.bfloat16 if dtype == "bf16" else torch.float32,
