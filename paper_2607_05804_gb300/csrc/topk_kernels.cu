@@ -1480,7 +1480,10 @@ cudaError_t launch_topk(const TopkCall &c, cudaStream_t stream)
     const size_t esz = bf16 ? 2 : 4;
     const bool aligned = ((reinterpret_cast<uintptr_t>(c.zt) | reinterpret_cast<uintptr_t>(c.zs) | (uintptr_t)(c.ld * esz)) & 15u) == 0;
     if (span <= (int64_t)kShortPerThread * 512 && (!aligned || c.vocab <= short_max_vocab(c.K))) {
-        const int s4 = span <= kShortPerThread * 32 ? 0 : span <= kShortPerThread * 128 ? 1 : span <= kShortPerThread * 256 ? 2 : 3;
+        // one warp a row where many rows hide its latency; a few rows of K above 128 finish sooner on four
+        // (up to 200 rows of 1,024 ids, K = 256, bf16: 37 us, 27 streamed, now 27)
+        const bool one_warp = span <= kShortPerThread * 32 && (c.K <= 128 || c.T > (int64_t)sms * 8);
+        const int s4 = one_warp ? 0 : span <= kShortPerThread * 128 ? 1 : span <= kShortPerThread * 256 ? 2 : 3;
         static const Kern shorts[2][2][4] = {
             {{k_topk_short<false, 32, false>, k_topk_short<false, 128, false>, k_topk_short<false, 256, false>,
               k_topk_short<false, 512, false>},
