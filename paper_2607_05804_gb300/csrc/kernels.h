@@ -89,7 +89,7 @@ struct RowIn {
     const int32_t *nvalid;
     int32_t *status;
     // split_den > 0: the cluster kernel takes rows [0, nvalid split_num / split_den) of the
-    // row list and the helper kernel the rest (set by launch_row_cluster)
+    // row list and the helper kernel the rest (set where the two are launched)
     int32_t split_num, split_den;
     int32_t split_ctas;  // CTAs of the helper grid (held-row kernels: its share comes in whole turns)
     int64_t elems;  // logits from the arrays' start to the last row's last column

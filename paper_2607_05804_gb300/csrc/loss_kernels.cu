@@ -224,7 +224,7 @@ k_row_portable(RowIn p)
         Teacher t = teacher_empty();
         // a sampled-token row leaves y out of the student statistics (add_sampled_term
         // brings its term back at the merge): in a vector its logit reads as the lowest
-        // finite value (never the maximum beside the other N - 1, adds 0); read alone
+        // finite value, which adds 0; read alone
         // it folds into the teacher only
         const int64_t ys = p.mode == TURNOPD_SAMPLED_TOKEN ? (int64_t)meta.z : -1;
         if (VEC) {

@@ -139,7 +139,7 @@ __device__ __forceinline__ void accumulate_teacher(Teacher &t, float b)
 
 // Sampled-token row (Eq. opd-rkl's one-token estimator): the student statistics leave y
 // out altogether -- within a vector of finite logits its logit is replaced by the
-// lowest finite value, which is then never the maximum and adds 0 to every sum; a y
+// lowest finite value, which adds 0 to every sum (scale_of), whatever the maximum; a y
 // read alone folds into the teacher only -- so s holds S' = sum_{v != y} exp(z_s - m')
 // at the maximum m' of the other logits.  This adds y's own term at M = max(m', z_y):
 // S = S' e^{m' - M} + e^{z_y - M}, and returns 1 - p_y = S' e^{m' - M} / S, which

@@ -804,8 +804,11 @@ constexpr int kHelpU = 4;  // vectors of each model per thread and batch
 // cp.async, kHelpStages - 1 batches ahead (each thread copies and reads only its own
 // slots): twice the loads in flight of the register path, with no registers held by
 // them.  The helper beside the clusters takes it (packed 8 x 4096, V = 151,936: 2.776 ->
-// 2.743 ms per loss call with the split rate raised to 0.7); the helper alone on every
-// SM keeps the register path (V = 16,384: 0.405 against 0.433 ms).
+// 2.743 ms per loss call with the split rate raised to 0.7).  The helper alone, which
+// takes rows that no cluster holds, has the register path, from when short rows took it
+// (V = 16,384: 0.405 against 0.433 ms); at its present lengths the ring would be faster
+// with a gradient (us at 6e8 bf16 logits, registers and ring: V = 400,000 908 and 874,
+// sampled 820 and 744, forward 427 and 389; fp32 forward at 200,001 382 and 416).
 constexpr int kHelpStages = 3;
 constexpr size_t kHelperSmem = (size_t)kHelpStages * 2 * kHelpU * kHelpThreads * 16;  // AS
 

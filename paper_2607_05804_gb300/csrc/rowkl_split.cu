@@ -129,7 +129,7 @@ __device__ __forceinline__ float lane4(const float4 &v, int i)
     return i == 0 ? v.x : (i == 1 ? v.y : (i == 2 ? v.z : v.w));
 }
 
-// v with lane i replaced by the lowest finite float (never a maximum, adds 0)
+// v with lane i replaced by the lowest finite float (adds 0)
 __device__ __forceinline__ float4 fill_lane4(float4 v, int i)
 {
     v.x = i == 0 ? -FLT_MAX : v.x;
@@ -617,7 +617,7 @@ __global__ void __launch_bounds__(NTH, 1) k_split_helper(RowIn p)
                     a[u] = hring4[slot(bi % kSplitHelpStages, 0, u)];
                     b[u] = hring4[slot(bi % kSplitHelpStages, 1, u)];
                 } else {
-                    a[u] = b[u] = kFill4;  // adds 0, never the maximum
+                    a[u] = b[u] = kFill4;  // adds 0
                 }
             }
             // a sampled-token row leaves y out of the student statistics (lowest finite

@@ -89,7 +89,7 @@ __device__ __forceinline__ void fold_row(const TIn *rs, const TIn *rt, int64_t V
 __device__ __forceinline__ void fold_row_bf16(const uint4 *vs, const uint4 *vt, int64_t nvec, Student &s,
                                               Teacher &t)
 {
-    constexpr uint32_t kFill = 0xff7fff7fu;  // lowest finite bf16 pair: adds 0, never the max
+    constexpr uint32_t kFill = 0xff7fff7fu;  // lowest finite bf16 pair: adds 0
     const float2 L2 = splat(kLog2e);
     float ms = -INFINITY, mt = -INFINITY, dd = 0.f;
     float2 S2 = make_float2(0.f, 0.f), A2 = S2, T2 = S2;
